@@ -5,7 +5,11 @@
 // and ||b||).
 #include "rtproj_internal.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
+
+namespace cg = cooperative_groups;
 
 namespace rtp {
 namespace {
@@ -108,19 +112,39 @@ __global__ void sqrt_sum_kernel(const double* part, int nparts, double* out) {
     if (threadIdx.x == 0) *out = sqrt(s);
 }
 
-// One CTA per row.
-__global__ void row_norms_kernel(const double* __restrict__ X, int64_t ldx, int n, double* out) {
-    __shared__ double red[BT / 32];
-    const double* row = X + (int64_t)blockIdx.x * ldx;
-    double s0 = 0.0, s1 = 0.0;
-    int c = threadIdx.x;
-    for (; c + BT < n; c += 2 * BT) {
-        s0 = fma(row[c], row[c], s0);
-        s1 = fma(row[c + BT], row[c + BT], s1);
+// A cluster of CTAs per row: each CTA sums a contiguous part, the first adds the parts in
+// order through distributed shared memory (deterministic). One 256-thread CTA per row left
+// most SMs idle and each of them latency-bound: 137 us for one row of 300,000 and 33 us for 64
+// rows of 65,536, against 5 us for the bytes of the latter.
+constexpr int RN_T = 512;
+__global__ void __launch_bounds__(RN_T) row_norms_kernel(const double* __restrict__ X, int64_t ldx, int n, double* out) {
+    __shared__ double red[RN_T / 32];
+    __shared__ double mine;
+    cg::cluster_group cl = cg::this_cluster();
+    const int parts = (int)cl.num_blocks(), q = (int)cl.block_rank();
+    const int j = blockIdx.x / parts;
+    const double* row = X + (int64_t)j * ldx;
+    const int per = (n + parts - 1) / parts;
+    const int64_t e = min((int64_t)n, (int64_t)(q + 1) * per);
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    int64_t c = (int64_t)q * per + threadIdx.x;
+    for (; c + 3 * RN_T < e; c += 4 * RN_T) {
+        const double a0 = row[c], a1 = row[c + RN_T], a2 = row[c + 2 * RN_T], a3 = row[c + 3 * RN_T];
+        s0 = fma(a0, a0, s0);
+        s1 = fma(a1, a1, s1);
+        s2 = fma(a2, a2, s2);
+        s3 = fma(a3, a3, s3);
     }
-    if (c < n) s0 = fma(row[c], row[c], s0);
-    const double s = block_sum(s0 + s1, red);
-    if (threadIdx.x == 0) out[blockIdx.x] = sqrt(s);
+    for (; c < e; c += RN_T) s0 = fma(row[c], row[c], s0);
+    const double s = block_sum((s0 + s1) + (s2 + s3), red);
+    if (threadIdx.x == 0) mine = s;
+    cl.sync();
+    if (q == 0 && threadIdx.x == 0) {
+        double t = 0.0;
+        for (int r = 0; r < parts; ++r) t += *cl.map_shared_rank(&mine, r);
+        out[j] = sqrt(t);
+    }
+    cl.sync();   // a CTA's partial sum stays readable until the first has added it
 }
 
 __device__ __forceinline__ void max_bits(unsigned long long* p, double v) {
@@ -223,7 +247,22 @@ cudaError_t frobenius(const double* X, int64_t ldx, int rows, int cols, double* 
 
 cudaError_t row_norms(const double* X, int64_t ldx, int k, int n, double* out, cudaStream_t s) {
     if (k <= 0) return cudaSuccess;
-    row_norms_kernel<<<k, BT, 0, s>>>(X, ldx, n, out);
+    // CTAs per row: enough for about two per SM, each with at least two passes of its threads
+    int parts = 1;
+    while (parts < 8 && (int64_t)k * parts < 2 * sm_count() && n / (2 * parts) >= 2 * RN_T) parts *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(k * parts));
+    cfg.blockDim = dim3(RN_T);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)parts;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, row_norms_kernel, X, ldx, n, out);
+    if (e != cudaSuccess) return e;
     note_launch();
     return cudaGetLastError();
 }

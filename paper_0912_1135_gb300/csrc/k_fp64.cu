@@ -276,16 +276,18 @@ cudaError_t check_finite(const double* X, int64_t rs, int rows, int cols, int* s
 // ---------------------------------------------------------------------------------
 // Narrow products C (M x N) = A (M x K) B (K x N) with M <= 64 (the rows of a low-rank
 // factor) and a long K: the 64 x 64 tiles of gemm64 would waste most of their rows. The K
-// range is cut into chunks; a CTA takes one chunk and a range of columns j and keeps NR
-// rows' partial sums per column in registers, reading A's chunk from shared memory. B is
-// read with the columns j contiguous (one thread per column), or with K contiguous (a warp
-// per column, lanes over k), or generated (G of Eq. 12). The chunks' partial sums are
-// added in chunk order by a second kernel (deterministic).
+// range is cut into chunks; a CTA takes one chunk and a range of columns j and keeps up to
+// 16 rows' partial sums per column in registers (a multiple of 4 rows: a padded row costs a
+// full FP64 instruction), reading A's chunk from shared memory. B is read with the columns j
+// contiguous (one thread per column; with fewer than 129 columns the CTA's threads also split
+// the chunk's K among them), or with K contiguous (a warp per column, lanes over k), or
+// generated (G of Eq. 12). The chunks' partial sums are added in chunk order by a second
+// kernel (deterministic).
 // ---------------------------------------------------------------------------------
 namespace {
 
-constexpr int NR_ROWS = 16;     // rows per register pass
-constexpr int NR_KC = 64;       // K entries of A staged per pass
+constexpr int NR_ROWS = 16;     // most rows of one register pass
+constexpr int NR_KC = 128;      // K entries of A staged per pass
 constexpr int NR_T = 256;
 
 struct NarrowDev {
@@ -320,55 +322,76 @@ __device__ __forceinline__ void narrow_b4(const NarrowDev& p, int k0, int ke, in
     }
 }
 
-// one thread per column j; rows [r0, r0 + NR_ROWS) of A; chunk blockIdx.y
-__global__ void __launch_bounds__(NR_T) narrow_rows_kernel(NarrowDev p) {
-    __shared__ double As[NR_ROWS][NR_KC];
-    const int j = blockIdx.x * NR_T + threadIdx.x;
+// NL = 2^jl threads side by side take NL columns j; the NR_T / NL groups of them take turns at
+// four K entries each, and their sums are added through shared memory. Rows [r0, r0 + NR) of A
+// per pass; chunk blockIdx.y.
+template <int NR>
+__global__ void __launch_bounds__(NR_T) narrow_rows_kernel(NarrowDev p, int jl) {
+    __shared__ double As[NR][NR_KC];
+    __shared__ double red[NR][NR_T];
+    const int nl = 1 << jl, groups = NR_T >> jl;
+    const int jj = threadIdx.x & (nl - 1), grp = threadIdx.x >> jl;
+    const int j = blockIdx.x * nl + jj;
     const int kb = blockIdx.y * p.kchunk, ke = min(p.K, kb + p.kchunk);
-    for (int r0 = 0; r0 < p.M; r0 += NR_ROWS) {
-        double acc[NR_ROWS];
+    for (int r0 = 0; r0 < p.M; r0 += NR) {
+        double acc[NR];
 #pragma unroll
-        for (int i = 0; i < NR_ROWS; ++i) acc[i] = 0.0;
+        for (int i = 0; i < NR; ++i) acc[i] = 0.0;
         for (int k0 = kb; k0 < ke; k0 += NR_KC) {
             __syncthreads();
-            for (int e = threadIdx.x; e < NR_ROWS * NR_KC; e += NR_T) {
+            for (int e = threadIdx.x; e < NR * NR_KC; e += NR_T) {
                 const int i = e / NR_KC, k = k0 + e % NR_KC;
                 As[i][e % NR_KC] = (r0 + i < p.M && k < ke) ? p.A[(int64_t)(r0 + i) * p.a_rs + k] : 0.0;
             }
             __syncthreads();
             if (j < p.N) {
                 const int kn = min(NR_KC, ke - k0);
-                for (int kk = 0; kk < kn; kk += 4) {
+                for (int kk = 4 * grp; kk < kn; kk += 4 * groups) {
                     double b[4];
                     narrow_b4(p, k0 + kk, ke, j, b);
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
 #pragma unroll
-                        for (int i = 0; i < NR_ROWS; ++i) acc[i] = fma(As[i][kk + u], b[u], acc[i]);
+                        for (int i = 0; i < NR; ++i) acc[i] = fma(As[i][kk + u], b[u], acc[i]);
                 }
             }
         }
-        if (j < p.N) {
+        if (groups > 1) {
 #pragma unroll
-            for (int i = 0; i < NR_ROWS; ++i)
+            for (int i = 0; i < NR; ++i) red[i][threadIdx.x] = acc[i];
+            __syncthreads();
+            for (int e = threadIdx.x; e < NR * nl; e += NR_T) {
+                const int i = e >> jl, q = e & (nl - 1);
+                const int jq = blockIdx.x * nl + q;
+                if (r0 + i < p.M && jq < p.N) {
+                    double t = 0.0;
+                    for (int g = 0; g < groups; ++g) t += red[i][(g << jl) + q];
+                    p.part[((int64_t)blockIdx.y * p.M + r0 + i) * p.N + jq] = t;
+                }
+            }
+            __syncthreads();
+        } else if (j < p.N) {
+#pragma unroll
+            for (int i = 0; i < NR; ++i)
                 if (r0 + i < p.M) p.part[((int64_t)blockIdx.y * p.M + r0 + i) * p.N + j] = acc[i];
         }
     }
 }
 
 // one warp per column j, lanes over k (B with K contiguous: b_rs == 1)
+template <int NR>
 __global__ void __launch_bounds__(NR_T) narrow_cols_kernel(NarrowDev p) {
-    __shared__ double As[NR_ROWS][NR_KC];
+    __shared__ double As[NR][NR_KC];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int j = blockIdx.x * (NR_T / 32) + warp;
     const int kb = blockIdx.y * p.kchunk, ke = min(p.K, kb + p.kchunk);
-    for (int r0 = 0; r0 < p.M; r0 += NR_ROWS) {
-        double acc[NR_ROWS];
+    for (int r0 = 0; r0 < p.M; r0 += NR) {
+        double acc[NR];
 #pragma unroll
-        for (int i = 0; i < NR_ROWS; ++i) acc[i] = 0.0;
+        for (int i = 0; i < NR; ++i) acc[i] = 0.0;
         for (int k0 = kb; k0 < ke; k0 += NR_KC) {
             __syncthreads();
-            for (int e = threadIdx.x; e < NR_ROWS * NR_KC; e += NR_T) {
+            for (int e = threadIdx.x; e < NR * NR_KC; e += NR_T) {
                 const int i = e / NR_KC, k = k0 + e % NR_KC;
                 As[i][e % NR_KC] = (r0 + i < p.M && k < ke) ? p.A[(int64_t)(r0 + i) * p.a_rs + k] : 0.0;
             }
@@ -377,17 +400,23 @@ __global__ void __launch_bounds__(NR_T) narrow_cols_kernel(NarrowDev p) {
                 for (int kk = lane; kk < NR_KC && k0 + kk < ke; kk += 32) {
                     const double b = p.B[(int64_t)(k0 + kk) + (int64_t)j * p.b_cs];
 #pragma unroll
-                    for (int i = 0; i < NR_ROWS; ++i) acc[i] = fma(As[i][kk], b, acc[i]);
+                    for (int i = 0; i < NR; ++i) acc[i] = fma(As[i][kk], b, acc[i]);
                 }
         }
 #pragma unroll
-        for (int i = 0; i < NR_ROWS; ++i) acc[i] = narrow_warp_sum(acc[i]);
+        for (int i = 0; i < NR; ++i) acc[i] = narrow_warp_sum(acc[i]);
         if (j < p.N && lane == 0) {
 #pragma unroll
-            for (int i = 0; i < NR_ROWS; ++i)
+            for (int i = 0; i < NR; ++i)
                 if (r0 + i < p.M) p.part[((int64_t)blockIdx.y * p.M + r0 + i) * p.N + j] = acc[i];
         }
     }
+}
+
+template <int NR>
+void launch_narrow(const NarrowDev& p, bool cols, int jl, dim3 grid, cudaStream_t s) {
+    if (cols) narrow_cols_kernel<NR><<<grid, NR_T, 0, s>>>(p);
+    else narrow_rows_kernel<NR><<<grid, NR_T, 0, s>>>(p, jl);
 }
 
 __global__ void narrow_reduce_kernel(const double* part, int chunks, int M, int N, double* C, int64_t c_rs) {
@@ -405,7 +434,9 @@ cudaError_t gemm64_narrow(const Narrow64& g, double* part, size_t part_elems, cu
     if (g.M <= 0 || g.N <= 0) return cudaSuccess;
     if (g.M > 64 || g.K <= 0) return cudaErrorInvalidValue;
     const bool cols = g.omega_dist < 0 && g.b_rs == 1;
-    const int per_block = cols ? NR_T / 32 : NR_T;
+    int jl = 3;                             // threads per row of columns: 8 .. 256
+    while (jl < 8 && (1 << jl) < g.N) ++jl;
+    const int per_block = cols ? NR_T / 32 : 1 << jl;
     const int gx = (g.N + per_block - 1) / per_block;
     // chunks: about four CTAs per SM in all, each chunk a multiple of 16 (whole Philox blocks)
     const int want = std::max(1, 4 * sm_count() / gx);
@@ -423,8 +454,11 @@ cudaError_t gemm64_narrow(const Narrow64& g, double* part, size_t part_elems, cu
     p.key0 = (uint32_t)(g.seed & 0xFFFFFFFFull); p.key1 = (uint32_t)(g.seed >> 32);
     p.part = part;
     const dim3 grid((unsigned)gx, (unsigned)chunks);
-    if (cols) narrow_cols_kernel<<<grid, NR_T, 0, s>>>(p);
-    else narrow_rows_kernel<<<grid, NR_T, 0, s>>>(p);
+    const int nr = std::min(NR_ROWS, (g.M + 3) / 4 * 4);
+    if (nr <= 4) launch_narrow<4>(p, cols, jl, grid, s);
+    else if (nr <= 8) launch_narrow<8>(p, cols, jl, grid, s);
+    else if (nr <= 12) launch_narrow<12>(p, cols, jl, grid, s);
+    else launch_narrow<16>(p, cols, jl, grid, s);
     const int64_t total = (int64_t)g.M * g.N;
     narrow_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(part, chunks, g.M, g.N, g.C, g.c_rs);
     note_launch(2);

@@ -10,11 +10,12 @@
 //     E = A D                 (m x m) one CTA per row of A
 //     X = R^{-*} Pi E         one float64 product with the triangular R^{-*}
 //   apply (the seven steps) and its refinement (Remark 4.3) with every product with A or
-//   A^* summed in double-double and rounded once: c = A b, s = b - A^* h, r = A s,
-//   s <- s - A^* dh. The sparse part of each of these is exact to double-double rounding,
-//   so the refinement converges to the projection of the stored matrix; the low-rank
-//   part (V b, U^* h and their products with U, V) is float64.
+//   A^* summed from exact products in 128-bit integers and rounded once: c = A b,
+//   s = b - A^* h, r = A s, s <- s - A^* dh. The sparse part of each of these is exact to
+//   about 2^-105 of its largest term, so the refinement converges to the projection of the
+//   stored matrix; the low-rank part's inner products (V b, U^* h) are float64.
 #include "rtproj_internal.cuh"
+#include "i128.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -33,23 +34,12 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
     } while (0)
 
 // ---------------------------------------------------------------------------------
-// Double-double building blocks: Knuth's TwoSum and the fma form of TwoProduct.
+// Double-double building block: Knuth's TwoSum.
 // ---------------------------------------------------------------------------------
 __device__ __forceinline__ void two_sum_d(double a, double b, double& s, double& e) {
     s = a + b;
     const double bb = s - a;
     e = (a - (s - bb)) + (b - bb);
-}
-
-// (hi, lo) += a b to double-double accuracy
-__device__ __forceinline__ void dd_fma_acc(double& hi, double& lo, double a, double b) {
-    const double p = a * b;
-    const double pe = fma(a, b, -p);
-    double s, e;
-    two_sum_d(hi, p, s, e);
-    e += lo + pe;
-    hi = s + e;
-    lo = e - (hi - s);
 }
 
 __device__ __forceinline__ void dd_add(double& hi, double& lo, double bh, double bl) {
@@ -58,15 +48,6 @@ __device__ __forceinline__ void dd_add(double& hi, double& lo, double bh, double
     e += lo + bl;
     hi = s + e;
     lo = e - (hi - s);
-}
-
-__device__ __forceinline__ void dd_warp_sum(double& hi, double& lo) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double oh = __shfl_xor_sync(0xffffffffu, hi, o);
-        const double ol = __shfl_xor_sync(0xffffffffu, lo, o);
-        dd_add(hi, lo, oh, ol);
-    }
 }
 
 // ---------------------------------------------------------------------------------
@@ -323,28 +304,104 @@ __global__ void sparse_e_kernel(const int64_t* __restrict__ rptr, const int32_t*
 }
 
 // ---------------------------------------------------------------------------------
-// Products of the apply, in double-double.
+// Products of the apply: exact products summed in 128-bit integers (i128.cuh).
+//
+// The right-hand sides are kept as an n x k block (row c holds entry c of every vector), so
+// that a nonzero's gather reads k consecutive doubles. A warp is cut into groups of
+// 2^LG lanes, one lane per right-hand side: 32 lanes from k = 17 up, fewer below, when the
+// groups take different nonzeros (A x) or columns (A^* h). Bound: the integer pipes, about 60
+// instructions per nonzero and right-hand side; the double-double form on the FP64 pipe took
+// 832 cycles per warp of them, and gathered one double per 32-byte sector. An apply of 100
+// vectors with two refinement passes at 1000 x 300,000, 1.5e6 nonzeros: 40.6 -> 5.7 ms.
 // ---------------------------------------------------------------------------------
 // Rows are cut into chunks of at most SP_CHUNK nonzeros (a table built at create), so that
-// a few long rows still spread over many warps. part(c, j) = the double-double sum over
-// chunk c of val x_j[col]: one warp per (chunk, right-hand side j).
+// a few long rows still spread over many warps, and no sum exceeds the 128 bits' capacity.
 constexpr int SP_CHUNK = 2048;
+static_assert(SP_CHUNK <= I128_MAX_TERMS, "a chunk's sum must fit 128 bits");
+constexpr int SP_WARPS = 8;
 
-__global__ void spmv_chunk_kernel(const int32_t* __restrict__ crow_of, const int64_t* __restrict__ cbeg,
-                                  const int64_t* __restrict__ rptr, const int32_t* __restrict__ col,
-                                  const double* __restrict__ val, const double* __restrict__ X, int64_t ldx,
-                                  int nchunks, int k, double2* __restrict__ part) {
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (wid >= (int64_t)nchunks * k) return;
-    const int c = (int)(wid / k), j = (int)(wid % k);
+__device__ __forceinline__ void ldg_words(const double* p, uint32_t& lo, uint32_t& hi) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    lo = u.x;
+    hi = u.y;
+}
+
+__device__ __forceinline__ i128acc i128_shfl_xor(const i128acc& a, int o) {
+    return {__shfl_xor_sync(0xffffffffu, a.w0, o), __shfl_xor_sync(0xffffffffu, a.w1, o),
+            __shfl_xor_sync(0xffffffffu, a.w2, o), __shfl_xor_sync(0xffffffffu, a.w3, o),
+            __shfl_xor_sync(0xffffffffu, a.E, o)};
+}
+
+// part(c, j) = the sum over chunk c of val x_j[col], as an unevaluated pair of doubles: one
+// warp per (chunk, 2^LG right-hand sides), X n x k (ld ldx). 32 nonzeros are decoded at a time
+// (one per lane) into shared memory, from which every group reads the ones it takes; four
+// gathers are in flight per lane.
+template <int LG>
+__global__ void __launch_bounds__(32 * SP_WARPS)
+    spmv_chunk_kernel(const int32_t* __restrict__ crow_of, const int64_t* __restrict__ cbeg,
+                      const int64_t* __restrict__ rptr, const int32_t* __restrict__ col,
+                      const double* __restrict__ val, const double* __restrict__ X, int64_t ldx, int nchunks, int k,
+                      double2* __restrict__ part) {
+    constexpr int KL = 1 << LG, SUB = 32 / KL, UN = 4;
+    __shared__ uint4 entries[SP_WARPS][32];      // left factor: low word, high word | sign, exponent, column
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int jb = (k + KL - 1) / KL;
+    const int64_t wid = (int64_t)blockIdx.x * SP_WARPS + warp;
+    if (wid >= (int64_t)nchunks * jb) return;
+    const int c = (int)(wid / jb), j = (int)(wid % jb) * KL + (lane & (KL - 1)), g = lane >> LG;
+    const bool live = j < k;
+    const double* x = X + (live ? j : 0);
     const int64_t b = cbeg[c];
     const int64_t e = min(b + (int64_t)SP_CHUNK, rptr[crow_of[c] + 1]);
-    const double* x = X + (int64_t)j * ldx;
-    double hi = 0.0, lo = 0.0;
-    for (int64_t p = b + lane; p < e; p += 32) dd_fma_acc(hi, lo, val[p], x[col[p]]);
-    dd_warp_sum(hi, lo);
-    if (lane == 0) part[(int64_t)c * k + j] = make_double2(hi, lo);
+    uint4* ent = entries[warp];
+    i128acc acc = i128_zero();
+    bool bad = false;
+    for (int64_t p0 = b; p0 < e; p0 += 32) {
+        uint4 w = make_uint4(0u, 0u, (uint32_t)(I128_E_EMPTY / 2), 0u);   // past the end: a zero
+        if (p0 + lane < e) {
+            uint32_t lo, hi;
+            ldg_words(val + p0 + lane, lo, hi);
+            const i128op o = i128_left(i128_decode(lo, hi));
+            w = make_uint4(o.lo, o.hi | (o.neg & 0x80000000u), (uint32_t)o.e, (uint32_t)col[p0 + lane]);
+        }
+        __syncwarp();
+        ent[lane] = w;
+        __syncwarp();
+        const int steps = ((int)min((int64_t)32, e - p0) + SUB - 1) / SUB;
+        for (int t0 = 0; t0 < steps; t0 += UN) {
+            uint32_t xl[UN], xh[UN];
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                const int at = (t0 + u) * SUB + g;
+                ldg_words(x + (int64_t)ent[at & 31].w * ldx, xl[u], xh[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                const int at = (t0 + u) * SUB + g;
+                if (at >= 32) break;             // the same for every group of the warp
+                const uint4 v = ent[at];
+                i128op a;
+                a.lo = v.x;
+                a.hi = v.y & 0x7FFFFFFFu;
+                a.e = (int)v.z;
+                a.neg = (uint32_t)((int32_t)v.y >> 31);
+                bad |= !i128_finite(xh[u]) && v.z != (uint32_t)(I128_E_EMPTY / 2);
+                i128_mac(acc, a, i128_decode(xl[u], xh[u]));
+            }
+        }
+    }
+    int any_bad = bad ? 1 : 0;
+#pragma unroll
+    for (int o = KL; o < 32; o <<= 1) {
+        i128_merge(acc, i128_shfl_xor(acc, o));
+        any_bad |= __shfl_xor_sync(0xffffffffu, any_bad, o);
+    }
+    if (g == 0 && live) {
+        double hi, lo;
+        i128_to_pair(acc, hi, lo);
+        if (any_bad) hi = __longlong_as_double(0x7FF8000000000000ll);   // an infinity or NaN among the x
+        part[(int64_t)c * k + j] = make_double2(hi, lo);
+    }
 }
 
 // out(i, j) (m x k, ld k) = (A x_j)_i: the chunks of row i added in order in double-double,
@@ -368,25 +425,87 @@ __global__ void spmv_rows_kernel(const int32_t* __restrict__ rchunk, const doubl
     out[idx] = hi + lo;
 }
 
-// out(j, c) = Y(j, c) - (A^* h_j)_c for h (m x k, ld k), rounded once from double-double:
-// one thread per (j, c). The low-rank part adds sum_q V(q, c) (U^* h)(q, j) as one float64
-// sum. out may be Y.
-__global__ void spmvT_dd_kernel(const int64_t* __restrict__ cptr, const int32_t* __restrict__ crow,
-                                const double* __restrict__ cval, const double* __restrict__ H, int k, int n, int r,
-                                const double* __restrict__ V, const double* __restrict__ UtH, const double* Y,
-                                int64_t ldy, double* out, int64_t ldo) {
-    const int j = blockIdx.y;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-        double hi = 0.0, lo = 0.0;
-        for (int64_t p = cptr[c]; p < cptr[c + 1]; ++p) dd_fma_acc(hi, lo, cval[p], H[(int64_t)crow[p] * k + j]);
-        if (r > 0) {
-            double t = 0.0;
-            for (int q = 0; q < r; ++q) t = fma(V[(int64_t)q * n + c], UtH[(int64_t)q * k + j], t);
-            dd_add(hi, lo, t, 0.0);
+// out(c, j) = Y(c, j) - (A^* h_j)_c for h (m x k, ld k), rounded once: a group of 2^LG lanes
+// per column c, JB right-hand sides per lane. The low-rank part subtracts
+// sum_q V(q, c) (U^* h)(q, j) the same way. out may be Y. Y and out: n x k (ld ldy, ldo).
+template <int LG, int JB>
+__global__ void __launch_bounds__(32 * SP_WARPS)
+    spmvT_kernel(const int64_t* __restrict__ cptr, const int32_t* __restrict__ crow, const double* __restrict__ cval,
+                 const double* __restrict__ H, int k, int n, int r, const double* __restrict__ V,
+                 const double* __restrict__ UtH, const double* Y, int64_t ldy, double* out, int64_t ldo) {
+    constexpr int KL = 1 << LG, SUB = 32 / KL;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j0 = blockIdx.y * (KL * JB) + (lane & (KL - 1));
+    const int64_t step = (int64_t)gridDim.x * SP_WARPS * SUB;
+    for (int64_t c = ((int64_t)blockIdx.x * SP_WARPS + warp) * SUB + (lane >> LG); c < n; c += step) {
+        i128acc acc[JB];
+        bool bad[JB];
+        const i128op one = i128_left(i128_decode(0u, 0x3FF00000u));
+#pragma unroll
+        for (int q = 0; q < JB; ++q) {
+            acc[q] = i128_zero();
+            bad[q] = false;
+            const int j = j0 + q * KL;
+            uint32_t lo = 0u, hi = 0u;
+            if (j < k) {
+                const double y = Y[c * ldy + j];
+                lo = (uint32_t)__double2loint(y);
+                hi = (uint32_t)__double2hiint(y);
+            }
+            bad[q] |= !i128_finite(hi);
+            i128_mac(acc[q], one, i128_decode(lo, hi));
         }
-        double z, e;
-        two_sum_d(Y[(int64_t)j * ldy + c], -hi, z, e);
-        out[(int64_t)j * ldo + c] = z + (e - lo);
+        int terms = 1;
+        auto term = [&](double v, const double* h) {
+            const i128op a = i128_left(i128_decode((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v)));
+            uint32_t lo[JB], hi[JB];
+#pragma unroll
+            for (int q = 0; q < JB; ++q) {
+                lo[q] = hi[q] = 0u;
+                if (j0 + q * KL < k) ldg_words(h + j0 + q * KL, lo[q], hi[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < JB; ++q) {
+                bad[q] |= !i128_finite(hi[q]);
+                i128_mac(acc[q], a, i128_decode(lo[q], hi[q]), ~0u);
+            }
+            if (++terms == I128_MAX_TERMS / 2) {   // room for as many more (a very long column)
+#pragma unroll
+                for (int q = 0; q < JB; ++q) {
+                    i128_sar(acc[q], 11);
+                    acc[q].E += 11;
+                }
+                terms = 0;
+            }
+        };
+        const int64_t pe = cptr[c + 1];
+        for (int64_t p = cptr[c]; p < pe; ++p) term(cval[p], H + (int64_t)crow[p] * k);
+        for (int q = 0; q < r; ++q) term(V[(int64_t)q * n + c], UtH + (int64_t)q * k);
+#pragma unroll
+        for (int q = 0; q < JB; ++q) {
+            const int j = j0 + q * KL;
+            if (j < k)
+                out[c * ldo + j] = bad[q] ? __longlong_as_double(0x7FF8000000000000ll) : i128_to_double(acc[q]);
+        }
+    }
+}
+
+// dst (k x n, ld ldd) = B - X or X for X n x k (ld k): 32 x 32 tiles through shared memory.
+__global__ void __launch_bounds__(256) finish_rows_kernel(const double* __restrict__ X, int n, int k,
+                                                          const double* __restrict__ B, int64_t ldb, double* dst,
+                                                          int64_t ldd) {
+    __shared__ double tile[32][33];
+    const int c0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int y = ty; y < 32; y += 8)
+        tile[y][tx] = (c0 + y < n && j0 + tx < k) ? X[(int64_t)(c0 + y) * k + j0 + tx] : 0.0;
+    __syncthreads();
+    for (int y = ty; y < 32; y += 8) {
+        const int j = j0 + y, c = c0 + tx;
+        if (j < k && c < n) {
+            const double v = tile[tx][y];
+            dst[(int64_t)j * ldd + c] = B ? B[(int64_t)j * ldb + c] - v : v;
+        }
     }
 }
 
@@ -402,7 +521,7 @@ unsigned grid_of(int64_t total, int threads) {
 int row_threads(int m) { return std::min(256, (m + 31) / 32 * 32); }
 
 // Low-rank helpers on the float64 GEMM: C (r x cols, ld ldc) = U^* Y for Y m x cols
-// (ld ldy), and C = V Y^* for Y cols x n (ld ldy).
+// (ld ldy), and C = V Y for Y n x k.
 cudaError_t ut_times(const rtproj_ctx* h, const double* Y, int64_t ldy, int cols, double* C, int64_t ldc) {
     Gemm64 g;
     g.M = h->lr; g.N = cols; g.K = (int)h->m;
@@ -412,11 +531,12 @@ cudaError_t ut_times(const rtproj_ctx* h, const double* Y, int64_t ldy, int cols
     return gemm64(g, h->part, h->part_elems, h->stream);
 }
 
-cudaError_t v_times_t(const rtproj_ctx* h, const double* Y, int64_t ldy, int cols, double* C, int64_t ldc) {
+// C (r x k, ld ldc) = V Y for Y n x k (ld k)
+cudaError_t v_times(const rtproj_ctx* h, const double* Y, int k, double* C, int64_t ldc) {
     Narrow64 g;
-    g.M = h->lr; g.N = cols; g.K = (int)h->n;
+    g.M = h->lr; g.N = k; g.K = (int)h->n;
     g.A = h->lrV; g.a_rs = h->n;
-    g.B = Y; g.b_rs = 1; g.b_cs = ldy;
+    g.B = Y; g.b_rs = k; g.b_cs = 1;
     g.C = C; g.c_rs = ldc;
     return gemm64_narrow(g, h->part, h->part_elems, h->stream);
 }
@@ -602,46 +722,82 @@ rtproj_status sparse_project(rtproj_ctx* h, const double* B, int64_t ldb, int k,
     const int m = (int)h->m, n = (int)h->n, r = h->lr;
     cudaStream_t s = h->stream;
     const int64_t mk = (int64_t)m * k;
-    const int64_t ck = (int64_t)h->nchunks * k;
-    const unsigned chunk_blocks = (unsigned)((ck * 32 + 255) / 256);
     double2* part = reinterpret_cast<double2*>(h->chunk_part);
-    const dim3 tgrid((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, sm_count() * 8 / k + 1)),
-                     (unsigned)k);
+    // lanes per right-hand side group: the smallest power of two that holds k, at most a warp
+    int lg = 0;
+    while (lg < 5 && (1 << lg) < k) ++lg;
+    const int kl = 1 << lg;
+    const int64_t warps_a = (int64_t)h->nchunks * ((k + kl - 1) / kl);
+    const unsigned grid_a = (unsigned)((warps_a + SP_WARPS - 1) / SP_WARPS);
+    const int jb = k > 64 ? 4 : k > 32 ? 2 : 1;          // right-hand sides per lane of A^* h
+    const int per_cta = SP_WARPS * (32 / kl);
+    const dim3 grid_t((unsigned)std::min<int64_t>((n + per_cta - 1) / per_cta, (int64_t)sm_count() * 32),
+                      (unsigned)((k + kl * jb - 1) / (kl * jb)));
     SP_CHECK(row_norms(B, ldb, k, n, h->bnorm, s));
     SP_CHECK(cudaMemsetAsync(h->stats, 0, 16, s));
-    auto apply_a = [&](const double* Xr, int64_t ldxr, double* out) -> rtproj_status {   // out = A x
+    // the vectors as an n x k block; one vector is already that
+    const double* Bt = B;
+    if (k > 1) {
+        SP_CHECK(store_transposed(B, ldb, k, n, h->sbuf, k, RTPROJ_F64, s));
+        Bt = h->sbuf;
+    }
+    auto apply_a = [&](const double* Xt, double* out) -> rtproj_status {   // out = A x
         phase_begin(h, RTPROJ_PHASE_APPLY_A);
-        if (r > 0) SP_CHECK(v_times_t(h, Xr, ldxr, k, h->lr_b, k));
-        spmv_chunk_kernel<<<chunk_blocks, 256, 0, s>>>(h->chunk_row, h->chunk_beg, h->csr_ptr, h->csr_col,
-                                                       h->csr_val, Xr, ldxr, h->nchunks, k, part);
+        if (r > 0) SP_CHECK(v_times(h, Xt, k, h->lr_b, k));
+        auto run = [&](auto kern) {
+            kern<<<grid_a, 32 * SP_WARPS, 0, s>>>(h->chunk_row, h->chunk_beg, h->csr_ptr, h->csr_col, h->csr_val, Xt,
+                                                  (int64_t)k, h->nchunks, k, part);
+        };
+        switch (lg) {
+            case 0: run(spmv_chunk_kernel<0>); break;
+            case 1: run(spmv_chunk_kernel<1>); break;
+            case 2: run(spmv_chunk_kernel<2>); break;
+            case 3: run(spmv_chunk_kernel<3>); break;
+            case 4: run(spmv_chunk_kernel<4>); break;
+            default: run(spmv_chunk_kernel<5>); break;
+        }
         spmv_rows_kernel<<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(h->row_chunk, part, m, k, r, h->lrU, h->lr_b,
                                                                       out);
         note_launch(2);
         phase_end(h, RTPROJ_PHASE_APPLY_A);
         return RTPROJ_OK;
     };
-    auto apply_at = [&](const double* Hm, const double* Y, int64_t ldy) -> rtproj_status {   // sbuf = Y - A^* h
+    auto apply_at = [&](const double* Hm, const double* Yt) -> rtproj_status {   // sbuf = Y - A^* h
         phase_begin(h, RTPROJ_PHASE_APPLY_AT);
         if (r > 0) SP_CHECK(ut_times(h, Hm, k, k, h->lr_b, k));
-        spmvT_dd_kernel<<<tgrid, 256, 0, s>>>(h->csc_ptr, h->csc_row, h->csc_val, Hm, k, n, r, h->lrV, h->lr_b, Y,
-                                              ldy, h->sbuf, n);
+        auto run = [&](auto kern) {
+            kern<<<grid_t, 32 * SP_WARPS, 0, s>>>(h->csc_ptr, h->csc_row, h->csc_val, Hm, k, n, r, h->lrV, h->lr_b,
+                                                  Yt, (int64_t)k, h->sbuf, (int64_t)k);
+        };
+        switch (lg) {
+            case 0: run(spmvT_kernel<0, 1>); break;
+            case 1: run(spmvT_kernel<1, 1>); break;
+            case 2: run(spmvT_kernel<2, 1>); break;
+            case 3: run(spmvT_kernel<3, 1>); break;
+            case 4: run(spmvT_kernel<4, 1>); break;
+            default:
+                if (jb == 1) run(spmvT_kernel<5, 1>);
+                else if (jb == 2) run(spmvT_kernel<5, 2>);
+                else run(spmvT_kernel<5, 4>);
+                break;
+        }
         note_launch();
         phase_end(h, RTPROJ_PHASE_APPLY_AT);
         return RTPROJ_OK;
     };
     // c = A b; h0 = Pi^* T1^* T1 Pi c; s = b - A^* h0
-    rtproj_status st = apply_a(B, ldb, h->cbuf);
+    rtproj_status st = apply_a(Bt, h->cbuf);
     if (st != RTPROJ_OK) return st;
     phase_begin(h, RTPROJ_PHASE_APPLY_M);
     st = middle_fp64(h, h->cbuf, h->hbuf, k);
     if (st != RTPROJ_OK) return st;
     phase_end(h, RTPROJ_PHASE_APPLY_M);
-    st = apply_at(h->hbuf, B, ldb);
+    st = apply_at(h->hbuf, Bt);
     if (st != RTPROJ_OK) return st;
     int passes = 0;
     for (int pass = 0; pass < o.refine_passes; ++pass) {
         // r = A s; dh = Pi^* T1^* T1 Pi r; h += dh; s <- s - A^* dh (Remark 4.3)
-        st = apply_a(h->sbuf, n, h->cbuf);
+        st = apply_a(h->sbuf, h->cbuf);
         if (st != RTPROJ_OK) return st;
         phase_begin(h, RTPROJ_PHASE_APPLY_M);
         st = middle_fp64(h, h->cbuf, h->dhbuf, k);
@@ -661,13 +817,20 @@ rtproj_status sparse_project(rtproj_ctx* h, const double* B, int64_t ldb, int k,
             std::memcpy(v, bits, 16);
             if (v[1] <= o.refine_tol) last = true;
         }
-        st = apply_at(h->dhbuf, h->sbuf, n);   // in place: each entry reads its own s first
+        st = apply_at(h->dhbuf, h->sbuf);   // in place: each entry reads its own s first
         if (st != RTPROJ_OK) return st;
         if (last) break;
     }
     h->last_passes = passes;
-    if (ROW) SP_CHECK(store_rows(h->sbuf, n, B, ldb, ROW, ldr, k, n, 1, RTPROJ_F64, s));
-    if (Z) SP_CHECK(store_rows(h->sbuf, n, nullptr, 0, Z, ldz, k, n, 0, RTPROJ_F64, s));
+    const dim3 fgrid((unsigned)((n + 31) / 32), (unsigned)((k + 31) / 32));
+    if (k == 1) {
+        if (ROW) SP_CHECK(store_rows(h->sbuf, n, B, ldb, ROW, ldr, k, n, 1, RTPROJ_F64, s));
+        if (Z) SP_CHECK(store_rows(h->sbuf, n, nullptr, 0, Z, ldz, k, n, 0, RTPROJ_F64, s));
+    } else {   // ROW before Z, since Z may alias B
+        if (ROW) finish_rows_kernel<<<fgrid, 256, 0, s>>>(h->sbuf, n, k, B, ldb, (double*)ROW, ldr);
+        if (Z) finish_rows_kernel<<<fgrid, 256, 0, s>>>(h->sbuf, n, k, nullptr, 0, (double*)Z, ldz);
+        note_launch((ROW ? 1 : 0) + (Z ? 1 : 0));
+    }
     if (X) SP_CHECK(store_transposed(h->hbuf, k, m, k, X, ldx, RTPROJ_F64, s));
     SP_CHECK(cudaGetLastError());
     return RTPROJ_OK;

@@ -24,6 +24,7 @@
 // 128-byte swizzle row per operand row). Thread 0 issues the MMAs; all threads stage
 // operands with cp.async into the SWIZZLE_128B K-major layout and read TMEM back.
 #include "rtproj_internal.cuh"
+#include "i128.cuh"
 
 #include <utility>
 
@@ -177,49 +178,12 @@ __device__ __forceinline__ void fold_level(int g, int D, const uint32_t (&r)[32]
 // every sign and magnitude: the earlier form with a branch per shift range took about
 // 1000 cycles per element in the epilogue. A result outside the normal range is delegated
 // to ldexp.
-__device__ __forceinline__ double u128_to_double(unsigned long long H, unsigned long long L, int e);
-
 __device__ __forceinline__ double words_to_double(long long hi, long long lo, int e) {
     // V = hi * 2^40 + lo as a 128-bit two's complement value (H:L)
     const unsigned long long L = ((unsigned long long)hi << 40) + (unsigned long long)lo;
     const unsigned long long carry = L < ((unsigned long long)hi << 40) ? 1ull : 0ull;
     const unsigned long long H = (unsigned long long)(hi >> 24) + (unsigned long long)(lo >> 63) + carry;
     return u128_to_double(H, L, e);
-}
-
-// V * 2^e for the 128-bit two's-complement integer V = (H:L), rounded to nearest even.
-__device__ __forceinline__ double u128_to_double(unsigned long long H, unsigned long long L, int e) {
-    // |V| by a masked negation (no branch: the lanes of a warp hold values of either sign)
-    const unsigned long long sg = (unsigned long long)((long long)H >> 63);
-    L ^= sg;
-    H ^= sg;
-    const unsigned long long one = sg & 1ull;
-    const unsigned long long L1 = L + one;
-    H += one & (L1 == 0 ? 1ull : 0ull);
-    L = L1;
-    if ((H | L) == 0) return 0.0;
-    // normalise: shift left by the leading zeros so that the leading one is bit 127
-    const int s = H != 0 ? __clzll((long long)H) : 64 + __clzll((long long)L);
-    const int s1 = s & 63;
-    const unsigned long long hl = s1 ? (H << s1) | (L >> (64 - s1)) : H;
-    const unsigned long long Hn = s < 64 ? hl : (L << s1);
-    const unsigned long long Ln = s < 64 ? (L << s1) : 0ull;
-    // 53 bits, round to nearest even on the round bit and the sticky bits below it
-    unsigned long long m = Hn >> 11;
-    const unsigned long long rb = (Hn >> 10) & 1ull;
-    const unsigned long long st = ((Hn & 0x3FFull) | Ln) != 0 ? 1ull : 0ull;
-    m += rb & (st | (m & 1ull));
-    const unsigned long long ovf = m >> 53;       // rounding carried into bit 53
-    m >>= ovf;
-    const int ex = 127 - s + (int)ovf;             // position of the leading bit of |V|
-    const int biased = ex + e + 1023;
-    if (biased <= 0 || biased >= 2047) {
-        const double mag = ldexp((double)m, ex - 52 + e);
-        return sg ? -mag : mag;
-    }
-    const unsigned long long bits =
-        ((unsigned long long)biased << 52) | (m & 0xFFFFFFFFFFFFFull) | (sg & 0x8000000000000000ull);
-    return __longlong_as_double((long long)bits);
 }
 
 // alpha * v + beta * cin with the common cases decided on the host: amode 0 (alpha = 1),

@@ -1,0 +1,43 @@
+// Host build of the 128-bit sums of exact products (csrc/i128.cuh) for the CPU tests: reads
+// "sum N" or "two N" and N pairs of doubles (hexadecimal), prints the rounded sum of their
+// products and the pair form; "two" forms the sum from two halves merged.
+#include <cmath>
+#include <cstdint>
+#include <cstdio>
+#include <cstring>
+
+#define __device__
+#define __forceinline__ inline
+static inline int __clzll(long long x) { return x ? __builtin_clzll((unsigned long long)x) : 64; }
+static inline double __longlong_as_double(long long x) {
+    double d;
+    std::memcpy(&d, &x, 8);
+    return d;
+}
+using std::ldexp;
+#include "i128.cuh"
+
+static rtp::i128op dec(double x) {
+    uint64_t u;
+    std::memcpy(&u, &x, 8);
+    return rtp::i128_decode((uint32_t)u, (uint32_t)(u >> 32));
+}
+
+int main() {
+    char op[16];
+    int n;
+    while (std::scanf("%15s %d", op, &n) == 2) {
+        rtp::i128acc a = rtp::i128_zero(), b = rtp::i128_zero();
+        const bool two = op[0] == 't';
+        for (int i = 0; i < n; ++i) {
+            double x, y;
+            if (std::scanf("%la %la", &x, &y) != 2) return 1;
+            rtp::i128_mac(two && (i & 1) ? b : a, rtp::i128_left(dec(x)), dec(y), i % 3 == 2 ? ~0u : 0u);
+        }
+        rtp::i128_merge(a, b);
+        double hi, lo;
+        rtp::i128_to_pair(a, hi, lo);
+        std::printf("%a %a %a\n", rtp::i128_to_double(a), hi, lo);
+    }
+    return 0;
+}
