@@ -25,6 +25,14 @@ struct i128acc {
     int E;                     // unit 2^E
 };
 
+__device__ __forceinline__ double i128_from_words(uint32_t hi, uint32_t lo) {
+#ifdef __CUDA_ARCH__
+    return __hiloint2double((int)hi, (int)lo);
+#else
+    return __longlong_as_double((long long)(((uint64_t)hi << 32) | lo));
+#endif
+}
+
 // One operand decoded: |x| = (hi 2^32 + lo) 2^e, neg = all ones for a negative x.
 struct i128op {
     uint32_t lo, hi;
@@ -85,13 +93,13 @@ __device__ __forceinline__ void i128_add_signed(i128acc& a, uint32_t p0, uint32_
                                                 uint32_t m) {
     p0 ^= m; p1 ^= m; p2 ^= m; p3 ^= m;
 #ifdef __CUDA_ARCH__
-    uint32_t t;
-    asm("add.cc.u32 %4, %9, %9;\n\t"          // the carry in: 1 when m is all ones
-        "addc.cc.u32 %0, %0, %5;\n\t"
-        "addc.cc.u32 %1, %1, %6;\n\t"
-        "addc.cc.u32 %2, %2, %7;\n\t"
-        "addc.u32 %3, %3, %8;\n\t"
-        : "+r"(a.w0), "+r"(a.w1), "+r"(a.w2), "+r"(a.w3), "=&r"(t)
+    asm("{\n\t.reg .u32 t;\n\t"
+        "add.cc.u32 t, %8, %8;\n\t"            // the carry in: 1 when m is all ones
+        "addc.cc.u32 %0, %0, %4;\n\t"
+        "addc.cc.u32 %1, %1, %5;\n\t"
+        "addc.cc.u32 %2, %2, %6;\n\t"
+        "addc.u32 %3, %3, %7;\n\t}\n"
+        : "+r"(a.w0), "+r"(a.w1), "+r"(a.w2), "+r"(a.w3)
         : "r"(p0), "r"(p1), "r"(p2), "r"(p3), "r"(m));
 #else
     uint64_t c = (uint64_t)a.w0 + p0 + (m & 1u);
@@ -145,39 +153,93 @@ __device__ __forceinline__ void i128_merge(i128acc& a, i128acc b) {
     i128_add_signed(a, b.w0, b.w1, b.w2, b.w3, 0u);
 }
 
-// V * 2^e for the 128-bit two's-complement integer V = (H:L), rounded to nearest even.
+// A result outside the normal range (rare): m 2^e for the 53-bit m, by ldexp.
+static __device__ __noinline__ double i128_edge_result(unsigned long long m, int e, uint32_t neg) {
+    const double mag = ldexp((double)m, e);
+    return neg ? -mag : mag;
+}
+
+// The magnitude (w3:w0) 2^e, negative when neg = ~0, rounded to nearest (ties to even). All in
+// 32-bit operations and without branches (the lanes of a warp hold values of every size): the
+// three words from the leading nonzero one on are selected and normalised by one count of
+// leading zeros and two funnel shifts, the rest joins the sticky bits; about 45 instructions.
+// (Written with 64-bit shifts by variable amounts the conversion took about 290 cycles per warp,
+// which bounded the sliced products with a short contraction.)
+__device__ __forceinline__ double i128_round(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, int e, uint32_t neg) {
+    const bool n3 = w3 != 0u, n2 = w2 != 0u, n1 = w1 != 0u;
+    const uint32_t t2 = n3 ? w3 : n2 ? w2 : n1 ? w1 : w0;
+    const uint32_t t1 = n3 ? w2 : n2 ? w1 : n1 ? w0 : 0u;
+    const uint32_t t0 = n3 ? w1 : n2 ? w0 : 0u;
+    const uint32_t rest = n3 ? w0 : 0u;
+    const int top = n3 ? 127 : n2 ? 95 : n1 ? 63 : 31;          // bit of t2's most significant place
+#ifdef __CUDA_ARCH__
+    const int z = __clz((int)t2);
+    const uint32_t a = __funnelshift_l(t1, t2, z), b = __funnelshift_l(t0, t1, z), c = t0 << (z & 31);
+#else
+    const int z = t2 ? __builtin_clz(t2) : 32;
+    const int y = z & 31;
+    const uint32_t a = y ? (t2 << y) | (t1 >> (32 - y)) : t2, b = y ? (t1 << y) | (t0 >> (32 - y)) : t1, c = t0 << y;
+#endif
+    const uint32_t mlo = (a << 21) | (b >> 11), mhi = a >> 11;  // 53 bits, the leading one at bit 20 of mhi
+    const bool up = (b & 0x400u) && (((b & 0xBFFu) | c | rest) != 0u);   // round bit; sticky bits or the last bit
+    const int biased = top - z + e + 1023;
+    if (t2 == 0u) return 0.0;
+    if (biased <= 0 || biased >= 2046)                          // 2046: the rounding could carry into 2047
+        return i128_edge_result((((unsigned long long)mhi << 32) | mlo) + (up ? 1ull : 0ull), top - z - 52 + e, neg);
+    const unsigned long long bits = ((((unsigned long long)(uint32_t)(biased - 1) << 20) + mhi) << 32 | mlo) + (up ? 1ull : 0ull);
+    const uint32_t hi = (uint32_t)(bits >> 32) | (neg & 0x80000000u), lo = (uint32_t)bits;
+    return i128_from_words(hi, lo);
+}
+
+// V * 2^e for the 128-bit two's-complement integer V = (v3:v0), rounded to nearest even.
+__device__ __forceinline__ double i128_round_signed(uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, int e) {
+    const uint32_t neg = (uint32_t)((int32_t)v3 >> 31);
+    i128acc a = {0u, 0u, 0u, 0u, 0};
+    i128_add_signed(a, v0, v1, v2, v3, neg);                    // |V|: (V xor neg) - neg
+    return i128_round(a.w0, a.w1, a.w2, a.w3, e, neg);
+}
+
 __device__ __forceinline__ double u128_to_double(unsigned long long H, unsigned long long L, int e) {
-    // |V| by a masked negation (no branch: the lanes of a warp hold values of either sign)
-    const unsigned long long sg = (unsigned long long)((long long)H >> 63);
-    L ^= sg;
-    H ^= sg;
-    const unsigned long long one = sg & 1ull;
-    const unsigned long long L1 = L + one;
-    H += one & (L1 == 0 ? 1ull : 0ull);
-    L = L1;
-    if ((H | L) == 0) return 0.0;
-    // normalise: shift left by the leading zeros so that the leading one is bit 127
-    const int s = H != 0 ? __clzll((long long)H) : 64 + __clzll((long long)L);
-    const int s1 = s & 63;
-    const unsigned long long hl = s1 ? (H << s1) | (L >> (64 - s1)) : H;
-    const unsigned long long Hn = s < 64 ? hl : (L << s1);
-    const unsigned long long Ln = s < 64 ? (L << s1) : 0ull;
-    // 53 bits, round to nearest even on the round bit and the sticky bits below it
-    unsigned long long m = Hn >> 11;
-    const unsigned long long rb = (Hn >> 10) & 1ull;
-    const unsigned long long st = ((Hn & 0x3FFull) | Ln) != 0 ? 1ull : 0ull;
-    m += rb & (st | (m & 1ull));
-    const unsigned long long ovf = m >> 53;       // rounding carried into bit 53
-    m >>= ovf;
-    const int ex = 127 - s + (int)ovf;             // position of the leading bit of |V|
-    const int biased = ex + e + 1023;
-    if (biased <= 0 || biased >= 2047) {
-        const double mag = ldexp((double)m, ex - 52 + e);
-        return sg ? -mag : mag;
+    return i128_round_signed((uint32_t)L, (uint32_t)(L >> 32), (uint32_t)H, (uint32_t)(H >> 32), e);
+}
+
+// 2^sh times the 128-bit integer (v3:v0), 0 <= sh < 32 (bits past the top are lost).
+__device__ __forceinline__ void i128_shl(uint32_t& v0, uint32_t& v1, uint32_t& v2, uint32_t& v3, int sh) {
+#ifdef __CUDA_ARCH__
+    v3 = __funnelshift_l(v2, v3, sh);
+    v2 = __funnelshift_l(v1, v2, sh);
+    v1 = __funnelshift_l(v0, v1, sh);
+#else
+    if (sh) {
+        v3 = (v3 << sh) | (v2 >> (32 - sh));
+        v2 = (v2 << sh) | (v1 >> (32 - sh));
+        v1 = (v1 << sh) | (v0 >> (32 - sh));
     }
-    const unsigned long long bits =
-        ((unsigned long long)biased << 52) | (m & 0xFFFFFFFFFFFFFull) | (sg & 0x8000000000000000ull);
-    return __longlong_as_double((long long)bits);
+#endif
+    v0 <<= sh;
+}
+
+// x - V 2^e rounded once, for V = (v3:v0) two's complement and a double x given by its bits: the
+// two are brought to a common unit (x's significand moves up by at most 63 bits, or V by at most
+// 22) and subtracted exactly. false (out untouched) when their units lie further apart, V is not
+// within 2^103, or x is not finite.
+__device__ __forceinline__ bool i128_sub_from(uint32_t xl, uint32_t xh, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3,
+                                              int e, double& out) {
+    const i128op o = i128_decode(xl, xh);
+    const int sh = o.e - e;
+    if (sh > 63 || sh < -22 || v3 + 0x80u >= 0x100u || !i128_finite(xh)) return false;
+    const int sv = sh < 0 ? -sh : 0, sx = sh > 0 ? sh : 0;
+    i128_shl(v0, v1, v2, v3, sv);
+    // -V
+    i128acc a = {0u, 0u, 0u, 0u, 0};
+    i128_add_signed(a, v0, v1, v2, v3, ~0u);
+    // the significand's two words at bit sx
+    const bool w = sx >= 32;
+    uint32_t x0 = w ? 0u : o.lo, x1 = w ? o.lo : o.hi, x2 = w ? o.hi : 0u, x3 = 0u;
+    i128_shl(x0, x1, x2, x3, sx & 31);
+    i128_add_signed(a, x0, x1, x2, x3, o.neg);
+    out = i128_round_signed(a.w0, a.w1, a.w2, a.w3, e - sv);
+    return true;
 }
 
 __device__ __forceinline__ unsigned long long i128_high(const i128acc& a) { return ((unsigned long long)a.w3 << 32) | a.w2; }

@@ -26,6 +26,7 @@
 #include "rtproj_internal.cuh"
 #include "i128.cuh"
 
+#include <type_traits>
 #include <utility>
 
 #include <cuda.h>
@@ -170,43 +171,57 @@ __device__ __forceinline__ void fold_level(int g, int D, const uint32_t (&r)[32]
     }
 }
 
-// (hi * 2^40 + lo) * 2^e rounded to nearest (ties to even), from integer operations: the
-// two words form a 128-bit two's-complement integer, whose magnitude is normalised by its
-// leading-zero count and cut to 53 bits with a round bit and a sticky bit. Integer
-// instructions keep the conversion off GB300's FP64 pipe (64 cycles per warp instruction),
-// and it is branch-free (selects and masks) because the lanes of a warp hold values of
-// every sign and magnitude: the earlier form with a branch per shift range took about
-// 1000 cycles per element in the epilogue. A result outside the normal range is delegated
-// to ldexp.
-__device__ __forceinline__ double words_to_double(long long hi, long long lo, int e) {
-    // V = hi * 2^40 + lo as a 128-bit two's complement value (H:L)
-    const unsigned long long L = ((unsigned long long)hi << 40) + (unsigned long long)lo;
-    const unsigned long long carry = L < ((unsigned long long)hi << 40) ? 1ull : 0ull;
-    const unsigned long long H = (unsigned long long)(hi >> 24) + (unsigned long long)(lo >> 63) + carry;
-    return u128_to_double(H, L, e);
+// The two words of an entry (0 <= lo < 2^40) as one 128-bit two's-complement integer
+// hi * 2^40 + lo.
+__device__ __forceinline__ void words_to_i128(long long hi, long long lo, uint32_t& w0, uint32_t& w1, uint32_t& w2,
+                                              uint32_t& w3) {
+    const uint32_t hl = (uint32_t)hi, hh = (uint32_t)((unsigned long long)hi >> 32);
+    w0 = (uint32_t)lo;
+    w1 = (uint32_t)((unsigned long long)lo >> 32) | (hl << 8);
+    w2 = (hl >> 24) | (hh << 8);
+    w3 = (uint32_t)((int32_t)hh >> 24);
 }
 
 // alpha * v + beta * cin with the common cases decided on the host: amode 0 (alpha = 1),
 // 1 (alpha = -1: a sign flip), 2 (general); bmode 0 (beta = 0), 1 (beta = 1), 2 (general).
 // The cases cost no float64 comparisons on the device.
-__device__ __forceinline__ double epilogue_value(double v, int amode, double alpha, int bmode, double beta,
-                                                 const double* cin) {
-    double out = amode == 0 ? v
-               : amode == 1 ? __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull)
-                            : alpha * v;
-    if (bmode == 1) out += *cin;
-    else if (bmode == 2) out = fma(beta, *cin, out);
-    return out;
-}
-// The same with the Cin entry already loaded.
-__device__ __forceinline__ double epilogue_value_v(double v, int amode, double alpha, int bmode, double beta,
-                                                   double cin) {
+__device__ __forceinline__ double epilogue_value(double v, int amode, double alpha, int bmode, double beta, double cin) {
     double out = amode == 0 ? v
                : amode == 1 ? __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull)
                             : alpha * v;
     if (bmode == 1) out += cin;
     else if (bmode == 2) out = fma(beta, cin, out);
     return out;
+}
+
+// An entry's output value from its exact integer sum V (v3:v0), unit 2^e. Cin - V 2^e (the
+// residuals b - A^* h and s - A^* dh) is formed in integers and rounded once (i128_sub_from; a
+// float64 subtraction would also hold the FP64 pipe for 64 cycles a warp); the other forms round
+// V 2^e to float64 first.
+__device__ __noinline__ double general_value(uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, int e, int amode,
+                                             double alpha, int bmode, double beta, double cin) {
+    return epilogue_value(i128_round_signed(v0, v1, v2, v3, e), amode, alpha, bmode, beta, cin);
+}
+template <bool CIN>
+__device__ __forceinline__ double entry_value(uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, int e, int amode,
+                                              double alpha, int bmode, double beta, double cin) {
+    if constexpr (CIN) {
+        double out;
+        if (amode == 1 && bmode == 1 &&
+            i128_sub_from((uint32_t)__double2loint(cin), (uint32_t)__double2hiint(cin), v0, v1, v2, v3, e, out))
+            return out;
+        return general_value(v0, v1, v2, v3, e, amode, alpha, bmode, beta, cin);
+    } else {
+        return epilogue_value(i128_round_signed(v0, v1, v2, v3, e), amode, alpha, 0, 0.0, 0.0);
+    }
+}
+// The same from the two words hi 2^40 + lo.
+template <bool CIN>
+__device__ __forceinline__ double entry_value_words(long long hi, long long lo, int e, int amode, double alpha, int bmode,
+                                                    double beta, double cin) {
+    uint32_t w0, w1, w2, w3;
+    words_to_i128(hi, lo, w0, w1, w2, w3);
+    return entry_value<CIN>(w0, w1, w2, w3, e, amode, alpha, bmode, beta, cin);
 }
 __host__ inline int alpha_mode(double a) { return a == 1.0 ? 0 : (a == -1.0 ? 1 : 2); }
 __host__ inline int beta_mode(double b) { return b == 0.0 ? 0 : (b == 1.0 ? 1 : 2); }
@@ -239,86 +254,187 @@ __device__ __forceinline__ void add_shifted(unsigned long long& acc, int v) {
     }
 }
 
-// Sum over levels [G0, G1) (positions g + D) that land in word `hi_word` of
-// 0x4B400000 * 2^level_shift, modulo 2^64: the offset that the magic-number conversion
-// adds to every value (0x4B400000 / 2^8 at position 10, exactly).
-__host__ __device__ constexpr unsigned long long magic_bias(int G0, int G1, bool hi_word, int D) {
+// acc += c * 2^SH for an unsigned c.
+template <int SH>
+__device__ __forceinline__ void add_shifted_u(unsigned long long& acc, uint32_t c) {
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc) : "r"(c), "r"(1u << SH));
+}
+
+// Readout groups. Levels g and g + 1 (g even, g < 8) lie one digit apart in the same word, so
+// they are joined before they enter it: the raw bits of x + 1.5 * 2^23 are the integer x plus
+// 0x4B400000 (|x| <= 2^22), and 256 bits_g + bits_{g+1} modulo 2^32 is the joined integer plus
+// kPairBias, which lies in (0, 2^32) for every such pair: one 32-bit and one wide
+// multiply-add for two values. Levels 8 and 9 enter one at a time. The offsets of all groups are
+// removed together (magic_bias).
+constexpr uint32_t kMagic = 0x4B400000u;
+constexpr uint32_t kPairBias = kMagic * 256u + kMagic;      // modulo 2^32: 0x8B400000
+// Whether levels g and g + 1 of a readout that ends before level `end` are joined.
+__host__ __device__ constexpr bool is_pair(int g, int end) { return g % 2 == 0 && g < 8 && g + 1 < end; }
+
+// The accumulators of a tile are read in two sets: levels [0, level_split) and [level_split, terms).
+// While the tensor cores work on one set, the other is read out, so a tile needs a single
+// accumulator per level (see sliced_gemm2_kernel).
+__host__ __device__ constexpr int level_split(int terms) { return terms >= 6 ? 4 : terms >= 3 ? 2 : terms; }
+
+// Sum over the groups of levels [L0, L1) that land in word `hi_word` of the offset each value
+// enters with, modulo 2^64.
+__host__ __device__ constexpr unsigned long long magic_bias(int L0, int L1, bool hi_word) {
     unsigned long long b = 0;
-    for (int g = G0; g < G1; ++g) {
-        const int P = g + D;
-        if ((P <= 4) != hi_word) continue;
-        b += P > 9 ? (0x4B400000ull >> 8) : (0x4B400000ull << level_shift(P));
+    for (int g = L0; g < L1; ++g) {
+        const int P = g + 1;                                   // level_offset
+        const bool pair = is_pair(g, L1);
+        if ((P <= 4) == hi_word)
+            b += pair ? (unsigned long long)kPairBias << level_shift(P + 1)
+                  : P > 9 ? (unsigned long long)(kMagic >> 8) : (unsigned long long)kMagic << level_shift(P);
+        if (pair) ++g;
     }
     return b;
 }
 
-// Adds level L of one 16-column unit (columns CB*16 .. CB*16+15 of the warp's NCOL) into
-// its word. Every value enters with the same offset 0x4B400000: the raw bits of
-// x + 1.5 * 2^23 (FAST, exact when |x| < 2^22) or the exact integer plus that offset; the
-// sum of the offsets is removed once per chunk.
-template <int P, bool FAST, int CB, int NCOL>
-__device__ __forceinline__ void fold_one(const uint32_t (&r)[16], unsigned long long (&hi)[NCOL],
-                                         unsigned long long (&lo)[NCOL]) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        const int v = FAST ? __float_as_int(__fadd_rn(__uint_as_float(r[j]), 12582912.0f))
-                           : exact_f2i(__uint_as_float(r[j])) + 0x4B400000;
-        if constexpr (P <= 4) add_shifted<level_shift(P)>(hi[CB * 16 + j], v);
-        else if constexpr (P <= 9) add_shifted<level_shift(P)>(lo[CB * 16 + j], v);
-        else add_shifted<0>(lo[CB * 16 + j], v >> 8);   // v > 0: the offset keeps it positive
-    }
+// x + 1.5 * 2^23 for two values at once (one packed add), as raw bits.
+__device__ __forceinline__ void magic_add2(uint32_t x0, uint32_t x1, uint32_t& b0, uint32_t& b1) {
+    asm("{\n\t.reg .b64 x, m;\n\t"
+        "mov.b64 x, {%2, %3};\n\t"
+        "mov.b64 m, {%4, %4};\n\t"
+        "add.rn.f32x2 x, x, m;\n\t"
+        "mov.b64 {%0, %1}, x;\n\t}\n"
+        : "=r"(b0), "=r"(b1)
+        : "r"(x0), "r"(x1), "r"(kMagic));
 }
-template <int P0, bool FAST, int CB, int NCOL, int... I>
-__device__ __forceinline__ void fold_levels(const uint32_t (&r)[sizeof...(I)][16], unsigned long long (&hi)[NCOL],
-                                            unsigned long long (&lo)[NCOL], std::integer_sequence<int, I...>) {
-    (fold_one<P0 + I, FAST, CB, NCOL>(r[I], hi, lo), ...);
+// max(|a|, |b|, m) for m >= 0
+__device__ __forceinline__ float max_abs3(float m, uint32_t a, uint32_t b) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(m), "f"(__uint_as_float(a)), "f"(__uint_as_float(b)));
+    return d;
 }
 
-// Loads levels L0 .. L0+NG-1 of one 16-column unit (TMEM address `addr` + level * tn),
-// checks them, and folds them in; with `release` the TMEM buffer is handed back to the
-// MMA warp as soon as the values are in registers.
-template <int L0, int NG, int CB, int NCOL, int D>
-__device__ __forceinline__ void fold_group(uint32_t addr, uint32_t tn, unsigned long long (&hi)[NCOL],
-                                           unsigned long long (&lo)[NCOL], bool release, uint64_t* empty_bar) {
-    uint32_t r[NG][16];
+// Folds one group (level G, with G + 1 when PAIR) of 16 columns. FAST: every value is within
+// 2^22; otherwise the two-part exact conversion, with the same offset added explicitly.
+template <int G, bool PAIR, bool FAST>
+__device__ __forceinline__ void fold_group(const uint32_t (&r)[PAIR ? 2 : 1][16], unsigned long long* hi,
+                                           unsigned long long* lo) {
+    constexpr int P = G + 1;                                   // level_offset
+    unsigned long long* acc = P <= 4 ? hi : lo;
 #pragma unroll
-    for (int g = 0; g < NG; ++g) tmem_ld16(addr + (uint32_t)(L0 + g) * tn, r[g]);
+    for (int j = 0; j < 16; j += 2) {
+        if constexpr (FAST) {
+            uint32_t a0, a1;
+            magic_add2(r[0][j], r[0][j + 1], a0, a1);
+            if constexpr (PAIR) {
+                constexpr int SH1 = level_shift(P + 1);
+                uint32_t b0, b1;
+                magic_add2(r[1][j], r[1][j + 1], b0, b1);
+                add_shifted_u<SH1>(acc[j], a0 * 256u + b0);
+                add_shifted_u<SH1>(acc[j + 1], a1 * 256u + b1);
+            } else if constexpr (P <= 9) {
+                add_shifted<level_shift(P)>(acc[j], (int)a0);
+                add_shifted<level_shift(P)>(acc[j + 1], (int)a1);
+            } else {                                           // positive: the offset keeps it so
+                add_shifted<0>(acc[j], (int)a0 >> 8);
+                add_shifted<0>(acc[j + 1], (int)a1 >> 8);
+            }
+        } else {
+#pragma unroll
+            for (int q = j; q < j + 2; ++q) {
+                const int v = exact_f2i(__uint_as_float(r[0][q]));
+                if constexpr (PAIR) {
+                    add_shifted<level_shift(P)>(acc[q], v);
+                    add_shifted<level_shift(P + 1)>(acc[q], exact_f2i(__uint_as_float(r[1][q])));
+                    acc[q] += (unsigned long long)kPairBias << level_shift(P + 1);
+                } else if constexpr (P <= 9) {
+                    add_shifted<level_shift(P)>(acc[q], v + (int)kMagic);
+                } else {
+                    add_shifted<0>(acc[q], (v + (int)kMagic) >> 8);
+                }
+            }
+        }
+    }
+}
+
+// Waits for the thread's TMEM loads; the registers pass through, so that no use of them can be
+// placed before the wait.
+template <int N>
+__device__ __forceinline__ void tmem_ld_wait_regs(uint32_t (&r)[N][16]) {
     tmem_ld_wait();
-    if (release) {
+#pragma unroll
+    for (int g = 0; g < N; ++g)
+#pragma unroll
+        for (int j = 0; j < 16; ++j) asm volatile("" : "+r"(r[g][j]));
+}
+
+template <int N>
+__device__ __forceinline__ void tmem_ld_group(uint32_t addr, uint32_t tn, uint32_t (&r)[N][16]) {
+#pragma unroll
+    for (int g = 0; g < N; ++g) tmem_ld16(addr + (uint32_t)g * tn, r[g]);
+}
+
+// A set's groups in order (16-column units, then level groups): the next group's TMEM loads are
+// issued before this one is folded, so that their latency is hidden; after the last loads have
+// arrived the set is handed back to the MMA warp. r holds group (CB, G), already waited for.
+template <int L0, int L1, int NCOL, int CB, int G>
+__device__ __forceinline__ void readout_rec(uint32_t addr0, uint32_t tn, unsigned long long (&hi)[NCOL],
+                                            unsigned long long (&lo)[NCOL], uint64_t* empty_bar,
+                                            uint32_t (&r)[is_pair(G, L1) ? 2 : 1][16]) {
+    constexpr bool PAIR = is_pair(G, L1);
+    constexpr int GN = G + (PAIR ? 2 : 1);
+    constexpr bool last_g = GN >= L1, last = last_g && CB == NCOL / 16 - 1;
+    constexpr int CBN = last_g ? CB + 1 : CB, G2 = last_g ? L0 : GN;
+    uint32_t rn[last ? 1 : is_pair(G2, L1) ? 2 : 1][16];
+    if constexpr (!last) {
+        tmem_ld_group(addr0 + (uint32_t)(CBN * 16) + (uint32_t)G2 * tn, tn, rn);
+    } else {
         tc_fence_before();
         mbar_arrive(empty_bar);
     }
     float mx = 0.0f;
 #pragma unroll
-    for (int g = 0; g < NG; ++g)
+    for (int g = 0; g < (PAIR ? 2 : 1); ++g)
 #pragma unroll
-        for (int j = 0; j < 16; ++j) mx = fmaxf(mx, fabsf(__uint_as_float(r[g][j])));
-    if (__all_sync(0xffffffffu, mx < 4194304.0f))
-        fold_levels<L0 + D, true, CB, NCOL>(r, hi, lo, std::make_integer_sequence<int, NG>{});
-    else
-        fold_levels<L0 + D, false, CB, NCOL>(r, hi, lo, std::make_integer_sequence<int, NG>{});
+        for (int j = 0; j < 16; j += 2) mx = max_abs3(mx, r[g][j], r[g][j + 1]);
+    if (__all_sync(0xffffffffu, mx <= 4194304.0f)) fold_group<G, PAIR, true>(r, hi + CB * 16, lo + CB * 16);
+    else fold_group<G, PAIR, false>(r, hi + CB * 16, lo + CB * 16);
+    if constexpr (!last) {
+        tmem_ld_wait_regs(rn);
+        readout_rec<L0, L1, NCOL, CBN, G2>(addr0, tn, hi, lo, empty_bar, rn);
+    }
 }
 
-// Level groups of one chunk readout: 16-column units in order, levels in groups of GS.
-template <int TERMS, int NCOL, int CB, int L0>
-__device__ __forceinline__ void readout_rec(uint32_t addr0, uint32_t tn, unsigned long long (&hi)[NCOL],
-                                            unsigned long long (&lo)[NCOL], uint64_t* empty_bar) {
-    constexpr int GS = NCOL == 16 ? 5 : 1;
-    constexpr int NG = (TERMS - L0) < GS ? (TERMS - L0) : GS;
-    constexpr bool last = (CB == NCOL / 16 - 1) && (L0 + NG >= TERMS);
-    fold_group<L0, NG, CB, NCOL, level_offset(TERMS)>(addr0 + CB * 16, tn, hi, lo, last, empty_bar);
-    if constexpr (L0 + NG < TERMS) readout_rec<TERMS, NCOL, CB, L0 + NG>(addr0, tn, hi, lo, empty_bar);
-    else if constexpr (CB + 1 < NCOL / 16) readout_rec<TERMS, NCOL, CB + 1, 0>(addr0, tn, hi, lo, empty_bar);
-}
-
-// One chunk readout of TERMS levels for the warp's NCOL columns, then the offsets are
-// removed and the carry of lo moved into hi (afterwards |lo| < 2^40).
-template <int TERMS, int NCOL>
+// One readout of levels [L0, L1) for the warp's NCOL columns. The groups' offsets stay in the
+// words (remove_bias takes them out, and moves the carry of lo into hi).
+template <int L0, int L1, int NCOL>
 __device__ __forceinline__ void readout(uint32_t addr0, uint32_t tn, unsigned long long (&hi)[NCOL],
                                         unsigned long long (&lo)[NCOL], uint64_t* empty_bar) {
-    readout_rec<TERMS, NCOL, 0, 0>(addr0, tn, hi, lo, empty_bar);
-    constexpr int D = level_offset(TERMS);
-    constexpr unsigned long long bh = magic_bias(0, TERMS, true, D), bl = magic_bias(0, TERMS, false, D);
+    if constexpr (L0 < L1) {
+        uint32_t r[is_pair(L0, L1) ? 2 : 1][16];
+        tmem_ld_group(addr0 + (uint32_t)L0 * tn, tn, r);
+        tmem_ld_wait_regs(r);
+        readout_rec<L0, L1, NCOL, 0, L0>(addr0, tn, hi, lo, empty_bar, r);
+    }
+}
+
+// Removes the offsets of n0 readouts of the lower set and n1 of the upper one, and moves the
+// carry of lo into hi (0 <= lo < 2^40 afterwards). A readout adds less than 2^57 to |lo|, so every
+// kCarryChunks readouts is enough.
+constexpr int kCarryChunks = 32;
+struct MagicBias {
+    unsigned long long lower[11], upper_hi[11], upper_lo[11];   // the lower set lies in hi
+};
+__host__ __device__ constexpr MagicBias make_magic_bias() {
+    MagicBias m{};
+    for (int t = 1; t <= 10; ++t) {
+        m.lower[t] = magic_bias(0, level_split(t), true);
+        m.upper_hi[t] = magic_bias(level_split(t), t, true);
+        m.upper_lo[t] = magic_bias(level_split(t), t, false);
+    }
+    return m;
+}
+__constant__ MagicBias kMagicBias = make_magic_bias();
+
+template <int NCOL>
+__device__ __forceinline__ void remove_bias(int terms, int n0, int n1, unsigned long long (&hi)[NCOL],
+                                            unsigned long long (&lo)[NCOL]) {
+    const unsigned long long bh = kMagicBias.lower[terms] * (unsigned)n0 + kMagicBias.upper_hi[terms] * (unsigned)n1;
+    const unsigned long long bl = kMagicBias.upper_lo[terms] * (unsigned)n1;
 #pragma unroll
     for (int j = 0; j < NCOL; ++j) {
         hi[j] -= bh;
@@ -329,20 +445,28 @@ __device__ __forceinline__ void readout(uint32_t addr0, uint32_t tn, unsigned lo
     }
 }
 
-template <int NCOL>
-__device__ __forceinline__ void readout_terms(int terms, uint32_t addr0, uint32_t tn, unsigned long long (&hi)[NCOL],
-                                              unsigned long long (&lo)[NCOL], uint64_t* empty_bar) {
-    switch (terms) {
-        case 1: readout<1, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        case 2: readout<2, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        case 3: readout<3, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        case 4: readout<4, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        case 5: readout<5, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        case 6: readout<6, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        case 7: readout<7, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        case 8: readout<8, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        case 9: readout<9, NCOL>(addr0, tn, hi, lo, empty_bar); break;
-        default: readout<10, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+// A readout of the lower (UPPER = false) or upper set of a product of `terms` levels.
+template <int NCOL, bool UPPER, int T = 1>
+__device__ __forceinline__ void readout_set(int terms, uint32_t addr0, uint32_t tn, unsigned long long (&hi)[NCOL],
+                                            unsigned long long (&lo)[NCOL], uint64_t* empty_bar) {
+    if constexpr (!UPPER) {                    // 1, 2 or 4 levels whatever the product's
+        switch (level_split(terms)) {
+            case 1: readout<0, 1, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            case 2: readout<0, 2, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            default: readout<0, 4, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+        }
+    } else {
+        switch (terms) {
+            case 3: readout<2, 3, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            case 4: readout<2, 4, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            case 5: readout<2, 5, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            case 6: readout<4, 6, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            case 7: readout<4, 7, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            case 8: readout<4, 8, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            case 9: readout<4, 9, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            case 10: readout<4, 10, NCOL>(addr0, tn, hi, lo, empty_bar); break;
+            default: break;
+        }
     }
 }
 
@@ -502,10 +626,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) sliced_gemm_kernel(SgDev p) {
             for (int j = 0; j < TN; ++j) {
                 const int gj = j0 + j;
                 if (gj >= p.N || (p.lower_only && gj > i)) continue;
-                const double v =
-                    words_to_double(hi[j], lo[j], ea + (p.eb ? p.eb[gj] : 0) - 86 + 8 * level_offset(p.terms));
+                const int e = ea + (p.eb ? p.eb[gj] : 0) - 86 + 8 * level_offset(p.terms);
+                const double cin = p.bmode ? p.Cin[(int64_t)i * p.cin_rs + (int64_t)gj * p.cin_cs] : 0.0;
                 p.C[row * p.c_rs + (int64_t)gj * p.c_cs] =
-                    epilogue_value(v, p.amode, p.alpha, p.bmode, p.beta, p.Cin + (int64_t)i * p.cin_rs + (int64_t)gj * p.cin_cs);
+                    p.bmode ? entry_value_words<true>(hi[j], lo[j], e, p.amode, p.alpha, p.bmode, p.beta, cin)
+                            : entry_value_words<false>(hi[j], lo[j], e, p.amode, p.alpha, 0, 0.0, 0.0);
             }
         }
     }
@@ -538,10 +663,15 @@ __global__ void sliced_reduce_kernel(SgReduceDev r) {
     }
     // all 128 bits: the sum of the splits may exceed what one split's hi word can hold
     const int e = (r.ea ? r.ea[i] : 0) + (r.eb ? r.eb[j] : 0) + r.eoff;
-    const double v = u128_to_double((unsigned long long)(acc >> 64), (unsigned long long)acc, e);
+    const uint32_t w0 = (uint32_t)acc, w1 = (uint32_t)(acc >> 32), w2 = (uint32_t)(acc >> 64), w3 = (uint32_t)(acc >> 96);
     const int64_t row = r.crow ? (int64_t)r.crow[i] : (int64_t)i;
-    r.C[row * r.c_rs + (int64_t)j * r.c_cs] =
-        epilogue_value(v, r.amode, r.alpha, r.bmode, r.beta, r.Cin + (int64_t)i * r.cin_rs + (int64_t)j * r.cin_cs);
+    double& out = r.C[row * r.c_rs + (int64_t)j * r.c_cs];
+    if (r.bmode == 0) {
+        out = entry_value<false>(w0, w1, w2, w3, e, r.amode, r.alpha, 0, 0.0, 0.0);
+    } else {
+        const double cin = r.Cin[(int64_t)i * r.cin_rs + (int64_t)j * r.cin_cs];
+        out = entry_value<true>(w0, w1, w2, w3, e, r.amode, r.alpha, r.bmode, r.beta, cin);
+    }
 }
 
 
@@ -549,27 +679,44 @@ __global__ void sliced_reduce_kernel(SgReduceDev r) {
 // Pipelined form (sliced_gemm2_kernel): TMA loads, warp specialisation, windowed B.
 //
 // The digit planes of the B operand for one K block are loaded by a single 3-D TMA box
-// (64 k x 32 rows x sb planes) and lie back to back in shared memory, so that "B planes
-// q = 0..w-1" is one contiguous N = 32 w operand. One MMA per (A plane p, 16-k step)
-// then forms every pair (p, q), q < min(sb, terms - p), at once, writing level p + q to
-// TMEM columns (p + q) * 32: the D address is offset by p * 32 columns. The first MMA of
-// a 128-k chunk (p = 0) covers every level (terms <= sb is required), so it alone
-// carries accumulate = 0. Warp 0 issues the TMA loads into a ring of A-plane stages and
-// a ring of B-plane stages; warp 1 issues the MMAs and commits each stage back to its
-// producer; warps 2-9 (two per TMEM lane quarter, 16 columns each) read the level sums of
-// each chunk from TMEM (double-buffered when 2 * terms * 32 <= 512 columns), hand the
-// buffer back as soon as the values are in registers, and fold them into the same int64
+// (64 k x tn rows x sb planes) and lie back to back in shared memory, so that "B planes
+// q0 .. q0 + w - 1" is one contiguous N = w tn operand. One MMA per (A plane p, 16-k step) then
+// forms every pair (p, q) of a range of levels p + q at once, writing level g to TMEM columns
+// g * tn.
+//
+// Every K block is issued in two phases: first the pairs of the lower levels (below level_split,
+// four of them from 5 levels up), plane by plane, then those of the upper ones. The two level
+// sets have accumulators, barriers and readout periods of their own: when a set's period ends, the
+// epilogue reads it while the tensor cores work on the other set's phase. So the readout
+// is hidden without a second accumulator buffer, and 64-row B tiles, which take all 512 TMEM
+// columns at 8 levels and move a third fewer operand bytes per flop than 32-row ones, cost no wait
+// at all. The lower levels hold at most four digit pairs per k and are read every 256 k, the
+// upper ones every 128 (period_for). Splitting a K block's MMAs adds none at 7 levels (11 against
+// 10 of the same total width) and narrows few.
+// Before, the MMAs waited for each readout of a single set, or 32-row tiles kept two: 2048 x 32768 x
+// 2048 with 7 x 7 digits 7.73 -> 4.45 ms (1.73 PFLOP/s of digit pairs), 256 x 4096 x 8192 523 -> 333 us,
+// 512 x 65536 x 512 773 -> 660 us, 65536 x 64 x 512 with 9 x 9 232 -> 179 us, 2048 x 256 x 65536 with
+// 10 x 10 3.92 -> 2.71 ms. Measured and not kept: two accumulators per set where they fit (the
+// issuing warp slows more than the overlap gives), and fetching operands into L2 three to six K
+// blocks ahead (the loads' own rate is the limit: 512 x 64 x 65536 130 -> 166 us).
+//
+// Warp 0 issues the TMA loads into a ring of A planes and a ring of B-plane stages; warp 1
+// issues the MMAs and commits each plane or stage back to its producer (an A plane after its
+// second use); warps 4-11 (two per TMEM lane quarter, 16 or 32 columns each) read the level sums,
+// hand the set back as soon as the values are in registers, and fold them into the same int64
 // words as the synchronous form. Every mbarrier wait is bounded; expiry raises RTPROJ_ETIMEOUT.
 // =====================================================================================
 constexpr int W_EPI_WARPS = 8;                  // two per TMEM lane quarter, 16 columns each
-constexpr int W_THREADS = 64 + 32 * W_EPI_WARPS;
+// Three warpgroups: warps 0 and 1 load and issue (2 and 3 idle), warps 4-11 read and fold. The
+// first hands registers to the others: 128 x 56 + 256 x 224 = 384 x 168, the launch's total (an
+// epilogue thread of a 64-row tile holds 128 words of sums and two 32-value groups).
+constexpr int W_THREADS = 128 + 32 * W_EPI_WARPS;
+constexpr int W_REGS_ISSUE = 56, W_REGS_EPI = 224;
 constexpr int W_MAX_A_STAGES = 16;
 constexpr int W_MAX_B_STAGES = 8;
-constexpr int A_PPS = 2;                       // A planes per pipeline slot (one TMA box, one barrier)
-constexpr int A_SLOT_BYTES = A_PPS * A_PLANE_BYTES;
-
 struct Sg2Dev {
-    int M, N, Kp, sa, sb, terms, k_per_split, chunk_kb, splits;
+    int M, N, Kp, sa, sb, terms, k_per_split, splits;
+    int period[2];                // K blocks between readouts of the lower and the upper levels
     int eoff;                     // -86 + 8 level_offset(terms) = -78: exponent of the output words
     const int32_t* ea; const int32_t* eb;
     long long* part;
@@ -581,7 +728,7 @@ struct Sg2Dev {
     int* status;
     long long timeout;
     uint32_t tmem_cols;
-    int acc_bufs, a_stages, b_stages;
+    int a_stages, b_stages;
     int tn;                       // B rows per tile: 32 or 64
     int m_fast;                   // tile order: A-row tiles fastest
     int vec2;                     // C rows contiguous and 16-byte aligned: paired stores
@@ -721,59 +868,135 @@ struct TileSched {
     }
 };
 
-// Epilogue role of one warp: NCOL = tn / 2 columns of each tile, for TMEM lanes
-// 32 * quarter ... + 31 (tile rows), chunk by chunk, then the tile's partial words or its
-// final values.
-// The MMA issuer's work on one k block for a fixed digit configuration (SA A planes,
-// TERMS levels, TN B rows per level): A slots SLOT, SLOT+1, ... are awaited in turn and
-// each of their planes pa meets B levels 0 .. TERMS-pa-1 in windows of 256/TN levels, four
-// K steps of 16. Plane, window and K offsets, instruction descriptors and the accumulate
-// flag are compile-time constants, so between two MMAs the issuing warp only adds a
-// constant to a base: with the general loop's run-time bounds the issue path, not the
-// tensor pipe, set the pace for windows narrower than 256 columns. Returns false on abort.
-template <int SA, int TERMS, int TN, int SLOT = 0>
+// The MMA issuer's state for one of the two level sets (lower, upper): K blocks since the set's
+// accumulators were last started, the phase of its barriers, and whether it has been read once.
+struct LevelSet {
+    int kc = 0;
+    uint32_t phase = 0;
+    bool used = false;
+};
+
+// Waits until the epilogue has taken the set's previous sums, when this K block starts new ones.
+__device__ __forceinline__ bool set_ready(LevelSet& ls, uint64_t* tempty, volatile int* abort_v, const Sg2Dev& p) {
+    if (ls.kc != 0) return true;
+    if (ls.used && !wait_phase_warp(tempty, ls.phase ^ 1u, abort_v, p.status, p.timeout)) return false;
+    tc_fence_after();
+    return true;
+}
+// Ends the set's part of a K block: at the end of its period, or of the tile, its sums are handed
+// to the epilogue.
+__device__ __forceinline__ void set_done(LevelSet& ls, uint64_t* tfull, int period, bool last_kb) {
+    if (++ls.kc == period || last_kb) {
+        umma_commit_lane0(tfull);
+        ls.phase ^= 1u;
+        ls.used = true;
+        ls.kc = 0;
+    }
+}
+
+// The MMA issuer's work on one K block for a fixed digit configuration (SA A planes, TERMS
+// levels, TN B rows per level): plane, window and K offsets, instruction descriptors and the
+// accumulate flag are compile-time constants, so between two MMAs the issuing warp only adds a
+// constant to a base: with the general loop's run-time bounds the issue path, not the tensor
+// pipe, set the pace. Returns false on abort.
+template <int SA, int TERMS, int TN>
 __device__ __forceinline__ bool issue_kblock(Ring& ra, uint32_t a_lo0, uint32_t b_lo, uint32_t desc_hi, uint32_t dbase,
-                                             uint32_t acc0, uint64_t* fullA, uint64_t* emptyA, volatile int* abort_v,
-                                             const Sg2Dev& p) {
-    constexpr int WMAX = 256 / TN;
-    constexpr uint32_t B_WIN = (uint32_t)WMAX * (uint32_t)((TN * KB * 2) >> 4);
-    const int as = ra.idx;
-    if (!wait_phase_warp(fullA + as, ra.phase, abort_v, p.status, p.timeout)) return false;
-    const uint32_t a_slot = a_lo0 + (uint32_t)as * (A_SLOT_BYTES >> 4);
+                                             LevelSet (&sets)[2], bool last_kb, uint64_t* fullA, uint64_t* emptyA,
+                                             uint64_t* tfull, uint64_t* tempty, volatile int* abort_v, const Sg2Dev& p) {
+    constexpr int S = level_split(TERMS);
+    Ring r = ra;
 #pragma unroll
-    for (int q = 0; q < A_PPS; ++q) {
-        const int pa = SLOT * A_PPS + q;
-        if (pa < SA) {
-            const int nwin = TERMS - pa;
+    for (int ph = 0; ph < (TERMS > S ? 2 : 1); ++ph) {
+        constexpr int kOnlyPhase = TERMS > S ? 0 : 1;
+        const int lo_level = ph == 0 ? 0 : S, hi_level = ph == 0 ? S : TERMS;
+        if (!set_ready(sets[ph], tempty + ph, abort_v, p)) return false;
+        const uint32_t acc0 = sets[ph].kc == 0 ? 0u : 1u;
+        Ring q = ra;
 #pragma unroll
-            for (int w0 = 0; w0 < nwin; w0 += WMAX) {
-                const int nw = (nwin - w0) < WMAX ? (nwin - w0) : WMAX;
-                const uint32_t id = idesc_bf16(TM, nw * TN);
-                const uint32_t d = dbase + (uint32_t)((pa + w0) * TN);
+        for (int pa = 0; pa < SA; ++pa) {
+            if (pa < hi_level) {
+                const int as = q.idx;
+                if (!wait_phase_warp(fullA + as, q.phase, abort_v, p.status, p.timeout)) return false;
+                uint32_t a_slot = a_lo0 + (uint32_t)as * (A_PLANE_BYTES >> 4);
+                uint32_t b = b_lo, d0 = dbase;
+                // opaque bases: the constants are added where they are used, not kept in registers
+                // across the configurations (the issuing warp has W_REGS_ISSUE of them)
+                asm volatile("" : "+r"(a_slot), "+r"(b), "+r"(d0));
+                const int l0 = pa > lo_level ? pa : lo_level;
+                const uint32_t id = idesc_bf16(TM, (hi_level - l0) * TN);
+                const uint32_t d = d0 + (uint32_t)(l0 * TN);
+                b += (uint32_t)((l0 - pa) * TN * 8);
 #pragma unroll
                 for (int kk = 0; kk < KB / 16; ++kk) {
-                    const uint64_t ad = make_desc(a_slot + (uint32_t)(q * (A_PLANE_BYTES >> 4) + 2 * kk), desc_hi);
-                    const uint64_t bd = make_desc(b_lo + (uint32_t)w0 / WMAX * B_WIN + (uint32_t)(2 * kk), desc_hi);
+                    const uint64_t ad = make_desc(a_slot + (uint32_t)(2 * kk), desc_hi);
+                    const uint64_t bd = make_desc(b + (uint32_t)(2 * kk), desc_hi);
                     if (pa == 0 && kk == 0) umma_bf16_lane0(d, ad, bd, id, acc0);
                     else umma_bf16_lane0_acc(d, ad, bd, id);
                 }
+                if (ph == 1 || kOnlyPhase) umma_commit_lane0(emptyA + as);
+                q.next();
             }
         }
+        r = q;
+        set_done(sets[ph], tfull + ph, p.period[ph], last_kb);
     }
-    umma_commit_lane0(emptyA + as);
-    ra.next();
-    constexpr int NSLOTS = (SA + A_PPS - 1) / A_PPS;
-    if constexpr (SLOT + 1 < NSLOTS)
-        return issue_kblock<SA, TERMS, TN, SLOT + 1>(ra, a_lo0, b_lo, desc_hi, dbase, acc0, fullA, emptyA, abort_v, p);
-    else
-        return true;
+    ra = r;
+    return true;
+}
+
+// The same for any digit counts (sa <= terms).
+__device__ __forceinline__ bool issue_kblock_any(Ring& ra, uint32_t a_lo0, uint32_t b_lo, uint32_t desc_hi,
+                                                 uint32_t dbase, LevelSet (&sets)[2], bool last_kb, uint64_t* fullA,
+                                                 uint64_t* emptyA, uint64_t* tfull, uint64_t* tempty,
+                                                 volatile int* abort_v, const Sg2Dev& p) {
+    const int S = level_split(p.terms), phases = p.terms > S ? 2 : 1;
+    Ring r = ra;
+#pragma unroll
+    for (int ph = 0; ph < 2; ++ph) {
+        if (ph >= phases) break;
+        const int lo_level = ph == 0 ? 0 : S, hi_level = ph == 0 ? S : p.terms;
+        if (!set_ready(sets[ph], tempty + ph, abort_v, p)) return false;
+        const uint32_t acc0 = sets[ph].kc == 0 ? 0u : 1u;
+        Ring q = ra;
+#pragma unroll 1
+        for (int pa = 0; pa < p.sa && pa < hi_level; ++pa) {
+            const int as = q.idx;
+            if (!wait_phase_warp(fullA + as, q.phase, abort_v, p.status, p.timeout)) return false;
+            const uint32_t a_slot = a_lo0 + (uint32_t)as * (A_PLANE_BYTES >> 4);
+            const int l0 = pa > lo_level ? pa : lo_level;
+            const uint32_t id = idesc_bf16(TM, (hi_level - l0) * p.tn);
+            const uint32_t d = dbase + (uint32_t)(l0 * p.tn);
+            const uint32_t b = b_lo + (uint32_t)((l0 - pa) * p.tn * 8);
+#pragma unroll
+            for (int kk = 0; kk < KB / 16; ++kk)
+                umma_bf16_lane0(d, make_desc(a_slot + (uint32_t)(2 * kk), desc_hi), make_desc(b + (uint32_t)(2 * kk), desc_hi),
+                                id, pa == 0 && kk == 0 ? acc0 : 1u);
+            if (ph == phases - 1) umma_commit_lane0(emptyA + as);
+            q.next();
+        }
+        r = q;
+        set_done(sets[ph], tfull + ph, p.period[ph], last_kb);
+    }
+    ra = r;
+    return true;
 }
 
 // Configurations with a compile-time issue path (digit planes of A, levels, B rows per
-// level); issue_cfg is the position in this list plus one.
+// level); issue_cfg is the position in this list plus one. With the general loop's run-time
+// bounds the issuing warp sets the pace: without an entry here, 10 x 10 digits at 2048 x 256 x
+// 65536 took 3.92 ms (3.27 with one), 4 x 4 at 512 x 512 x 65536 (lower triangle) 240 us (180).
+#define SG2_ISSUE_CFGS(X)                                                                                   \
+    X(1, 5, 32) X(2, 5, 32) X(4, 4, 32) X(7, 7, 32) X(9, 9, 32) X(10, 10, 32)                               \
+    X(1, 5, 64) X(2, 5, 64) X(1, 6, 64) X(2, 6, 64) X(3, 3, 64) X(4, 4, 64) X(5, 5, 64) X(7, 7, 64)
 struct IssueCfg { int sa, terms, tn; };
-constexpr IssueCfg kIssueCfgs[] = {{7, 7, 32}, {9, 9, 32}, {3, 3, 64}, {1, 5, 64}, {5, 5, 64}, {7, 7, 64},
-                                   {2, 5, 64}};   // the last: the Gaussian sketch (two G planes, five of A)
+#define X(sa, terms, tn) {sa, terms, tn},
+constexpr IssueCfg kIssueCfgs[] = {SG2_ISSUE_CFGS(X)};
+#undef X
+constexpr int issue_cfg_of(int sa, int terms, int tn) {
+    for (int i = 0; i < (int)(sizeof(kIssueCfgs) / sizeof(kIssueCfgs[0])); ++i)
+        if (kIssueCfgs[i].sa == sa && kIssueCfgs[i].terms == terms && kIssueCfgs[i].tn == tn) return i + 1;
+    return 0;
+}
 
 // Running record of max |v| for the row exponent, in two integer operations per value:
 // the largest sign-cleared upper word (sign, exponent field, top 20 mantissa bits) and the
@@ -801,28 +1024,42 @@ __device__ __forceinline__ void epilogue_role(const Sg2Dev& p, uint32_t tmem, ui
     const TileSched ts{(p.M + TM - 1) / TM, (p.N + tn - 1) / tn, tn, p.lower_only, p.m_fast};
     const int per_z = ts.per_split();
     const int ntiles = per_z * p.splits;
-    const int cb = p.chunk_kb;
-    const uint32_t buf_cols = (uint32_t)(p.terms * tn);
-    Ring tr(p.acc_bufs);
+    const bool two = p.terms > level_split(p.terms);
+    uint32_t ph0 = 0u, ph1 = 0u;                    // phases of the two sets' full barriers
     bool ok = true;
     for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
         const TileCoord c = ts.at(tile, per_z);
         const int kbeg = c.z * p.k_per_split;
         const int nkb = (min(p.Kp, kbeg + p.k_per_split) - kbeg) / KB;
-        const int nchunks = (nkb + cb - 1) / cb;
         unsigned long long hi[NCOL], lo[NCOL];
 #pragma unroll
         for (int j = 0; j < NCOL; ++j) { hi[j] = 0; lo[j] = 0; }
-        for (int cc = 0; cc < nchunks; ++cc, tr.next()) {
-            const int buf = tr.idx;
-            if (!wait_phase(tfull + buf, tr.phase, abort_v, p.status, p.timeout)) {
-                ok = false;
-                break;
+        const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * NCOL);
+        int c0 = 0, c1 = 0;                         // K blocks since each set's last readout
+        int n0 = 0, n1 = 0;                         // readouts whose offsets are still in the words
+#pragma unroll 1
+        for (int kb = 0; kb < nkb; ++kb) {
+            const bool last = kb == nkb - 1;
+            if (++c0 == p.period[0] || last) {
+                if (!wait_phase(tfull, ph0, abort_v, p.status, p.timeout)) { ok = false; break; }
+                tc_fence_after();
+                readout_set<NCOL, false>(p.terms, base, (uint32_t)tn, hi, lo, tempty);
+                ph0 ^= 1u;
+                c0 = 0;
+                ++n0;
             }
-            tc_fence_after();
-            const uint32_t base =
-                tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * buf_cols + (uint32_t)(half * NCOL);
-            readout_terms<NCOL>(p.terms, base, (uint32_t)tn, hi, lo, tempty + buf);
+            if (two && (++c1 == p.period[1] || last)) {
+                if (!wait_phase(tfull + 1, ph1, abort_v, p.status, p.timeout)) { ok = false; break; }
+                tc_fence_after();
+                readout_set<NCOL, true>(p.terms, base, (uint32_t)tn, hi, lo, tempty + 1);
+                ph1 ^= 1u;
+                c1 = 0;
+                ++n1;
+            }
+            if (n0 == kCarryChunks || n1 == kCarryChunks || last) {
+                remove_bias<NCOL>(p.terms, n0, n1, hi, lo);
+                n0 = n1 = 0;
+            }
         }
         if (!ok) break;
         const int i = c.i0 + quarter * 32 + lane;
@@ -843,88 +1080,61 @@ __device__ __forceinline__ void epilogue_role(const Sg2Dev& p, uint32_t tmem, ui
             const int64_t row = p.crow && valid ? (int64_t)p.crow[i] : (int64_t)i;
             double* crow_p = p.C + row * p.c_rs;
             const double* cin_p = p.Cin + (int64_t)i * p.cin_rs;
+            // NE columns at a time in a rolled loop (the words are rotated down after each turn): the
+            // conversions are about 60 instructions each, and fetching their unrolled code took most of
+            // the time of a product of a few tiles (64 x 16 x 64: 33 -> 18 us with the shorter readout)
+            uint32_t mxh = 0, orl = 0;             // the stored values' largest magnitude (track_abs_max)
+            // Cin is read in full ahead of the stores: C may alias Cin (an update in place), so a load
+            // placed after a store would wait for the previous element's whole round trip
+            double cv[NCOL];
+            if (p.bmode != 0) {
+#pragma unroll
+                for (int q = 0; q < NCOL; ++q) {
+                    const int gj = jb + q;
+                    cv[q] = (valid && gj < p.N && !(p.lower_only && gj > i)) ? __ldcg(cin_p + (int64_t)gj * p.cin_cs) : 0.0;
+                }
+            }
+            auto turn = [&](auto ne_tag, auto cin_tag, int j0) {
+                constexpr int NE = decltype(ne_tag)::value;
+                constexpr bool CIN = decltype(cin_tag)::value;
+#pragma unroll
+                for (int q = 0; q < NE; q += 2) {
+                    const int gj = jb + j0 + q;
+                    const int e0 = __shfl_sync(0xffffffffu, ebl, j0 + q), e1 = __shfl_sync(0xffffffffu, ebl, j0 + q + 1);
+                    const bool s0 = valid && gj < p.N && !(p.lower_only && gj > i);
+                    const bool s1 = valid && gj + 1 < p.N && !(p.lower_only && gj + 1 > i);
+                    const double v0 = entry_value_words<CIN>(
+                        (long long)hi[q], (long long)lo[q], ea + e0, p.amode, p.alpha, p.bmode, p.beta, cv[q]);
+                    const double v1 = entry_value_words<CIN>(
+                        (long long)hi[q + 1], (long long)lo[q + 1], ea + e1, p.amode, p.alpha, p.bmode, p.beta, cv[q + 1]);
+                    if (!CIN && s0) track_abs_max(v0, mxh, orl);
+                    if (!CIN && s1) track_abs_max(v1, mxh, orl);
+                    if (p.vec2 && s0 && s1) {      // row-contiguous output: two columns as one 16-byte store
+                        *reinterpret_cast<double2*>(crow_p + gj) = make_double2(v0, v1);
+                    } else {
+                        if (s0) crow_p[(int64_t)gj * p.c_cs] = v0;
+                        if (s1) crow_p[(int64_t)(gj + 1) * p.c_cs] = v1;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q + NE < NCOL; ++q) {
+                    hi[q] = hi[q + NE];
+                    lo[q] = lo[q + NE];
+                    if (CIN) cv[q] = cv[q + NE];
+                }
+            };
             if (p.bmode == 0) {
-                // no Cin: the stores follow the conversions directly
-                if (p.vec2) {
-                    // row-contiguous output: pairs of columns as one 16-byte store; with row_exp
-                    // the stored values' maximum magnitude is recorded (track_abs_max)
-                    uint32_t mxh = 0, orl = 0;
-#pragma unroll
-                    for (int j = 0; j < NCOL; j += 2) {
-                        const int gj = jb + j;
-                        const int e0 = __shfl_sync(0xffffffffu, ebl, j), e1 = __shfl_sync(0xffffffffu, ebl, j + 1);
-                        if (!valid || gj >= p.N || (p.lower_only && gj > i)) continue;
-                        const double v0 = epilogue_value_v(words_to_double((long long)hi[j], (long long)lo[j], ea + e0),
-                                                           p.amode, p.alpha, 0, 0.0, 0.0);
-                        track_abs_max(v0, mxh, orl);
-                        if (gj + 1 < p.N && !(p.lower_only && gj + 1 > i)) {
-                            const double v1 = epilogue_value_v(
-                                words_to_double((long long)hi[j + 1], (long long)lo[j + 1], ea + e1), p.amode,
-                                p.alpha, 0, 0.0, 0.0);
-                            track_abs_max(v1, mxh, orl);
-                            *reinterpret_cast<double2*>(crow_p + gj) = make_double2(v0, v1);
-                        } else {
-                            crow_p[gj] = v0;
-                        }
-                    }
-                    if (p.row_exp && valid) {
-                        if (mxh >= 0x7FF00000u) set_status(p.status, RTPROJ_ENONFINITE);
-                        else if ((mxh | orl) != 0) atomicMax(p.row_exp + row, frexp_exponent_of_words(mxh, orl));
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < NCOL; ++j) {
-                        const int gj = jb + j;
-                        const int ej = __shfl_sync(0xffffffffu, ebl, j);
-                        if (!valid || gj >= p.N || (p.lower_only && gj > i)) continue;
-                        crow_p[(int64_t)gj * p.c_cs] = epilogue_value_v(
-                            words_to_double((long long)hi[j], (long long)lo[j], ea + ej), p.amode, p.alpha, 0, 0.0, 0.0);
-                    }
+#pragma unroll 1
+                for (int j0 = 0; j0 < NCOL; j0 += 4)
+                    turn(std::integral_constant<int, 4>{}, std::false_type{}, j0);
+                if (p.row_exp && valid) {
+                    if (mxh >= 0x7FF00000u) set_status(p.status, RTPROJ_ENONFINITE);
+                    else if ((mxh | orl) != 0) atomicMax(p.row_exp + row, frexp_exponent_of_words(mxh, orl));
                 }
             } else {
-                // Cin is read eight entries ahead of the stores, in groups: C may alias Cin (an
-                // update in place), so a load placed after a store would wait for the previous
-                // element's whole round trip
-                constexpr int CG = 8;
-#pragma unroll
-                for (int g0 = 0; g0 < NCOL; g0 += CG) {
-                    double cv[CG];
-#pragma unroll
-                    for (int q = 0; q < CG; ++q) {
-                        const int gj = jb + g0 + q;
-                        cv[q] = (p.bmode != 0 && valid && gj < p.N && !(p.lower_only && gj > i))
-                                    ? __ldcg(cin_p + (int64_t)gj * p.cin_cs) : 0.0;
-                    }
-                    if (p.vec2) {
-                        // row-contiguous output: pairs of columns as one 16-byte store
-#pragma unroll
-                        for (int q = 0; q < CG; q += 2) {
-                            const int j = g0 + q, gj = jb + j;
-                            const int e0 = __shfl_sync(0xffffffffu, ebl, j), e1 = __shfl_sync(0xffffffffu, ebl, j + 1);
-                            if (!valid || gj >= p.N || (p.lower_only && gj > i)) continue;
-                            const double v0 = epilogue_value_v(words_to_double((long long)hi[j], (long long)lo[j], ea + e0),
-                                                               p.amode, p.alpha, p.bmode, p.beta, cv[q]);
-                            if (gj + 1 < p.N && !(p.lower_only && gj + 1 > i)) {
-                                const double v1 = epilogue_value_v(
-                                    words_to_double((long long)hi[j + 1], (long long)lo[j + 1], ea + e1), p.amode,
-                                    p.alpha, p.bmode, p.beta, cv[q + 1]);
-                                *reinterpret_cast<double2*>(crow_p + gj) = make_double2(v0, v1);
-                            } else {
-                                crow_p[gj] = v0;
-                            }
-                        }
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < CG; ++q) {
-                            const int j = g0 + q, gj = jb + j;
-                            const int ej = __shfl_sync(0xffffffffu, ebl, j);
-                            if (!valid || gj >= p.N || (p.lower_only && gj > i)) continue;
-                            crow_p[(int64_t)gj * p.c_cs] =
-                                epilogue_value_v(words_to_double((long long)hi[j], (long long)lo[j], ea + ej), p.amode,
-                                                 p.alpha, p.bmode, p.beta, cv[q]);
-                        }
-                    }
-                }
+#pragma unroll 1
+                for (int j0 = 0; j0 < NCOL; j0 += 4)
+                    turn(std::integral_constant<int, 4>{}, std::true_type{}, j0);
             }
         }
     }
@@ -940,7 +1150,7 @@ __global__ void __launch_bounds__(W_THREADS, 1)
     const uint32_t b_plane_bytes = (uint32_t)tn * KB * 2;
     const uint32_t b_stage_bytes = (uint32_t)p.sb * b_plane_bytes;
     unsigned char* sA = smem;
-    unsigned char* sB = sA + (size_t)AS * A_SLOT_BYTES;
+    unsigned char* sB = sA + (size_t)AS * A_PLANE_BYTES;
     uint64_t* bars = (uint64_t*)(sB + (size_t)BSN * b_stage_bytes);
     uint64_t* fullA = bars;
     uint64_t* emptyA = fullA + W_MAX_A_STAGES;
@@ -955,8 +1165,6 @@ __global__ void __launch_bounds__(W_THREADS, 1)
     const TileSched ts{(p.M + TM - 1) / TM, (p.N + tn - 1) / tn, tn, p.lower_only, p.m_fast};
     const int per_z = ts.per_split();
     const int ntiles = per_z * p.splits;
-    const int cb = p.chunk_kb;
-    const uint32_t buf_cols = (uint32_t)(p.terms * tn);
 
     if (t == 0) {
         abort_s = 0;
@@ -977,6 +1185,8 @@ __global__ void __launch_bounds__(W_THREADS, 1)
 
     // Every role walks the same tile sequence (blockIdx.x, + gridDim.x, ...), skipping the
     // tiles strictly above the diagonal when only the lower triangle is wanted.
+    if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(W_REGS_ISSUE));
     if (warp == 0) {
         // ---------------- TMA producer (whole warp, lane 0 issues)
         Ring ra(AS), rb(BSN);
@@ -995,15 +1205,14 @@ __global__ void __launch_bounds__(W_THREADS, 1)
                 tma_load_3d_lane0(smem_addr(sB + (size_t)bs * b_stage_bytes), &tmB, k0, c.j0, 0, fullB + bs,
                                   b_stage_bytes);
                 rb.next();
-                for (int pa = 0; pa < p.sa; pa += A_PPS) {
-                    // A_PPS planes per slot; a plane past the stack reads as zeros (no MMA uses it)
+                for (int pa = 0; pa < p.sa; ++pa) {
                     const int as = ra.idx;
                     if (ra.wrapped && !wait_phase_warp(emptyA + as, ra.phase ^ 1u, abort_v, p.status, p.timeout)) {
                         ok = false;
                         break;
                     }
-                    tma_load_3d_lane0(smem_addr(sA + (size_t)as * A_SLOT_BYTES), &tmA, k0, c.i0, pa, fullA + as,
-                                      A_SLOT_BYTES);
+                    tma_load_3d_lane0(smem_addr(sA + (size_t)as * A_PLANE_BYTES), &tmA, k0, c.i0, pa, fullA + as,
+                                      A_PLANE_BYTES);
                     ra.next();
                 }
             }
@@ -1013,90 +1222,45 @@ __global__ void __launch_bounds__(W_THREADS, 1)
         const uint64_t d0desc = sw128_desc(smem_addr(sA));
         const uint32_t a_lo0 = (uint32_t)d0desc, desc_hi = (uint32_t)(d0desc >> 32);
         const uint32_t b_lo0 = (uint32_t)sw128_desc(smem_addr(sB));
-        const int wmax = 256 / tn;                                     // levels per MMA window
-        const uint32_t b_win = (uint32_t)wmax * (b_plane_bytes >> 4);  // second window's B offset
-        Ring ra(AS), rb(BSN), rt(p.acc_bufs);
-        int buf = 0;
+        Ring ra(AS), rb(BSN);
+        LevelSet sets[2];
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
             const TileCoord c = ts.at(tile, per_z);
             const int kbeg = c.z * p.k_per_split;
             const int nkb = (min(p.Kp, kbeg + p.k_per_split) - kbeg) / KB;
-            int kc = 0;                                  // k blocks into the current chunk
             for (int kb = 0; kb < nkb && ok; ++kb) {
-                const bool chunk_start = kc == 0;
-                if (chunk_start) {
-                    buf = rt.idx;
-                    if (rt.wrapped && !wait_phase_warp(tempty + buf, rt.phase ^ 1u, abort_v, p.status, p.timeout)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                }
+                const bool last_kb = kb == nkb - 1;
                 const int bs = rb.idx;
                 if (!wait_phase_warp(fullB + bs, rb.phase, abort_v, p.status, p.timeout)) {
                     ok = false;
                     break;
                 }
                 const uint32_t b_lo = b_lo0 + (uint32_t)bs * (b_stage_bytes >> 4);
-                if (p.issue_cfg > 0) {
-                    const uint32_t dbase = tmem + (uint32_t)buf * buf_cols;
-                    const uint32_t acc0 = chunk_start ? 0u : 1u;
-                    switch (p.issue_cfg) {
-                    case 1: ok = issue_kblock<7, 7, 32>(ra, a_lo0, b_lo, desc_hi, dbase, acc0, fullA, emptyA, abort_v, p); break;
-                    case 2: ok = issue_kblock<9, 9, 32>(ra, a_lo0, b_lo, desc_hi, dbase, acc0, fullA, emptyA, abort_v, p); break;
-                    case 3: ok = issue_kblock<3, 3, 64>(ra, a_lo0, b_lo, desc_hi, dbase, acc0, fullA, emptyA, abort_v, p); break;
-                    case 4: ok = issue_kblock<1, 5, 64>(ra, a_lo0, b_lo, desc_hi, dbase, acc0, fullA, emptyA, abort_v, p); break;
-                    case 5: ok = issue_kblock<5, 5, 64>(ra, a_lo0, b_lo, desc_hi, dbase, acc0, fullA, emptyA, abort_v, p); break;
-                    case 6: ok = issue_kblock<7, 7, 64>(ra, a_lo0, b_lo, desc_hi, dbase, acc0, fullA, emptyA, abort_v, p); break;
-                    default: ok = issue_kblock<2, 5, 64>(ra, a_lo0, b_lo, desc_hi, dbase, acc0, fullA, emptyA, abort_v, p); break;
-                    }
-                } else
-                for (int pa0 = 0; pa0 < p.sa; pa0 += A_PPS) {
-                    const int as = ra.idx;
-                    if (!wait_phase_warp(fullA + as, ra.phase, abort_v, p.status, p.timeout)) {
-                        ok = false;
+                switch (p.issue_cfg) {
+#define X(sa, terms, tn)                                                                                             \
+    case issue_cfg_of(sa, terms, tn):                                                                                \
+        ok = issue_kblock<sa, terms, tn>(ra, a_lo0, b_lo, desc_hi, tmem, sets, last_kb, fullA, emptyA, tfull, tempty, \
+                                         abort_v, p);                                                                \
+        break;
+                    SG2_ISSUE_CFGS(X)
+#undef X
+                    default:
+                        ok = issue_kblock_any(ra, a_lo0, b_lo, desc_hi, tmem, sets, last_kb, fullA, emptyA, tfull,
+                                              tempty, abort_v, p);
                         break;
-                    }
-                    // Plane pa against B levels 0 .. nwin-1: one MMA per window of up to 256 / tn
-                    // levels (N = tn per level), at most two windows. Descriptors are built from
-                    // precomputed words: the K step adds 32 bytes (2 units) to the start address.
-#pragma unroll
-                    for (int q = 0; q < A_PPS; ++q) {
-                        const int pa = pa0 + q;
-                        const int nwin = pa < p.sa ? min(p.sb, p.terms - pa) : 0;
-                        if (nwin > 0) {
-                            const int n1 = min(wmax, nwin), n2 = nwin - n1;
-                            const uint32_t a_lo = a_lo0 + (uint32_t)as * (A_SLOT_BYTES >> 4) + (uint32_t)q * (A_PLANE_BYTES >> 4);
-                            const uint32_t d = tmem + (uint32_t)buf * buf_cols + (uint32_t)(pa * tn);
-                            const uint32_t id1 = idesc_bf16(TM, n1 * tn), id2 = idesc_bf16(TM, (n2 > 0 ? n2 : 1) * tn);
-#pragma unroll
-                            for (int kk = 0; kk < KB / 16; ++kk) {
-                                const uint32_t acc = (chunk_start && pa == 0 && kk == 0) ? 0u : 1u;
-                                const uint64_t ad = make_desc(a_lo + 2 * kk, desc_hi);
-                                umma_bf16_lane0(d, ad, make_desc(b_lo + 2 * kk, desc_hi), id1, acc);
-                                if (n2 > 0)
-                                    umma_bf16_lane0(d + 256, ad, make_desc(b_lo + b_win + 2 * kk, desc_hi), id2, acc);
-                            }
-                        }
-                    }
-                    umma_commit_lane0(emptyA + as);
-                    ra.next();
                 }
                 if (!ok) break;
                 umma_commit_lane0(emptyB + bs);
                 rb.next();
-                if (++kc == cb || kb == nkb - 1) {
-                    umma_commit_lane0(tfull + buf);
-                    rt.next();
-                    kc = 0;
-                }
             }
         }
+    }
     } else {
-        // ---------------- epilogue: warps 2..9; warp w reads TMEM lanes 32 * (w % 4) ... + 31
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(W_REGS_EPI));
+        // ---------------- epilogue: warps 4..11; warp w reads TMEM lanes 32 * (w % 4) ... + 31
         // (the lane quarter it may access) and columns tn/2 * half ... of each level.
-        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        const int quarter = warp & 3, half = (warp - 4) >> 2;
         if (tn == 64) epilogue_role<32>(p, tmem, tfull, tempty, abort_v, quarter, half, lane);
         else epilogue_role<16>(p, tmem, tfull, tempty, abort_v, quarter, half, lane);
     }
@@ -1226,16 +1390,17 @@ static cudaError_t sliced_gemm_sync(const SlicedGemm& g, void* scratch, size_t s
 }
 
 
-// Largest readout interval (128, 256 or 512 k) that keeps every level g <= 7 exact: each
-// level holds at most min(sa, sb, terms) digit pairs per k, each product at most
+// Largest readout interval (128, 256 or 512 k) that keeps every level g < min(levels, 8) exact:
+// each level holds at most min(sa, sb, levels) digit pairs per k, each product at most
 // max_digit_a * max_digit_b, and a float32 sum is exact while it stays within 2^24.
-static int chunk_for(const SlicedGemm& g) {
-    const long long pairs = std::max(1, std::min(std::min(g.a.s, g.b.s), std::min(g.terms, 8)));
+static int period_for(const SlicedGemm& g, int levels) {
+    const long long pairs = std::max(1, std::min(std::min(g.a.s, g.b.s), std::min(levels, 8)));
     const long long prod = (long long)g.a.max_digit * g.b.max_digit;
     int kc = 128;
     while (kc < 512 && pairs * (2 * kc) * prod <= (1ll << 24)) kc *= 2;
     return kc;
 }
+static int chunk_for(const SlicedGemm& g) { return period_for(g, g.terms); }
 
 // Split-K factor for a persistent grid of one CTA per SM: the number of rounds of work units
 // (tiles x splits) times the K blocks of one unit, plus a fixed cost per round (pipeline
@@ -1294,20 +1459,23 @@ cudaError_t sliced_gemm_impl(const SlicedGemm& g0, void* scratch, size_t scratch
                            g.terms <= 10 && g.terms <= g.b.s && g.b.cols == K && g.a.ld % 64 == 0 &&
                            g.b.ld % 64 == 0 && g.a.ld >= K && g.b.ld >= K;
     if (!shapes_ok || pipelined_disabled()) return sliced_gemm_sync(g, scratch, scratch_bytes, status, s);
-    // 64 B rows per tile when the levels of one accumulator set fit TMEM at that width
-    // (terms * 64 <= 512 columns) and the output is wider than 64: half the A-plane reads
-    // per flop and twice the MMA work per pipeline stage. 32 otherwise, and also when 64
-    // would leave a single TMEM accumulator set on a short contraction (K <= 1024: few
-    // chunks per tile, so the per-tile output must overlap the next tile's MMAs, which
-    // takes two sets). Both choices were measured faster where they apply.
-    const int Kp0 = (K + KB - 1) / KB * KB;
-    const bool wide_ok = g.terms * 64 <= 512 && N > 64 && (2 * g.terms * 64 <= 512 || Kp0 > 1024);
-    const int tn = wide_ok ? 64 : 32;
+    // planes past the last level form no pair that is kept
+    g.a.s = std::min(g.a.s, g.terms);
+    g.b.s = std::min(g.b.s, g.terms);
+    // 64 B rows per tile when the levels fit TMEM at that width (terms * 64 <= 512 columns): a third
+    // fewer operand bytes per flop and wider MMAs than 32-row tiles (2048 x 32768 x 2048, 7 x 7
+    // digits: 4.45 against 6.05 ms; 512 x 65536 x 512: 0.66 against 0.84). 32 rows for outputs up to
+    // 64 wide, whose large operand streams from DRAM (the smaller B stages leave more A planes in
+    // flight: 155 against 178 us for 65536 x 64 x 512), and when 64 would leave SMs without a tile
+    // (of one readout period of K at least).
+    const int kmin = 128;
+    const long long wide_units = (long long)((M + TM - 1) / TM) * ((N + 63) / 64) * ((K + kmin - 1) / kmin);
+    const int tn = g.terms * 64 <= 512 && N > 64 && wide_units >= sm_count() ? 64 : 32;
     CUtensorMap mapA, mapB;
-    if (!make_stack_map(&mapA, g.a, TM, A_PPS) || !make_stack_map(&mapB, g.b, tn, g.b.s))
+    if (!make_stack_map(&mapA, g.a, TM, 1) || !make_stack_map(&mapB, g.b, tn, g.b.s))
         return sliced_gemm_sync(g, scratch, scratch_bytes, status, s);
     const int Kp = (K + KB - 1) / KB * KB;
-    const int kchunk = chunk_for(g);
+    const int kchunk = kmin;                 // a split ends with a readout of both sets
     int kps = 0;
     const int tiles_m = (M + TM - 1) / TM, tiles_n = (N + tn - 1) / tn;
     const TileSched ts{tiles_m, tiles_n, tn, g.lower_only ? 1 : 0, tiles_m <= tiles_n ? 1 : 0};
@@ -1315,7 +1483,8 @@ cudaError_t sliced_gemm_impl(const SlicedGemm& g0, void* scratch, size_t scratch
     Sg2Dev p;
     p.M = M; p.N = N; p.Kp = Kp; p.sa = g.a.s; p.sb = g.b.s; p.terms = g.terms; p.k_per_split = kps;
     p.eoff = -86 + 8 * level_offset(g.terms);
-    p.chunk_kb = kchunk / KB;
+    p.period[0] = period_for(g, level_split(g.terms)) / KB;
+    p.period[1] = period_for(g, g.terms) / KB;
     p.ea = g.a.e; p.eb = g.b.e;
     p.part = (long long*)scratch;
     p.C = g.C; p.c_rs = g.c_rs; p.c_cs = g.c_cs; p.crow = g.crow;
@@ -1327,34 +1496,30 @@ cudaError_t sliced_gemm_impl(const SlicedGemm& g0, void* scratch, size_t scratch
     p.tn = tn;
     p.m_fast = ts.m_fast;
     p.vec2 = (g.c_cs == 1 && g.c_rs % 2 == 0 && ((uintptr_t)g.C & 15) == 0) ? 1 : 0;
-    p.issue_cfg = 0;
-    for (int i = 0; i < (int)(sizeof(kIssueCfgs) / sizeof(kIssueCfgs[0])); ++i)
-        if (kIssueCfgs[i].sa == g.a.s && kIssueCfgs[i].terms == g.terms && kIssueCfgs[i].tn == tn) p.issue_cfg = i + 1;
-    p.acc_bufs = (2 * g.terms * tn <= 512) ? 2 : 1;
+    p.issue_cfg = issue_cfg_of(g.a.s, g.terms, tn);
     p.tmem_cols = 32;
-    while (p.tmem_cols < (uint32_t)(p.acc_bufs * g.terms * tn)) p.tmem_cols <<= 1;
-    // Split shared memory between the A-plane ring (sa slots per K block) and the B-stage
+    while (p.tmem_cols < (uint32_t)(g.terms * tn)) p.tmem_cols <<= 1;
+    // Split shared memory between the A-plane ring (sa planes per K block) and the B-stage
     // ring (one stage per K block) so that the producer can run as many K blocks ahead as
     // possible: maximise min(b_stages, a_stages / sa).
     const size_t b_stage = (size_t)g.b.s * tn * KB * 2;
     const size_t fixed = 1024 + (2 * W_MAX_A_STAGES + 2 * W_MAX_B_STAGES + 4) * 8 + 16;
-    // 200 KB, not the 227 KB a CTA may take: an SM then also holds one CTA of the pivoted QR
-    // (about 23 KB), so that a step's products can run while the next step's latency-bound
-    // QR occupies the SMs
-    const size_t budget = 200 * 1024 - fixed;
+    // all of the 227 KB a CTA may take: the rings hold about one K block of A planes, and 27 KB more
+    // than the 200 KB taken before were worth 7% at 2048 x 32768 x 2048 and 12% for the sketch at
+    // 512 x 516 x 65536
+    const size_t budget = 227 * 1024 - 1024 - fixed;
     int best_bs = 0, best_as = 0;
     double best_depth = -1.0;
-    const int a_slots_per_kb = (g.a.s + A_PPS - 1) / A_PPS;
     for (int bsn = 2; bsn <= W_MAX_B_STAGES; ++bsn) {
-        if ((size_t)bsn * b_stage + 2 * A_SLOT_BYTES > budget) break;
-        const int asn = (int)std::min<size_t>(W_MAX_A_STAGES, (budget - (size_t)bsn * b_stage) / A_SLOT_BYTES);
-        const double depth = std::min<double>(bsn, (double)asn / a_slots_per_kb);
+        if ((size_t)bsn * b_stage + 5 * A_PLANE_BYTES > budget) break;      // the lower levels keep 4 planes
+        const int asn = (int)std::min<size_t>(W_MAX_A_STAGES, (budget - (size_t)bsn * b_stage) / A_PLANE_BYTES);
+        const double depth = std::min<double>(bsn, (double)asn / g.a.s);
         if (depth > best_depth + 1e-9) { best_depth = depth; best_bs = bsn; best_as = asn; }
     }
-    if (best_as < 2 || best_bs < 2) return sliced_gemm_sync(g, scratch, scratch_bytes, status, s);
+    if (best_as < 5 || best_bs < 2) return sliced_gemm_sync(g, scratch, scratch_bytes, status, s);
     p.a_stages = best_as;
     p.b_stages = best_bs;
-    const size_t smem = fixed + (size_t)best_bs * b_stage + (size_t)best_as * A_SLOT_BYTES;
+    const size_t smem = fixed + (size_t)best_bs * b_stage + (size_t)best_as * A_PLANE_BYTES;
     cudaError_t e = cudaFuncSetAttribute(sliced_gemm2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     p.splits = splits;

@@ -1,6 +1,7 @@
 // Host build of the 128-bit sums of exact products (csrc/i128.cuh) for the CPU tests: reads
 // "sum N" or "two N" and N pairs of doubles (hexadecimal), prints the rounded sum of their
-// products and the pair form; "two" forms the sum from two halves merged.
+// products and the pair form; "two" forms the sum from two halves merged. "sub N" prints x - V 2^e
+// and V 2^e, each rounded once, for 128-bit integers V.
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -8,6 +9,7 @@
 
 #define __device__
 #define __forceinline__ inline
+#define __noinline__
 static inline int __clzll(long long x) { return x ? __builtin_clzll((unsigned long long)x) : 64; }
 static inline double __longlong_as_double(long long x) {
     double d;
@@ -27,6 +29,19 @@ int main() {
     char op[16];
     int n;
     while (std::scanf("%15s %d", op, &n) == 2) {
+        if (!std::strcmp(op, "sub")) {       // n lines: x, the words of V (lowest first), e
+            for (int i = 0; i < n; ++i) {
+                double x, out = 0.0;
+                unsigned w[4];
+                int e;
+                if (std::scanf("%la %x %x %x %x %d", &x, &w[0], &w[1], &w[2], &w[3], &e) != 6) return 1;
+                uint64_t u;
+                std::memcpy(&u, &x, 8);
+                const bool ok = rtp::i128_sub_from((uint32_t)u, (uint32_t)(u >> 32), w[0], w[1], w[2], w[3], e, out);
+                std::printf("%d %a %a\n", (int)ok, out, rtp::i128_round_signed(w[0], w[1], w[2], w[3], e));
+            }
+            continue;
+        }
         rtp::i128acc a = rtp::i128_zero(), b = rtp::i128_zero();
         const bool two = op[0] == 't';
         for (int i = 0; i < n; ++i) {

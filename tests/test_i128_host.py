@@ -25,6 +25,12 @@ def i128(tmp_path_factory):
                     os.path.join(ROOT, "tests", "i128_host_check.cpp"), "-o", exe], check=True)
 
     def run(op, xs, ys):
+        if op == "sub":
+            text = f"sub {len(xs)}\n" + "\n".join(
+                f"{x.hex()} " + " ".join("%x" % ((v >> (32 * i)) & 0xFFFFFFFF) for i in range(4)) + f" {e}"
+                for x, (v, e) in zip(xs, ys)) + "\n"
+            out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True)
+            return [(int(a), float.fromhex(b), float.fromhex(c)) for a, b, c in map(str.split, out.stdout.splitlines())]
         text = f"{op} {len(xs)}\n" + "\n".join(f"{x.hex()} {y.hex()}" for x, y in zip(xs, ys)) + "\n"
         out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True)
         return [float.fromhex(v) for v in out.stdout.split()]
@@ -62,3 +68,35 @@ def test_sum_of_products(i128, op, kind, n):
         assert abs(F(hi) + F(lo) - exact) <= bound + abs(exact) / 2 ** 105 + F(1, 2 ** 1074)
         assert abs(F(got) - exact) <= bound + abs(exact) / 2 ** 53 + F(1, 2 ** 1074)
         assert abs(lo) <= abs(hi) * 2.0 ** -51 or hi == 0.0
+
+
+def test_rounding_and_difference(i128):
+    """V 2^e is rounded to the nearest double, ties to even, and x - V 2^e is the exact
+    difference rounded once wherever the two units lie close enough for it to be taken (always
+    when x's last place is within 22 bits below and 63 above V's unit)."""
+    rng = np.random.default_rng(9)
+    xs, vs = [], []
+    for i in range(4000):
+        bits = int(rng.integers(1, 104))
+        v = int.from_bytes(rng.bytes(16), "little") >> (128 - bits)
+        if i % 5 == 0 and bits > 54:                     # exact ties and their neighbours
+            v = (v >> (bits - 53) << (bits - 53)) + (1 << (bits - 54)) + int(rng.integers(-1, 2))
+        v = -v if rng.random() < 0.5 else v
+        e = int(rng.integers(-200, 100))
+        x = float(rng.standard_normal()) * 2.0 ** (e + int(rng.integers(-30, 130)))
+        if i % 7 == 0:
+            x = float(F(v) * F(2) ** e) * (1 + 2.0 ** -52 * int(rng.integers(-2, 3)))   # cancels
+        xs.append(x if i % 11 else 0.0)
+        vs.append((v, e))
+    taken = 0
+    for x, (v, e), (ok, diff, val) in zip(xs, vs, i128("sub", xs, vs)):
+        exact = F(v) * F(2) ** e
+        assert val == float(exact)                       # Fraction to float rounds to nearest even
+        m, ex = np.frexp(x)
+        place = int(ex) - 53 - e                         # x's last place above V's unit
+        if x != 0.0:
+            assert bool(ok) == (-22 <= place <= 63)
+        if ok:
+            taken += 1
+            assert diff == float(F(x) - exact)
+    assert taken > 1000
