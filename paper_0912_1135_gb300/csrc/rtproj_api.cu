@@ -543,7 +543,7 @@ rtproj_status rtproj_precondition(rtproj_t h, uint64_t seed, int64_t l) {
             RT_CHECK(pivoted_qr_cluster(h->S, m, (int)l, l, h->R, h->perm, qr_flag, s, &ff_first));
         else if (h->opts.qr_form == 0)
             RT_CHECK(pivoted_qr_ff(h->S, m, (int)l, l, h->R, h->perm, h->qr_work, h->status, s, h->spin_limit,
-                                   qr_flag, &ff_first));
+                                   qr_flag, h->opts.async != 0, &ff_first));
     }
     RT_CHECK(pivoted_qr(h->S, m, (int)l, l, h->R, h->perm, h->qr_work, h->status, s, h->spin_limit,
                         ff_first ? qr_flag : nullptr));

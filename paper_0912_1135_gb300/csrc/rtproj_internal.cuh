@@ -141,11 +141,17 @@ cudaError_t pivoted_qr(double* S, int m, int l, int64_t lds, double* R, int32_t*
                        double* work, int* status, cudaStream_t s, long long spin_limit,
                        const int* run_if = nullptr);
 bool pivoted_qr_persistent_ok(int m, int l);
-// The mixed form's QR in float-float on the whole grid (k_qr.cu): sets *launched when the
+// The mixed form's QR in float-float on the whole grid (k_qr.cu); side_by_side: other factorizations
+// run at the same time (asynchronous handles). Sets *launched when the
 // kernel was enqueued; the kernel writes *fallback = 1 when the entries' range needs the
 // float64 kernel, which must follow with run_if = fallback.
 cudaError_t pivoted_qr_ff(double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work, int* status,
-                          cudaStream_t s, long long spin_limit, int* fallback, bool* launched);
+                          cudaStream_t s, long long spin_limit, int* fallback, bool side_by_side, bool* launched);
+// Its form with the columns in registers (k_qr_ff.cu), taken first; not launched when a column does
+// not fit a warp's registers. qr_ff_work_doubles: its part of the work area.
+cudaError_t pivoted_qr_ff_regs(const double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work, int* status,
+                               cudaStream_t s, long long spin_limit, int* fallback, bool* launched);
+size_t qr_ff_work_doubles(int m, int l);
 // The mixed form's QR on one 16-CTA cluster in float-float arithmetic (k_qr_cluster.cu).
 // Sets *launched when the kernel was enqueued; the kernel then writes *fallback = 1 if the
 // entries' range needs the float64 kernel (which must follow with run_if = fallback).
