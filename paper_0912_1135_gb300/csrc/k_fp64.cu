@@ -280,9 +280,8 @@ cudaError_t check_finite(const double* X, int64_t rs, int rows, int cols, int* s
 // 16 rows' partial sums per column in registers (a multiple of 4 rows: a padded row costs a
 // full FP64 instruction), reading A's chunk from shared memory. B is read with the columns j
 // contiguous (one thread per column; with fewer than 129 columns the CTA's threads also split
-// the chunk's K among them), or with K contiguous (a warp per column, lanes over k), or
-// generated (G of Eq. 12). The chunks' partial sums are added in chunk order by a second
-// kernel (deterministic).
+// the chunk's K among them), or with K contiguous (a warp per column, lanes over k). The chunks'
+// partial sums are added in a fixed order by a second kernel.
 // ---------------------------------------------------------------------------------
 namespace {
 
@@ -294,7 +293,6 @@ struct NarrowDev {
     int M, N, K, kchunk;
     const double* A; int64_t a_rs;
     const double* B; int64_t b_rs, b_cs;
-    int omega_dist; uint32_t key0, key1;
     double* part;               // [chunk][M][N]
 };
 
@@ -304,22 +302,10 @@ __device__ __forceinline__ double narrow_warp_sum(double v) {
     return v;
 }
 
-// B(k, j) for k = k0 .. k0 + 3 (k0 a multiple of 4), zero at k >= ke, into b[0..3]
+// B(k, j) for k = k0 .. k0 + 3, zero at k >= ke, into b[0..3]
 __device__ __forceinline__ void narrow_b4(const NarrowDev& p, int k0, int ke, int j, double (&b)[4]) {
-    if (p.omega_dist == RTPROJ_OMEGA_GAUSSIAN) {
-        int N4[4];
-        gauss_quad((uint32_t)(k0 >> 2), (uint32_t)j, p.key0, p.key1, N4);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) b[u] = k0 + u < ke ? (double)N4[u] * (1.0 / 4096.0) : 0.0;
-    } else if (p.omega_dist >= 0) {
-        const uint4 w = philox4x32_10(make_uint4((uint32_t)(k0 >> 4), (uint32_t)j, 0u, 0u), p.key0, p.key1);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            b[u] = k0 + u < ke ? (double)omega_from_byte(block_byte(w, (k0 & 15) + u), p.omega_dist) : 0.0;
-    } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) b[u] = k0 + u < ke ? p.B[(int64_t)(k0 + u) * p.b_rs + (int64_t)j * p.b_cs] : 0.0;
-    }
+    for (int u = 0; u < 4; ++u) b[u] = k0 + u < ke ? p.B[(int64_t)(k0 + u) * p.b_rs + (int64_t)j * p.b_cs] : 0.0;
 }
 
 // NL = 2^jl threads side by side take NL columns j; the NR_T / NL groups of them take turns at
@@ -419,13 +405,15 @@ void launch_narrow(const NarrowDev& p, bool cols, int jl, dim3 grid, cudaStream_
     else narrow_rows_kernel<NR><<<grid, NR_T, 0, s>>>(p, jl);
 }
 
+// One warp per entry, its lanes over the chunks.
 __global__ void narrow_reduce_kernel(const double* part, int chunks, int M, int N, double* C, int64_t c_rs) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t idx = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (idx >= (int64_t)M * N) return;
-    const int i = (int)(idx / N), j = (int)(idx % N);
+    const int i = (int)(idx / N), j = (int)(idx % N), lane = threadIdx.x & 31;
     double s = 0.0;
-    for (int z = 0; z < chunks; ++z) s += part[((int64_t)z * M + i) * N + j];
-    C[(int64_t)i * c_rs + j] = s;
+    for (int z = lane; z < chunks; z += 32) s += part[((int64_t)z * M + i) * N + j];
+    s = narrow_warp_sum(s);
+    if (lane == 0) C[(int64_t)i * c_rs + j] = s;
 }
 
 }  // namespace
@@ -433,12 +421,12 @@ __global__ void narrow_reduce_kernel(const double* part, int chunks, int M, int 
 cudaError_t gemm64_narrow(const Narrow64& g, double* part, size_t part_elems, cudaStream_t s) {
     if (g.M <= 0 || g.N <= 0) return cudaSuccess;
     if (g.M > 64 || g.K <= 0) return cudaErrorInvalidValue;
-    const bool cols = g.omega_dist < 0 && g.b_rs == 1;
+    const bool cols = g.b_rs == 1;
     int jl = 3;                             // threads per row of columns: 8 .. 256
     while (jl < 8 && (1 << jl) < g.N) ++jl;
     const int per_block = cols ? NR_T / 32 : 1 << jl;
     const int gx = (g.N + per_block - 1) / per_block;
-    // chunks: about four CTAs per SM in all, each chunk a multiple of 16 (whole Philox blocks)
+    // chunks: about four CTAs per SM in all, each chunk a multiple of 16
     const int want = std::max(1, 4 * sm_count() / gx);
     const size_t cap = std::max<size_t>(1, part_elems / ((size_t)g.M * g.N));
     int chunks = (int)std::min<size_t>((size_t)std::min(want, 65535), cap);
@@ -450,8 +438,6 @@ cudaError_t gemm64_narrow(const Narrow64& g, double* part, size_t part_elems, cu
     p.M = g.M; p.N = g.N; p.K = g.K; p.kchunk = kchunk;
     p.A = g.A; p.a_rs = g.a_rs;
     p.B = g.B; p.b_rs = g.b_rs; p.b_cs = g.b_cs;
-    p.omega_dist = g.omega_dist;
-    p.key0 = (uint32_t)(g.seed & 0xFFFFFFFFull); p.key1 = (uint32_t)(g.seed >> 32);
     p.part = part;
     const dim3 grid((unsigned)gx, (unsigned)chunks);
     const int nr = std::min(NR_ROWS, (g.M + 3) / 4 * 4);
@@ -460,7 +446,7 @@ cudaError_t gemm64_narrow(const Narrow64& g, double* part, size_t part_elems, cu
     else if (nr <= 12) launch_narrow<12>(p, cols, jl, grid, s);
     else launch_narrow<16>(p, cols, jl, grid, s);
     const int64_t total = (int64_t)g.M * g.N;
-    narrow_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(part, chunks, g.M, g.N, g.C, g.c_rs);
+    narrow_reduce_kernel<<<(unsigned)((total + 7) / 8), 256, 0, s>>>(part, chunks, g.M, g.N, g.C, g.c_rs);
     note_launch(2);
     return cudaGetLastError();
 }

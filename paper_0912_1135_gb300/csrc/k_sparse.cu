@@ -3,7 +3,7 @@
 // Section 5: the sparse test matrix of Eq. 21 (five nonzeros per column) and its sum with
 // a rank-10 term (Eq. 22), applied as operators at O(nnz + r(m + n)) per vector.
 //
-//   S_k = A G                 one CTA per (row, 32 columns of G); G generated per nonzero
+//   S_k = A G                 one CTA per (row, 64 columns of G); G generated a panel at a time
 //                             (the same entries as the dense forms), Eq. 12
 //   X column by column as in steps a-e that follow Eq. 15, all m columns at once:
 //     D = A^* P^-             (n x m) one CTA per column of A, a gather over its nonzeros
@@ -205,55 +205,295 @@ __global__ void frobenius_total_kernel(const double* part_s, int np, const doubl
     *out = sqrt(fmax(s + 2.0 * x + t, 0.0));
 }
 
-// ---------------------------------------------------------------------------------
-// S = A G. G(c, j) is generated where it is used, from the counter-based Philox words
-// that the dense forms use: entries 16q .. 16q+15 of column j from the block at (q, j, 0, 0)
-// (uniform or +-1 bytes), Gaussian entries 4q .. 4q+3 from the block at (q, j, 1, 0).
-// ---------------------------------------------------------------------------------
-__device__ __forceinline__ double omega_at(int c, int j, int dist, uint32_t k0, uint32_t k1) {
-    if (dist == RTPROJ_OMEGA_GAUSSIAN) {
-        const uint4 w = philox4x32_10(make_uint4((uint32_t)(c >> 2), (uint32_t)j, 1u, 0u), k0, k1);
-        int ncos, nsin;
-        if (c & 2) gauss_pair(w.z, w.w, ncos, nsin);
-        else gauss_pair(w.x, w.y, ncos, nsin);
-        return (double)((c & 1) ? nsin : ncos) * (1.0 / 4096.0);
-    }
-    const uint4 w = philox4x32_10(make_uint4((uint32_t)(c >> 4), (uint32_t)j, 0u, 0u), k0, k1);
-    return (double)omega_from_byte(block_byte(w, c & 15), dist);
+__device__ __forceinline__ void ldg_words(const double* p, uint32_t& lo, uint32_t& hi) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    lo = u.x;
+    hi = u.y;
 }
 
-constexpr int SK_WARPS = 8;
+// ---------------------------------------------------------------------------------
+// S = A G in panels of SK_COLS columns of G. A panel's entries are generated once, as the integers
+// behind them (N = 4096 G, 256 G or G; 16 bits; the counter-based Philox words that the dense
+// forms use: entries 16q .. 16q+15 of column j from the block at (q, j, 0, 0), Gaussian entries
+// 4q .. 4q+3 from the block at (q, j, 1, 0)), into n x SK_COLS words that stay in L2, and every
+// nonzero of a row reads SK_COLS consecutive ones. The products run on the integer pipes: a row's
+// values are 61-bit multiples of 2^-61 of a power of two above its largest, in two limbs, and
+// sums of limb times N are exact in 64 bits; each entry of S is rounded once. Its error is below
+// nnz 2^-61 of the largest value times |N|, against about 2^-53 of every partial sum in float64.
+// (Generated per nonzero and multiplied in float64 - 192 FP64 cycles a warp and nonzero with the
+// conversions - the sketch at 1000 x 300,000, l = 1004, took 8.7 ms and V G of a rank-10 term 7.3;
+// now 2.0 with the panels' generation, and 2.3.)
+// ---------------------------------------------------------------------------------
+constexpr int SK_COLS = 64;
+constexpr int SK_T = 256;
+constexpr int SK_WARPS = SK_T / 32;
+constexpr int SK_LIMB = 30;                      // bits of the lower limb
+constexpr int SK_FLUSH = 1 << 16;                // products whose lower-limb sums fit 62 bits
 
-// one CTA per (row i, 32 columns j): the 8 warps take interleaved nonzeros of the row, each
-// lane one column j; the warps' partial sums are added in a fixed order. With a low-rank
-// term, S(i, j) += sum_q U(i, q) (V G)(q, j).
-__global__ void sparse_sketch_kernel(const int64_t* __restrict__ rptr, const int32_t* __restrict__ col,
-                                     const double* __restrict__ val, int l, int dist, uint32_t k0, uint32_t k1,
-                                     int r, const double* __restrict__ U, const double* __restrict__ VG, int64_t ldvg,
-                                     double* S, int64_t lds) {
-    const int i = blockIdx.y;
-    const int lane = threadIdx.x & 31, wsub = threadIdx.x >> 5;
-    const int j = blockIdx.x * 32 + lane;
-    __shared__ double part[SK_WARPS][32];
-    double acc0 = 0.0, acc1 = 0.0;
-    if (j < l) {
-        const int64_t e = rptr[i + 1];
-        int64_t p = rptr[i] + wsub;
-        for (; p + SK_WARPS < e; p += 2 * SK_WARPS) {
-            acc0 = fma(val[p], omega_at(col[p], j, dist, k0, k1), acc0);
-            acc1 = fma(val[p + SK_WARPS], omega_at(col[p + SK_WARPS], j, dist, k0, k1), acc1);
-        }
-        if (p < e) acc0 = fma(val[p], omega_at(col[p], j, dist, k0, k1), acc0);
-    }
-    part[wsub][lane] = acc0 + acc1;
-    __syncthreads();
-    if (wsub == 0 && j < l) {
-        double s = 0.0;
+// Panel entries (c, jj), jj < SK_COLS: N of G(c, j0 + jj), zero past column l. One warp per 4
+// (Gaussian) or 16 rows, two columns a lane.
+__global__ void __launch_bounds__(SK_T) omega_panel_kernel(int n, int l, int j0, int dist, uint32_t k0, uint32_t k1,
+                                                           int16_t* __restrict__ P) {
+    const int lane = threadIdx.x & 31;
+    const int j = j0 + 2 * lane;
+    const int per = dist == RTPROJ_OMEGA_GAUSSIAN ? 4 : 16;
+    const int64_t groups = ((int64_t)n + per - 1) / per;
+    for (int64_t q = (int64_t)blockIdx.x * SK_WARPS + (threadIdx.x >> 5); q < groups; q += (int64_t)gridDim.x * SK_WARPS) {
+        if (dist == RTPROJ_OMEGA_GAUSSIAN) {
+            int a[4], b[4];
+            gauss_quad((uint32_t)q, (uint32_t)j, k0, k1, a);
+            gauss_quad((uint32_t)q, (uint32_t)(j + 1), k0, k1, b);
 #pragma unroll
-        for (int w = 0; w < SK_WARPS; ++w) s += part[w][lane];
+            for (int u = 0; u < 4; ++u) {
+                const int64_t c = 4 * q + u;
+                if (c < n)
+                    *reinterpret_cast<short2*>(P + c * SK_COLS + 2 * lane) =
+                        make_short2((short)(j < l ? a[u] : 0), (short)(j + 1 < l ? b[u] : 0));
+            }
+        } else {
+            const uint4 wa = philox4x32_10(make_uint4((uint32_t)q, (uint32_t)j, 0u, 0u), k0, k1);
+            const uint4 wb = philox4x32_10(make_uint4((uint32_t)q, (uint32_t)(j + 1), 0u, 0u), k0, k1);
+            const float sc = dist == RTPROJ_OMEGA_RADEMACHER ? 1.0f : 256.0f;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+                const int64_t c = 16 * q + u;
+                const int a = (int)(omega_from_byte(block_byte(wa, u), dist) * sc);
+                const int b = (int)(omega_from_byte(block_byte(wb, u), dist) * sc);
+                if (c < n)
+                    *reinterpret_cast<short2*>(P + c * SK_COLS + 2 * lane) =
+                        make_short2((short)(j < l ? a : 0), (short)(j + 1 < l ? b : 0));
+            }
+        }
+    }
+}
+// G = N 2^omega_exp
+int omega_exp(int dist) { return dist == RTPROJ_OMEGA_GAUSSIAN ? -12 : dist == RTPROJ_OMEGA_RADEMACHER ? 0 : -8; }
+
+// top[i] = the frexp exponent of the largest magnitude in row i (0 for an empty or zero row).
+__device__ __forceinline__ int block_top(uint32_t mxh, uint32_t orl, uint32_t* buf) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mxh = max(mxh, __shfl_xor_sync(0xffffffffu, mxh, o));
+        orl |= __shfl_xor_sync(0xffffffffu, orl, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        buf[2 * (threadIdx.x >> 5)] = mxh;
+        buf[2 * (threadIdx.x >> 5) + 1] = orl;
+    }
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        mxh = max(mxh, buf[2 * w]);
+        orl |= buf[2 * w + 1];
+    }
+    if ((mxh | orl) == 0u) return 0;
+    if (mxh >> 20) return (int)(mxh >> 20) - 1022;
+    return mxh ? 32 - __clz((int)mxh) + 32 - 1074 : 32 - __clz((int)orl) - 1074;
+}
+__global__ void __launch_bounds__(256) row_tops_kernel(const int64_t* __restrict__ rptr, const double* __restrict__ val,
+                                                       int64_t ld, int len, int32_t* __restrict__ top) {
+    __shared__ uint32_t buf[16];
+    const int i = blockIdx.x;
+    const int64_t b = rptr ? rptr[i] : (int64_t)i * ld, e = rptr ? rptr[i + 1] : b + len;
+    uint32_t mxh = 0u, orl = 0u;
+    for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) {
+        uint32_t lo, hi;
+        ldg_words(val + p, lo, hi);
+        mxh = max(mxh, hi & 0x7FFFFFFFu);
+        orl |= lo;
+    }
+    const int t = block_top(mxh, orl, buf);
+    if (threadIdx.x == 0) top[i] = t;
+}
+
+// x 2^(bits - top) rounded to an integer (|x| < 2^top, bits <= 61), in a signed upper and a
+// SK_LIMB-bit lower limb.
+__device__ __forceinline__ int2 to_limbs(double x, int top, int bits) {
+    const i128op o = i128_decode((uint32_t)__double2loint(x), (uint32_t)__double2hiint(x));
+    long long v = (long long)(((unsigned long long)o.hi << 32) | o.lo);
+    const int sh = o.e - top + bits;               // the significand's last place in units
+    if (sh >= 0) v <<= sh;                         // at most bits - 53
+    else if (sh > -62) v = (v + (1ll << (-sh - 1))) >> -sh;
+    else v = 0;
+    if (o.neg) v = -v;
+    return make_int2((int)(v >> SK_LIMB), (int)(v & ((1ll << SK_LIMB) - 1)));
+}
+// acc += a N for a signed 32-bit a
+__device__ __forceinline__ void mad_limb(long long& acc, int a, int N) {
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(N));
+}
+// (hi 2^SK_LIMB + lo) 2^e rounded once
+__device__ __forceinline__ double limbs_to_double(__int128 hi, __int128 lo, int e) {
+    const __int128 v = (hi << SK_LIMB) + lo;
+    return u128_to_double((unsigned long long)(v >> 64), (unsigned long long)v, e);
+}
+// bits of a value in a sum of `count` products with N (16 bits): the upper limb's sum stays
+// below 2^62
+__host__ __device__ __forceinline__ int limb_bits(int64_t count) {
+    int b = 61;
+    while (b > 40 && count > ((int64_t)1 << (16 + 61 - b))) --b;
+    return b;
+}
+
+// S(i, j0 .. j0 + SK_COLS - 1) for row i: the CTA's warps take the row's nonzeros in turn, two
+// columns a lane. With a low-rank term, S(i, j) += sum_q U(i, q) (V G)(q, j).
+__global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __restrict__ rptr, const int32_t* __restrict__ col,
+                                                             const double* __restrict__ val, const int32_t* __restrict__ top,
+                                                             const int16_t* __restrict__ P, int l, int j0, int gexp, int r,
+                                                             const double* __restrict__ U, const double* __restrict__ VG,
+                                                             int64_t ldvg, double* S, int64_t lds) {
+    __shared__ int4 ent[SK_T];                     // upper limb, lower limb, column
+    __shared__ unsigned long long sum[2][SK_COLS];
+    const int i = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t b = rptr[i], e = rptr[i + 1];
+    const int tp = top[i], bits = limb_bits(e - b);
+    if (t < SK_COLS) sum[0][t] = sum[1][t] = 0ull;
+    long long h0 = 0, h1 = 0, l0 = 0, l1 = 0;
+    int held = 0;
+    for (int64_t p0 = b; p0 < e; p0 += SK_T) {
+        __syncthreads();
+        if (p0 + t < e) {
+            const int2 v = to_limbs(val[p0 + t], tp, bits);
+            ent[t] = make_int4(v.x, v.y, col[p0 + t], 0);
+        } else {
+            ent[t] = make_int4(0, 0, 0, 0);
+        }
+        __syncthreads();
+        const int cnt = (int)min((int64_t)SK_T, e - p0);
+        for (int q = warp; q < cnt; q += 4 * SK_WARPS) {
+            int4 v[4];
+            int N[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                v[u] = ent[(q + u * SK_WARPS) & (SK_T - 1)];
+                N[u] = __ldg(reinterpret_cast<const int*>(P + (int64_t)v[u].z * SK_COLS) + lane);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (q + u * SK_WARPS >= SK_T) break;
+                const int n0 = (int)(short)(N[u] & 0xFFFF), n1 = N[u] >> 16;
+                mad_limb(h0, v[u].x, n0);
+                mad_limb(l0, v[u].y, n0);
+                mad_limb(h1, v[u].x, n1);
+                mad_limb(l1, v[u].y, n1);
+            }
+        }
+        if ((held += SK_T) >= SK_FLUSH) {          // the lower sums' upper part moves over
+            h0 += l0 >> SK_LIMB;
+            l0 &= (1ll << SK_LIMB) - 1;
+            h1 += l1 >> SK_LIMB;
+            l1 &= (1ll << SK_LIMB) - 1;
+            held = 0;
+        }
+    }
+    h0 += l0 >> SK_LIMB;
+    l0 &= (1ll << SK_LIMB) - 1;
+    h1 += l1 >> SK_LIMB;
+    l1 &= (1ll << SK_LIMB) - 1;
+    __syncthreads();                               // integer sums: the order does not matter
+    atomicAdd(&sum[0][2 * lane], (unsigned long long)h0);
+    atomicAdd(&sum[1][2 * lane], (unsigned long long)l0);
+    atomicAdd(&sum[0][2 * lane + 1], (unsigned long long)h1);
+    atomicAdd(&sum[1][2 * lane + 1], (unsigned long long)l1);
+    __syncthreads();
+    const int j = j0 + t;
+    if (t < SK_COLS && j < l) {
+        double s = limbs_to_double((long long)sum[0][t], (long long)sum[1][t], tp - bits + gexp);
         for (int q = 0; q < r; ++q) s = fma(U[(int64_t)i * r + q], VG[(int64_t)q * ldvg + j], s);
         S[(int64_t)i * lds + j] = s;
     }
+}
+
+// Partial sums of (V G)(q, j0 ..) over chunk blockIdx.x of the rows of G: rows q0 .. q0 + VG_ROWS - 1
+// of V (blockIdx.y; as many as cover r in equal parts of at most 12), the warps take G's rows in
+// turn, two columns a lane.
+constexpr int VG_KC = 128;
+template <int VG_ROWS>
+__global__ void __launch_bounds__(SK_T) lowrank_panel_kernel(const double* __restrict__ V, const int32_t* __restrict__ top,
+                                                             int r, int n, int chunk, int bits, const int16_t* __restrict__ P,
+                                                             longlong2* __restrict__ part) {
+    __shared__ int2 vs[VG_KC][VG_ROWS];
+    __shared__ unsigned long long sum[2][VG_ROWS][SK_COLS];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, q0 = blockIdx.y * VG_ROWS;
+    const int64_t kb = (int64_t)blockIdx.x * chunk, ke = min((int64_t)n, kb + chunk);
+    for (int e = t; e < 2 * VG_ROWS * SK_COLS; e += SK_T) (&sum[0][0][0])[e] = 0ull;
+    long long h[VG_ROWS][2], lo[VG_ROWS][2];
+#pragma unroll
+    for (int q = 0; q < VG_ROWS; ++q) h[q][0] = h[q][1] = lo[q][0] = lo[q][1] = 0;
+    int held = 0;
+    for (int64_t k0 = kb; k0 < ke; k0 += VG_KC) {
+        __syncthreads();
+        for (int e = t; e < VG_KC * VG_ROWS; e += SK_T) {
+            const int q = e / VG_KC, k = e % VG_KC;
+            int2 v = make_int2(0, 0);
+            if (q0 + q < r && k0 + k < ke) v = to_limbs(V[(int64_t)(q0 + q) * n + k0 + k], top[q0 + q], bits);
+            vs[k][q] = v;
+        }
+        __syncthreads();
+        const int cnt = (int)min((int64_t)VG_KC, ke - k0);
+        for (int k = warp; k < cnt; k += SK_WARPS) {
+            const int N = __ldg(reinterpret_cast<const int*>(P + (k0 + k) * SK_COLS) + lane);
+            const int n0 = (int)(short)(N & 0xFFFF), n1 = N >> 16;
+#pragma unroll
+            for (int q = 0; q < VG_ROWS; ++q) {
+                const int2 v = vs[k][q];
+                mad_limb(h[q][0], v.x, n0);
+                mad_limb(lo[q][0], v.y, n0);
+                mad_limb(h[q][1], v.x, n1);
+                mad_limb(lo[q][1], v.y, n1);
+            }
+        }
+        if ((held += VG_KC) >= SK_FLUSH) {
+#pragma unroll
+            for (int q = 0; q < VG_ROWS; ++q)
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    h[q][u] += lo[q][u] >> SK_LIMB;
+                    lo[q][u] &= (1ll << SK_LIMB) - 1;
+                }
+            held = 0;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < VG_ROWS; ++q)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            h[q][u] += lo[q][u] >> SK_LIMB;
+            lo[q][u] &= (1ll << SK_LIMB) - 1;
+            atomicAdd(&sum[0][q][2 * lane + u], (unsigned long long)h[q][u]);
+            atomicAdd(&sum[1][q][2 * lane + u], (unsigned long long)lo[q][u]);
+        }
+    __syncthreads();
+    for (int e = t; e < VG_ROWS * SK_COLS; e += SK_T) {
+        const int q = e / SK_COLS, j = e % SK_COLS;
+        if (q0 + q < r)
+            part[((int64_t)blockIdx.x * r + q0 + q) * SK_COLS + j] =
+                make_longlong2((long long)sum[0][q][j], (long long)sum[1][q][j]);
+    }
+}
+// (V G)(q, j0 + j) from the chunks' partial sums: one warp per entry.
+__global__ void lowrank_panel_sum_kernel(const longlong2* __restrict__ part, const int32_t* __restrict__ top, int chunks, int r,
+                                         int l, int j0, int bits, int gexp, double* __restrict__ VG, int64_t ldvg) {
+    const int idx = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    const int q = idx / SK_COLS, j = idx % SK_COLS;
+    if (q >= r || j0 + j >= l) return;
+    // the upper limbs' sums are below 2^62 a chunk: kept as a high and a low half
+    long long hh = 0, hl = 0, lo = 0;
+    for (int z = lane; z < chunks; z += 32) {
+        const longlong2 v = part[((int64_t)z * r + q) * SK_COLS + j];
+        hh += v.x >> 32;
+        hl += v.x & 0xFFFFFFFFll;
+        lo += v.y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        hh += __shfl_xor_sync(0xffffffffu, hh, o);
+        hl += __shfl_xor_sync(0xffffffffu, hl, o);
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+    }
+    if (lane != 0) return;
+    const __int128 h = ((__int128)hh << 32) + hl;
+    VG[(int64_t)q * ldvg + j0 + j] = limbs_to_double(h, lo, top[q] - bits + gexp);
 }
 
 // ---------------------------------------------------------------------------------
@@ -319,12 +559,6 @@ __global__ void sparse_e_kernel(const int64_t* __restrict__ rptr, const int32_t*
 constexpr int SP_CHUNK = 2048;
 static_assert(SP_CHUNK <= I128_MAX_TERMS, "a chunk's sum must fit 128 bits");
 constexpr int SP_WARPS = 8;
-
-__device__ __forceinline__ void ldg_words(const double* p, uint32_t& lo, uint32_t& hi) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
-    lo = u.x;
-    hi = u.y;
-}
 
 __device__ __forceinline__ i128acc i128_shfl_xor(const i128acc& a, int o) {
     return {__shfl_xor_sync(0xffffffffu, a.w0, o), __shfl_xor_sync(0xffffffffu, a.w1, o),
@@ -547,6 +781,9 @@ namespace rtp {
 
 int64_t sparse_max_chunks(int64_t m, int64_t nnz) { return m + nnz / SP_CHUNK + 1; }
 
+// G's panel lies in D's region, which is free during the sketch, when that holds it.
+size_t panel_bytes(int64_t m, int64_t n) { return m * 8 >= SK_COLS * 2 ? 0 : (size_t)n * SK_COLS * 2; }
+
 size_t sparse_bytes(int64_t m, int64_t n, int64_t nnz, int64_t r, int64_t l_max, int64_t k_max) {
     const int64_t nb = (n + SCAN_T - 1) / SCAN_T;
     const int64_t nz = std::max<int64_t>(nnz, 1);
@@ -555,7 +792,8 @@ size_t sparse_bytes(int64_t m, int64_t n, int64_t nnz, int64_t r, int64_t l_max,
            align_up((size_t)n * 8) + align_up((size_t)nb * 8) + 2 * align_up((size_t)m * m * 8) +
            align_up((size_t)r * std::max(l_max, m) * 8) + align_up((size_t)r * k_max * 8) +
            align_up((size_t)(2 * r * r + norm_parts()) * 8) + align_up((size_t)nc * 4) + align_up((size_t)nc * 8) +
-           align_up((size_t)(m + 1) * 4) + align_up((size_t)nc * k_max * 16);
+           align_up((size_t)(m + 1) * 4) + align_up((size_t)nc * k_max * 16) + align_up((size_t)m * 4) +
+           align_up((size_t)r * 4) + align_up(panel_bytes(m, n));
 }
 
 void sparse_bind(rtproj_ctx* h, char* base) {
@@ -578,6 +816,10 @@ void sparse_bind(rtproj_ctx* h, char* base) {
     h->chunk_beg = (int64_t*)take((size_t)nc * 8);
     h->row_chunk = (int32_t*)take((size_t)(m + 1) * 4);
     h->chunk_part = (double*)take((size_t)nc * h->k_max * 16);
+    h->row_top = (int32_t*)take((size_t)m * 4);
+    h->lr_top = (int32_t*)take((size_t)r * 4);
+    int16_t* own = (int16_t*)take(panel_bytes(m, n));
+    h->panel = panel_bytes(m, n) ? own : reinterpret_cast<int16_t*>(h->W);
 }
 
 // The chunk table from the row pointers (on the host): row i is cut into
@@ -632,6 +874,12 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
         check_values_kernel<<<grid_of((int64_t)r * n, 256), 256, 0, s>>>(h->lrV, (int64_t)r * n, h->status);
         note_launch(2);
     }
+    row_tops_kernel<<<(unsigned)m, 256, 0, s>>>(h->csr_ptr, h->csr_val, 0, 0, h->row_top);
+    note_launch();
+    if (r > 0) {
+        row_tops_kernel<<<(unsigned)r, 256, 0, s>>>(nullptr, h->lrV, n, n, h->lr_top);
+        note_launch();
+    }
     // ||A||_F
     const unsigned np = std::min<unsigned>(grid_of(std::max<int64_t>(nnz, 1), 256), (unsigned)norm_parts());
     sumsq_vals_kernel<<<np, 256, 0, s>>>(h->csr_val, nnz, h->norm_part);
@@ -665,19 +913,38 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
 
 rtproj_status sparse_sketch(rtproj_ctx* h, uint64_t seed, int64_t l, double* S, int64_t lds) {
     const uint32_t k0 = (uint32_t)(seed & 0xFFFFFFFFull), k1 = (uint32_t)(seed >> 32);
-    if (h->lr > 0) {   // V G (r x l), G generated where it is used
-        Narrow64 g;
-        g.M = h->lr; g.N = (int)l; g.K = (int)h->n;
-        g.A = h->lrV; g.a_rs = h->n;
-        g.omega_dist = h->opts.omega; g.seed = seed;
-        g.C = h->lr_a; g.c_rs = l;
-        SP_CHECK(gemm64_narrow(g, h->part, h->part_elems, h->stream));
+    const int m = (int)h->m, n = (int)h->n, r = h->lr, dist = h->opts.omega, gexp = omega_exp(dist);
+    cudaStream_t s = h->stream;
+    // the chunks of V G: up to four CTAs an SM, their partial sums within the scratch
+    const int64_t cap = std::max<int64_t>(1, (int64_t)(h->part_elems / ((size_t)std::max(r, 1) * SK_COLS * 2)));
+    int64_t chunks = std::min<int64_t>(cap, std::min<int64_t>(4 * sm_count(), ((int64_t)n + VG_KC - 1) / VG_KC));
+    const int64_t chunk = (((int64_t)n + chunks - 1) / chunks + VG_KC - 1) / VG_KC * VG_KC;
+    chunks = ((int64_t)n + chunk - 1) / chunk;
+    const int vbits = limb_bits(chunk);
+    const int per = dist == RTPROJ_OMEGA_GAUSSIAN ? 4 : 16;
+    const unsigned pgrid = (unsigned)std::max<int64_t>(
+        1, std::min<int64_t>(((int64_t)n + per * SK_WARPS - 1) / (per * SK_WARPS), (int64_t)sm_count() * 32));
+    for (int j0 = 0; j0 < (int)l; j0 += SK_COLS) {
+        omega_panel_kernel<<<pgrid, SK_T, 0, s>>>(n, (int)l, j0, dist, k0, k1, h->panel);
+        if (r > 0) {   // V G (r x l), this panel's columns
+            longlong2* part = reinterpret_cast<longlong2*>(h->part);
+            const int groups = (r + 11) / 12, rows = (r + groups - 1) / groups;   // 1 .. 12 rows a CTA
+            const dim3 grid((unsigned)chunks, (unsigned)groups);
+            auto run = [&](auto kern) {
+                kern<<<grid, SK_T, 0, s>>>(h->lrV, h->lr_top, r, n, (int)chunk, vbits, h->panel, part);
+            };
+            if (rows <= 4) run(lowrank_panel_kernel<4>);
+            else if (rows <= 8) run(lowrank_panel_kernel<8>);
+            else if (rows <= 10) run(lowrank_panel_kernel<10>);
+            else run(lowrank_panel_kernel<12>);
+            lowrank_panel_sum_kernel<<<(unsigned)((r * SK_COLS + 7) / 8), 256, 0, s>>>(part, h->lr_top, (int)chunks, r, (int)l, j0,
+                                                                                       vbits, gexp, h->lr_a, l);
+            note_launch(2);
+        }
+        sparse_sketch_kernel<<<(unsigned)m, SK_T, 0, s>>>(h->csr_ptr, h->csr_col, h->csr_val, h->row_top, h->panel, (int)l, j0,
+                                                          gexp, r, h->lrU, h->lr_a, l, S, lds);
+        note_launch(2);
     }
-    const dim3 grid((unsigned)((l + 31) / 32), (unsigned)h->m);
-    sparse_sketch_kernel<<<grid, 32 * SK_WARPS, 0, h->stream>>>(h->csr_ptr, h->csr_col, h->csr_val, (int)l,
-                                                                h->opts.omega, k0, k1, h->lr, h->lrU, h->lr_a, l, S,
-                                                                lds);
-    note_launch();
     SP_CHECK(cudaGetLastError());
     return RTPROJ_OK;
 }

@@ -111,13 +111,12 @@ struct Gemm64 {
 cudaError_t gemm64(const Gemm64& g, double* part, size_t part_elems, cudaStream_t s);
 
 // C (M x N, M <= 64, ld c_rs) = A (M x K, ld a_rs) B (K x N) for a long K, where
-// B(k, j) = B[k b_rs + j b_cs] or, with omega_dist >= 0, G(k, j) of Eq. 12 (k_fp64.cu).
+// B(k, j) = B[k b_rs + j b_cs] (k_fp64.cu).
 // part: chunks x M x N doubles of scratch.
 struct Narrow64 {
     int M = 0, N = 0, K = 0;
     const double* A = nullptr; int64_t a_rs = 0;
     const double* B = nullptr; int64_t b_rs = 0, b_cs = 0;
-    int omega_dist = -1; uint64_t seed = 0;
     double* C = nullptr; int64_t c_rs = 0;
 };
 cudaError_t gemm64_narrow(const Narrow64& g, double* part, size_t part_elems, cudaStream_t s);
@@ -402,6 +401,9 @@ struct rtproj_ctx {
     int64_t* chunk_beg = nullptr;     // first nonzero of each chunk
     int32_t* row_chunk = nullptr;     // m + 1: first chunk of each row
     double* chunk_part = nullptr;     // chunks x k_max double-double partial sums
+    int32_t* row_top = nullptr;       // m: frexp exponents of the rows' largest values
+    int32_t* lr_top = nullptr;        // r: the same of V's rows
+    int16_t* panel = nullptr;         // n x 64 entries of G (as integers), the sketch's current panel
 
     rtp::PhaseTimer timer;
     int64_t l = 0;
