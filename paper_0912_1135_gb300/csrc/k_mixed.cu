@@ -234,10 +234,17 @@ rtproj_status mixed_gram(rtproj_ctx* h) {
 // inverse, so the first product runs as D' c' with D' = D diag(2^{e_A}) and c' = c
 // diag(2^{-e_A}): digits sliced per right-hand side then keep every row's digits whatever
 // the spread of A's row scales (rows scaled apart leave the projection unchanged).
+// Small blocks sum the products with T1 itself instead (k_middle.cu): where every call of the
+// handle will, only T1's transpose is made.
 rtproj_status mixed_prepare_middle(rtproj_ctx* h) {
     const int m = (int)h->m;
     const int64_t total = (int64_t)m * m;
     phase_begin(h, RTPROJ_PHASE_SLICE);
+    if (middle_direct_ok(m, h->k_max)) {       // no call will read the digits
+        MX_CHECK(middle_direct_prepare(h->T1, m, h->Mprime, h->status, h->stream));
+        phase_end(h, RTPROJ_PHASE_SLICE);
+        return RTPROJ_OK;
+    }
     permute_columns_kernel<<<(unsigned)((total + 255) / 256), 256, 0, h->stream>>>(h->T1, h->perm, m, h->Mprime);
     note_launch();
     MX_CHECK(cudaGetLastError());
@@ -247,6 +254,7 @@ rtproj_status mixed_prepare_middle(rtproj_ctx* h) {
     note_launch();
     MX_CHECK(cudaGetLastError());
     MX_CHECK(slice_rows(h->Mprime, m, 1, nullptr, nullptr, h->Ts, h->status, h->stream));      // D'
+    if (middle_direct_ok(m, 1)) MX_CHECK(middle_direct_prepare(h->T1, m, h->Mprime, h->status, h->stream));
     phase_end(h, RTPROJ_PHASE_SLICE);
     return RTPROJ_OK;
 }
@@ -256,6 +264,10 @@ namespace {
 // out = D^* (D c) for the m x k block c (row-major, leading dimension k).
 rtproj_status middle_mixed(rtproj_ctx* h, const double* c, double* out, int k) {
     const int ap = h->opts.apply_slices;
+    if (middle_direct_ok(h->m, k)) {
+        MX_CHECK(middle_direct(h->T1, h->Mprime, h->perm, (int)h->m, c, k, h->ebuf, out, h->status, h->stream));
+        return RTPROJ_OK;
+    }
     const SliceStack Hk = rows_of(h->Hs, k, ap);
     MX_CHECK(slice_rows(c, 1, k, nullptr, h->neg_eA, Hk, h->status, h->stream));           // c'^*: k x m
     rtproj_status st = gemm(h, h->Ts, Hk, ap, h->ebuf, k, 1);                              // u = D' c' = D c

@@ -280,6 +280,12 @@ rtproj_status sparse_project(rtproj_ctx* h, const double* B, int64_t ldb, int k,
                              int64_t ldr, void* X, int64_t ldx);
 void phase_begin(rtproj_ctx* h, int phase);
 void phase_end(rtproj_ctx* h, int phase);
+// k_middle.cu: steps 2-6 of the apply for small m and k, from T1 and its transpose.
+constexpr int64_t MIDDLE_DIRECT_PRODUCTS = (int64_t)4 << 20;
+bool middle_direct_ok(int64_t m, int64_t k);
+cudaError_t middle_direct_prepare(const double* T1, int m, double* T1t, int* status, cudaStream_t s);
+cudaError_t middle_direct(const double* T1, const double* T1t, const int32_t* perm, int m, const double* c, int k, double* u,
+                          double* out, int* status, cudaStream_t s);
 // Steps 2-6 of the apply in float64: out = Pi^* T1^* T1 Pi c (c, out: m x k, ld k).
 rtproj_status middle_fp64(rtproj_ctx* h, const double* c, double* out, int k);
 }  // namespace rtp
