@@ -147,11 +147,6 @@ __global__ void __launch_bounds__(RN_T) row_norms_kernel(const double* __restric
     cl.sync();   // a CTA's partial sum stays readable until the first has added it
 }
 
-__device__ __forceinline__ void max_bits(unsigned long long* p, double v) {
-    // non-negative doubles order like their bit patterns; NaN lands above every finite value
-    atomicMax(p, (unsigned long long)__double_as_longlong(v));
-}
-
 // One CTA per right-hand side j (column j of the m x k blocks).
 __global__ void column_stats_kernel(const double* r, const double* h, const double* dh, int m, int k,
                                     const double* bnorm, const double* normA, unsigned long long* stats) {
@@ -168,20 +163,12 @@ __global__ void column_stats_kernel(const double* r, const double* h, const doub
     }
     if (r) {
         const double t = block_sum(sr, red);
-        if (threadIdx.x == 0) {
-            const double den = *normA * bnorm[j];
-            max_bits(&stats[0], den > 0.0 ? sqrt(t) / den : sqrt(t));
-        }
+        if (threadIdx.x == 0) report_residual(t, bnorm[j], *normA, stats);
     }
     if (dh) {
-        // relative to ||h||, or to ||b|| / ||A||_F when h is smaller than that (a b already
-        // near the null space): ||A||_F ||dh|| bounds the change A^* dh makes to Zb
         const double th = block_sum(sh, red);
         const double td = block_sum(sd, red);
-        if (threadIdx.x == 0) {
-            const double scale = fmax(sqrt(th), *normA > 0.0 ? bnorm[j] / *normA : 0.0);
-            max_bits(&stats[1], scale > 0.0 ? sqrt(td) / scale : sqrt(td));
-        }
+        if (threadIdx.x == 0) report_change(th, td, bnorm[j], *normA, stats);
     }
 }
 

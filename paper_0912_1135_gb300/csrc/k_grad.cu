@@ -125,8 +125,8 @@ rtproj_status rtproj_grad_A(rtproj_t h, int64_t k, const void* H, int64_t ldh, c
         const int sl = h->opts.apply_slices;
         SliceStack SA = make_stack(b, L.SA, L.eA, m, K2, sl);
         SliceStack SB = make_stack(b, L.SB, L.eB, n, K2, sl);
-        GR_CHECK(slice_rows(TA, K2, 1, nullptr, nullptr, SA, h->status, s));
-        GR_CHECK(slice_rows(TB, K2, 1, nullptr, nullptr, SB, h->status, s));
+        GR_CHECK(slice_rows(TA, K2, SA, h->status, s));
+        GR_CHECK(slice_rows(TB, K2, SB, h->status, s));
         SlicedGemm g;
         g.a = SA;
         g.b = SB;

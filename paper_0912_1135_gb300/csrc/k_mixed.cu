@@ -130,11 +130,6 @@ __global__ void scale_columns_pow2_kernel(double* D, const int32_t* e, int m, in
     if (idx < m) ne[idx] = -e[idx];
 }
 
-__global__ void axpy_kernel(double* y, const double* x, int64_t n) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < n) y[idx] += x[idx];
-}
-
 #define MX_CHECK(expr)                              \
     do {                                            \
         cudaError_t e_ = (expr);                    \
@@ -214,7 +209,7 @@ rtproj_status mixed_gram(rtproj_ctx* h) {
     mprime_kernel<<<(unsigned)((total + 255) / 256), 256, 0, h->stream>>>(h->RinvT, h->perm, h->As.e, m, h->Mprime);
     note_launch();
     MX_CHECK(cudaGetLastError());
-    MX_CHECK(slice_rows(h->Mprime, m, 1, nullptr, nullptr, h->Ms, h->status, h->stream));
+    MX_CHECK(slice_rows(h->Mprime, m, h->Ms, h->status, h->stream));
     // W's row exponents are gathered by the product's output stage, so slicing W reads it once
     MX_CHECK(fill_int(h->Ws.e, m, kZeroRowExp, h->stream));
     rtproj_status st = gemm(h, h->Ms, first(h->Ats, h->opts.gram_slices), h->opts.gram_slices, h->W, n, 1, 1.0, 0.0,
@@ -248,12 +243,12 @@ rtproj_status mixed_prepare_middle(rtproj_ctx* h) {
     permute_columns_kernel<<<(unsigned)((total + 255) / 256), 256, 0, h->stream>>>(h->T1, h->perm, m, h->Mprime);
     note_launch();
     MX_CHECK(cudaGetLastError());
-    MX_CHECK(slice_rows(h->Mprime, 1, m, nullptr, nullptr, h->Tts, h->status, h->stream));      // D^*
+    MX_CHECK(slice_columns(h->Mprime, m, nullptr, h->Tts, h->status, h->stream));      // D^*
     scale_columns_pow2_kernel<<<(unsigned)((total + 255) / 256), 256, 0, h->stream>>>(h->Mprime, h->As.e, m,
                                                                                         h->neg_eA);
     note_launch();
     MX_CHECK(cudaGetLastError());
-    MX_CHECK(slice_rows(h->Mprime, m, 1, nullptr, nullptr, h->Ts, h->status, h->stream));      // D'
+    MX_CHECK(slice_rows(h->Mprime, m, h->Ts, h->status, h->stream));      // D'
     if (middle_direct_ok(m, 1)) MX_CHECK(middle_direct_prepare(h->T1, m, h->Mprime, h->status, h->stream));
     phase_end(h, RTPROJ_PHASE_SLICE);
     return RTPROJ_OK;
@@ -269,28 +264,30 @@ rtproj_status middle_mixed(rtproj_ctx* h, const double* c, double* out, int k) {
         return RTPROJ_OK;
     }
     const SliceStack Hk = rows_of(h->Hs, k, ap);
-    MX_CHECK(slice_rows(c, 1, k, nullptr, h->neg_eA, Hk, h->status, h->stream));           // c'^*: k x m
+    MX_CHECK(slice_columns(c, k, h->neg_eA, Hk, h->status, h->stream));           // c'^*: k x m
     rtproj_status st = gemm(h, h->Ts, Hk, ap, h->ebuf, k, 1);                              // u = D' c' = D c
     if (st != RTPROJ_OK) return st;
-    MX_CHECK(slice_rows(h->ebuf, 1, k, nullptr, nullptr, Hk, h->status, h->stream));        // u^*: k x m
+    MX_CHECK(slice_columns(h->ebuf, k, nullptr, Hk, h->status, h->stream));        // u^*: k x m
     return gemm(h, h->Tts, Hk, ap, out, k, 1);                                             // D^* u
 }
 
 }  // namespace
 
-rtproj_status mixed_project(rtproj_ctx* h, const double* B, int64_t ldb, int k, void* Z, int64_t ldz, void* ROW,
+rtproj_status mixed_project(rtproj_ctx* h, const void* Bin, int64_t ldbin, int k, void* Z, int64_t ldz, void* ROW,
                             int64_t ldr, void* X, int64_t ldx) {
     const rtproj_opts& o = h->opts;
     const int m = (int)h->m, n = (int)h->n;
     cudaStream_t s = h->stream;
     rtproj_status st;
-    // residual report: ||b_j|| once per apply, the maxima cleared
-    MX_CHECK(row_norms(B, ldb, k, n, h->bnorm, s));
-    MX_CHECK(cudaMemsetAsync(h->stats, 0, 16, s));
-    // c = A b
+    // digits of B; with them its float64 form, and for the residual report ||b_j|| and the maxima
+    // cleared
     phase_begin(h, RTPROJ_PHASE_SLICE);
     const SliceStack Bk = rows_of(h->Bs, k, o.apply_slices);
-    MX_CHECK(slice_rows(B, ldb, 1, nullptr, nullptr, Bk, h->status, s));
+    MX_CHECK(slice_rhs(Bin, h->dtype, ldbin, h->B64, n, h->bnorm, h->stats, Bk, h->status, s));
+    const bool f32 = h->dtype == RTPROJ_F32;
+    const double* B = f32 ? h->B64 : (const double*)Bin;
+    const int64_t ldb = f32 ? n : ldbin;
+    // c = A b
     phase_end(h, RTPROJ_PHASE_SLICE);
     phase_begin(h, RTPROJ_PHASE_APPLY_A);
     st = gemm(h, first(h->As, o.apply_slices), Bk, o.apply_slices, h->cbuf, k, 1);
@@ -304,7 +301,7 @@ rtproj_status mixed_project(rtproj_ctx* h, const double* B, int64_t ldb, int k, 
     // s = b - A^* h0
     phase_begin(h, RTPROJ_PHASE_SLICE);
     const SliceStack Hr = rows_of(h->Hs, k, o.resid_slices);
-    MX_CHECK(slice_rows(h->hbuf, 1, k, nullptr, h->As.e, Hr, h->status, s));
+    MX_CHECK(slice_columns(h->hbuf, k, h->As.e, Hr, h->status, s));
     phase_end(h, RTPROJ_PHASE_SLICE);
     phase_begin(h, RTPROJ_PHASE_APPLY_AT);
     st = gemm(h, first(h->Ats, o.resid_slices), Hr, o.resid_slices, h->sbuf, 1, n, -1.0, 1.0, B, 1, ldb);
@@ -318,7 +315,7 @@ rtproj_status mixed_project(rtproj_ctx* h, const double* B, int64_t ldb, int k, 
         // r = A s
         phase_begin(h, RTPROJ_PHASE_SLICE);
         const SliceStack Sk = rows_of(h->Ss, k, o.resid_slices);
-        MX_CHECK(slice_rows(h->sbuf, n, 1, nullptr, nullptr, Sk, h->status, s));
+        MX_CHECK(slice_rows(h->sbuf, n, Sk, h->status, s, h->stats));    // and the report's maxima cleared
         phase_end(h, RTPROJ_PHASE_SLICE);
         phase_begin(h, RTPROJ_PHASE_APPLY_A);
         st = gemm(h, first(h->As, o.resid_slices), Sk, o.resid_slices, h->cbuf, k, 1);
@@ -328,13 +325,12 @@ rtproj_status mixed_project(rtproj_ctx* h, const double* B, int64_t ldb, int k, 
         phase_begin(h, RTPROJ_PHASE_APPLY_M);
         st = middle_mixed(h, h->cbuf, h->dhbuf, k);
         if (st != RTPROJ_OK) return st;
-        const int64_t mk = (int64_t)m * k;
-        axpy_kernel<<<(unsigned)((mk + 255) / 256), 256, 0, s>>>(h->hbuf, h->dhbuf, mk);
-        note_launch();
-        // the pass's report: ||r_j|| = ||A s_j|| and ||dh_j|| / ||h_j||
-        MX_CHECK(cudaMemsetAsync(h->stats, 0, 16, s));
-        MX_CHECK(column_stats(h->cbuf, h->hbuf, h->dhbuf, m, k, h->bnorm, h->normA, h->stats, s));
         phase_end(h, RTPROJ_PHASE_APPLY_M);
+        // h += dh, the pass's report (||r_j|| = ||A s_j|| and ||dh_j|| / ||h_j||), digits of dh
+        phase_begin(h, RTPROJ_PHASE_SLICE);
+        const SliceStack Hd = rows_of(h->Hs, k, o.apply_slices);
+        MX_CHECK(slice_correction(h->dhbuf, k, h->hbuf, h->cbuf, h->bnorm, h->normA, h->stats, h->As.e, Hd, h->status, s));
+        phase_end(h, RTPROJ_PHASE_SLICE);
         passes = pass + 1;
         bool last = passes == o.refine_passes;
         if (o.refine_tol > 0.0 && !last) {
@@ -347,10 +343,6 @@ rtproj_status mixed_project(rtproj_ctx* h, const double* B, int64_t ldb, int k, 
             if (v[1] <= o.refine_tol) last = true;
         }
         // s = s - A^* dh
-        phase_begin(h, RTPROJ_PHASE_SLICE);
-        const SliceStack Hd = rows_of(h->Hs, k, o.apply_slices);
-        MX_CHECK(slice_rows(h->dhbuf, 1, k, nullptr, h->As.e, Hd, h->status, s));
-        phase_end(h, RTPROJ_PHASE_SLICE);
         phase_begin(h, RTPROJ_PHASE_APPLY_AT);
         if (last && direct_z) {
             st = gemm(h, first(h->Ats, o.apply_slices), Hd, o.apply_slices, (double*)Z, 1, ldz, -1.0, 1.0, h->sbuf, 1,

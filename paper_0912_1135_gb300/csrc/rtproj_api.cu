@@ -285,7 +285,7 @@ rtproj_status mixed_prepare_a(rtproj_ctx* h);
 rtproj_status mixed_sketch(rtproj_ctx* h, uint64_t seed, int64_t l, double* S, int64_t lds);
 rtproj_status mixed_gram(rtproj_ctx* h);
 rtproj_status mixed_prepare_middle(rtproj_ctx* h);
-rtproj_status mixed_project(rtproj_ctx* h, const double* B, int64_t ldb, int k, void* Z, int64_t ldz,
+rtproj_status mixed_project(rtproj_ctx* h, const void* B, int64_t ldb, int k, void* Z, int64_t ldz,
                             void* ROW, int64_t ldr, void* X, int64_t ldx);
 }  // namespace rtp
 
@@ -612,6 +612,8 @@ rtproj_status rtproj_project(rtproj_t h, const void* B, int64_t ldb, int64_t k, 
     if (!Z && !ROW && !X) return RTPROJ_EINVAL;
     if ((Z && ldz < h->n) || (ROW && ldr < h->n) || (X && ldx < h->m)) return RTPROJ_EINVAL;
     if (!h->preconditioned) return RTPROJ_ESTATE;
+    if (h->opts.mode == RTPROJ_MIXED_REFINED && !h->sparse)
+        return mixed_project(h, B, ldb, (int)k, Z, ldz, ROW, ldr, X, ldx);
     const double* Bd = (const double*)B;
     int64_t ldbd = ldb;
     if (h->dtype == RTPROJ_F32) {   // right-hand sides widened exactly; outputs stored as float32
@@ -620,7 +622,6 @@ rtproj_status rtproj_project(rtproj_t h, const void* B, int64_t ldb, int64_t k, 
         ldbd = h->n;
     }
     if (h->sparse) return sparse_project(h, Bd, ldbd, (int)k, Z, ldz, ROW, ldr, X, ldx);
-    if (h->opts.mode == RTPROJ_MIXED_REFINED) return mixed_project(h, Bd, ldbd, (int)k, Z, ldz, ROW, ldr, X, ldx);
     return project_fp64(h, Bd, ldbd, (int)k, Z, ldz, ROW, ldr, X, ldx);
 }
 

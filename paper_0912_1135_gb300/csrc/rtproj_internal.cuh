@@ -217,25 +217,37 @@ struct SliceStack {
 // parts of a row start from it); slicing reads it as exponent 0.
 constexpr int kZeroRowExp = -(1 << 30);
 
-// Slices X (element (r, c) at X[r*x_rs + c*x_cs], multiplied by 2^cexp[c] when cexp is
-// given) into the stack; optional row gather. Columns cols..ld-1 are written as zeros.
-cudaError_t slice_rows(const double* X, int64_t x_rs, int64_t x_cs, const int32_t* rowidx, const int32_t* cexp,
-                       const SliceStack& st, int* status, cudaStream_t s);
-// Digit planes of src transposed into dst (dst.rows = src.cols, dst.ld >= src.rows).
+// Slices X (contiguous rows, leading dimension x_rs) into the stack. Columns cols..ld-1 are
+// written as zeros; non-finite entries raise RTPROJ_ENONFINITE in status (digits 0). clear
+// (optional): two words zeroed on the way.
+cudaError_t slice_rows(const double* X, int64_t x_rs, const SliceStack& st, int* status, cudaStream_t s,
+                       unsigned long long* clear = nullptr);
+// The same for right-hand sides of element type dt (ld ldb), with the 2-norm of every row and,
+// for float32, the rows widened to float64 (wide, ld ldw) in the same pass.
+cudaError_t slice_rhs(const void* B, int dt, int64_t ldb, double* wide, int64_t ldw, double* norms,
+                      unsigned long long* clear, const SliceStack& st, int* status, cudaStream_t s);
+// Slices the columns of X (st.cols x st.rows row-major, ld ldx): row j of the stack is column j
+// of X, entry i multiplied by 2^cexp[i] when cexp is given.
+cudaError_t slice_columns(const double* X, int64_t ldx, const int32_t* cexp, const SliceStack& st, int* status,
+                          cudaStream_t s);
+// slice_columns of a correction dh (m x k, ld ldx as h's and r's), which is also added to h; then
+// column_stats of r, the new h and dh.
+cudaError_t slice_correction(const double* dh, int64_t ldx, double* h, const double* r, const double* bnorm,
+                             const double* normA, unsigned long long* stats, const int32_t* cexp, const SliceStack& st,
+                             int* status, cudaStream_t s);
 // Row exponents of X (rows x cols, contiguous rows): e[r] <- max(e[r], the frexp exponent
 // of max_c |X[r][c]|), e pre-filled with kZeroRowExp; non-finite entries raise
 // RTPROJ_ENONFINITE in status.
 cudaError_t row_exponents(const double* X, int64_t x_rs, int rows, int cols, int32_t* e, int* status, cudaStream_t s);
 // Slices X (contiguous rows) into st with the row exponents already in st.e (gathered as
 // by row_exponents, kZeroRowExp for an all-zero row): one read of X, spread over spans of
-// every row. Falls back to slice_rows when the fast layout conditions do not hold.
+// every row.
 cudaError_t slice_rows_given_exp(const double* X, int64_t x_rs, const SliceStack& st, int* status, cudaStream_t s);
 // Row-major digits of X (rows x cols, contiguous rows) into st and the same digits
 // transposed into tst (tst.rows = st.cols, tst.cols = st.rows, same s), in one pass over
 // the digits: the row exponents first, then 64 x 64 tiles that write both layouts.
 cudaError_t slice_rows_dual(const double* X, int64_t x_rs, const SliceStack& st, const SliceStack& tst, int* status,
                             cudaStream_t s);
-cudaError_t transpose_planes(const SliceStack& src, const SliceStack& dst, cudaStream_t s);
 // Writes G^* (l x n, reduction over n) as digit planes plus row exponents (exact): one
 // plane for the uniform and Rademacher entries, two for the Gaussian ones (st.s >= 2).
 cudaError_t omega_plane(uint64_t seed, int dist, int n, int l, const SliceStack& st, cudaStream_t s);
@@ -313,6 +325,19 @@ int norm_parts();
 cudaError_t frobenius(const double* X, int64_t ldx, int rows, int cols, double* part, double* out, cudaStream_t s);
 // out[j] = ||row j of X|| for the k rows of X (k x n float64, ld ldx).
 cudaError_t row_norms(const double* X, int64_t ldx, int k, int n, double* out, cudaStream_t s);
+// The residual report's maxima for one right-hand side, from the squared norms of its r, h and dh
+// (see column_stats). Non-negative doubles order like their bit patterns; a NaN lands above
+// every finite value.
+__device__ __forceinline__ void report_residual(double rr, double bnorm, double normA, unsigned long long* stats) {
+    const double den = normA * bnorm;
+    atomicMax(&stats[0], (unsigned long long)__double_as_longlong(den > 0.0 ? sqrt(rr) / den : sqrt(rr)));
+}
+__device__ __forceinline__ void report_change(double hh, double dd, double bnorm, double normA, unsigned long long* stats) {
+    // relative to ||h||, or to ||b|| / ||A||_F when h is smaller than that (a b already
+    // near the null space): ||A||_F ||dh|| bounds the change A^* dh makes to Zb
+    const double scale = fmax(sqrt(hh), normA > 0.0 ? bnorm / normA : 0.0);
+    atomicMax(&stats[1], (unsigned long long)__double_as_longlong(scale > 0.0 ? sqrt(dd) / scale : sqrt(dd)));
+}
 // For the m x k blocks r, h, dh (row-major, ld k; right-hand side j is column j):
 // stats[0] <- max(stats[0], max_j ||r_j|| / (normA ||b_j||)) and
 // stats[1] <- max(stats[1], max_j ||dh_j|| / max(||h_j||, ||b_j|| / normA)), as bit patterns of non-negative
