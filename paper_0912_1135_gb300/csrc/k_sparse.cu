@@ -306,7 +306,8 @@ __global__ void __launch_bounds__(256) row_tops_kernel(const int64_t* __restrict
 }
 
 // x 2^(bits - top) rounded to an integer (|x| < 2^top, bits <= 61), in a signed upper and a
-// SK_LIMB-bit lower limb.
+// LIMB-bit lower limb.
+template <int LIMB = SK_LIMB>
 __device__ __forceinline__ int2 to_limbs(double x, int top, int bits) {
     const i128op o = i128_decode((uint32_t)__double2loint(x), (uint32_t)__double2hiint(x));
     long long v = (long long)(((unsigned long long)o.hi << 32) | o.lo);
@@ -315,7 +316,7 @@ __device__ __forceinline__ int2 to_limbs(double x, int top, int bits) {
     else if (sh > -62) v = (v + (1ll << (-sh - 1))) >> -sh;
     else v = 0;
     if (o.neg) v = -v;
-    return make_int2((int)(v >> SK_LIMB), (int)(v & ((1ll << SK_LIMB) - 1)));
+    return make_int2((int)(v >> LIMB), (int)(v & ((1ll << LIMB) - 1)));
 }
 // acc += a N for a signed 32-bit a
 __device__ __forceinline__ void mad_limb(long long& acc, int a, int N) {
@@ -508,18 +509,208 @@ __global__ void pminus_kernel(const double* __restrict__ RinvT, const int32_t* _
     Pm[(int64_t)perm[t] * m + k] = RinvT[(int64_t)k * m + t];
 }
 
-// D(c, :) = sum over column c's nonzeros of val P^-(row, :)  [+ sum_q V(q, c) (U^* P^-)(q, :)]
-__global__ void sparse_d_kernel(const int64_t* __restrict__ cptr, const int32_t* __restrict__ crow,
-                                const double* __restrict__ cval, const double* __restrict__ Pm, int m, int n, int r,
-                                const double* __restrict__ V, const double* __restrict__ UtP, double* D) {
-    for (int c = blockIdx.x; c < n; c += gridDim.x) {
-        const int64_t b = cptr[c], e = cptr[c + 1];
-        for (int k = threadIdx.x; k < m; k += blockDim.x) {
-            double s = 0.0;
-            for (int64_t p = b; p < e; ++p) s = fma(cval[p], Pm[(int64_t)crow[p] * m + k], s);
-            for (int q = 0; q < r; ++q) s = fma(V[(int64_t)q * n + c], UtP[(int64_t)q * m + k], s);
-            D[(int64_t)c * m + k] = s;
+// D = A^* P^-: its sparse part on the FP64 pipe (the entries of P^- span too many binades for
+// fixed point), the low-rank part V^* (U^* P^-) and then V D on the integer pipes. In both, V(q, :) is
+// taken in units of 2^{lr_top[q]} and the other factor (times 2^{lr_top[q]} for U^* P^-) in units of its
+// largest value in column k, each as LR_BITS = 57 bits in two limbs; a product is the three upper of
+// the four limb products, so its error is below 2^-56 of the two units -- 2^-53 of the partial sums
+// in float64. An FP64 multiply-add holds an SM sub-partition for 64 cycles, the three limb products
+// for 12: with r = 10 at 1000 x 300,000 D took 7.5 ms and V D 6.0.
+constexpr int LR_LO = 28;
+constexpr int LR_BITS = 57;            // 29 bits and the sign in the upper limb
+constexpr int LR_TERMS = 16;           // products whose upper sums (2^58 each) stay below 2^62
+constexpr int DC_STAGE = 32;           // columns of V staged at a time
+constexpr int DC_COLS = 4;             // columns c a thread works on at once
+
+// An upper sum and the sum of the two middle products (2^-LR_LO of it).
+struct LimbSum { long long h, m; };
+__device__ __forceinline__ void mad_limbs(LimbSum& s, int2 a, int2 b) {
+    mad_limb(s.h, a.x, b.x);
+    mad_limb(s.m, a.x, b.y);
+    mad_limb(s.m, a.y, b.x);
+}
+// The middle sum's upper part moves over.
+__device__ __forceinline__ void fold(LimbSum& s) {
+    s.h += s.m >> LR_LO;
+    s.m &= (1ll << LR_LO) - 1;
+}
+
+// h 2^e rounded once
+__device__ __forceinline__ double limb_value(long long h, int e) {
+    const unsigned long long neg = (unsigned long long)(h >> 63), w = ((unsigned long long)h ^ neg) - neg;
+    return i128_round((uint32_t)w, (uint32_t)(w >> 32), 0u, 0u, e, (uint32_t)neg);
+}
+
+__device__ __forceinline__ int top_of(double x) {          // |x| < 2^top, tight for a normal x
+    const int e = (int)(((uint32_t)__double2hiint(x) & 0x7FF00000u) >> 20);
+    return (e ? e : 1) - 1022;
+}
+
+// D(c, k): a thread per k (blockIdx.y picks blockDim of them), the CTA walks the columns c.
+// dtop[k] (pre-filled with kZeroRowExp) gathers the frexp exponents of D(:, k)'s maxima.
+template <bool LOWRANK>
+__global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict__ cptr, const int32_t* __restrict__ crow,
+                                                       const double* __restrict__ cval, const double* __restrict__ Pm, int m,
+                                                       int n, int r, const double* __restrict__ V,
+                                                       const int32_t* __restrict__ vtop, const double* __restrict__ UtP,
+                                                       double* __restrict__ D, int32_t* __restrict__ dtop) {
+    extern __shared__ __align__(16) int2 d_smem[];
+    const int t = threadIdx.x, nt = blockDim.x, k = blockIdx.y * nt + t;
+    int2* ts = d_smem;                                     // [r][nt]: (U^* P^-)(q, k) 2^{vtop[q]}
+    int2* vs = d_smem + (LOWRANK ? r * nt : 0);            // [DC_STAGE][r]
+    int ek = 0, tmax = kZeroRowExp;
+    bool bad = false;
+    if (LOWRANK) {
+        int e = kZeroRowExp;
+        for (int q = 0; q < r; ++q) {
+            const double x = k < m ? UtP[(int64_t)q * m + k] : 0.0;
+            bad |= !isfinite(x);
+            if (x != 0.0) e = max(e, top_of(x) + vtop[q]);
         }
+        ek = e == kZeroRowExp ? 0 : e;
+        for (int q = 0; q < r; ++q)
+            ts[q * nt + t] = to_limbs<LR_LO>(k < m && !bad ? UtP[(int64_t)q * m + k] : 0.0, ek - vtop[q], LR_BITS);
+    }
+    for (int64_t c0 = (int64_t)blockIdx.x * DC_STAGE; c0 < n; c0 += (int64_t)gridDim.x * DC_STAGE) {
+        if (LOWRANK) {
+            __syncthreads();
+            for (int e = t; e < DC_STAGE * r; e += nt) {
+                const int q = e / DC_STAGE, cc = e % DC_STAGE;
+                vs[cc * r + q] = to_limbs<LR_LO>(c0 + cc < n ? V[(int64_t)q * n + c0 + cc] : 0.0, vtop[q], LR_BITS);
+            }
+            __syncthreads();
+        }
+        if (k >= m) continue;
+        const int cnt = (int)min((int64_t)DC_STAGE, n - c0);
+#pragma unroll 1
+        for (int cc = 0; cc < cnt; cc += DC_COLS) {
+            double s[DC_COLS];
+            int64_t b[DC_COLS];
+            int len[DC_COLS], most = 0;
+#pragma unroll
+            for (int u = 0; u < DC_COLS; ++u) {
+                const bool live = cc + u < cnt;
+                b[u] = live ? cptr[c0 + cc + u] : 0;
+                len[u] = live ? (int)(cptr[c0 + cc + u + 1] - b[u]) : 0;
+                most = max(most, len[u]);
+                s[u] = 0.0;
+            }
+            for (int p = 0; p < most; ++p)
+#pragma unroll
+                for (int u = 0; u < DC_COLS; ++u)
+                    if (p < len[u]) s[u] = fma(cval[b[u] + p], __ldg(Pm + (int64_t)crow[b[u] + p] * m + k), s[u]);
+            if (LOWRANK) {
+                for (int q0 = 0; q0 < r; q0 += LR_TERMS) {
+                    LimbSum w[DC_COLS];
+#pragma unroll
+                    for (int u = 0; u < DC_COLS; ++u) w[u].h = w[u].m = 0;
+                    const int qe = min(r, q0 + LR_TERMS);
+#pragma unroll 2
+                    for (int q = q0; q < qe; ++q) {
+                        const int2 x = ts[q * nt + t];
+#pragma unroll
+                        for (int u = 0; u < DC_COLS; ++u) mad_limbs(w[u], x, vs[(cc + u) * r + q]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < DC_COLS; ++u) {
+                        fold(w[u]);
+                        s[u] += limb_value(w[u].h, ek - 58);
+                    }
+                }
+                if (bad)
+#pragma unroll
+                    for (int u = 0; u < DC_COLS; ++u) s[u] = __longlong_as_double(0x7FF8000000000000ll);
+            }
+#pragma unroll
+            for (int u = 0; u < DC_COLS; ++u)
+                if (cc + u < cnt) {
+                    D[(c0 + cc + u) * m + k] = s[u];
+                    if (LOWRANK && s[u] != 0.0) tmax = max(tmax, top_of(s[u]));
+                }
+        }
+    }
+    if (LOWRANK && k < m && tmax != kZeroRowExp) atomicMax(dtop + k, tmax);
+}
+
+// Partial sums of (V D)(q, k) over chunk blockIdx.x of D's rows: 32 columns k a CTA (a lane each),
+// rows q0 .. q0 + ROWS - 1 of V (blockIdx.z), the warps take D's rows in turn. part[chunk][q][k].
+constexpr int VD_KC = 128;
+template <int ROWS>
+__global__ void __launch_bounds__(SK_T) lowrank_d_kernel(const double* __restrict__ V, const int32_t* __restrict__ vtop, int r,
+                                                         int n, int m, int chunk, const double* __restrict__ D,
+                                                         const int32_t* __restrict__ dtop, double* __restrict__ part) {
+    __shared__ int2 vs[VD_KC][ROWS];
+    __shared__ unsigned long long sum[2][ROWS][32];
+    __shared__ int bad_s[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, q0 = blockIdx.z * ROWS, k = blockIdx.y * 32 + lane;
+    const int64_t kb = (int64_t)blockIdx.x * chunk, ke = min((int64_t)n, kb + chunk);
+    for (int e = t; e < 2 * ROWS * 32; e += SK_T) (&sum[0][0][0])[e] = 0ull;
+    if (t < 32) bad_s[t] = 0;
+    const int top = k < m ? max(dtop[k], -1022) : 0;      // a column of zeros or subnormals: the smallest normal's
+    LimbSum a[ROWS];
+    long long up[ROWS];                                    // the upper sums' own upper words
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) a[q].h = a[q].m = up[q] = 0;
+    bool bad = false;
+    for (int64_t c0 = kb; c0 < ke; c0 += VD_KC) {
+        __syncthreads();
+        for (int e = t; e < VD_KC * ROWS; e += SK_T) {
+            const int q = e / VD_KC, c = e % VD_KC;
+            vs[c][q] = q0 + q < r && c0 + c < ke ? to_limbs<LR_LO>(V[(int64_t)(q0 + q) * n + c0 + c], vtop[q0 + q], LR_BITS)
+                                                 : make_int2(0, 0);
+        }
+        __syncthreads();
+        const int cnt = (int)min((int64_t)VD_KC, ke - c0);
+        if (k < m) {
+#pragma unroll 4
+            for (int c = warp; c < cnt; c += SK_WARPS) {   // VD_KC / SK_WARPS = LR_TERMS rows a stage at most
+                const double x = __ldg(D + (c0 + c) * m + k);
+                bad |= !isfinite(x);
+                const int2 d = to_limbs<LR_LO>(x, top, LR_BITS);
+#pragma unroll
+                for (int q = 0; q < ROWS; ++q) mad_limbs(a[q], d, vs[c][q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q) {
+            fold(a[q]);
+            up[q] += a[q].h >> 32;
+            a[q].h &= 0xFFFFFFFFll;
+        }
+    }
+    // integer sums: the order does not matter. Below 2^60 a warp: h and m; above: up
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+        atomicAdd(&sum[0][q][lane], (unsigned long long)up[q]);
+        atomicAdd(&sum[1][q][lane], (unsigned long long)((a[q].h << LR_LO) + a[q].m));
+    }
+    if (bad) bad_s[lane] = 1;
+    __syncthreads();
+    for (int e = t; e < ROWS * 32; e += SK_T) {
+        const int q = e >> 5, l = e & 31, kk = blockIdx.y * 32 + l;
+        if (q0 + q >= r || kk >= m) continue;
+        const __int128 v = ((__int128)(long long)sum[0][q][l] << (32 + LR_LO)) + (__int128)sum[1][q][l];
+        const int e2 = vtop[q0 + q] + max(dtop[kk], -1022) - 58 - LR_LO;
+        part[((int64_t)blockIdx.x * r + q0 + q) * m + kk] =
+            bad_s[l] ? __longlong_as_double(0x7FF8000000000000ll)
+                     : u128_to_double((unsigned long long)(v >> 64), (unsigned long long)v, e2);
+    }
+}
+static_assert(VD_KC <= SK_WARPS * LR_TERMS, "a stage's upper sums must fit before they are folded");
+
+// VD(q, k) from the chunks' partial sums, 32 entries a CTA, eight threads an entry.
+__global__ void __launch_bounds__(256) lowrank_d_sum_kernel(const double* __restrict__ part, int chunks, int total,
+                                                            double* __restrict__ VD) {
+    __shared__ double s[8][32];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, idx = blockIdx.x * 32 + lane;
+    double a = 0.0;
+    if (idx < total)
+        for (int z = g; z < chunks; z += 8) a += part[(int64_t)z * total + idx];
+    s[g][lane] = a;
+    __syncthreads();
+    if (g == 0 && idx < total) {
+        for (int w = 1; w < 8; ++w) a += s[w][lane];
+        VD[idx] = a;
     }
 }
 
@@ -793,7 +984,7 @@ size_t sparse_bytes(int64_t m, int64_t n, int64_t nnz, int64_t r, int64_t l_max,
            align_up((size_t)r * std::max(l_max, m) * 8) + align_up((size_t)r * k_max * 8) +
            align_up((size_t)(2 * r * r + norm_parts()) * 8) + align_up((size_t)nc * 4) + align_up((size_t)nc * 8) +
            align_up((size_t)(m + 1) * 4) + align_up((size_t)nc * k_max * 16) + align_up((size_t)m * 4) +
-           align_up((size_t)r * 4) + align_up(panel_bytes(m, n));
+           align_up((size_t)r * 4) + align_up((size_t)m * 4) + align_up(panel_bytes(m, n));
 }
 
 void sparse_bind(rtproj_ctx* h, char* base) {
@@ -818,6 +1009,7 @@ void sparse_bind(rtproj_ctx* h, char* base) {
     h->chunk_part = (double*)take((size_t)nc * h->k_max * 16);
     h->row_top = (int32_t*)take((size_t)m * 4);
     h->lr_top = (int32_t*)take((size_t)r * 4);
+    h->d_top = (int32_t*)take((size_t)m * 4);
     int16_t* own = (int16_t*)take(panel_bytes(m, n));
     h->panel = panel_bytes(m, n) ? own : reinterpret_cast<int16_t*>(h->W);
 }
@@ -958,16 +1150,35 @@ rtproj_status sparse_gram(rtproj_ctx* h) {
     pminus_kernel<<<(unsigned)((mm + 255) / 256), 256, 0, s>>>(h->RinvT, h->perm, m, h->Pminus);
     note_launch();
     if (r > 0) SP_CHECK(ut_times(h, h->Pminus, m, m, h->lr_a, m));                    // U^* P^-
-    sparse_d_kernel<<<(unsigned)std::min(n, sm_count() * 64), row_threads(m), 0, s>>>(
-        h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, r, h->lrV, h->lr_a, D);
-    note_launch();
-    if (r > 0) {                                                                        // V D
-        Narrow64 g;
-        g.M = r; g.N = m; g.K = n;
-        g.A = h->lrV; g.a_rs = n;
-        g.B = D; g.b_rs = m; g.b_cs = 1;
-        g.C = h->lr_a; g.c_rs = m;
-        SP_CHECK(gemm64_narrow(g, h->part, h->part_elems, s));
+    const int nt = row_threads(m), kgroups = (m + nt - 1) / nt;
+    const dim3 dgrid((unsigned)std::max(1, std::min((n + DC_STAGE - 1) / DC_STAGE, sm_count() * 32 / kgroups)), (unsigned)kgroups);
+    if (r == 0) {
+        sparse_d_kernel<false><<<dgrid, nt, 0, s>>>(h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, 0, nullptr, nullptr,
+                                                    nullptr, D, nullptr);
+        note_launch();
+    } else {
+        SP_CHECK(fill_int(h->d_top, m, kZeroRowExp, s));
+        const size_t smem = (size_t)r * (nt + DC_STAGE) * sizeof(int2);
+        SP_CHECK(cudaFuncSetAttribute(sparse_d_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        sparse_d_kernel<true><<<dgrid, nt, smem, s>>>(h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, r, h->lrV, h->lr_top,
+                                                      h->lr_a, D, h->d_top);
+        note_launch();
+        // V D: about four CTAs an SM, their partial sums within the scratch
+        const int groups = (r + 11) / 12, rows = (r + groups - 1) / groups, kg = (m + 31) / 32;
+        const int64_t cap = std::max<int64_t>(1, (int64_t)(h->part_elems / ((size_t)r * m)));
+        int64_t chunks = std::min<int64_t>(std::min<int64_t>(cap, 65535), std::max(1, 4 * sm_count() / (kg * groups)));
+        const int64_t chunk = (((int64_t)n + chunks - 1) / chunks + VD_KC - 1) / VD_KC * VD_KC;
+        chunks = ((int64_t)n + chunk - 1) / chunk;
+        const dim3 grid((unsigned)chunks, (unsigned)kg, (unsigned)groups);
+        auto run = [&](auto kern) {
+            kern<<<grid, SK_T, 0, s>>>(h->lrV, h->lr_top, r, n, m, (int)chunk, D, h->d_top, h->part);
+        };
+        if (rows <= 4) run(lowrank_d_kernel<4>);
+        else if (rows <= 8) run(lowrank_d_kernel<8>);
+        else if (rows <= 10) run(lowrank_d_kernel<10>);
+        else run(lowrank_d_kernel<12>);
+        lowrank_d_sum_kernel<<<(unsigned)((r * m + 31) / 32), 256, 0, s>>>(h->part, (int)chunks, r * m, h->lr_a);
+        note_launch(2);
     }
     sparse_e_kernel<<<m, row_threads(m), 0, s>>>(h->csr_ptr, h->csr_col, h->csr_val, D, m, r, h->lrU, h->lr_a,
                                                  h->Esp);

@@ -434,6 +434,7 @@ struct rtproj_ctx {
     double* chunk_part = nullptr;     // chunks x k_max double-double partial sums
     int32_t* row_top = nullptr;       // m: frexp exponents of the rows' largest values
     int32_t* lr_top = nullptr;        // r: the same of V's rows
+    int32_t* d_top = nullptr;         // m: the same of the columns of D = A^* P^- (with a low-rank term)
     int16_t* panel = nullptr;         // n x 64 entries of G (as integers), the sketch's current panel
 
     rtp::PhaseTimer timer;
