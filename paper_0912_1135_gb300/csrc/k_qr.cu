@@ -158,7 +158,8 @@ __global__ void qr_extract_r_kernel(const double* S, int m, int64_t lds, double*
 
 
 // ---------------------------------------------------------------------------------
-// Persistent form: one cooperative launch for all m steps. CTA b keeps columns
+// Persistent form: one cooperative launch for all m steps; taken where the register form
+// (k_qr_regs.cu) is not: longer columns, factorizations side by side, a range it refuses. CTA b keeps columns
 // [b*cpc, b*cpc + cpc) of S^* (rows of S) in shared memory for the whole factorization,
 // one warp per column, and consecutive steps are separated by one grid-wide exchange.
 // The pivot rule is the textbook one (Businger-Golub with the norms recomputed every
@@ -707,7 +708,7 @@ size_t pivoted_qr_work_doubles(int m, int l) {
     const size_t steps = (size_t)3 * m + 3 * (size_t)l + 2048;                       // per-step form
     // staging slots (G * cpc < m + cpc columns per parity), candidates, counter and flag
     const size_t persistent = (size_t)2 * ((size_t)m + PQ_MAXC) * l + 5 * (size_t)PQ_MAX_G + (size_t)m + 65;
-    return std::max(std::max(steps, persistent), qr_ff_work_doubles(m, l));
+    return std::max(std::max(steps, persistent), qr_regs_work_doubles(m, l));
 }
 
 // One CTA: perm must hold every index 0..m-1 once (m <= 4096: a bitmap in shared
@@ -754,12 +755,12 @@ constexpr int ff_cols_per_cta() { return 4; }
 cudaError_t pivoted_qr_ff(double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work, int* status,
                           cudaStream_t s, long long spin_limit, int* fallback, bool side_by_side, bool* launched) {
     *launched = false;
-    // The register form (k_qr_ff.cu) is the faster one alone (512 x 516: 1.50 against 1.89 ms) but takes
+    // The register form (k_qr_regs.cu) is the faster one alone (512 x 516: 1.50 against 1.89 ms) but takes
     // up to three times the registers of an SM. Factorizations that run side by side on several
     // streams wait for one another's SMs then: a batch of 64 instances took 16.1 ms with it throughout,
     // 15.0 with it up to 100 columns only, 15.1 without it.
     if (!side_by_side || m <= 100) {
-        const cudaError_t er = pivoted_qr_ff_regs(S, m, l, lds, R, perm, work, status, s, spin_limit, fallback, launched);
+        const cudaError_t er = pivoted_qr_regs(S, m, l, lds, R, perm, work, status, s, spin_limit, fallback, false, launched);
         if (er != cudaSuccess || *launched) return er;
     }
     int dev = 0, sms = 0, coop = 0, smem_optin = 0;

@@ -1,10 +1,11 @@
-// Pivoted Householder QR of S^* (Section 4, Eq. 13) for the mixed form: float-float, one
-// cooperative launch, columns in registers, exchanges through self-validating packets.
+// Pivoted Householder QR of S^* (Section 4, Eq. 13): one cooperative launch, columns in registers,
+// exchanges through self-validating packets; in float-float for the mixed form, in float64 for the
+// others.
 //
 // The factorization is m strictly sequential steps, so a step's latency is its cost. CTA b keeps
 // columns [b cpc, b cpc + cpc) of S^* (rows of S), WPC warps each, in registers: the warps take
-// 64-row groups in turn, lane t rows 2 t and 2 t + 1 of a group. All column arithmetic runs two rows
-// at a time in packed float32 instructions (add/mul/fma.f32x2; ff2.cuh). Step j:
+// 64-row groups in turn, lane t rows 2 t and 2 t + 1 of a group. Float-float column arithmetic runs
+// two rows at a time in packed float32 instructions (add/mul/fma.f32x2; ff2.cuh). Step j:
 //  1. warp 0 polls the CTAs' candidate records of step j (one 16-byte word each) until all carry the
 //     step's tag, and takes the largest key: the squared trailing norm to 44 mantissa bits, lowest
 //     column on ties (Businger-Golub);
@@ -26,7 +27,8 @@
 // on expiry the kernel raises RTPROJ_ETIMEOUT and all CTAs leave.
 // Measured: 512 x 516 1.89 -> 1.50 ms (2.9 us a step), 64 x 256 246 -> 172 us, 333 x 698 1.37 -> 1.15 ms,
 // 256 x 1024 1.27 -> 1.02 ms, 1024 x 2080 7.55 -> 7.09 ms (there the column arithmetic counts: seven
-// columns of 2080 rows a CTA). Not kept: one 16-CTA cluster with the same columns and a hardware
+// columns of 2080 rows a CTA). Float64, against the persistent kernel: 1000 x 1004 10.4 -> 7.2 ms, 256 x
+// 544 1.49 -> 1.12 ms; the FP64 pipe (64 cycles a warp instruction) bounds its columns. Not kept: one 16-CTA cluster with the same columns and a hardware
 // barrier a step (5 to 8 us a step: distributed shared memory answers no sooner than L2 here),
 // per-column records polled by every warp, scalars formed after the packets' barrier.
 //
@@ -34,19 +36,20 @@
 // has cancelled by more than 2^10 the candidates are exchanged once more with their fresh
 // sums, so the choice never rests on fewer than 37 bits. The reflector always uses the fresh sum.
 // Range: S^* is scaled by a power of two below 1 / sqrt(l) of its largest entry; columns whose largest
-// entries span more than 2^40, or a pivot whose squared norm falls below 2^-112, send the
-// factorization to the float64 kernel enqueued behind (*fallback), and S is not modified. Accuracy: R
-// is the exact factor of S^* + E with ||E|| of order l 2^-48 ||S||.
+// entries span more than 2^40 (2^400 in float64), or a pivot whose squared norm falls below 2^-112
+// (2^-900), send the factorization to the float64 kernel enqueued behind (*fallback), and S is not
+// modified. Accuracy: R is the exact factor of S^* + E with ||E|| of order l 2^-48 ||S|| (l 2^-53).
 #include "rtproj_internal.cuh"
 #include "ff2.cuh"
 
 #include <climits>
 #include <algorithm>
+#include <iterator>
 
 namespace rtp {
 namespace {
 
-struct QrFfDev {
+struct QrRegsDev {
     const double* S; int m, l; int64_t lds;
     double* R; int32_t* perm;
     int cpc;
@@ -61,6 +64,8 @@ struct QrFfDev {
     long long timeout;
     int* fallback;
 };
+
+constexpr int MAX_SCALE = 1000;                      // largest scale's exponent that is taken here
 
 // ---- 128-bit words in global memory, single-copy atomic at GPU scope
 __device__ __forceinline__ ulonglong2 ld_word(const ulonglong2* p) {
@@ -77,29 +82,154 @@ __device__ __forceinline__ void st_word(ulonglong2* p, unsigned long long x, uns
                  : "memory");
 }
 
-// A packet is the pair's high and low parts as they are, with a step's 4-bit tag in the top exponent
-// bits of the four floats, which are zero: S^* is scaled so that no column's norm exceeds 1, and
-// reflections keep the norms, so every part is below 2 in magnitude. A slot's previous content is
-// the packet of two steps before (or the zero written at the start), whose tag differs.
-constexpr f2 TAG_BITS = 0x4000000040000000ull;
 struct Tag {
-    f2 h, l;                 // the tag's bits in the two words
+    f2 h, l;                 // the tag's bits in a packet's two words
 };
-__device__ __forceinline__ Tag step_tag(int j) {
-    const uint32_t n = ((uint32_t)(j >> 1) + 1u) & 15u;
-    return {((f2)((n & 1u) << 30)) | ((f2)((n & 2u) << 29) << 32), ((f2)((n & 4u) << 28)) | ((f2)((n & 8u) << 27) << 32)};
-}
+
+// The arithmetic: a scalar S, and a pair of rows (2 q, 2 q + 1) as two 64-bit words. A packet is the
+// pair's words as they are, with a tag of step j in exponent bits that are zero: S^* is scaled so that
+// no column's norm exceeds 1, and reflections keep the norms, so every entry is below 2 in magnitude.
+// A slot's previous content is the packet of two steps before (or the zero written at the start),
+// whose tag differs.
+
+// Float-float: the words are both rows' high parts and both rows' low parts; 4 tag bits.
+struct FfArith {
+    using S = ff;
+    static constexpr f2 TAG_BITS = 0x4000000040000000ull;
+    static constexpr int RANGE = 40;                          // binades between the columns' largest entries
+    static constexpr int ACCS = 3;                            // independent partial sums of a lane
+    static constexpr bool SHARED_SCALARS = false;             // every thread forms the reflector's scalars
+    static __device__ __forceinline__ bool too_small(S n) { return !(n.hi >= 0x1p-112f); }
+    static __device__ __forceinline__ Tag tag(int j) {
+        const uint32_t n = ((uint32_t)(j >> 1) + 1u) & 15u;
+        return {((f2)((n & 1u) << 30)) | ((f2)((n & 2u) << 29) << 32), ((f2)((n & 4u) << 28)) | ((f2)((n & 8u) << 27) << 32)};
+    }
+    static __device__ __forceinline__ S zero() { return {0.f, 0.f}; }
+    static __device__ __forceinline__ S add(S a, S b) { return ff_add(a, b); }
+    static __device__ __forceinline__ S mul(S a, S b) { return ff_mul(a, b); }
+    static __device__ __forceinline__ S neg(S a) { return ff_neg(a); }
+    static __device__ __forceinline__ S sqrt(S a) { return ff_sqrt_newton(a); }
+    static __device__ __forceinline__ S recip(S a) { return ff_recip_newton(a); }
+    static __device__ __forceinline__ bool nonneg(S a) { return a.hi >= 0.f; }
+    static __device__ __forceinline__ S clamp(S a) { return a.hi > 0.f ? a : zero(); }
+    static __device__ __forceinline__ bool cancelled(S now, S before) { return now.hi < before.hi * 0x1p-10f; }
+    static __device__ __forceinline__ f2 bits(S a) { return pack2(a.hi, a.lo); }
+    static __device__ __forceinline__ S of(f2 w) { return {lo2(w), hi2(w)}; }
+    static __device__ __forceinline__ double to_double(S a) { return ff_to_double(a); }
+    static __device__ __forceinline__ unsigned long long key(S n, int c) { return norm_key(n, c); }
+    static __device__ __forceinline__ S row(const ffp& x, bool odd) {
+        return odd ? S{hi2(x.h), hi2(x.l)} : S{lo2(x.h), lo2(x.l)};
+    }
+    static __device__ __forceinline__ ffp pair(double a, double b) {
+        const ff x = ff_from_double(a), y = ff_from_double(b);
+        return {pack2(x.hi, y.hi), pack2(x.lo, y.lo)};
+    }
+    static __device__ __forceinline__ ffp both(S a) { return {pack2(a.hi, a.hi), pack2(a.lo, a.lo)}; }
+    // the reflector's pair that holds row j (odd: its second row), whose entry there is v0
+    static __device__ __forceinline__ ffp first(const ffp& v, bool odd, S v0) {
+        if (odd) return {pack2(0.f, v0.hi), pack2(0.f, v0.lo)};
+        return {pack2(v0.hi, hi2(v.h)), pack2(v0.lo, hi2(v.l))};
+    }
+    // the pair, its second row only, or nothing
+    static __device__ __forceinline__ ffp keep(const ffp& x, bool all, bool second) {
+        const f2 k = all ? ~0ull : second ? 0xFFFFFFFF00000000ull : 0ull;
+        return {x.h & k, x.l & k};
+    }
+    static __device__ __forceinline__ void dot(ffp& acc, const ffp& x, const ffp& y) { dot_acc2(acc, x, y); }
+    static __device__ __forceinline__ ffp update(const ffp& c, const ffp& w, const ffp& v) { return update2(c, w, v); }
+    static __device__ __forceinline__ S total(const ffp (&a)[ACCS]) { return warp_total(sum3(a)); }
+};
+
+// Float64: the words are the two rows; 2 tag bits (1, 2, 3 in turn, 0 at the start). The FP64 pipe
+// holds a sub-partition for 64 cycles a warp instruction, whatever depends on what and however many
+// lanes count: one chain of partial sums, comparisons on the bits, and the reflector's scalars formed
+// by one warp (by all 14 of a CTA, with three partial sums, 1000 x 1004 took 11.3 ms; the persistent
+// kernel 10.4).
+struct F64Arith {
+    using S = double;
+    static constexpr f2 TAG_BITS = 0x4000000000000000ull;
+    static constexpr int RANGE = 400;
+    static constexpr int ACCS = 1;
+    static constexpr bool SHARED_SCALARS = true;
+    // the order of non-negative doubles is that of their bits; a NaN counts as small
+    static __device__ __forceinline__ bool too_small(S n) {
+        return bits(n) - (123ull << 52) >= (2047ull - 123ull) << 52;      // below 2^-900
+    }
+    static __device__ __forceinline__ Tag tag(int j) {
+        const uint32_t n = (uint32_t)(j >> 1) % 3u + 1u;
+        return {(f2)(n & 1u) << 62, (f2)(n & 2u) << 61};
+    }
+    static __device__ __forceinline__ double d(f2 w) { return __longlong_as_double((long long)w); }
+    static __device__ __forceinline__ f2 bits(S a) { return (f2)__double_as_longlong(a); }
+    static __device__ __forceinline__ S of(f2 w) { return d(w); }
+    static __device__ __forceinline__ S zero() { return 0.0; }
+    static __device__ __forceinline__ S add(S a, S b) { return a + b; }
+    static __device__ __forceinline__ S mul(S a, S b) { return a * b; }
+    static __device__ __forceinline__ S neg(S a) { return d(bits(a) ^ (1ull << 63)); }
+    // Newton's iterations from the approximate functions (20 bits): x r^2 = 1 twice, then s^2 = x with
+    // the residual exact; 1 / a twice. Within an ulp or so, a third of the FP64 pipe's chain.
+    static __device__ __forceinline__ S sqrt(S a) {
+        double r;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+        r = fma(r * 0.5, fma(-a * r, r, 1.0), r);
+        r = fma(r * 0.5, fma(-a * r, r, 1.0), r);
+        const double s = a * r;
+        return fma(fma(-s, s, a), 0.5 * r, s);
+    }
+    static __device__ __forceinline__ S recip(S a) {
+        double q;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(q) : "d"(a));
+        q = fma(fma(-a, q, 1.0), q, q);
+        return fma(fma(-a, q, 1.0), q, q);
+    }
+    static __device__ __forceinline__ bool nonneg(S a) { return (long long)bits(a) >= 0; }
+    static __device__ __forceinline__ S clamp(S a) { return (long long)bits(a) > 0 ? a : 0.0; }
+    static __device__ __forceinline__ bool cancelled(S now, S before) {
+        return (long long)bits(now) < (long long)bits(before) - (10ll << 52);
+    }
+    static __device__ __forceinline__ double to_double(S a) { return a; }
+    // the bits of a norm below 2 (two leading zeros) without the 10 lowest, then 4095 - c
+    static __device__ __forceinline__ unsigned long long key(S n, int c) {
+        return ((bits(n) << 2) & ~4095ull) | (unsigned long long)(4095 - c);
+    }
+    static __device__ __forceinline__ S row(const ffp& x, bool odd) { return d(odd ? x.l : x.h); }
+    static __device__ __forceinline__ ffp pair(double a, double b) { return {bits(a), bits(b)}; }
+    static __device__ __forceinline__ ffp both(S a) { return {bits(a), bits(a)}; }
+    static __device__ __forceinline__ ffp first(const ffp& v, bool odd, S v0) {
+        if (odd) return {0ull, bits(v0)};
+        return {bits(v0), v.l};
+    }
+    static __device__ __forceinline__ ffp keep(const ffp& x, bool all, bool second) {
+        return {all ? x.h : 0ull, all || second ? x.l : 0ull};
+    }
+    static __device__ __forceinline__ void dot(ffp& acc, const ffp& x, const ffp& y) {
+        acc.h = bits(fma(d(x.h), d(y.h), d(acc.h)));
+        acc.l = bits(fma(d(x.l), d(y.l), d(acc.l)));
+    }
+    static __device__ __forceinline__ ffp update(const ffp& c, const ffp& w, const ffp& v) {
+        return {bits(fma(d(w.h), d(v.h), d(c.h))), bits(fma(d(w.l), d(v.l), d(c.l)))};
+    }
+    static __device__ __forceinline__ S total(const ffp (&a)[ACCS]) {
+        double s = d(a[0].h) + d(a[0].l);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    }
+};
+
+template <class A>
 __device__ __forceinline__ bool has_tag(const ulonglong2& w, const Tag& t) {
-    return (w.x & TAG_BITS) == t.h && (w.y & TAG_BITS) == t.l;
+    return (w.x & A::TAG_BITS) == t.h && (w.y & A::TAG_BITS) == t.l;
 }
 __device__ __forceinline__ void st_packet(ulonglong2* p, const ffp& x, const Tag& t) { st_word(p, x.h | t.h, x.l | t.l); }
-__device__ __forceinline__ ffp unpack(const ulonglong2& w) { return {w.x & ~TAG_BITS, w.y & ~TAG_BITS}; }
+template <class A>
+__device__ __forceinline__ ffp unpack(const ulonglong2& w) { return {w.x & ~A::TAG_BITS, w.y & ~A::TAG_BITS}; }
 
 // A wait's deadline: true while it may go on.
 struct Deadline {
     long long t0 = 0;
     unsigned int it = 0;
-    __device__ __forceinline__ bool more(const QrFfDev& p) {
+    __device__ __forceinline__ bool more(const QrRegsDev& p) {
         if (it == 0u) t0 = clock64();
         if (clock64() - t0 >= p.timeout && it > 0u) {
             atomicExch(p.abort_flag, 1);
@@ -112,7 +242,7 @@ struct Deadline {
 
 // Warp-wide: waits until the G records carry `tag`, returns the largest key and whether its norm
 // has cancelled; false on expiry.
-__device__ __forceinline__ bool poll_records(const QrFfDev& p, const ulonglong2* rec, int G, uint32_t tag, int lane,
+__device__ __forceinline__ bool poll_records(const QrRegsDev& p, const ulonglong2* rec, int G, uint32_t tag, int lane,
                                              unsigned long long& key, bool& cancelled) {
     Deadline d;
     while (true) {
@@ -140,15 +270,17 @@ __device__ __forceinline__ void column_barrier(int c) {
 }
 
 // NP: row pairs per lane; WPC: warps per column (l <= 64 NP WPC); MAXW: most warps of a CTA.
-template <int NP, int WPC, int MAXW>
-__global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
-    __shared__ ulonglong2 vs[32 * NP * WPC];         // the reflector, zero above row j: high pairs, low pairs
+template <class A, int NP, int WPC, int MAXW>
+__global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
+    using S = typename A::S;
+    __shared__ ulonglong2 vs[32 * NP * WPC];         // the reflector, zero above row j
     __shared__ double col_mx[MAXW];
     __shared__ unsigned long long key_s[MAXW];       // the columns' keys (0: retired)
     __shared__ uint32_t flag_s[MAXW];                // whether a column's early norm has cancelled
     __shared__ unsigned long long win_s[2];          // the winner by round
     __shared__ int state_s[2];                       // 0: expired, 1: winner, 2: winner has cancelled
-    __shared__ float2 dot_s[MAXW], nsq_s[MAXW], cj_s[MAXW];
+    __shared__ f2 dot_s[MAXW], nsq_s[MAXW], cj_s[MAXW];
+    __shared__ f2 scal_s[3];                         // alpha, v0, beta where one warp forms them
     __shared__ int ok_s, e_s, range_s;
     const int l = p.l, m = p.m, cpc = p.cpc, npk = (l + 1) >> 1;
     const int b = blockIdx.x, G = gridDim.x, t = threadIdx.x, lane = t & 31, warp = t >> 5, NT = blockDim.x;
@@ -163,7 +295,10 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
     //    smallest largest entry, exchanged once (see the top)
     if (mine) {
         double cm = 0.0;
-        for (int i = 32 * part + lane; i < l; i += 32 * WPC) cm = fmax(cm, fabs(p.S[(int64_t)col * p.lds + i]));
+        for (int i = 32 * part + lane; i < l; i += 32 * WPC) {
+            const double x = fabs(p.S[(int64_t)col * p.lds + i]);
+            cm = fmax(cm, isfinite(x) ? x : INFINITY);
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) cm = fmax(cm, __shfl_xor_sync(0xffffffffu, cm, o));
         if (lane == 0) col_mx[warp] = cm;
@@ -180,7 +315,8 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
             double cm = col_mx[q * WPC];
             for (int u = 1; u < WPC; ++u) cm = fmax(cm, col_mx[q * WPC + u]);
             int e = INT_MIN / 2;
-            if (cm > 0.0) frexp(cm, &e);                     // cm < 2^e
+            if (isinf(cm)) e = 2 * MAX_SCALE;                // an entry that is not finite
+            else if (cm > 0.0) frexp(cm, &e);                // cm < 2^e
             e_hi = max(e_hi, e);
             e_lo = min(e_lo, e);
         }
@@ -209,7 +345,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
     }
     __syncthreads();
     if (!ok_s) return;
-    if (range_s > 40) {                                     // the same decision in every CTA
+    if (range_s > A::RANGE || abs(e_s) > MAX_SCALE) {            // the same decision in every CTA
         if (b == 0 && t == 0) *p.fallback = 1;
         return;
     }
@@ -217,18 +353,18 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
 
     // the column, its norm and its packets for step 0
     f2 ch[NP], cl[NP];
-    ff nsq = {0.f, 0.f};
+    S nsq = A::zero();
     bool active = mine;
     int pos = -1;
-    ff alpha_mine = {0.f, 0.f};
+    S alpha_mine = A::zero();
     // the column's sum over its warps of each warp's total (every lane receives it)
-    auto column_sum = [&](ff x, float2* buf) {
+    auto column_sum = [&](S x, f2* buf) {
         if (WPC == 1) return x;
-        if (lane == 0) buf[warp] = make_float2(x.hi, x.lo);
+        if (lane == 0) buf[warp] = A::bits(x);
         column_barrier<WPC>(cw);
-        ff sum = {buf[cw * WPC].x, buf[cw * WPC].y};
+        S sum = A::of(buf[cw * WPC]);
 #pragma unroll
-        for (int u = 1; u < WPC; ++u) sum = ff_add(sum, {buf[cw * WPC + u].x, buf[cw * WPC + u].y});
+        for (int u = 1; u < WPC; ++u) sum = A::add(sum, A::of(buf[cw * WPC + u]));
         return sum;
     };
     // the CTA's record of step s (warp 0, after a barrier): its largest key, and that column's flag
@@ -248,21 +384,20 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
     if (mine) {
         const double sc = ldexp(1.0, -E);
         const double* src = p.S + (int64_t)col * p.lds;
-        ffp a = {0ull, 0ull};
+        ffp a[A::ACCS] = {};
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             const int q = pair_of(i), r0 = 2 * q;
-            const ff x = r0 < l ? ff_from_double(src[r0] * sc) : ff{0.f, 0.f};
-            const ff y = r0 + 1 < l ? ff_from_double(src[r0 + 1] * sc) : ff{0.f, 0.f};
-            ch[i] = pack2(x.hi, y.hi);
-            cl[i] = pack2(x.lo, y.lo);
-            dot_acc2(a, {ch[i], cl[i]}, {ch[i], cl[i]});
-            if (q < npk) st_packet(p.slots + (size_t)col * npk + q, {ch[i], cl[i]}, step_tag(0));
+            const ffp x = A::pair(r0 < l ? src[r0] * sc : 0.0, r0 + 1 < l ? src[r0 + 1] * sc : 0.0);
+            ch[i] = x.h;
+            cl[i] = x.l;
+            A::dot(a[i % A::ACCS], x, x);
+            if (q < npk) st_packet(p.slots + (size_t)col * npk + q, x, A::tag(0));
         }
-        nsq = column_sum(warp_total(a), nsq_s);
+        nsq = column_sum(A::total(a), nsq_s);
         if (lane == 0 && part == 0) {
-            st_word(p.nrm + col, pack2(nsq.hi, nsq.lo), 1ull);
-            key_s[cw] = norm_key(nsq, col);
+            st_word(p.nrm + col, A::bits(nsq), 1ull);
+            key_s[cw] = A::key(nsq, col);
         }
     } else {
 #pragma unroll
@@ -279,7 +414,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
         int round = 0;
         for (; round < 2; ++round) {
             if (round == 1) {
-                if (active && lane == 0 && part == 0) key_s[cw] = norm_key(nsq, col);
+                if (active && lane == 0 && part == 0) key_s[cw] = A::key(nsq, col);
                 __syncthreads();
                 if (warp == 0) publish(p.rec_exact, j, false);
             }
@@ -302,7 +437,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
         if (piv < 0 || piv >= m) return;                      // cannot happen while columns remain
         // 2. the reflector: the pivot's packets of rows j .. l-1, the row-j packet and the norm
         const ulonglong2* slot = p.slots + (size_t)par * par_stride + (size_t)piv * npk;
-        const Tag tag = step_tag(j);
+        const Tag tag = A::tag(j);
         const int q0 = j >> 1;
         bool good = true;
         constexpr int VL = (32 * NP * WPC + 127) / 128;      // packets per thread at 128 threads
@@ -310,36 +445,45 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
 #pragma unroll
         for (int k = 0; k < VL; ++k)
             if (q0 + t + k * NT < npk) w[k] = ld_word(slot + q0 + t + k * NT);
-        ulonglong2 wj = ld_word(slot + q0), wn = ld_word(p.nrm + (size_t)par * m + piv);
+        const bool scalars = !A::SHARED_SCALARS || warp == 0;
+        S alpha = A::zero(), v0 = A::zero(), beta = A::zero();
+        bool small = false;                                  // the kernel enqueued behind takes over
         if (t == 0 && q0 > 0) vs[q0 - 1] = make_ulonglong2(0ull, 0ull);
-        {
+        if (scalars) {
+            ulonglong2 wj = ld_word(slot + q0), wn = ld_word(p.nrm + (size_t)par * m + piv);
             Deadline d;
-            while (!has_tag(wj, tag) && good) { good = d.more(p); wj = ld_word(slot + q0); }
+            while (!has_tag<A>(wj, tag) && good) { good = d.more(p); wj = ld_word(slot + q0); }
             while ((uint32_t)wn.y != (uint32_t)(j + 1) && good) { good = d.more(p); wn = ld_word(p.nrm + (size_t)par * m + piv); }
+            const S npiv = A::of(wn.x);
+            small = A::too_small(npiv);
+            const S x0 = A::row(unpack<A>(wj), (j & 1) != 0);
+            const S nx = A::sqrt(npiv);
+            alpha = A::nonneg(x0) ? A::neg(nx) : nx;
+            v0 = A::add(x0, A::neg(alpha));
+            beta = A::recip(A::mul(nx, A::add(nx, A::nonneg(x0) ? x0 : A::neg(x0))));
+            if (A::SHARED_SCALARS && t == 0) {
+                scal_s[0] = A::bits(alpha);
+                scal_s[1] = A::bits(v0);
+                scal_s[2] = A::bits(beta);
+            }
         }
-        const ff npiv = {lo2(wn.x), hi2(wn.x)};
-        const bool small = !(npiv.hi >= 0x1p-112f);          // the float64 kernel takes over
-        const ffp pj = unpack(wj);
-        const ff x0 = (j & 1) ? ff{hi2(pj.h), hi2(pj.l)} : ff{lo2(pj.h), lo2(pj.l)};
-        const ff nx = ff_sqrt_newton(npiv);
-        const ff alpha = x0.hi >= 0.f ? ff_neg(nx) : nx;
-        const ff v0 = ff_add(x0, ff_neg(alpha));
-        const ff beta = ff_recip_newton(ff_mul(nx, ff_add(nx, x0.hi >= 0.f ? x0 : ff_neg(x0))));
 #pragma unroll
         for (int k = 0; k < VL; ++k) {
             const int q = q0 + t + k * NT;
             if (q < npk) {
                 Deadline d;
-                while (!has_tag(w[k], tag) && good) { good = d.more(p); w[k] = ld_word(slot + q); }
-                ffp v = unpack(w[k]);
-                if (q == q0) {                               // rows above j stay out, row j: x0 - alpha
-                    if (j & 1) v = {pack2(0.f, v0.hi), pack2(0.f, v0.lo)};
-                    else v = {pack2(v0.hi, hi2(v.h)), pack2(v0.lo, hi2(v.l))};
-                }
+                while (!has_tag<A>(w[k], tag) && good) { good = d.more(p); w[k] = ld_word(slot + q); }
+                ffp v = unpack<A>(w[k]);
+                if (q == q0) v = A::first(v, (j & 1) != 0, v0);   // rows above j stay out, row j: x0 - alpha
                 vs[q] = make_ulonglong2(v.h, v.l);
             }
         }
         good = __syncthreads_and(good && !small);
+        if (A::SHARED_SCALARS) {
+            alpha = A::of(scal_s[0]);
+            v0 = A::of(scal_s[1]);
+            beta = A::of(scal_s[2]);
+        }
         if (!good) {
             if (small && b == 0 && t == 0) *p.fallback = 1;   // every thread of every CTA reads the same norm
             return;
@@ -354,40 +498,36 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
             }
         }
         // 3. the dot product (v is zero outside rows j .. l - 1, so whole groups of rows go through;
-        //    three at a time keep independent chains in flight) and the next trailing norm
-        ff nw = {0.f, 0.f};
+        //    in float-float three at a time, to keep independent chains in flight) and the next trailing norm
+        S nw = A::zero();
         if (active) {
-            ffp a[3] = {{0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}};
+            ffp a[A::ACCS] = {};
             f2 xh = 0ull, xl = 0ull;                          // the pair that holds row j
 #pragma unroll
-            for (int i = 0; i < NP; i += 3)
-                if (64 * WPC * (i + 3) > j) {
+            for (int i = 0; i < NP; i += A::ACCS)
+                if (64 * WPC * (i + A::ACCS) > j && 64 * WPC * i < l) {
 #pragma unroll
-                    for (int u = 0; u < 3; ++u) {
+                    for (int u = 0; u < A::ACCS; ++u) {
                         const ulonglong2 v = vs[pair_of(i + u)];
-                        dot_acc2(a[u], {v.x, v.y}, {ch[i + u], cl[i + u]});
+                        A::dot(a[u], {v.x, v.y}, {ch[i + u], cl[i + u]});
                     }
                     if (64 * WPC * i <= j) {
 #pragma unroll
-                        for (int u = 0; u < 3; ++u)
+                        for (int u = 0; u < A::ACCS; ++u)
                             if (pair_of(i + u) == q0) { xh = ch[i + u]; xl = cl[i + u]; }
                     }
                 }
-            ff cj;
-            if (WPC == 1) {
-                cj = {__shfl_sync(0xffffffffu, (j & 1) ? hi2(xh) : lo2(xh), q0 & 31),
-                      __shfl_sync(0xffffffffu, (j & 1) ? hi2(xl) : lo2(xl), q0 & 31)};
-            } else if ((q0 >> 5) % WPC == part && lane == (q0 & 31)) {
-                cj_s[cw] = (j & 1) ? make_float2(hi2(xh), hi2(xl)) : make_float2(lo2(xh), lo2(xl));
-            }
-            nw = ff_neg(ff_mul(column_sum(warp_total(sum3(a)), dot_s), beta));
-            if (WPC > 1) cj = {cj_s[cw].x, cj_s[cw].y};
+            S cj = A::row({xh, xl}, (j & 1) != 0);
+            if (WPC == 1) cj = A::of(__shfl_sync(0xffffffffu, A::bits(cj), q0 & 31));
+            else if ((q0 >> 5) % WPC == part && lane == (q0 & 31)) cj_s[cw] = A::bits(cj);
+            nw = A::neg(A::mul(column_sum(A::total(a), dot_s), beta));
+            if (WPC > 1) cj = A::of(cj_s[cw]);
             if (part == 0) {
-                const ff r = ff_add(cj, ff_mul(nw, v0));      // R's entry
-                const ff ne = ff_add(nsq, ff_neg(ff_mul(r, r)));
+                const S r = A::add(cj, A::mul(nw, v0));       // R's entry
+                const S ne = A::add(nsq, A::neg(A::mul(r, r)));
                 if (lane == 0) {
-                    key_s[cw] = norm_key(ne.hi > 0.f ? ne : ff{0.f, 0.f}, col);
-                    flag_s[cw] = ne.hi < nsq.hi * 0x1p-10f ? 1u : 0u;
+                    key_s[cw] = A::key(A::clamp(ne), col);
+                    flag_s[cw] = A::cancelled(ne, nsq) ? 1u : 0u;
                 }
             }
         }
@@ -395,32 +535,30 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
         if (warp == 0) publish(p.rec, j + 1, true);
         // 4. the update, the fresh norm, the packets of step j + 1
         if (active) {
-            const ffp w2 = {pack2(nw.hi, nw.hi), pack2(nw.lo, nw.lo)};
+            const ffp w2 = A::both(nw);
             ulonglong2* dst = p.slots + (size_t)(par ^ 1) * par_stride + (size_t)col * npk;
-            const Tag ntag = step_tag(j + 1);
+            const Tag ntag = A::tag(j + 1);
             const int qn = (j + 1) >> 1;
-            // rows j + 1 .. count in the fresh norm: of the pair that holds row j its second row, or none
-            const f2 edge = (j & 1) ? 0ull : 0xFFFFFFFF00000000ull;
-            ffp a[3] = {{0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}};
+            ffp a[A::ACCS] = {};
 #pragma unroll
-            for (int i = 0; i < NP; i += 3)
-                if (64 * WPC * (i + 3) > j) {
+            for (int i = 0; i < NP; i += A::ACCS)
+                if (64 * WPC * (i + A::ACCS) > j && 64 * WPC * i < l) {
 #pragma unroll
-                    for (int u = 0; u < 3; ++u) {
+                    for (int u = 0; u < A::ACCS; ++u) {
                         const int q = pair_of(i + u);
                         const ulonglong2 v = vs[q];
-                        const ffp x = update2({ch[i + u], cl[i + u]}, w2, {v.x, v.y});
+                        const ffp x = A::update({ch[i + u], cl[i + u]}, w2, {v.x, v.y});
                         ch[i + u] = x.h;
                         cl[i + u] = x.l;
                         if (q >= qn && q < npk) st_packet(dst + q, x, ntag);
-                        const f2 keep = q > q0 ? ~0ull : q == q0 ? edge : 0ull;
-                        const ffp y = {x.h & keep, x.l & keep};
-                        dot_acc2(a[u], y, y);
+                        // rows j + 1 .. count in the fresh norm: of the pair that holds row j its second, or none
+                        const ffp y = A::keep(x, q > q0, q == q0 && !(j & 1));
+                        A::dot(a[u], y, y);
                     }
                 }
-            nsq = column_sum(warp_total(sum3(a)), nsq_s);
+            nsq = column_sum(A::total(a), nsq_s);
             if (lane == 0 && part == 0)
-                st_word(p.nrm + (size_t)(par ^ 1) * m + col, pack2(nsq.hi, nsq.lo), (unsigned long long)(uint32_t)(j + 2));
+                st_word(p.nrm + (size_t)(par ^ 1) * m + col, A::bits(nsq), (unsigned long long)(uint32_t)(j + 2));
         }
     }
     // R[:, pos] = rows 0 .. pos of the retired column, scaled back by 2^E
@@ -432,8 +570,8 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_ff_kernel(QrFfDev p) {
         for (int u = 0; u < 2; ++u) {
             const int row = r0 + u;
             if (row >= m) continue;
-            const ff x = row == pos ? alpha_mine : u ? ff{hi2(ch[i]), hi2(cl[i])} : ff{lo2(ch[i]), lo2(cl[i])};
-            p.R[(int64_t)row * m + pos] = row <= pos ? ldexp(ff_to_double(x), E) : 0.0;
+            const S x = row == pos ? alpha_mine : A::row({ch[i], cl[i]}, u != 0);
+            p.R[(int64_t)row * m + pos] = row <= pos ? ldexp(A::to_double(x), E) : 0.0;
         }
     }
 }
@@ -446,30 +584,38 @@ struct Shape {
 }  // namespace
 
 // Workspace: the packets, the records, the norms and the scale exchange.
-size_t qr_ff_work_doubles(int m, int l) {
+size_t qr_regs_work_doubles(int m, int l) {
     const size_t npk = ((size_t)l + 1) / 2;
     return 2 * (2 * (size_t)m * npk) + 2 * 6 * (size_t)m + (size_t)m + 64;
 }
 
-cudaError_t pivoted_qr_ff_regs(const double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work,
-                               int* status, cudaStream_t s, long long spin_limit, int* fallback, bool* launched) {
+cudaError_t pivoted_qr_regs(const double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work,
+                            int* status, cudaStream_t s, long long spin_limit, int* fallback, bool f64, bool* launched) {
     *launched = false;
     int dev = 0, coop = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     const int sms = sm_count();
     if (!coop) return cudaSuccess;
-    // Warps per column, and rows a lane holds. Four columns a CTA while that fits the chip, more beyond.
-    const Shape shapes[] = {{(const void*)qr_ff_kernel<3, 1, 16>, 3, 1, 16}, {(const void*)qr_ff_kernel<6, 1, 16>, 6, 1, 16},
-                            {(const void*)qr_ff_kernel<9, 1, 16>, 9, 1, 16}, {(const void*)qr_ff_kernel<6, 2, 16>, 6, 2, 16},
-                            {(const void*)qr_ff_kernel<12, 1, 16>, 12, 1, 16}, {(const void*)qr_ff_kernel<9, 2, 16>, 9, 2, 16},
-                            {(const void*)qr_ff_kernel<12, 2, 16>, 12, 2, 16}, {(const void*)qr_ff_kernel<24, 1, 12>, 24, 1, 12},
-                            {(const void*)qr_ff_kernel<9, 4, 16>, 9, 4, 16}, {(const void*)qr_ff_kernel<33, 1, 8>, 33, 1, 8}};
-    const int cpc = std::max((m + sms - 1) / sms, std::min(4, m));
+    // Warps per column, and row pairs a lane holds.
+#define QR_SHAPE(A, NP, WPC, MAXW) {(const void*)qr_regs_kernel<A, NP, WPC, MAXW>, NP, WPC, MAXW}
+    const Shape ff_shapes[] = {QR_SHAPE(FfArith, 3, 1, 16),  QR_SHAPE(FfArith, 6, 1, 16),  QR_SHAPE(FfArith, 9, 1, 16),
+                               QR_SHAPE(FfArith, 6, 2, 16),  QR_SHAPE(FfArith, 12, 1, 16), QR_SHAPE(FfArith, 9, 2, 16),
+                               QR_SHAPE(FfArith, 12, 2, 16), QR_SHAPE(FfArith, 24, 1, 12), QR_SHAPE(FfArith, 9, 4, 16),
+                               QR_SHAPE(FfArith, 33, 1, 8)};
+    const Shape f64_shapes[] = {QR_SHAPE(F64Arith, 3, 2, 16), QR_SHAPE(F64Arith, 6, 2, 16), QR_SHAPE(F64Arith, 9, 2, 16),
+                                QR_SHAPE(F64Arith, 12, 2, 16), QR_SHAPE(F64Arith, 9, 4, 16)};
+#undef QR_SHAPE
+    // Four columns a CTA while that fits the chip (float64: two, whose arithmetic then has a sub-
+    // partition each; 256 x 544 took 1.35 ms by fours, 1.17 by twos), more beyond.
+    const int few = f64 ? 2 : 4;
+    const int cpc = std::max((m + sms - 1) / sms, std::min(few, m));
     const int G = (m + cpc - 1) / cpc;
     const Shape* sh = nullptr;
-    for (const Shape& x : shapes)
-        if (l <= 64 * x.np * x.wpc && cpc * x.wpc <= x.maxw) { sh = &x; break; }
+    const Shape* first = f64 ? std::begin(f64_shapes) : std::begin(ff_shapes);
+    const Shape* last = f64 ? std::end(f64_shapes) : std::end(ff_shapes);
+    for (const Shape* x = first; x != last && !sh; ++x)
+        if (l <= 64 * x->np * x->wpc && cpc * x->wpc <= x->maxw) sh = x;
     if (!sh) return cudaSuccess;
     const int nt = 32 * std::max(cpc * sh->wpc, 4);   // at least 128 threads load the pivot column's packets
     int per_sm = 0;
@@ -478,7 +624,7 @@ cudaError_t pivoted_qr_ff_regs(const double* S, int m, int l, int64_t lds, doubl
         cudaGetLastError();
         return cudaSuccess;
     }
-    QrFfDev p;
+    QrRegsDev p;
     p.S = S; p.m = m; p.l = l; p.lds = lds; p.R = R; p.perm = perm; p.cpc = cpc;
     const size_t npk = ((size_t)l + 1) / 2;
     ulonglong2* w = reinterpret_cast<ulonglong2*>(work);

@@ -545,6 +545,10 @@ rtproj_status rtproj_precondition(rtproj_t h, uint64_t seed, int64_t l) {
             RT_CHECK(pivoted_qr_ff(h->S, m, (int)l, l, h->R, h->perm, h->qr_work, h->status, s, h->spin_limit,
                                    qr_flag, h->opts.async != 0, &ff_first));
     }
+    // float64: the register form first where it has the chip to itself (k_qr.cu, pivoted_qr_ff)
+    if (!ff_first && !h->opts.async)
+        RT_CHECK(pivoted_qr_regs(h->S, m, (int)l, l, h->R, h->perm, h->qr_work, h->status, s, h->spin_limit, qr_flag, true,
+                                 &ff_first));
     RT_CHECK(pivoted_qr(h->S, m, (int)l, l, h->R, h->perm, h->qr_work, h->status, s, h->spin_limit,
                         ff_first ? qr_flag : nullptr));
     // default threshold: 8 times the sketch's relative precision -- 2^-52 in float64, 2^(-8 s)

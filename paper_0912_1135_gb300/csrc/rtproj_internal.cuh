@@ -146,11 +146,12 @@ bool pivoted_qr_persistent_ok(int m, int l);
 // float64 kernel, which must follow with run_if = fallback.
 cudaError_t pivoted_qr_ff(double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work, int* status,
                           cudaStream_t s, long long spin_limit, int* fallback, bool side_by_side, bool* launched);
-// Its form with the columns in registers (k_qr_ff.cu), taken first; not launched when a column does
-// not fit a warp's registers. qr_ff_work_doubles: its part of the work area.
-cudaError_t pivoted_qr_ff_regs(const double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work, int* status,
-                               cudaStream_t s, long long spin_limit, int* fallback, bool* launched);
-size_t qr_ff_work_doubles(int m, int l);
+// The form with the columns in registers (k_qr_regs.cu), float-float or float64 (f64), taken first; not
+// launched when a column does not fit a warp's registers. As above, *fallback = 1 asks for the
+// persistent float64 kernel behind it. qr_regs_work_doubles: its part of the work area.
+cudaError_t pivoted_qr_regs(const double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work, int* status,
+                            cudaStream_t s, long long spin_limit, int* fallback, bool f64, bool* launched);
+size_t qr_regs_work_doubles(int m, int l);
 // The mixed form's QR on one 16-CTA cluster in float-float arithmetic (k_qr_cluster.cu).
 // Sets *launched when the kernel was enqueued; the kernel then writes *fallback = 1 if the
 // entries' range needs the float64 kernel (which must follow with run_if = fallback).
