@@ -15,22 +15,25 @@
 //  3. each active column's dot product with the reflector gives its row-j entry r, hence its next
 //     trailing norm n - r^2 before the column is updated: the CTA's record for step j + 1 is
 //     published here, and the exchange overlaps the update;
-//  4. the update, which also sums the new norm afresh and writes the column's packets (into
-//     the other of two buffers) and norm for step j + 1.
+//  4. the update, which also sums the new norm afresh and writes the column's packets and norm for
+//     step j + 1.
 // A packet, record or norm is one 128-bit store and one 128-bit load, which are single-copy
 // atomic, so a reader needs neither a fence nor a flag behind the data: the former kernel's
 // release fence, arrival counter, winner word and column load were four L2 round trips in a row
 // (3.7 us a step at 512 x 516). What remains is the exchange (about 2800 cycles from a record's store
 // until every CTA has seen all of them, across both dies) and one column load (850). A retired
-// column's slot is never rewritten, so late readers of a pivot column are safe; a record buffer is
+// column's packets are never rewritten, so late readers of a pivot column are safe; a record buffer is
 // rewritten only after every CTA has published the step between. Every wait has a clock deadline;
 // on expiry the kernel raises RTPROJ_ETIMEOUT and all CTAs leave.
 // Measured: 512 x 516 1.89 -> 1.50 ms (2.9 us a step), 64 x 256 246 -> 172 us, 333 x 698 1.37 -> 1.15 ms,
-// 256 x 1024 1.27 -> 1.02 ms, 1024 x 2080 7.55 -> 7.09 ms (there the column arithmetic counts: seven
-// columns of 2080 rows a CTA). Float64, against the persistent kernel: 1000 x 1004 10.4 -> 7.2 ms, 256 x
-// 544 1.49 -> 1.12 ms; the FP64 pipe (64 cycles a warp instruction) bounds its columns. Not kept: one 16-CTA cluster with the same columns and a hardware
-// barrier a step (5 to 8 us a step: distributed shared memory answers no sooner than L2 here),
-// per-column records polled by every warp, scalars formed after the packets' barrier.
+// 256 x 1024 1.27 -> 1.02 ms, 1024 x 2080 7.6 -> 6.9 ms. Past what registers hold (LONG), against the
+// kernels with the columns in shared memory or in L2: 700 x 1900 5.1 -> 4.3 ms, 1500 x 1504 10.0 -> 8.8,
+// 1024 x 4096 23 -> 12, 2048 x 4128 52 -> 39; there the column arithmetic of the CTA with most columns left
+// counts. Float64, against the persistent kernel: 1000 x 1004 10.4 -> 7.2 ms, 256 x 544 1.49 -> 1.12 ms;
+// the FP64 pipe (64 cycles a warp instruction) bounds its columns. Not kept: one 16-CTA cluster with
+// the same columns and a hardware barrier a step (5 to 8 us a step: distributed shared memory answers
+// no sooner than L2 here), per-column records polled by every warp, scalars formed after the packets'
+// barrier.
 //
 // The early norm n - r^2 is exact to 2^-47 of n (n is summed afresh every step). When the winner's
 // has cancelled by more than 2^10 the candidates are exchanged once more with their fresh
@@ -53,7 +56,8 @@ struct QrRegsDev {
     const double* S; int m, l; int64_t lds;
     double* R; int32_t* perm;
     int cpc;
-    ulonglong2* slots;       // 2 x m x npk: packets by step parity
+    ulonglong2* slots;       // m x npk: the columns' packets
+    int tg, ts;              // LONG: row pairs of a column kept in its packets only, and in shared memory
     ulonglong2* rec;         // 2 x G: candidate records by step parity
     ulonglong2* rec_exact;   // 2 x G: the same with fresh norms (only when a winner has cancelled)
     ulonglong2* nrm;         // 2 x m: fresh squared norms
@@ -65,6 +69,7 @@ struct QrRegsDev {
     int* fallback;
 };
 
+constexpr int LB = 4;                                // packets of a column in flight per lane (LONG)
 constexpr int MAX_SCALE = 1000;                      // largest scale's exponent that is taken here
 
 // ---- 128-bit words in global memory, single-copy atomic at GPU scope
@@ -89,7 +94,7 @@ struct Tag {
 // The arithmetic: a scalar S, and a pair of rows (2 q, 2 q + 1) as two 64-bit words. A packet is the
 // pair's words as they are, with a tag of step j in exponent bits that are zero: S^* is scaled so that
 // no column's norm exceeds 1, and reflections keep the norms, so every entry is below 2 in magnitude.
-// A slot's previous content is the packet of two steps before (or the zero written at the start),
+// A slot's previous content is the packet of the step before (or the zero written at the start),
 // whose tag differs.
 
 // Float-float: the words are both rows' high parts and both rows' low parts; 4 tag bits.
@@ -101,7 +106,7 @@ struct FfArith {
     static constexpr bool SHARED_SCALARS = false;             // every thread forms the reflector's scalars
     static __device__ __forceinline__ bool too_small(S n) { return !(n.hi >= 0x1p-112f); }
     static __device__ __forceinline__ Tag tag(int j) {
-        const uint32_t n = ((uint32_t)(j >> 1) + 1u) & 15u;
+        const uint32_t n = ((uint32_t)j & 7u) + 1u;
         return {((f2)((n & 1u) << 30)) | ((f2)((n & 2u) << 29) << 32), ((f2)((n & 4u) << 28)) | ((f2)((n & 8u) << 27) << 32)};
     }
     static __device__ __forceinline__ S zero() { return {0.f, 0.f}; }
@@ -156,7 +161,7 @@ struct F64Arith {
         return bits(n) - (123ull << 52) >= (2047ull - 123ull) << 52;      // below 2^-900
     }
     static __device__ __forceinline__ Tag tag(int j) {
-        const uint32_t n = (uint32_t)(j >> 1) % 3u + 1u;
+        const uint32_t n = (uint32_t)j % 3u + 1u;
         return {(f2)(n & 1u) << 62, (f2)(n & 2u) << 61};
     }
     static __device__ __forceinline__ double d(f2 w) { return __longlong_as_double((long long)w); }
@@ -269,11 +274,20 @@ __device__ __forceinline__ void column_barrier(int c) {
     else asm volatile("barrier.sync %0, %1;" ::"r"(c + 1), "n"(32 * WPC) : "memory");
 }
 
-// NP: row pairs per lane; WPC: warps per column (l <= 64 NP WPC); MAXW: most warps of a CTA.
-template <class A, int NP, int WPC, int MAXW>
+// NP: row pairs per lane; WPC: warps per column; MAXW: most warps of a CTA. l <= 64 NP WPC, or with
+// LONG any l: a column's first pairs p.tg live in its packets (read back from L2 in both passes), the
+// next p.ts in shared memory, the rest in registers -- the rows that leave the factorization first
+// are the ones whose reads cost most. tg and ts are multiples of 32 WPC. Few pairs in registers and
+// few packets in flight, so that nothing spills: 12 and 6 of them took 51 ms at 2048 x 4128, 3 and 4
+// take 39.
+template <class A, int NP, int WPC, int MAXW, bool LONG>
 __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
     using S = typename A::S;
-    __shared__ ulonglong2 vs[32 * NP * WPC];         // the reflector, zero above row j
+    constexpr int GR = 32 * WPC;                     // pairs of a column's group: one a lane
+    extern __shared__ __align__(16) ulonglong2 qr_smem[];
+    __shared__ ulonglong2 vs_short[LONG ? 1 : NP * GR];
+    const int base = LONG ? p.tg + p.ts : 0;         // the first pair in registers
+    ulonglong2* vs = LONG ? qr_smem : vs_short;      // the reflector, zero above row j
     __shared__ double col_mx[MAXW];
     __shared__ unsigned long long key_s[MAXW];       // the columns' keys (0: retired)
     __shared__ uint32_t flag_s[MAXW];                // whether a column's early norm has cancelled
@@ -287,9 +301,11 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
     const int c0 = b * cpc, nc = max(0, min(cpc, m - c0));
     const int cw = warp / WPC, part = warp % WPC, col = c0 + cw;      // the warp's column and its share of the rows
     const bool mine = cw < nc;
-    const size_t par_stride = (size_t)m * npk;
-    // pair (u) of the warp's i-th group of rows
-    auto pair_of = [&](int i) { return 32 * (i * WPC + part) + lane; };
+    // pair of the warp's i-th group in registers, and of the column's g-th group
+    auto pair_of = [&](int i) { return base + 32 * (i * WPC + part) + lane; };
+    auto pair_in = [&](int g) { return g * GR + 32 * part + lane; };
+    ulonglong2* held = LONG ? qr_smem + base + NP * GR + (size_t)cw * p.ts - p.tg : nullptr;   // indexed by pair
+    const int g_l2 = LONG ? p.tg / GR : 0, g_sm = LONG ? base / GR : 0;   // groups: [0, g_l2) L2, [g_l2, g_sm) shared
 
     // 0. tags cleared; the scale: exponents of the CTAs' largest entries, and of their columns'
     //    smallest largest entry, exchanged once (see the top)
@@ -304,10 +320,9 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
         if (lane == 0) col_mx[warp] = cm;
         for (int q = 32 * part + lane; q < npk; q += 32 * WPC) {
             st_word(p.slots + (size_t)col * npk + q, 0ull, 0ull);
-            st_word(p.slots + par_stride + (size_t)col * npk + q, 0ull, 0ull);
         }
     }
-    for (int q = t; q < 32 * NP * WPC; q += NT) vs[q] = make_ulonglong2(0ull, 0ull);
+    for (int q = t; q < base + NP * GR; q += NT) vs[q] = make_ulonglong2(0ull, 0ull);
     __syncthreads();
     if (t == 0) {
         int e_hi = INT_MIN / 2, e_lo = INT_MAX / 2;
@@ -394,6 +409,15 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
             A::dot(a[i % A::ACCS], x, x);
             if (q < npk) st_packet(p.slots + (size_t)col * npk + q, x, A::tag(0));
         }
+        if constexpr (LONG) {
+            for (int g = 0; g < g_sm; ++g) {
+                const int q = pair_in(g), r0 = 2 * q;
+                const ffp x = A::pair(r0 < l ? src[r0] * sc : 0.0, r0 + 1 < l ? src[r0 + 1] * sc : 0.0);
+                A::dot(a[0], x, x);
+                if (q < npk) st_packet(p.slots + (size_t)col * npk + q, x, A::tag(0));
+                if (g >= g_l2) held[q] = make_ulonglong2(x.h, x.l);
+            }
+        }
         nsq = column_sum(A::total(a), nsq_s);
         if (lane == 0 && part == 0) {
             st_word(p.nrm + col, A::bits(nsq), 1ull);
@@ -436,11 +460,11 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
         const int piv = 4095 - (int)(win & 4095ull);
         if (piv < 0 || piv >= m) return;                      // cannot happen while columns remain
         // 2. the reflector: the pivot's packets of rows j .. l-1, the row-j packet and the norm
-        const ulonglong2* slot = p.slots + (size_t)par * par_stride + (size_t)piv * npk;
+        const ulonglong2* slot = p.slots + (size_t)piv * npk;
         const Tag tag = A::tag(j);
         const int q0 = j >> 1;
         bool good = true;
-        constexpr int VL = (32 * NP * WPC + 127) / 128;      // packets per thread at 128 threads
+        constexpr int VL = LONG ? 6 : (NP * GR + 127) / 128; // packets per thread (at 128 threads all of them)
         ulonglong2 w[VL];
 #pragma unroll
         for (int k = 0; k < VL; ++k)
@@ -478,6 +502,14 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
                 vs[q] = make_ulonglong2(v.h, v.l);
             }
         }
+        if constexpr (LONG)
+            for (int q = q0 + t + VL * NT; q < npk; q += NT) {
+                ulonglong2 x = ld_word(slot + q);
+                Deadline d;
+                while (!has_tag<A>(x, tag) && good) { good = d.more(p); x = ld_word(slot + q); }
+                const ffp v = unpack<A>(x);
+                vs[q] = make_ulonglong2(v.h, v.l);
+            }
         good = __syncthreads_and(good && !small);
         if (A::SHARED_SCALARS) {
             alpha = A::of(scal_s[0]);
@@ -503,15 +535,42 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
         if (active) {
             ffp a[A::ACCS] = {};
             f2 xh = 0ull, xl = 0ull;                          // the pair that holds row j
+            if constexpr (LONG) {
+                const ulonglong2* own = p.slots + (size_t)col * npk;
+                int g = q0 / GR;                              // the first group with a row from j on
+                for (; g < g_l2; g += LB) {
+                    ulonglong2 x[LB];
+#pragma unroll
+                    for (int u = 0; u < LB; ++u)
+                        if (g + u < g_l2) x[u] = ld_word(own + pair_in(g + u));
+#pragma unroll
+                    for (int u = 0; u < LB; ++u)
+                        if (g + u < g_l2) {
+                            const int q = pair_in(g + u);
+                            const ulonglong2 v = vs[q];
+                            const ffp c = unpack<A>(x[u]);
+                            A::dot(a[0], {v.x, v.y}, c);
+                            if (q == q0) { xh = c.h; xl = c.l; }
+                        }
+                }
+                g = max(q0 / GR, g_l2);
+#pragma unroll 2
+                for (; g < g_sm; ++g) {
+                    const int q = pair_in(g);
+                    const ulonglong2 v = vs[q], c = held[q];
+                    A::dot(a[0], {v.x, v.y}, {c.x, c.y});
+                    if (q == q0) { xh = c.x; xl = c.y; }
+                }
+            }
 #pragma unroll
             for (int i = 0; i < NP; i += A::ACCS)
-                if (64 * WPC * (i + A::ACCS) > j && 64 * WPC * i < l) {
+                if (base + GR * (i + A::ACCS) > q0 && (A::ACCS > 1 || base + GR * i < npk)) {
 #pragma unroll
                     for (int u = 0; u < A::ACCS; ++u) {
                         const ulonglong2 v = vs[pair_of(i + u)];
                         A::dot(a[u], {v.x, v.y}, {ch[i + u], cl[i + u]});
                     }
-                    if (64 * WPC * i <= j) {
+                    if (base + GR * i <= q0) {
 #pragma unroll
                         for (int u = 0; u < A::ACCS; ++u)
                             if (pair_of(i + u) == q0) { xh = ch[i + u]; xl = cl[i + u]; }
@@ -536,24 +595,52 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
         // 4. the update, the fresh norm, the packets of step j + 1
         if (active) {
             const ffp w2 = A::both(nw);
-            ulonglong2* dst = p.slots + (size_t)(par ^ 1) * par_stride + (size_t)col * npk;
+            ulonglong2* dst = p.slots + (size_t)col * npk;
             const Tag ntag = A::tag(j + 1);
             const int qn = (j + 1) >> 1;
             ffp a[A::ACCS] = {};
+            // one pair: the updated rows, counted in the fresh norm from row j + 1 on (of the pair that holds
+            // row j its second row, or none)
+            auto step = [&](const ffp& c, int q, ffp& acc, bool st) {
+                const ulonglong2 v = vs[q];
+                const ffp x = A::update(c, w2, {v.x, v.y});
+                if (st) st_packet(dst + q, x, ntag);
+                const ffp y = A::keep(x, q > q0, q == q0 && !(j & 1));
+                A::dot(acc, y, y);
+                return x;
+            };
+            if constexpr (LONG) {
+                int g = q0 / GR;
+                for (; g < g_l2; g += LB) {
+                    ulonglong2 x[LB];
+#pragma unroll
+                    for (int u = 0; u < LB; ++u)
+                        if (g + u < g_l2) x[u] = ld_word(dst + pair_in(g + u));
+#pragma unroll
+                    for (int u = 0; u < LB; ++u)
+                        if (g + u < g_l2) {
+                            const int q = pair_in(g + u);
+                            const ffp y = step(unpack<A>(x[u]), q, a[0], q >= q0);
+                        }
+                }
+                g = max(q0 / GR, g_l2);
+#pragma unroll 2
+                for (; g < g_sm; ++g) {
+                    const int q = pair_in(g);
+                    const ulonglong2 c = held[q];
+                    const ffp y = step({c.x, c.y}, q, a[0], q >= qn);
+                    held[q] = make_ulonglong2(y.h, y.l);
+                }
+            }
 #pragma unroll
             for (int i = 0; i < NP; i += A::ACCS)
-                if (64 * WPC * (i + A::ACCS) > j && 64 * WPC * i < l) {
+                if (base + GR * (i + A::ACCS) > q0 && (A::ACCS > 1 || base + GR * i < npk)) {
 #pragma unroll
                     for (int u = 0; u < A::ACCS; ++u) {
                         const int q = pair_of(i + u);
-                        const ulonglong2 v = vs[q];
-                        const ffp x = A::update({ch[i + u], cl[i + u]}, w2, {v.x, v.y});
+                        const ffp x = step({ch[i + u], cl[i + u]}, q, a[u], q >= qn && q < npk);
                         ch[i + u] = x.h;
                         cl[i + u] = x.l;
-                        if (q >= qn && q < npk) st_packet(dst + q, x, ntag);
-                        // rows j + 1 .. count in the fresh norm: of the pair that holds row j its second, or none
-                        const ffp y = A::keep(x, q > q0, q == q0 && !(j & 1));
-                        A::dot(a[u], y, y);
                     }
                 }
             nsq = column_sum(A::total(a), nsq_s);
@@ -563,22 +650,30 @@ __global__ void __launch_bounds__(32 * MAXW, 1) qr_regs_kernel(QrRegsDev p) {
     }
     // R[:, pos] = rows 0 .. pos of the retired column, scaled back by 2^E
     if (!mine || pos < 0) return;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-        const int r0 = 2 * pair_of(i);
+    auto store_pair = [&](int q, const ffp& c) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int row = r0 + u;
+            const int row = 2 * q + u;
             if (row >= m) continue;
-            const S x = row == pos ? alpha_mine : A::row({ch[i], cl[i]}, u != 0);
+            const S x = row == pos ? alpha_mine : A::row(c, u != 0);
             p.R[(int64_t)row * m + pos] = row <= pos ? ldexp(A::to_double(x), E) : 0.0;
         }
-    }
+    };
+#pragma unroll
+    for (int i = 0; i < NP; ++i) store_pair(pair_of(i), {ch[i], cl[i]});
+    if constexpr (LONG)
+        for (int g = 0; g < g_sm; ++g) {
+            const int q = pair_in(g);
+            if (2 * q >= m) break;
+            if (g >= g_l2) store_pair(q, {held[q].x, held[q].y});
+            else store_pair(q, unpack<A>(ld_word(p.slots + (size_t)col * npk + q)));
+        }
 }
 
 struct Shape {
     const void* kern;
     int np, wpc, maxw;
+    bool longer;
 };
 
 }  // namespace
@@ -586,7 +681,7 @@ struct Shape {
 // Workspace: the packets, the records, the norms and the scale exchange.
 size_t qr_regs_work_doubles(int m, int l) {
     const size_t npk = ((size_t)l + 1) / 2;
-    return 2 * (2 * (size_t)m * npk) + 2 * 6 * (size_t)m + (size_t)m + 64;
+    return 2 * ((size_t)m * npk) + 2 * 6 * (size_t)m + (size_t)m + 64;
 }
 
 cudaError_t pivoted_qr_regs(const double* S, int m, int l, int64_t lds, double* R, int32_t* perm, double* work,
@@ -598,14 +693,16 @@ cudaError_t pivoted_qr_regs(const double* S, int m, int l, int64_t lds, double* 
     const int sms = sm_count();
     if (!coop) return cudaSuccess;
     // Warps per column, and row pairs a lane holds.
-#define QR_SHAPE(A, NP, WPC, MAXW) {(const void*)qr_regs_kernel<A, NP, WPC, MAXW>, NP, WPC, MAXW}
+#define QR_SHAPE(A, NP, WPC, MAXW) {(const void*)qr_regs_kernel<A, NP, WPC, MAXW, false>, NP, WPC, MAXW, false}
+#define QR_LONG(A, NP, WPC, MAXW) {(const void*)qr_regs_kernel<A, NP, WPC, MAXW, true>, NP, WPC, MAXW, true}
     const Shape ff_shapes[] = {QR_SHAPE(FfArith, 3, 1, 16),  QR_SHAPE(FfArith, 6, 1, 16),  QR_SHAPE(FfArith, 9, 1, 16),
                                QR_SHAPE(FfArith, 6, 2, 16),  QR_SHAPE(FfArith, 12, 1, 16), QR_SHAPE(FfArith, 9, 2, 16),
-                               QR_SHAPE(FfArith, 12, 2, 16), QR_SHAPE(FfArith, 24, 1, 12), QR_SHAPE(FfArith, 9, 4, 16),
-                               QR_SHAPE(FfArith, 33, 1, 8)};
+                               QR_SHAPE(FfArith, 12, 2, 16), QR_SHAPE(FfArith, 30, 1, 8),  QR_SHAPE(FfArith, 33, 1, 8),
+                               QR_LONG(FfArith, 3, 4, 16),   QR_LONG(FfArith, 3, 2, 16),   QR_LONG(FfArith, 3, 1, 16)};
     const Shape f64_shapes[] = {QR_SHAPE(F64Arith, 3, 2, 16), QR_SHAPE(F64Arith, 6, 2, 16), QR_SHAPE(F64Arith, 9, 2, 16),
                                 QR_SHAPE(F64Arith, 12, 2, 16), QR_SHAPE(F64Arith, 9, 4, 16)};
 #undef QR_SHAPE
+#undef QR_LONG
     // Four columns a CTA while that fits the chip (float64: two, whose arithmetic then has a sub-
     // partition each; 256 x 544 took 1.35 ms by fours, 1.17 by twos), more beyond.
     const int few = f64 ? 2 : 4;
@@ -615,20 +712,44 @@ cudaError_t pivoted_qr_regs(const double* S, int m, int l, int64_t lds, double* 
     const Shape* first = f64 ? std::begin(f64_shapes) : std::begin(ff_shapes);
     const Shape* last = f64 ? std::end(f64_shapes) : std::end(ff_shapes);
     for (const Shape* x = first; x != last && !sh; ++x)
-        if (l <= 64 * x->np * x->wpc && cpc * x->wpc <= x->maxw) sh = x;
+        if ((x->longer || l <= 64 * x->np * x->wpc) && cpc * x->wpc <= x->maxw) {
+            // A warp with 30 or more pairs a lane pays from seven columns a CTA up (with fewer, two or four
+            // warps a column are faster: 900 x 2100, six columns, 5.6 ms as LONG, 6.3 so) and when its rows fill
+            // nine tenths of the registers (1000 x 1600 5.8 as LONG, 6.1 so; 1000 x 1900 6.6 and 6.2; 1024 x 2080
+            // 7.2 and 6.9).
+            if (x->np >= 30 && (cpc < 7 || 10 * l <= 9 * 64 * x->np)) continue;
+            sh = x;
+        }
     if (!sh) return cudaSuccess;
     const int nt = 32 * std::max(cpc * sh->wpc, 4);   // at least 128 threads load the pivot column's packets
+    // LONG: as many groups of each column in shared memory as fit beside the reflector, the rest in L2
+    const size_t npk = ((size_t)l + 1) / 2;
+    const int gr = 32 * sh->wpc, in_regs = gr * sh->np;
+    int tg = 0, ts = 0;
+    size_t smem = 0;
+    if (sh->longer) {
+        const int rest = std::max(0, ((int)npk - in_regs + gr - 1) / gr * gr);
+        const size_t room = (size_t)(220 << 10) / sizeof(ulonglong2), reflector = (size_t)rest + in_regs;
+        if (reflector + (size_t)cpc * gr > room) return cudaSuccess;
+        ts = std::min(rest, (int)((room - reflector) / cpc) / gr * gr);
+        tg = rest - ts;
+        smem = (reflector + (size_t)cpc * ts) * sizeof(ulonglong2);
+        if (cudaFuncSetAttribute(sh->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+            cudaGetLastError();
+            return cudaSuccess;
+        }
+    }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sh->kern, nt, 0) != cudaSuccess || per_sm < 1 ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sh->kern, nt, smem) != cudaSuccess || per_sm < 1 ||
         G > per_sm * sms) {
         cudaGetLastError();
         return cudaSuccess;
     }
     QrRegsDev p;
     p.S = S; p.m = m; p.l = l; p.lds = lds; p.R = R; p.perm = perm; p.cpc = cpc;
-    const size_t npk = ((size_t)l + 1) / 2;
+    p.tg = tg; p.ts = ts;
     ulonglong2* w = reinterpret_cast<ulonglong2*>(work);
-    p.slots = w;      w += 2 * (size_t)m * npk;
+    p.slots = w;      w += (size_t)m * npk;
     ulonglong2* cleared = w;                       // words whose tags must start at zero
     p.rec = w;        w += 2 * (size_t)G;
     p.rec_exact = w;  w += 2 * (size_t)G;
@@ -645,7 +766,7 @@ cudaError_t pivoted_qr_regs(const double* S, int m, int l, int64_t lds, double* 
     if (e == cudaSuccess) e = cudaMemsetAsync(fallback, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
     void* args[] = {&p};
-    e = cudaLaunchCooperativeKernel(sh->kern, dim3((unsigned)G), dim3((unsigned)nt), args, 0, s);
+    e = cudaLaunchCooperativeKernel(sh->kern, dim3((unsigned)G), dim3((unsigned)nt), args, smem, s);
     note_launch();
     if (e != cudaSuccess) {
         cudaGetLastError();   // clear; the caller's other kernels run
