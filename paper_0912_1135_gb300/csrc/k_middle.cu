@@ -50,7 +50,7 @@ __device__ __forceinline__ i128acc merge_lanes(i128acc a, int o) {
     return a;
 }
 
-// Block (r, g): row r of the product with T (row-major, leading dimension m; entries t of
+// Block (g, r): row r of the product with T (row-major, leading dimension m; entries t of
 // [r, m) when UPPER, of [0, r] otherwise) for the LG columns from g LG on. LG lanes of a warp
 // take a column each and the 32 / LG lane groups of all warps split the sum over t (so that
 // T's row is read coalesced where LG is small and once per warp where it is 32).
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(32 * MD_MAX_WARPS) middle_rows_kernel(const do
                                                                         double* __restrict__ out, int* status) {
     __shared__ i128acc part[MD_MAX_WARPS][LG];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    const int r = blockIdx.x, j = blockIdx.y * LG + (lane & (LG - 1));
+    const int r = blockIdx.y, j = blockIdx.x * LG + (lane & (LG - 1));
     constexpr int GROUPS = 32 / LG;
     const int lo = UPPER ? r : 0, hi = UPPER ? m : r + 1;
     const unsigned long long* row = reinterpret_cast<const unsigned long long*>(T) + (int64_t)r * m;
@@ -100,7 +100,7 @@ void launch_rows(const double* T, int m, const double* x, const int32_t* gather,
     while (lg < 32 && lg < k) lg <<= 1;
     int warps = 1;
     while (warps < MD_MAX_WARPS && (int64_t)m * lg > (int64_t)32 * MD_TERMS_PER_LANE * warps) warps <<= 1;
-    const dim3 grid((unsigned)m, (unsigned)((k + lg - 1) / lg));
+    const dim3 grid((unsigned)((k + lg - 1) / lg), (unsigned)m);   // m <= I128_MAX_TERMS; k may be any
     auto go = [&](auto kern) { kern<<<grid, 32 * warps, 0, s>>>(T, m, x, gather, scatter, k, out, status); };
     switch (lg) {
         case 1: go(middle_rows_kernel<1, UPPER>); break;

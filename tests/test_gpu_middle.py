@@ -48,3 +48,17 @@ def test_direct_and_sliced_forms_agree(m, ks):
         for k in ks:
             got = P.lstsq(B[:k].contiguous()).cpu().numpy()
             assert np.max(np.abs(got - want[:k])) <= 4 * m * 2.0 ** -52 * m * KAPPA ** 2 * np.max(np.abs(want))
+
+
+def test_more_columns_than_a_grid_dimension():
+    """m = 1 with k past 65535 groups of 32 columns: every row of Z is b - (a b) a^* / (a a^*)."""
+    torch, rt = torch_cuda(), rt_module()
+    k, n = 65535 * 32 + 33, 8
+    A = np.random.default_rng(1).standard_normal((1, n))
+    B = torch.randn(k, n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    with rt.Projector(to_dev(torch, A), l_max=n, k_max=k) as P:
+        P.precondition(seed=5, l=n)
+        Z = P.null_project(B)
+    a = to_dev(torch, A)
+    want = B - (B @ a.T) @ a / (a @ a.T)
+    assert float((Z - want).abs().max()) <= 64 * 2.0 ** -52 * float(B.abs().max())
