@@ -76,7 +76,7 @@ typedef enum {
        of X run in float-float on the FP32 pipe, each with the float64 kernel enqueued
        behind it for ranges float-float cannot hold; T1 = L^{-1} R^{-*} is formed in
        float64, and the m x m stage's products with it are sliced tensor-core products
-       (apply_slices). */
+       (apply_slices) or, for small m^2 k, exact integer sums rounded once. */
     RTPROJ_MIXED_REFINED = 1
 } rtproj_mode;
 
@@ -205,11 +205,12 @@ rtproj_status rtproj_create(rtproj_t* out, int64_t m, int64_t n, const void* A, 
    ld n) are float64 device matrices, r = 0 (U, V null) for S alone, 0 <= r <= min(m, 64);
    k_max <= 65535.
    All of them are borrowed: they must stay alive and unchanged until rtproj_destroy.
-   The handle runs the float64 arithmetic of the dense float64 form on the products that
-   build the preconditioner (S_k = A G with G generated per nonzero; X column by column
-   as in steps a-e after Eq. 15: D = A^* P^-, E = A D, X = R^{-*} Pi E) and sums every
-   product with A or A^* of the apply and its refinement passes (Remark 4.3; opts
-   refine_passes and refine_tol) in double-double, so that the refinement converges to
+   The preconditioner is built to float64's accuracy (S_k = A G with G generated a panel at
+   a time; X column by column as in steps a-e after Eq. 15: D = A^* P^-, E = A D,
+   X = R^{-*} Pi E; the sketch and the low-rank products as exact sums of fixed-point
+   values, the rest in float64), and every product with A or A^* of the apply and its
+   refinement passes (Remark 4.3; opts refine_passes and refine_tol) is a sum of exact
+   products in 128-bit integers, rounded once, so that the refinement converges to
    the projection of the stored matrix. A product with A costs O(nnz + r (m + n)).
    opts.mode, the slice counts and qr_form do not apply; dtype must be RTPROJ_F64 and
    scalable 0 (else RTPROJ_EUNSUPPORTED). rtproj_create_sparse synchronizes the stream:

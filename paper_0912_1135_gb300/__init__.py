@@ -347,7 +347,7 @@ class Projector:
 class SparseProjector(Projector):
     """A = S + U V with S sparse (compressed sparse row, on the device) and an optional
     low-rank term U V (``rtproj_create_sparse``): the products with A cost O(nnz + r(m + n))
-    and the apply's residuals are summed in double-double. The arrays are borrowed for the
+    and the apply's residuals are sums of exact products, rounded once. The arrays are borrowed for the
     handle's lifetime (kept referenced here). The other methods are those of Projector;
     set_scaling is not supported."""
 

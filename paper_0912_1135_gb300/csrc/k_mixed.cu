@@ -1,20 +1,21 @@
 // Mixed mode: every product with A on the tensor cores through exact digit slicing
-// (k_slice.cu, k_umma.cu), the m x m stage in float64, and refinement (Remark 4.3).
+// (k_slice.cu, k_umma.cu), the m x m stage there too or, for small blocks, summed exactly in
+// integers (k_middle.cu), and refinement (Remark 4.3).
 //
 // Preconditioner (Section 4):
 //   S = A G           sketch_slices digits of A times the one-digit G plane (Eq. 12)
-//   pivoted QR of S^* in float64 (Eq. 13); R^{-*} by a triangular solve
+//   pivoted QR of S^* in float-float (Eq. 13); R^{-*} by a triangular solve
 //   W = R^{-*} Pi A   = M' A^, where A^ is A with row i divided by 2^{e_i} (its slicing
 //                     exponent) and M'[i][k] = R^{-*}[i][t] 2^{e_k} for k = perm[t]:
 //                     gram_slices digits of M' against the transposed digits of A^
 //   X = W W^*         gram2_slices digits of W (Eq. 14 as a Gram product), then Cholesky
 // Apply, for right-hand sides b (rows of B):
 //   c  = A b                       apply_slices digits        (step 1)
-//   h0 = Pi^* T1^* T1 Pi c         float64                     (steps 2-6)
+//   h0 = Pi^* T1^* T1 Pi c         apply_slices digits, or exact sums (steps 2-6)
 //   s  = b - A^* h0                resid_slices digits of A^ and of 2^{e} h0
 //   repeat refine_passes times (Remark 4.3):
 //     r  = A s                     resid_slices digits
-//     dh = Pi^* T1^* T1 Pi r       float64
+//     dh = Pi^* T1^* T1 Pi r       as h0
 //     h  = h + dh;  s = s - A^* dh apply_slices digits
 //   Z = s, ROW = b - s, least squares h.
 // Because the digit products and their sums are exact, the residual products s and r

@@ -6,7 +6,8 @@
 //   S_k = A G                 one CTA per (row, 64 columns of G); G generated a panel at a time
 //                             (the same entries as the dense forms), Eq. 12
 //   X column by column as in steps a-e that follow Eq. 15, all m columns at once:
-//     D = A^* P^-             (n x m) one CTA per column of A, a gather over its nonzeros
+//     D = A^* P^-             (n x m) a thread per column of P^-, a gather over the nonzeros of A's
+//                             columns; the low-rank part, and V D after it, by limbs
 //     E = A D                 (m x m) one CTA per row of A
 //     X = R^{-*} Pi E         one float64 product with the triangular R^{-*}
 //   apply (the seven steps) and its refinement (Remark 4.3) with every product with A or

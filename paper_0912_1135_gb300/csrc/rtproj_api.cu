@@ -444,7 +444,7 @@ rtproj_status rtproj_create_sparse(rtproj_t* out, int64_t m, int64_t n, int64_t 
         return RTPROJ_EUNSUPPORTED;
     if (o.dtype != RTPROJ_F64 || o.scalable) return RTPROJ_EUNSUPPORTED;
     if (((uintptr_t)workspace) % kAlign) return RTPROJ_EINVAL;
-    o.mode = RTPROJ_PLAIN_FP64;   // the sparse form: float64 products, double-double residuals
+    o.mode = RTPROJ_PLAIN_FP64;   // the sparse form: float64 preconditioner, exact products in the apply
     const Layout L = make_layout(m, n, l_max, k_max, o);
     if (ws_bytes < L.total + sparse_bytes(m, n, nnz, r, l_max, k_max)) return RTPROJ_ENOMEM;
     // the row pointers bound every later read of col_idx and val: checked here, on the host
