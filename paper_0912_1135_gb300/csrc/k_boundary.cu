@@ -16,39 +16,45 @@ namespace {
 
 constexpr int BT = 256;
 
-__global__ void widen_kernel(const float* __restrict__ src, int64_t lds, int rows, int cols, double* __restrict__ dst,
-                             int64_t ldd) {
-    const int64_t total = (int64_t)rows * cols;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = idx / cols, c = idx % cols;
-        dst[r * ldd + c] = (double)src[r * lds + c];
+// A CTA's share of a rows x cols block: ROW_TILE columns of every gridDim.y-th row, four entries a
+// thread in flight (a flat index took a 64-bit division an entry). f(r, c) loads, g(r, c, x) stores.
+constexpr int ROW_TILE = 4 * BT;
+template <typename Load, typename Store>
+__device__ __forceinline__ void for_entries(int rows, int cols, Load f, Store g) {
+    const int c0 = blockIdx.x * ROW_TILE + threadIdx.x;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+        double x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = c0 + i * BT < cols ? f(r, c0 + i * BT) : 0.0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (c0 + i * BT < cols) g(r, c0 + i * BT, x[i]);
     }
+}
+dim3 entry_grid(int rows, int cols) {
+    return dim3((unsigned)((cols + ROW_TILE - 1) / ROW_TILE), (unsigned)std::min(rows, 65535));
+}
+
+__global__ void __launch_bounds__(BT) widen_kernel(const float* __restrict__ src, int64_t lds, int rows, int cols,
+                                                   double* __restrict__ dst, int64_t ldd) {
+    for_entries(rows, cols, [&](int64_t r, int c) { return widen_exact(src[r * lds + c]); },
+                [&](int64_t r, int c, double x) { dst[r * ldd + c] = x; });
 }
 
 // dst = src diag(d) (d optional), widened to float64
 template <typename T>
-__global__ void form_rows_kernel(const T* __restrict__ src, int64_t lds, int rows, int cols, const double* __restrict__ d,
-                                 double* __restrict__ dst, int64_t ldd) {
-    const int64_t total = (int64_t)rows * cols;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = idx / cols, c = idx % cols;
-        const double x = (double)src[r * lds + c];
-        dst[r * ldd + c] = d ? x * d[c] : x;
-    }
+__global__ void __launch_bounds__(BT) form_rows_kernel(const T* __restrict__ src, int64_t lds, int rows, int cols,
+                                                       const double* __restrict__ d, double* __restrict__ dst, int64_t ldd) {
+    for_entries(rows, cols, [&](int64_t r, int c) { return widen_exact(src[r * lds + c]); },
+                [&](int64_t r, int c, double x) { dst[r * ldd + c] = d ? x * d[c] : x; });
 }
 
 template <typename T>
-__global__ void store_rows_kernel(const double* __restrict__ X, int64_t ldx, const double* __restrict__ B, int64_t ldb,
-                                  T* __restrict__ dst, int64_t ldd, int rows, int cols, int sub) {
-    const int64_t total = (int64_t)rows * cols;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = idx / cols, c = idx % cols;
-        const double x = X[r * ldx + c];
-        dst[r * ldd + c] = (T)(sub ? B[r * ldb + c] - x : x);
-    }
+__global__ void __launch_bounds__(BT) store_rows_kernel(const double* __restrict__ X, int64_t ldx, const double* __restrict__ B,
+                                                        int64_t ldb, T* __restrict__ dst, int64_t ldd, int rows, int cols,
+                                                        int sub) {
+    for_entries(rows, cols, [&](int64_t r, int c) { return sub ? B[r * ldb + c] - X[r * ldx + c] : X[r * ldx + c]; },
+                [&](int64_t r, int c, double x) { dst[r * ldd + c] = narrow_rounded<T>(x); });
 }
 
 // 32 x 32 tiles through shared memory: reads of src and writes of dst both coalesced.
@@ -65,7 +71,7 @@ __global__ void store_transposed_kernel(const double* __restrict__ src, int64_t 
     __syncthreads();
     for (int y = ty; y < 32; y += 8) {
         const int c = c0 + y, r = r0 + tx;
-        if (c < cols && r < rows) dst[(int64_t)c * ldd + r] = (T)tile[tx][y];
+        if (c < cols && r < rows) dst[(int64_t)c * ldd + r] = narrow_rounded<T>(tile[tx][y]);
     }
 }
 
@@ -181,7 +187,7 @@ unsigned grid_for(int64_t total) {
 
 cudaError_t widen_rows(const float* src, int64_t lds, int rows, int cols, double* dst, int64_t ldd, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
-    widen_kernel<<<grid_for((int64_t)rows * cols), BT, 0, s>>>(src, lds, rows, cols, dst, ldd);
+    widen_kernel<<<entry_grid(rows, cols), BT, 0, s>>>(src, lds, rows, cols, dst, ldd);
     note_launch();
     return cudaGetLastError();
 }
@@ -189,7 +195,7 @@ cudaError_t widen_rows(const float* src, int64_t lds, int rows, int cols, double
 cudaError_t form_rows(const void* src, int dt, int64_t lds, int rows, int cols, const double* d, double* dst, int64_t ldd,
                       cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
-    const unsigned g = grid_for((int64_t)rows * cols);
+    const dim3 g = entry_grid(rows, cols);
     if (dt == RTPROJ_F32)
         form_rows_kernel<float><<<g, BT, 0, s>>>((const float*)src, lds, rows, cols, d, dst, ldd);
     else
@@ -201,7 +207,7 @@ cudaError_t form_rows(const void* src, int dt, int64_t lds, int rows, int cols, 
 cudaError_t store_rows(const double* X, int64_t ldx, const double* B, int64_t ldb, void* dst, int64_t ldd, int rows,
                        int cols, int sub, int dt, cudaStream_t s) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
-    const unsigned g = grid_for((int64_t)rows * cols);
+    const dim3 g = entry_grid(rows, cols);
     if (dt == RTPROJ_F32)
         store_rows_kernel<float><<<g, BT, 0, s>>>(X, ldx, B, ldb, (float*)dst, ldd, rows, cols, sub);
     else

@@ -145,14 +145,6 @@ __device__ __forceinline__ void store_digits(const DigitWord<W> (&a)[8], const f
     }
 }
 
-// A float32 as the bits of the float64 of the same value (a subnormal by the conversion).
-__device__ __forceinline__ uint2 widen_bits(float x) {
-    const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
-    if (m - 0x00800000u < 0x7F000000u) return make_uint2(u << 29, (u & 0x80000000u) | ((m >> 3) + 0x38000000u));
-    const double d = (double)x;
-    return make_uint2((uint32_t)__double2loint(d), (uint32_t)__double2hiint(d));
-}
-
 __device__ __forceinline__ uint2 entry_bits(const double* p) { return __ldg(reinterpret_cast<const uint2*>(p)); }
 __device__ __forceinline__ uint2 entry_bits(const float* p) { return widen_bits(__ldg(p)); }
 
