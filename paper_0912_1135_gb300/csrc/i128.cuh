@@ -10,7 +10,8 @@
 // product, and each addition loses less than one unit 2^E, so a sum of N products is within
 // N 2^-105 of the largest product's magnitude: the bound of a double-double sum, whose
 // every addition rounds at 2^-105 of the partial sum. Capacity: products enter at most
-// 2^115 units large, so 2^11 of them fit 127 bits (I128_MAX_TERMS).
+// 2^115 units large, so 2^11 of them fit 127 bits (I128_MAX_TERMS); a longer sum is taken in parts
+// of that many, which are added in double-double (i128_full, i128_flush).
 #pragma once
 
 #include <cstdint>
@@ -261,6 +262,37 @@ __device__ __forceinline__ void i128_to_pair(const i128acc& a, double& hi, doubl
     else if (cut > 0) mL = (1ull << cut) - 1ull;
     hi = u128_to_double(H & ~mH, L & ~mL, a.E);
     lo = u128_to_double(H & mH, L & mL, a.E);
+}
+
+// ---- sums of more products than one integer holds: each full sum joins a double-double pair
+
+__device__ __forceinline__ void two_sum_d(double a, double b, double& s, double& e) {   // Knuth's TwoSum
+    s = a + b;
+    const double bb = s - a;
+    e = (a - (s - bb)) + (b - bb);
+}
+
+__device__ __forceinline__ void dd_add(double& hi, double& lo, double bh, double bl) {
+    double s, e;
+    two_sum_d(hi, bh, s, e);
+    e += lo + bl;
+    hi = s + e;
+    lo = e - (hi - s);
+}
+
+// Counts a product; true when the sum is full: it has to be flushed before the next one.
+__device__ __forceinline__ bool i128_full(int& terms) {
+    if (++terms < I128_MAX_TERMS) return false;
+    terms = 0;
+    return true;
+}
+
+// The sum moves over to the pair hi + lo and starts anew.
+__device__ __forceinline__ void i128_flush(i128acc& a, double& hi, double& lo) {
+    double h, l;
+    i128_to_pair(a, h, l);
+    dd_add(hi, lo, h, l);
+    a = i128_zero();
 }
 
 }  // namespace rtp

@@ -35,23 +35,6 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
     } while (0)
 
 // ---------------------------------------------------------------------------------
-// Double-double building block: Knuth's TwoSum.
-// ---------------------------------------------------------------------------------
-__device__ __forceinline__ void two_sum_d(double a, double b, double& s, double& e) {
-    s = a + b;
-    const double bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-__device__ __forceinline__ void dd_add(double& hi, double& lo, double bh, double bl) {
-    double s, e;
-    two_sum_d(hi, bh, s, e);
-    e += lo + bl;
-    hi = s + e;
-    lo = e - (hi - s);
-}
-
-// ---------------------------------------------------------------------------------
 // The column-compressed copy: counting sort by column, then each column's entries put in
 // (row, value) order, so that every sum over a column runs in one fixed order whatever the
 // order in which the scatter's atomics landed.
@@ -860,6 +843,7 @@ __global__ void __launch_bounds__(32 * SP_WARPS)
                  const double* __restrict__ H, int k, int n, int r, const double* __restrict__ V,
                  const double* __restrict__ UtH, const double* Y, int64_t ldy, double* out, int64_t ldo) {
     constexpr int KL = 1 << LG, SUB = 32 / KL;
+    __shared__ double2 full[SP_WARPS][JB][32];   // full sums so far of a column with more terms than one sum holds
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int j0 = blockIdx.y * (KL * JB) + (lane & (KL - 1));
     const int64_t step = (int64_t)gridDim.x * SP_WARPS * SUB;
@@ -882,6 +866,12 @@ __global__ void __launch_bounds__(32 * SP_WARPS)
             i128_mac(acc[q], one, i128_decode(lo, hi));
         }
         int terms = 1;
+        bool longer = false;
+        auto flush = [&](int q) {
+            double2 v = longer ? full[warp][q][lane] : make_double2(0.0, 0.0);
+            i128_flush(acc[q], v.x, v.y);
+            return v;
+        };
         auto term = [&](double v, const double* h) {
             const i128op a = i128_left(i128_decode((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v)));
             uint32_t lo[JB], hi[JB];
@@ -895,13 +885,10 @@ __global__ void __launch_bounds__(32 * SP_WARPS)
                 bad[q] |= !i128_finite(hi[q]);
                 i128_mac(acc[q], a, i128_decode(lo[q], hi[q]), ~0u);
             }
-            if (++terms == I128_MAX_TERMS / 2) {   // room for as many more (a very long column)
+            if (i128_full(terms)) {              // a very long column
 #pragma unroll
-                for (int q = 0; q < JB; ++q) {
-                    i128_sar(acc[q], 11);
-                    acc[q].E += 11;
-                }
-                terms = 0;
+                for (int q = 0; q < JB; ++q) full[warp][q][lane] = flush(q);
+                longer = true;
             }
         };
         const int64_t pe = cptr[c + 1];
@@ -910,8 +897,14 @@ __global__ void __launch_bounds__(32 * SP_WARPS)
 #pragma unroll
         for (int q = 0; q < JB; ++q) {
             const int j = j0 + q * KL;
-            if (j < k)
-                out[c * ldo + j] = bad[q] ? __longlong_as_double(0x7FF8000000000000ll) : i128_to_double(acc[q]);
+            double v;
+            if (longer) {
+                const double2 f = flush(q);
+                v = f.x + f.y;
+            } else {
+                v = i128_to_double(acc[q]);
+            }
+            if (j < k) out[c * ldo + j] = bad[q] ? __longlong_as_double(0x7FF8000000000000ll) : v;
         }
     }
 }

@@ -1,7 +1,7 @@
 // Host build of the 128-bit sums of exact products (csrc/i128.cuh) for the CPU tests: reads
 // "sum N" or "two N" and N pairs of doubles (hexadecimal), prints the rounded sum of their
-// products and the pair form; "two" forms the sum from two halves merged. "sub N" prints x - V 2^e
-// and V 2^e, each rounded once, for 128-bit integers V.
+// products and the pair form; "two" forms the sum from two halves merged, "long" takes a sum of any
+// length in parts. "sub N" prints x - V 2^e and V 2^e, each rounded once, for 128-bit integers V.
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -43,14 +43,21 @@ int main() {
             continue;
         }
         rtp::i128acc a = rtp::i128_zero(), b = rtp::i128_zero();
-        const bool two = op[0] == 't';
+        const bool two = op[0] == 't', longer = op[0] == 'l';
+        int terms = 0;
+        double hi = 0.0, lo = 0.0;
         for (int i = 0; i < n; ++i) {
             double x, y;
             if (std::scanf("%la %la", &x, &y) != 2) return 1;
             rtp::i128_mac(two && (i & 1) ? b : a, rtp::i128_left(dec(x)), dec(y), i % 3 == 2 ? ~0u : 0u);
+            if (longer && rtp::i128_full(terms)) rtp::i128_flush(a, hi, lo);
+        }
+        if (longer) {
+            rtp::i128_flush(a, hi, lo);
+            std::printf("%a %a %a\n", hi + lo, hi, lo);
+            continue;
         }
         rtp::i128_merge(a, b);
-        double hi, lo;
         rtp::i128_to_pair(a, hi, lo);
         std::printf("%a %a %a\n", rtp::i128_to_double(a), hi, lo);
     }

@@ -70,6 +70,22 @@ def test_sum_of_products(i128, op, kind, n):
         assert abs(lo) <= abs(hi) * 2.0 ** -51 or hi == 0.0
 
 
+@pytest.mark.parametrize("kind,n", [("plain", 2047), ("plain", 2048), ("plain", 2049), ("plain", 4160), ("full", 4160),
+                                    ("wide", 4160), ("cancel", 10000), ("plain", 50000), ("full", 50000)])
+def test_sum_of_any_length(i128, kind, n):
+    """Sums longer than one integer holds, in P parts: each part's terms and its pair lose 2^-105 of the
+    largest product (of the part) a term, and each of the P additions in double-double at most 2^-103
+    of the two magnitudes added, N times the largest product each."""
+    for seed in range(2):
+        xs, ys = _draw(kind, n, 50 + seed)
+        prods = [F(x) * F(y) * (-1 if i % 3 == 2 else 1) for i, (x, y) in enumerate(zip(xs, ys))]
+        exact, top = sum(prods), max(abs(p) for p in prods)
+        got, hi, lo = i128("long", xs, ys)
+        bound = (2 + 8 * (n // 2048 + 1)) * (n + 1) * top / 2 ** 105
+        assert abs(F(hi) + F(lo) - exact) <= bound
+        assert abs(F(got) - exact) <= bound + abs(exact) / 2 ** 53
+
+
 def test_rounding_and_difference(i128):
     """V 2^e is rounded to the nearest double, ties to even, and x - V 2^e is the exact
     difference rounded once wherever the two units lie close enough for it to be taken (always
