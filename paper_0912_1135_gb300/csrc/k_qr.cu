@@ -788,7 +788,7 @@ cudaError_t pivoted_qr_ff(double* S, int m, int l, int64_t lds, double* R, int32
                                        : (const void*)qr_persistent_ff_kernel<false, 1024>;
     const int nt = !in_smem ? 512 : warps_s <= 4 ? 128 : warps_s <= 8 ? 256 : warps_s <= 16 ? 512 : 1024;
     if (cpc > PQ_MAXC || G > PQ_MAX_G || smem + 4096 > (size_t)smem_optin) return cudaSuccess;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_shared(kern, (size_t)smem_optin - 4096);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
     if (per_sm < 1 || G > per_sm * sms) return cudaSuccess;
@@ -856,7 +856,7 @@ cudaError_t pivoted_qr(double* S, int m, int l, int64_t lds, double* R, int32_t*
         const void* kern = in_smem ? (const void*)qr_persistent_kernel<false> : (const void*)qr_persistent_kernel<true>;
         const int nt = in_smem ? PqrShape<false>::NT : PqrShape<true>::NT;
         if (cpc <= PQ_MAXC && G <= PQ_MAX_G && smem + 4096 <= (size_t)smem_optin) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            allow_dynamic_shared(kern, (size_t)smem_optin - 4096);
             int per_sm = 0;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
             if (per_sm >= 1 && G <= per_sm * sms) {

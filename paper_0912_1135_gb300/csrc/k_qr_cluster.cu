@@ -44,6 +44,7 @@ namespace {
 constexpr int CQ_CTAS = 16;
 constexpr int CQ_THREADS = 512;
 constexpr int CQ_WARPS = CQ_THREADS / 32;
+constexpr size_t CQ_MAX_SMEM = 200 * 1024;
 constexpr int CQ_MAXC = 64;
 
 // Warp-wide maximum of (value, index): largest value, lowest index on ties; an index of m
@@ -333,7 +334,7 @@ __global__ void __launch_bounds__(CQ_THREADS, 1) qr_cluster_kernel(CqrDev p) {
 bool qr_cluster_fits(int m, int l) {
     const int cpc = (m + CQ_CTAS - 1) / CQ_CTAS;
     const size_t smem = ((size_t)cpc * l + l) * sizeof(float2);
-    return cpc <= CQ_MAXC && smem <= 200 * 1024;
+    return cpc <= CQ_MAXC && smem <= CQ_MAX_SMEM;
 }
 
 cudaError_t pivoted_qr_cluster(const double* S, int m, int l, int64_t lds, double* R, int32_t* perm, int* fallback,
@@ -343,7 +344,7 @@ cudaError_t pivoted_qr_cluster(const double* S, int m, int l, int64_t lds, doubl
     const int cpc = (m + CQ_CTAS - 1) / CQ_CTAS;
     const size_t smem = ((size_t)cpc * l + l) * sizeof(float2);
     cudaError_t e = cudaFuncSetAttribute(qr_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(qr_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = allow_dynamic_shared((const void*)qr_cluster_kernel, CQ_MAX_SMEM);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return cudaSuccess;   // the caller uses the float64 kernel

@@ -729,12 +729,13 @@ cudaError_t pivoted_qr_regs(const double* S, int m, int l, int64_t lds, double* 
     size_t smem = 0;
     if (sh->longer) {
         const int rest = std::max(0, ((int)npk - in_regs + gr - 1) / gr * gr);
-        const size_t room = (size_t)(220 << 10) / sizeof(ulonglong2), reflector = (size_t)rest + in_regs;
+        constexpr size_t most = (size_t)220 << 10;
+        const size_t room = most / sizeof(ulonglong2), reflector = (size_t)rest + in_regs;
         if (reflector + (size_t)cpc * gr > room) return cudaSuccess;
         ts = std::min(rest, (int)((room - reflector) / cpc) / gr * gr);
         tg = rest - ts;
         smem = (reflector + (size_t)cpc * ts) * sizeof(ulonglong2);
-        if (cudaFuncSetAttribute(sh->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        if (allow_dynamic_shared(sh->kern, most) != cudaSuccess) {
             cudaGetLastError();
             return cudaSuccess;
         }

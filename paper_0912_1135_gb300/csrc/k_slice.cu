@@ -733,12 +733,12 @@ cudaError_t slice_rows_dual(const double* X, int64_t x_rs, const SliceStack& st,
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(st.ld / SLD_TILE), (unsigned)(tst.ld / SLD_TILE));
     const size_t smem = (size_t)st.s * SLD_TILE * SLD_PAD * sizeof(__nv_bfloat16);
-    auto launch = [&](auto kern) {
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto launch = [&](auto kern, int most_planes) {
+        allow_dynamic_shared((const void*)kern, (size_t)most_planes * SLD_TILE * SLD_PAD * sizeof(__nv_bfloat16));
         kern<<<grid, SLD_THREADS, smem, s>>>(a, tst.d, tst.ld, tst.plane_stride, tst.rows);
     };
-    if (st.s <= 7) launch(slice_dual_kernel<2>);
-    else launch(slice_dual_kernel<3>);
+    if (st.s <= 7) launch(slice_dual_kernel<2>, 7);
+    else launch(slice_dual_kernel<3>, 10);
     note_launch();
     return cudaGetLastError();
 }

@@ -1153,7 +1153,7 @@ rtproj_status sparse_gram(rtproj_ctx* h) {
     } else {
         SP_CHECK(fill_int(h->d_top, m, kZeroRowExp, s));
         const size_t smem = (size_t)r * (nt + DC_STAGE) * sizeof(int2);
-        SP_CHECK(cudaFuncSetAttribute(sparse_d_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SP_CHECK(allow_dynamic_shared((const void*)sparse_d_kernel<true>, (size_t)kMaxLowRank * (256 + DC_STAGE) * sizeof(int2)));
         sparse_d_kernel<true><<<dgrid, nt, smem, s>>>(h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, r, h->lrV, h->lr_top,
                                                       h->lr_a, D, h->d_top);
         note_launch();

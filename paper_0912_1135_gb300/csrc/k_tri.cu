@@ -16,6 +16,7 @@ namespace {
 
 constexpr int TRSM_THREADS = 512;
 constexpr int TRSM_BS = 32;       // rows per diagonal block
+constexpr size_t TRSM_MAX_SMEM = 200 * 1024;   // the column being solved
 constexpr int TRSM_DPARTS = 4;    // partial sums per entry of the diagonal-block product (4 warps)
 
 // Inverse of each 32 x 32 diagonal block of T (lower or upper), one CTA of four warps per
@@ -525,7 +526,7 @@ cudaError_t trsm(const double* T, int64_t t_rs, int64_t t_cs, bool lower, int m,
                  const int* run_if) {
     if (m <= 0 || ncols <= 0) return cudaSuccess;
     const size_t smem = (size_t)m * sizeof(double);
-    if (smem > 200 * 1024) return cudaErrorInvalidValue;
+    if (smem > TRSM_MAX_SMEM) return cudaErrorInvalidValue;
     const int nblk = (m + TRSM_BS - 1) / TRSM_BS;
     unsigned int* next_col = (unsigned int*)(dinv_work + (size_t)nblk * TRSM_BS * TRSM_BS);
     int dev = 0, sms = 0;
@@ -536,14 +537,12 @@ cudaError_t trsm(const double* T, int64_t t_rs, int64_t t_cs, bool lower, int m,
     if (e != cudaSuccess) return e;
     if (lower) {
         tri_diag_inv_kernel<true><<<nblk, TDI_THREADS, 0, s>>>(T, t_rs, t_cs, m, dinv_work, status, run_if);
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(trsm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (smem > 48 * 1024) allow_dynamic_shared((const void*)trsm_kernel<true>, TRSM_MAX_SMEM);
         trsm_kernel<true><<<grid, TRSM_THREADS, smem, s>>>(T, t_rs, t_cs, m, Bm, b_rs, ncols, dinv_work,
                                                              rhs_lower ? 1 : 0, next_col, run_if);
     } else {
         tri_diag_inv_kernel<false><<<nblk, TDI_THREADS, 0, s>>>(T, t_rs, t_cs, m, dinv_work, status, run_if);
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(trsm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (smem > 48 * 1024) allow_dynamic_shared((const void*)trsm_kernel<false>, TRSM_MAX_SMEM);
         trsm_kernel<false><<<grid, TRSM_THREADS, smem, s>>>(T, t_rs, t_cs, m, Bm, b_rs, ncols, dinv_work, 0,
                                                               next_col, run_if);
     }
@@ -1035,7 +1034,7 @@ cudaError_t trsm_ff(const double* T, int64_t t_rs, int64_t t_cs, int m, double* 
                     double* dinv_work, void* ffbuf, int* ctl, int* status, cudaStream_t s, bool rhs_lower) {
     if (m <= 0 || ncols <= 0) return cudaSuccess;
     const size_t smem = (size_t)m * sizeof(float2);
-    if (smem > 200 * 1024) return trsm(T, t_rs, t_cs, true, m, Bm, b_rs, ncols, dinv_work, status, s, rhs_lower);
+    if (smem > TRSM_MAX_SMEM) return trsm(T, t_rs, t_cs, true, m, Bm, b_rs, ncols, dinv_work, status, s, rhs_lower);
     const int nblk = (m + TRSM_BS - 1) / TRSM_BS;
     // the column counters after the block inverses: [0] the float64 solve, [1] this one
     unsigned int* ctr = (unsigned int*)(dinv_work + (size_t)nblk * TRSM_BS * TRSM_BS);
@@ -1051,7 +1050,7 @@ cudaError_t trsm_ff(const double* T, int64_t t_rs, int64_t t_cs, int m, double* 
     tri_diag_inv_ff_kernel<<<nblk, TDI_THREADS, 0, s>>>(Tf, m, Df, ctl);
     cudaError_t e = cudaMemsetAsync(ctr + 1, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return e;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(trsm_ff_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024) allow_dynamic_shared((const void*)trsm_ff_kernel, TRSM_MAX_SMEM);
     const unsigned grid = (unsigned)std::min(ncols, std::max(sms, 1));
     trsm_ff_kernel<<<grid, TRSM_THREADS, smem, s>>>(Tf, m, Bm, b_rs, ncols, Df, rhs_lower ? 1 : 0, ctr + 1, ctl,
                                                      status);

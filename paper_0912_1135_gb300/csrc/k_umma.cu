@@ -1368,7 +1368,8 @@ static cudaError_t sliced_gemm_sync(const SlicedGemm& g, void* scratch, size_t s
     p.tmem_cols = 32;
     while (p.tmem_cols < (uint32_t)(TN * g.terms)) p.tmem_cols <<= 1;
     const size_t smem = 1024 + (size_t)p.sa * A_PLANE_BYTES + (size_t)p.sb * B_PLANE_BYTES + 64;
-    cudaError_t e = cudaFuncSetAttribute(sliced_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr size_t most = 1024 + (size_t)MAXS * (A_PLANE_BYTES + B_PLANE_BYTES) + 64;
+    cudaError_t e = allow_dynamic_shared((const void*)sliced_gemm_kernel, most);
     if (e != cudaSuccess) return e;
     dim3 grid(tiles_n, tiles_m, splits);
     sliced_gemm_kernel<<<grid, NTHREADS, smem, s>>>(p);
@@ -1520,7 +1521,7 @@ cudaError_t sliced_gemm_impl(const SlicedGemm& g0, void* scratch, size_t scratch
     p.a_stages = best_as;
     p.b_stages = best_bs;
     const size_t smem = fixed + (size_t)best_bs * b_stage + (size_t)best_as * A_PLANE_BYTES;
-    cudaError_t e = cudaFuncSetAttribute(sliced_gemm2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_shared((const void*)sliced_gemm2_kernel, fixed + budget);
     if (e != cudaSuccess) return e;
     p.splits = splits;
     p.row_exp = (g.row_exp && !swapped && splits == 1 && p.bmode == 0 && p.vec2 && !g.crow) ? g.row_exp : nullptr;

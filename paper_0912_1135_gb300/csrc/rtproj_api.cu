@@ -294,7 +294,6 @@ size_t mixed_workspace(int64_t m, int64_t n, int64_t l_max, int64_t k_max, const
     return rtp::mixed_bytes(m, n, l_max, k_max, o);
 }
 
-constexpr int64_t kMaxLowRank = 64;
 constexpr int64_t kMaxNnz = (int64_t)1 << 40;
 
 // A new handle over the caller's workspace with the float64 form's layout L bound.

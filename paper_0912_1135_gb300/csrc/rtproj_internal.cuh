@@ -17,6 +17,13 @@ void note_launch(int n = 1);
 // GB300). Grid sizes and split-K factors are derived from it.
 int sm_count();
 
+// Lets kern be launched with up to `most` bytes of dynamic shared memory: the largest size that any of
+// its launches asks for, whatever this one needs. The limit belongs to the function, so a thread with
+// a handle of another size may set it between this call and the launch; all set the same value.
+inline cudaError_t allow_dynamic_shared(const void* kern, size_t most) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Per-phase CUDA-event timing (opts.timing).
 struct PhaseTimer {
     static constexpr int kMax = 64;
@@ -285,6 +292,7 @@ namespace rtp {
 // the Gram matrix and the apply.
 size_t sparse_bytes(int64_t m, int64_t n, int64_t nnz, int64_t r, int64_t l_max, int64_t k_max);
 void sparse_bind(rtproj_ctx* h, char* base);
+constexpr int64_t kMaxLowRank = 64;   // largest rank of the low-rank term
 rtproj_status sparse_chunks(rtproj_ctx* h, const int64_t* rp_host);
 rtproj_status sparse_prepare(rtproj_ctx* h);
 rtproj_status sparse_sketch(rtproj_ctx* h, uint64_t seed, int64_t l, double* S, int64_t lds);
