@@ -274,12 +274,11 @@ __device__ __forceinline__ int block_top(uint32_t mxh, uint32_t orl, uint32_t* b
     return mxh ? 32 - __clz((int)mxh) + 32 - 1074 : 32 - __clz((int)orl) - 1074;
 }
 __global__ void __launch_bounds__(256) row_tops_kernel(const int64_t* __restrict__ rptr, const double* __restrict__ val,
-                                                       int64_t ld, int len, int32_t* __restrict__ top) {
+                                                       int32_t* __restrict__ top) {
     __shared__ uint32_t buf[16];
     const int i = blockIdx.x;
-    const int64_t b = rptr ? rptr[i] : (int64_t)i * ld, e = rptr ? rptr[i + 1] : b + len;
     uint32_t mxh = 0u, orl = 0u;
-    for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) {
+    for (int64_t p = rptr[i] + threadIdx.x; p < rptr[i + 1]; p += blockDim.x) {
         uint32_t lo, hi;
         ldg_words(val + p, lo, hi);
         mxh = max(mxh, hi & 0x7FFFFFFFu);
@@ -288,6 +287,13 @@ __global__ void __launch_bounds__(256) row_tops_kernel(const int64_t* __restrict
     const int t = block_top(mxh, orl, buf);
     if (threadIdx.x == 0) top[i] = t;
 }
+// The same for V's r long rows, whose maxima row_exponents gathers (a CTA a row took 64 us at 10 x
+// 300,000): what it leaves for a row of zeros becomes 0.
+__global__ void zero_row_tops_kernel(int32_t* top, int r) {
+    const int q = threadIdx.x;
+    if (q < r && top[q] == kZeroRowExp) top[q] = 0;
+}
+static_assert(kMaxLowRank <= 64, "one CTA of 64 threads");
 
 // x 2^(bits - top) rounded to an integer (|x| < 2^top, bits <= 61), in a signed upper and a
 // LIMB-bit lower limb.
@@ -1060,10 +1066,12 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
         check_values_kernel<<<grid_of((int64_t)r * n, 256), 256, 0, s>>>(h->lrV, (int64_t)r * n, h->status);
         note_launch(2);
     }
-    row_tops_kernel<<<(unsigned)m, 256, 0, s>>>(h->csr_ptr, h->csr_val, 0, 0, h->row_top);
+    row_tops_kernel<<<(unsigned)m, 256, 0, s>>>(h->csr_ptr, h->csr_val, h->row_top);
     note_launch();
     if (r > 0) {
-        row_tops_kernel<<<(unsigned)r, 256, 0, s>>>(nullptr, h->lrV, n, n, h->lr_top);
+        SP_CHECK(fill_int(h->lr_top, r, kZeroRowExp, s));
+        SP_CHECK(row_exponents(h->lrV, n, r, n, h->lr_top, h->status, s));
+        zero_row_tops_kernel<<<1, 64, 0, s>>>(h->lr_top, r);
         note_launch();
     }
     // ||A||_F
