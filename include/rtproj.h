@@ -207,8 +207,9 @@ rtproj_status rtproj_create(rtproj_t* out, int64_t m, int64_t n, const void* A, 
    All of them are borrowed: they must stay alive and unchanged until rtproj_destroy.
    The preconditioner is built to float64's accuracy (S_k = A G with G generated a panel at
    a time; X column by column as in steps a-e after Eq. 15: D = A^* P^-, E = A D,
-   X = R^{-*} Pi E; the sketch and the low-rank products as exact sums of fixed-point
-   values, the rest in float64), and every product with A or A^* of the apply and its
+   X = R^{-*} Pi E; the sketch and, for a V whose rows have no entry above 16 times their
+   root mean square, the low-rank products as exact sums of fixed-point values, with errors
+   bounded by norm per row or column; the rest in float64), and every product with A or A^* of the apply and its
    refinement passes (Remark 4.3; opts refine_passes and refine_tol) is a sum of exact
    products in 128-bit integers, rounded once, so that the refinement converges to
    the projection of the stored matrix. A product with A costs O(nnz + r (m + n)).

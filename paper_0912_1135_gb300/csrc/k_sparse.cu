@@ -288,10 +288,19 @@ __global__ void __launch_bounds__(256) row_tops_kernel(const int64_t* __restrict
     if (threadIdx.x == 0) top[i] = t;
 }
 // The same for V's r long rows, whose maxima row_exponents gathers (a CTA a row took 64 us at 10 x
-// 300,000): what it leaves for a row of zeros becomes 0.
-__global__ void zero_row_tops_kernel(int32_t* top, int r) {
+// 300,000): what it leaves for a row of zeros becomes 0. *flat = 1 when no other row's largest entry
+// (rounded up to a power of two) is above 2^LR_FLAT times its root mean square (GV: V V^*).
+constexpr int LR_FLAT = 4;
+__global__ void lowrank_rows_kernel(int32_t* top, int r, const double* __restrict__ GV, double n, int* flat) {
     const int q = threadIdx.x;
-    if (q < r && top[q] == kZeroRowExp) top[q] = 0;
+    bool ok = true;
+    if (q < r) {
+        const double g = GV[q * r + q];
+        if (top[q] == kZeroRowExp) top[q] = 0;
+        else ok = isfinite(g) && g > 1e-280 && ldexp(n, 2 * (top[q] - LR_FLAT)) <= g;
+    }
+    ok = __syncthreads_and(ok);
+    if (q == 0) *flat = ok ? 1 : 0;
 }
 static_assert(kMaxLowRank <= 64, "one CTA of 64 threads");
 
@@ -500,12 +509,18 @@ __global__ void pminus_kernel(const double* __restrict__ RinvT, const int32_t* _
 }
 
 // D = A^* P^-: its sparse part on the FP64 pipe (the entries of P^- span too many binades for
-// fixed point), the low-rank part V^* (U^* P^-) and then V D on the integer pipes. In both, V(q, :) is
-// taken in units of 2^{lr_top[q]} and the other factor (times 2^{lr_top[q]} for U^* P^-) in units of its
-// largest value in column k, each as LR_BITS = 57 bits in two limbs; a product is the three upper of
-// the four limb products, so its error is below 2^-56 of the two units -- 2^-53 of the partial sums
-// in float64. An FP64 multiply-add holds an SM sub-partition for 64 cycles, the three limb products
-// for 12: with r = 10 at 1000 x 300,000 D took 7.5 ms and V D 6.0.
+// fixed point), the low-rank part V^* (U^* P^-) and then V D on the integer pipes where V's rows are
+// flat, else on the FP64 pipe too. On the integer pipes V(q, :) is taken in units of 2^{lr_top[q]} and
+// the other factor (times 2^{lr_top[q]} for U^* P^-) in units of its largest value in column k, each
+// as LR_BITS = 57 bits in two limbs; a product is the three upper of the four limb products. An FP64
+// multiply-add holds an SM sub-partition for 64 cycles, the three limb products for 12: with r = 10
+// at 1000 x 300,000 D took 7.5 ms and V D 6.0 in float64, 4.5 and 2.9 so.
+// The line (lr_flat, decided at create): fixed point rounds every entry of V(q, :) to 2^-58 of the
+// largest, so over a column of D the term V(q, :)^* T(q, k) moves by 2^-58 2^{lr_top[q]} |T(q, k)| sqrt(n)
+// at most: with the largest entry up to 2^LR_FLAT root mean squares that is 2^-54 of the term's own
+// norm, float64's rounding of one product. Rows of normal variates stay below 13 for any n up to
+// 2^30. Rows with few large entries or scaled columns do not: one entry a row 2^10
+// times the others at 100 x 200,000 left a first correction of 2e-13 in fixed point, 6e-15 in float64.
 constexpr int LR_LO = 28;
 constexpr int LR_BITS = 57;            // 29 bits and the sign in the upper limb
 constexpr int LR_TERMS = 16;           // products whose upper sums (2^58 each) stay below 2^62
@@ -536,9 +551,11 @@ __device__ __forceinline__ int top_of(double x) {          // |x| < 2^top, tight
     return (e ? e : 1) - 1022;
 }
 
-// D(c, k): a thread per k (blockIdx.y picks blockDim of them), the CTA walks the columns c.
-// dtop[k] (pre-filled with kZeroRowExp) gathers the frexp exponents of D(:, k)'s maxima.
-template <bool LOWRANK>
+// D(c, k): a thread per k (blockIdx.y picks blockDim of them), the CTA walks the columns c. The low-rank
+// part by limbs or in float64 (the words of ts and vs are then doubles).
+// dtop[k] (limbs; pre-filled with kZeroRowExp) gathers the frexp exponents of D(:, k)'s maxima.
+enum LowRank { LR_NONE, LR_LIMBS, LR_FLOAT64 };
+template <LowRank LR>
 __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict__ cptr, const int32_t* __restrict__ crow,
                                                        const double* __restrict__ cval, const double* __restrict__ Pm, int m,
                                                        int n, int r, const double* __restrict__ V,
@@ -546,11 +563,16 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
                                                        double* __restrict__ D, int32_t* __restrict__ dtop) {
     extern __shared__ __align__(16) int2 d_smem[];
     const int t = threadIdx.x, nt = blockDim.x, k = blockIdx.y * nt + t;
+    constexpr bool LOWRANK = LR != LR_NONE;
     int2* ts = d_smem;                                     // [r][nt]: (U^* P^-)(q, k) 2^{vtop[q]}
     int2* vs = d_smem + (LOWRANK ? r * nt : 0);            // [DC_STAGE][r]
+    double* ts_d = reinterpret_cast<double*>(ts);
+    double* vs_d = reinterpret_cast<double*>(vs);
     int ek = 0, tmax = kZeroRowExp;
     bool bad = false;
-    if (LOWRANK) {
+    if (LR == LR_FLOAT64)
+        for (int q = 0; q < r; ++q) ts_d[q * nt + t] = k < m ? UtP[(int64_t)q * m + k] : 0.0;
+    if (LR == LR_LIMBS) {
         int e = kZeroRowExp;
         for (int q = 0; q < r; ++q) {
             const double x = k < m ? UtP[(int64_t)q * m + k] : 0.0;
@@ -566,7 +588,9 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
             __syncthreads();
             for (int e = t; e < DC_STAGE * r; e += nt) {
                 const int q = e / DC_STAGE, cc = e % DC_STAGE;
-                vs[cc * r + q] = to_limbs<LR_LO>(c0 + cc < n ? V[(int64_t)q * n + c0 + cc] : 0.0, vtop[q], LR_BITS);
+                const double v = c0 + cc < n ? V[(int64_t)q * n + c0 + cc] : 0.0;
+                if (LR == LR_FLOAT64) vs_d[cc * r + q] = v;
+                else vs[cc * r + q] = to_limbs<LR_LO>(v, vtop[q], LR_BITS);
             }
             __syncthreads();
         }
@@ -589,7 +613,15 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
 #pragma unroll
                 for (int u = 0; u < DC_COLS; ++u)
                     if (p < len[u]) s[u] = fma(cval[b[u] + p], __ldg(Pm + (int64_t)crow[b[u] + p] * m + k), s[u]);
-            if (LOWRANK) {
+            if (LR == LR_FLOAT64) {
+#pragma unroll 2
+                for (int q = 0; q < r; ++q) {
+                    const double x = ts_d[q * nt + t];
+#pragma unroll
+                    for (int u = 0; u < DC_COLS; ++u) s[u] = fma(vs_d[(cc + u) * r + q], x, s[u]);
+                }
+            }
+            if (LR == LR_LIMBS) {
                 for (int q0 = 0; q0 < r; q0 += LR_TERMS) {
                     LimbSum w[DC_COLS];
 #pragma unroll
@@ -615,11 +647,11 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
             for (int u = 0; u < DC_COLS; ++u)
                 if (cc + u < cnt) {
                     D[(c0 + cc + u) * m + k] = s[u];
-                    if (LOWRANK && s[u] != 0.0) tmax = max(tmax, top_of(s[u]));
+                    if (LR == LR_LIMBS && s[u] != 0.0) tmax = max(tmax, top_of(s[u]));
                 }
         }
     }
-    if (LOWRANK && k < m && tmax != kZeroRowExp) atomicMax(dtop + k, tmax);
+    if (LR == LR_LIMBS && k < m && tmax != kZeroRowExp) atomicMax(dtop + k, tmax);
 }
 
 // Partial sums of (V D)(q, k) over chunk blockIdx.x of D's rows: 32 columns k a CTA (a lane each),
@@ -1071,8 +1103,6 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
     if (r > 0) {
         SP_CHECK(fill_int(h->lr_top, r, kZeroRowExp, s));
         SP_CHECK(row_exponents(h->lrV, n, r, n, h->lr_top, h->status, s));
-        zero_row_tops_kernel<<<1, 64, 0, s>>>(h->lr_top, r);
-        note_launch();
     }
     // ||A||_F
     const unsigned np = std::min<unsigned>(grid_of(std::max<int64_t>(nnz, 1), 256), (unsigned)norm_parts());
@@ -1098,6 +1128,8 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
         v.B = h->lrV; v.b_rs = 1; v.b_cs = n;
         v.C = GV; v.c_rs = r; v.c_cs = 1;
         SP_CHECK(gemm64(v, h->part, h->part_elems, s));
+        lowrank_rows_kernel<<<1, 64, 0, s>>>(h->lr_top, r, GV, (double)n, h->lr_flat_dev);
+        note_launch();
     }
     frobenius_total_kernel<<<1, 32, 0, s>>>(h->norm_part, (int)np, px, (int)nx, GU, GV, r, h->normA);
     note_launch();
@@ -1154,17 +1186,29 @@ rtproj_status sparse_gram(rtproj_ctx* h) {
     if (r > 0) SP_CHECK(ut_times(h, h->Pminus, m, m, h->lr_a, m));                    // U^* P^-
     const int nt = row_threads(m), kgroups = (m + nt - 1) / nt;
     const dim3 dgrid((unsigned)std::max(1, std::min((n + DC_STAGE - 1) / DC_STAGE, sm_count() * 32 / kgroups)), (unsigned)kgroups);
-    if (r == 0) {
-        sparse_d_kernel<false><<<dgrid, nt, 0, s>>>(h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, 0, nullptr, nullptr,
-                                                    nullptr, D, nullptr);
+    auto run_d = [&](auto kern, size_t smem) {
+        const cudaError_t e = smem ? allow_dynamic_shared((const void*)kern, (size_t)kMaxLowRank * (256 + DC_STAGE) * sizeof(int2))
+                                   : cudaSuccess;
+        if (e != cudaSuccess) return e;
+        kern<<<dgrid, nt, smem, s>>>(h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, r, h->lrV, h->lr_top, h->lr_a, D,
+                                     h->d_top);
         note_launch();
+        return cudaGetLastError();
+    };
+    const size_t smem = (size_t)r * (nt + DC_STAGE) * sizeof(int2);
+    if (r == 0) {
+        SP_CHECK(run_d(sparse_d_kernel<LR_NONE>, 0));
+    } else if (!h->lr_flat) {
+        SP_CHECK(run_d(sparse_d_kernel<LR_FLOAT64>, smem));
+        Narrow64 g;                                                                     // V D
+        g.M = r; g.N = m; g.K = n;
+        g.A = h->lrV; g.a_rs = n;
+        g.B = D; g.b_rs = m; g.b_cs = 1;
+        g.C = h->lr_a; g.c_rs = m;
+        SP_CHECK(gemm64_narrow(g, h->part, h->part_elems, s));
     } else {
         SP_CHECK(fill_int(h->d_top, m, kZeroRowExp, s));
-        const size_t smem = (size_t)r * (nt + DC_STAGE) * sizeof(int2);
-        SP_CHECK(allow_dynamic_shared((const void*)sparse_d_kernel<true>, (size_t)kMaxLowRank * (256 + DC_STAGE) * sizeof(int2)));
-        sparse_d_kernel<true><<<dgrid, nt, smem, s>>>(h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, r, h->lrV, h->lr_top,
-                                                      h->lr_a, D, h->d_top);
-        note_launch();
+        SP_CHECK(run_d(sparse_d_kernel<LR_LIMBS>, smem));
         // V D: about four CTAs an SM, their partial sums within the scratch
         const int groups = (r + 11) / 12, rows = (r + groups - 1) / groups, kg = (m + 31) / 32;
         const int64_t cap = std::max<int64_t>(1, (int64_t)(h->part_elems / ((size_t)r * m)));

@@ -310,6 +310,7 @@ rtproj_ctx* bind_handle(int64_t m, int64_t n, int64_t l_max, int64_t k_max, void
     char* b = h->ws;
     h->status = (int*)(b + L.status);
     h->a_status_dev = h->status + 8;
+    h->lr_flat_dev = h->status + 14;
     h->S = (double*)(b + L.S);
     h->qr_work = (double*)(b + L.qr_work);
     h->perm = (int32_t*)(b + L.perm);
@@ -467,12 +468,13 @@ rtproj_status rtproj_create_sparse(rtproj_t* out, int64_t m, int64_t n, int64_t 
     if (st == RTPROJ_OK) st = sparse_prepare(h);
     if (st == RTPROJ_OK) {
         // column indices in range and values finite, or the handle is refused
-        int dev_status = 0;
+        int words[16] = {};
         if (cudaStreamSynchronize(h->stream) != cudaSuccess ||
-            cudaMemcpy(&dev_status, h->status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+            cudaMemcpy(words, h->status, sizeof(words), cudaMemcpyDeviceToHost) != cudaSuccess)
             st = RTPROJ_ECUDA;
         else
-            st = (rtproj_status)dev_status;
+            st = (rtproj_status)words[0];
+        h->lr_flat = r > 0 ? words[h->lr_flat_dev - h->status] : 0;
     }
     if (st != RTPROJ_OK) {
         rtproj_destroy(h);

@@ -472,6 +472,8 @@ struct rtproj_ctx {
     double* chunk_part = nullptr;     // chunks x k_max double-double partial sums
     int32_t* row_top = nullptr;       // m: frexp exponents of the rows' largest values
     int32_t* lr_top = nullptr;        // r: the same of V's rows
+    int* lr_flat_dev = nullptr;       // whether V's rows are flat enough for fixed point (k_sparse.cu)
+    int lr_flat = 0;                  // the same on the host
     int32_t* d_top = nullptr;         // m: the same of the columns of D = A^* P^- (with a low-rank term)
     int16_t* panel = nullptr;         // n x 64 entries of G (as integers), the sketch's current panel
 
