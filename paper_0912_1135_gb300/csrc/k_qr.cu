@@ -757,8 +757,11 @@ cudaError_t pivoted_qr_ff(double* S, int m, int l, int64_t lds, double* R, int32
     *launched = false;
     // The register form (k_qr_regs.cu) is the faster one alone (512 x 516: 1.50 against 1.89 ms) but takes
     // up to three times the registers of an SM. Factorizations that run side by side on several
-    // streams wait for one another's SMs then: a batch of 64 instances took 16.1 ms with it throughout,
-    // 15.0 with it up to 100 columns only, 15.1 without it.
+    // streams wait for one another's SMs then. Batches on eight streams, m log-uniform from 16, us with it
+    // never / up to 100 columns / always: 64 instances to m = 64 3,940 / 3,496 / 3,490; 32 to 100
+    // 2,553 / 2,250 / 2,250; 64 to 160 6,810 / 6,620 / 5,910; 64 to 256 8,450 / 8,270 / 7,900; 64 to 512
+    // 14,600 / 14,550 / 15,320; 32 to 512 8,620 / 8,450 / 9,520. Few large instances lose by it, so the
+    // line lies below them.
     if (!side_by_side || m <= 100) {
         const cudaError_t er = pivoted_qr_regs(S, m, l, lds, R, perm, work, status, s, spin_limit, fallback, false, launched);
         if (er != cudaSuccess || *launched) return er;

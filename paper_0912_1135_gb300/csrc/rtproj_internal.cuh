@@ -316,7 +316,8 @@ rtproj_status middle_fp64(rtproj_ctx* h, const double* c, double* out, int k);
 // ---------------------------------------------------------------------------
 namespace rtp {
 // Conversions between float32 and float64 by integer operations: the conversion instructions run
-// on the FP64 pipe, at 64 cycles a warp (storing 4096 x 8192 entries as float32: 86 -> 57 us, 7.1 TB/s).
+// on the FP64 pipe, at 64 cycles a warp (storing 4096 x 8192 entries as float32: 86 -> 57 us, 7.1 TB/s
+// of reads and writes, some of which L2 serves).
 // A float32 as the bits of the float64 of the same value (zeros, subnormals and non-finite values by
 // the conversion).
 __device__ __forceinline__ uint2 widen_bits(float x) {
