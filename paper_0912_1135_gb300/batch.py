@@ -3,8 +3,8 @@ sequence of interior-point-style column scalings A diag(d_j).
 
 Each instance has its own handle in the asynchronous mode (opts.async: no host
 synchronization inside precondition) on one of several CUDA streams, so independent
-instances run concurrently on the GPU: a small instance's pivoted QR occupies one 16-SM
-cluster and its products a fraction of the SMs, leaving the rest to the others. One step --
+instances run concurrently on the GPU: a small instance's pivoted QR and products occupy a
+fraction of the SMs, leaving the rest to the others. One step --
 every instance's precondition and null_project -- can be captured once into a CUDA graph and
 replayed with one host call, which removes the host's per-launch cost from the loop. Every
 kernel is librtproj's; conditions found on the device stay latched per handle
