@@ -11,7 +11,7 @@
 // N 2^-105 of the largest product's magnitude: the bound of a double-double sum, whose
 // every addition rounds at 2^-105 of the partial sum. Capacity: products enter at most
 // 2^115 units large, so 2^11 of them fit 127 bits (I128_MAX_TERMS); a longer sum is taken in parts
-// of that many, which are added in double-double (i128_full, i128_flush).
+// of at most that many, which are added in double-double (i128_flush).
 #pragma once
 
 #include <cstdint>
@@ -278,13 +278,6 @@ __device__ __forceinline__ void dd_add(double& hi, double& lo, double bh, double
     e += lo + bl;
     hi = s + e;
     lo = e - (hi - s);
-}
-
-// Counts a product; true when the sum is full: it has to be flushed before the next one.
-__device__ __forceinline__ bool i128_full(int& terms) {
-    if (++terms < I128_MAX_TERMS) return false;
-    terms = 0;
-    return true;
 }
 
 // The sum moves over to the pair hi + lo and starts anew.

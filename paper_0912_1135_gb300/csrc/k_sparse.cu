@@ -771,6 +771,7 @@ __global__ void sparse_e_kernel(const int64_t* __restrict__ rptr, const int32_t*
 // a few long rows still spread over many warps, and no sum exceeds the 128 bits' capacity.
 constexpr int SP_CHUNK = 2048;
 static_assert(SP_CHUNK <= I128_MAX_TERMS, "a chunk's sum must fit 128 bits");
+constexpr int SP_PART = I128_MAX_TERMS - 1 - (int)kMaxLowRank;   // a column's part, beside y and the low-rank terms
 constexpr int SP_WARPS = 8;
 
 __device__ __forceinline__ i128acc i128_shfl_xor(const i128acc& a, int o) {
@@ -903,7 +904,6 @@ __global__ void __launch_bounds__(32 * SP_WARPS)
             bad[q] |= !i128_finite(hi);
             i128_mac(acc[q], one, i128_decode(lo, hi));
         }
-        int terms = 1;
         bool longer = false;
         auto flush = [&](int q) {
             double2 v = longer ? full[warp][q][lane] : make_double2(0.0, 0.0);
@@ -923,14 +923,29 @@ __global__ void __launch_bounds__(32 * SP_WARPS)
                 bad[q] |= !i128_finite(hi[q]);
                 i128_mac(acc[q], a, i128_decode(lo[q], hi[q]), ~0u);
             }
-            if (i128_full(terms)) {              // a very long column
-#pragma unroll
-                for (int q = 0; q < JB; ++q) full[warp][q][lane] = flush(q);
-                longer = true;
-            }
         };
         const int64_t pe = cptr[c + 1];
-        for (int64_t p = cptr[c]; p < pe; ++p) term(cval[p], H + (int64_t)crow[p] * k);
+        int64_t p = cptr[c];
+        while (pe - p > SP_PART) {                // a very long column
+            const int64_t part_end = p + SP_PART;
+#pragma unroll 1
+            for (; p < part_end; ++p) term(cval[p], H + (int64_t)crow[p] * k);
+#pragma unroll
+            for (int q = 0; q < JB; ++q) full[warp][q][lane] = flush(q);
+            longer = true;
+        }
+        if (p < pe) {                             // the next entry is loaded ahead of this one's products
+            double v = cval[p];
+            int row = crow[p];
+            while (++p < pe) {
+                const double v1 = cval[p];
+                const int row1 = crow[p];
+                term(v, H + (int64_t)row * k);
+                v = v1;
+                row = row1;
+            }
+            term(v, H + (int64_t)row * k);
+        }
         for (int q = 0; q < r; ++q) term(V[(int64_t)q * n + c], UtH + (int64_t)q * k);
 #pragma unroll
         for (int q = 0; q < JB; ++q) {

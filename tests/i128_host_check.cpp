@@ -50,7 +50,10 @@ int main() {
             double x, y;
             if (std::scanf("%la %la", &x, &y) != 2) return 1;
             rtp::i128_mac(two && (i & 1) ? b : a, rtp::i128_left(dec(x)), dec(y), i % 3 == 2 ? ~0u : 0u);
-            if (longer && rtp::i128_full(terms)) rtp::i128_flush(a, hi, lo);
+            if (longer && ++terms == rtp::I128_MAX_TERMS) {
+                rtp::i128_flush(a, hi, lo);
+                terms = 0;
+            }
         }
         if (longer) {
             rtp::i128_flush(a, hi, lo);
