@@ -34,6 +34,11 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
         if ((expr) != cudaSuccess) return RTPROJ_ECUDA; \
     } while (0)
 
+// Rows are cut into chunks of at most SP_CHUNK nonzeros (a table built at create), so that
+// a few long rows still spread over many warps, and no sum exceeds the 128 bits' capacity.
+constexpr int SP_CHUNK = 2048;
+static_assert(SP_CHUNK <= I128_MAX_TERMS, "a chunk's sum must fit 128 bits");
+
 // ---------------------------------------------------------------------------------
 // The column-compressed copy: counting sort by column, then each column's entries put in
 // (row, value) order, so that every sum over a column runs in one fixed order whatever the
@@ -70,10 +75,12 @@ __global__ void block_totals_kernel(const int64_t* cnt, int n, int64_t* tot) {
     if (threadIdx.x == SCAN_T - 1) tot[blockIdx.x] = incl;
 }
 
-__global__ void scan_totals_kernel(int64_t* tot, int nb) {
+// fill[0 .. nfill) = kZeroRowExp on the way (row_tops_kernel's maxima start from it).
+__global__ void scan_totals_kernel(int64_t* tot, int nb, int32_t* fill, int nfill) {
     __shared__ int64_t buf[SCAN_T];
     __shared__ int64_t carry;
     if (threadIdx.x == 0) carry = 0;
+    for (int i = threadIdx.x; i < nfill; i += SCAN_T) fill[i] = kZeroRowExp;
     __syncthreads();
     for (int b0 = 0; b0 < nb; b0 += SCAN_T) {
         const int i = b0 + threadIdx.x;
@@ -133,11 +140,6 @@ __global__ void sort_columns_kernel(const int64_t* __restrict__ cptr, int n, int
     }
 }
 
-__global__ void check_values_kernel(const double* __restrict__ val, int64_t nnz, int* status) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x)
-        if (!isfinite(val[p])) set_status(status, RTPROJ_ENONFINITE);
-}
-
 // ---------------------------------------------------------------------------------
 // ||A||_F^2 = ||S||_F^2 + 2 <S, U V> + trace((U^* U)(V V^*)), each part summed in two
 // deterministic levels (per-CTA partials, then one thread).
@@ -176,17 +178,6 @@ __global__ void cross_term_kernel(const int64_t* __restrict__ rptr, const int32_
         }
     const double t = block_sum(s, red);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-__global__ void frobenius_total_kernel(const double* part_s, int np, const double* part_x, int nx, const double* GU,
-                                       const double* GV, int r, double* out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s = 0.0, x = 0.0, t = 0.0;
-    for (int i = 0; i < np; ++i) s += part_s[i];
-    for (int i = 0; i < nx; ++i) x += part_x[i];
-    for (int a = 0; a < r; ++a)
-        for (int b = 0; b < r; ++b) t = fma(GU[a * r + b], GV[b * r + a], t);
-    *out = sqrt(fmax(s + 2.0 * x + t, 0.0));
 }
 
 __device__ __forceinline__ void ldg_words(const double* p, uint32_t& lo, uint32_t& hi) {
@@ -253,56 +244,88 @@ __global__ void __launch_bounds__(SK_T) omega_panel_kernel(int n, int l, int j0,
 // G = N 2^omega_exp
 int omega_exp(int dist) { return dist == RTPROJ_OMEGA_GAUSSIAN ? -12 : dist == RTPROJ_OMEGA_RADEMACHER ? 0 : -8; }
 
-// top[i] = the frexp exponent of the largest magnitude in row i (0 for an empty or zero row).
-__device__ __forceinline__ int block_top(uint32_t mxh, uint32_t orl, uint32_t* buf) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        mxh = max(mxh, __shfl_xor_sync(0xffffffffu, mxh, o));
-        orl |= __shfl_xor_sync(0xffffffffu, orl, o);
+// The exponents of the largest values in the rows of S and of V, and the check that they and U are
+// finite: a CTA per chunk of S, then per TOPS_SPAN entries of a row of V, then of U. top[i]
+// (pre-filled with kZeroRowExp, and left so for an empty or zero row) is the frexp exponent of row i's
+// largest magnitude: S's m rows, then V's r. (A CTA a row took 165 us of 966 at create for 2 x 500,000.)
+constexpr int TOPS_SPAN = 4096;
+__global__ void __launch_bounds__(256) row_tops_kernel(const int32_t* __restrict__ crow_of, const int64_t* __restrict__ cbeg,
+                                                       const int64_t* __restrict__ rptr, const double* __restrict__ val,
+                                                       int nchunks, int m, int n, int r, const double* __restrict__ U,
+                                                       const double* __restrict__ V, int32_t* __restrict__ top, int* status) {
+    __shared__ uint32_t buf[8][2];
+    const int spans = (n + TOPS_SPAN - 1) / TOPS_SPAN;
+    const int64_t v = (int64_t)blockIdx.x - nchunks, u = v - (int64_t)spans * r;
+    const double* x = val;
+    int64_t b, e;
+    int row = -1;
+    if (v < 0) {
+        row = crow_of[blockIdx.x];
+        b = cbeg[blockIdx.x];
+        e = min(b + (int64_t)SP_CHUNK, rptr[row + 1]);
+    } else if (u < 0) {
+        const int q = (int)(v / spans);
+        row = m + q;
+        x = V;
+        b = (int64_t)q * n + (v % spans) * TOPS_SPAN;
+        e = min(b + (int64_t)TOPS_SPAN, (int64_t)(q + 1) * n);
+    } else {
+        x = U;
+        b = u * TOPS_SPAN;
+        e = min(b + (int64_t)TOPS_SPAN, (int64_t)m * r);
     }
-    if ((threadIdx.x & 31) == 0) {
-        buf[2 * (threadIdx.x >> 5)] = mxh;
-        buf[2 * (threadIdx.x >> 5) + 1] = orl;
-    }
-    __syncthreads();
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        mxh = max(mxh, buf[2 * w]);
-        orl |= buf[2 * w + 1];
-    }
-    if ((mxh | orl) == 0u) return 0;
-    if (mxh >> 20) return (int)(mxh >> 20) - 1022;
-    return mxh ? 32 - __clz((int)mxh) + 32 - 1074 : 32 - __clz((int)orl) - 1074;
-}
-__global__ void __launch_bounds__(256) row_tops_kernel(const int64_t* __restrict__ rptr, const double* __restrict__ val,
-                                                       int32_t* __restrict__ top) {
-    __shared__ uint32_t buf[16];
-    const int i = blockIdx.x;
     uint32_t mxh = 0u, orl = 0u;
-    for (int64_t p = rptr[i] + threadIdx.x; p < rptr[i + 1]; p += blockDim.x) {
+    for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) {
         uint32_t lo, hi;
-        ldg_words(val + p, lo, hi);
+        ldg_words(x + p, lo, hi);
         mxh = max(mxh, hi & 0x7FFFFFFFu);
         orl |= lo;
     }
-    const int t = block_top(mxh, orl, buf);
-    if (threadIdx.x == 0) top[i] = t;
-}
-// The same for V's r long rows, whose maxima row_exponents gathers (a CTA a row took 64 us at 10 x
-// 300,000): what it leaves for a row of zeros becomes 0. *flat = 1 when no other row's largest entry
-// (rounded up to a power of two) is above 2^LR_FLAT times its root mean square (GV: V V^*).
-constexpr int LR_FLAT = 4;
-__global__ void lowrank_rows_kernel(int32_t* top, int r, const double* __restrict__ GV, double n, int* flat) {
-    const int q = threadIdx.x;
-    bool ok = true;
-    if (q < r) {
-        const double g = GV[q * r + q];
-        if (top[q] == kZeroRowExp) top[q] = 0;
-        else ok = isfinite(g) && g > 1e-280 && ldexp(n, 2 * (top[q] - LR_FLAT)) <= g;
+    mxh = __reduce_max_sync(0xffffffffu, mxh);
+    orl = __reduce_or_sync(0xffffffffu, orl);
+    if ((threadIdx.x & 31) == 0) {
+        buf[threadIdx.x >> 5][0] = mxh;
+        buf[threadIdx.x >> 5][1] = orl;
     }
-    ok = __syncthreads_and(ok);
-    if (q == 0) *flat = ok ? 1 : 0;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < 8; ++w) {
+        mxh = max(mxh, buf[w][0]);
+        orl |= buf[w][1];
+    }
+    if (mxh >= 0x7FF00000u) set_status(status, RTPROJ_ENONFINITE);
+    if (row < 0 || (mxh | orl) == 0u) return;
+    atomicMax(top + row, mxh >> 20 ? (int)(mxh >> 20) - 1022
+                         : mxh     ? 32 - __clz((int)mxh) + 32 - 1074
+                                   : 32 - __clz((int)orl) - 1074);
 }
-static_assert(kMaxLowRank <= 64, "one CTA of 64 threads");
+
+// Whether V's row q is flat: its largest entry, rounded up to a power of two, at most 2^LR_FLAT times
+// its root mean square (g: its squared norm).
+constexpr int LR_FLAT = 4;
+__device__ __forceinline__ bool row_is_flat(int top, double g, int n) {
+    if (top == kZeroRowExp) return true;
+    return isfinite(g) && g > 1e-280 && ldexp((double)n, 2 * (top - LR_FLAT)) <= g;
+}
+
+// ||A||_F from its parts; V's rows: *flat, and the exponent of a row of zeros made 0.
+__global__ void frobenius_total_kernel(const double* part_s, int np, const double* part_x, int nx, const double* GU,
+                                       const double* GV, int r, int n, int32_t* lr_top, int* flat, double* out) {
+    bool ok = true;
+    for (int q = threadIdx.x; q < r; q += blockDim.x) {
+        ok &= row_is_flat(lr_top[q], GV[q * r + q], n);
+        if (lr_top[q] == kZeroRowExp) lr_top[q] = 0;
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (threadIdx.x != 0) return;
+    *flat = ok ? 1 : 0;
+    double s = 0.0, x = 0.0, t = 0.0;
+    for (int i = 0; i < np; ++i) s += part_s[i];
+    for (int i = 0; i < nx; ++i) x += part_x[i];
+    for (int a = 0; a < r; ++a)
+        for (int b = 0; b < r; ++b) t = fma(GU[a * r + b], GV[b * r + a], t);
+    *out = sqrt(fmax(s + 2.0 * x + t, 0.0));
+}
 
 // x 2^(bits - top) rounded to an integer (|x| < 2^top, bits <= 61), in a signed upper and a
 // LIMB-bit lower limb.
@@ -345,7 +368,7 @@ __global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __re
     __shared__ unsigned long long sum[2][SK_COLS];
     const int i = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t b = rptr[i], e = rptr[i + 1];
-    const int tp = top[i], bits = limb_bits(e - b);
+    const int tp = max(top[i], -1073), bits = limb_bits(e - b);   // -1073: the smallest value's, or an empty row
     if (t < SK_COLS) sum[0][t] = sum[1][t] = 0ull;
     long long h0 = 0, h1 = 0, l0 = 0, l1 = 0;
     int held = 0;
@@ -767,10 +790,6 @@ __global__ void sparse_e_kernel(const int64_t* __restrict__ rptr, const int32_t*
 // 832 cycles per warp of them, and gathered one double per 32-byte sector. An apply of 100
 // vectors with two refinement passes at 1000 x 300,000, 1.5e6 nonzeros: 40.6 -> 5.7 ms.
 // ---------------------------------------------------------------------------------
-// Rows are cut into chunks of at most SP_CHUNK nonzeros (a table built at create), so that
-// a few long rows still spread over many warps, and no sum exceeds the 128 bits' capacity.
-constexpr int SP_CHUNK = 2048;
-static_assert(SP_CHUNK <= I128_MAX_TERMS, "a chunk's sum must fit 128 bits");
 constexpr int SP_PART = I128_MAX_TERMS - 1 - (int)kMaxLowRank;   // a column's part, beside y and the low-rank terms
 constexpr int SP_WARPS = 8;
 
@@ -1030,8 +1049,8 @@ size_t sparse_bytes(int64_t m, int64_t n, int64_t nnz, int64_t r, int64_t l_max,
            align_up((size_t)n * 8) + align_up((size_t)nb * 8) + 2 * align_up((size_t)m * m * 8) +
            align_up((size_t)r * std::max(l_max, m) * 8) + align_up((size_t)r * k_max * 8) +
            align_up((size_t)(2 * r * r + norm_parts()) * 8) + align_up((size_t)nc * 4) + align_up((size_t)nc * 8) +
-           align_up((size_t)(m + 1) * 4) + align_up((size_t)nc * k_max * 16) + align_up((size_t)m * 4) +
-           align_up((size_t)r * 4) + align_up((size_t)m * 4) + align_up(panel_bytes(m, n));
+           align_up((size_t)(m + 1) * 4) + align_up((size_t)nc * k_max * 16) + align_up((size_t)(m + r) * 4) +
+           align_up((size_t)m * 4) + align_up(panel_bytes(m, n));
 }
 
 void sparse_bind(rtproj_ctx* h, char* base) {
@@ -1054,8 +1073,8 @@ void sparse_bind(rtproj_ctx* h, char* base) {
     h->chunk_beg = (int64_t*)take((size_t)nc * 8);
     h->row_chunk = (int32_t*)take((size_t)(m + 1) * 4);
     h->chunk_part = (double*)take((size_t)nc * h->k_max * 16);
-    h->row_top = (int32_t*)take((size_t)m * 4);
-    h->lr_top = (int32_t*)take((size_t)r * 4);
+    h->row_top = (int32_t*)take((size_t)(m + r) * 4);
+    h->lr_top = h->row_top + m;
     h->d_top = (int32_t*)take((size_t)m * 4);
     int16_t* own = (int16_t*)take(panel_bytes(m, n));
     h->panel = panel_bytes(m, n) ? own : reinterpret_cast<int16_t*>(h->W);
@@ -1096,11 +1115,10 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
     SP_CHECK(cudaMemsetAsync(h->csc_cursor, 0, (size_t)n * 8, s));
     if (nnz > 0) {
         count_cols_kernel<<<grid_of(nnz, 256), 256, 0, s>>>(h->csr_col, nnz, n, h->csc_cursor, h->status);
-        check_values_kernel<<<grid_of(nnz, 256), 256, 0, s>>>(h->csr_val, nnz, h->status);
-        note_launch(2);
+        note_launch();
     }
     block_totals_kernel<<<nb, SCAN_T, 0, s>>>(h->csc_cursor, n, h->scan_tot);
-    scan_totals_kernel<<<1, SCAN_T, 0, s>>>(h->scan_tot, nb);
+    scan_totals_kernel<<<1, SCAN_T, 0, s>>>(h->scan_tot, nb, h->row_top, m + r);
     block_scan_kernel<<<nb, SCAN_T, 0, s>>>(h->csc_cursor, n, h->scan_tot, h->csc_ptr);
     note_launch(3);
     SP_CHECK(cudaMemsetAsync(h->csc_cursor, 0, (size_t)n * 8, s));
@@ -1108,17 +1126,10 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
         h->csr_ptr, h->csr_col, h->csr_val, m, n, h->csc_ptr, h->csc_cursor, h->csc_row, h->csc_val);
     sort_columns_kernel<<<grid_of(n, 256), 256, 0, s>>>(h->csc_ptr, n, h->csc_row, h->csc_val);
     note_launch(2);
-    if (r > 0) {   // the low-rank factors must be finite too
-        check_values_kernel<<<grid_of((int64_t)m * r, 256), 256, 0, s>>>(h->lrU, (int64_t)m * r, h->status);
-        check_values_kernel<<<grid_of((int64_t)r * n, 256), 256, 0, s>>>(h->lrV, (int64_t)r * n, h->status);
-        note_launch(2);
-    }
-    row_tops_kernel<<<(unsigned)m, 256, 0, s>>>(h->csr_ptr, h->csr_val, h->row_top);
+    const int64_t tops = h->nchunks + (int64_t)((n + TOPS_SPAN - 1) / TOPS_SPAN) * r + ((int64_t)m * r + TOPS_SPAN - 1) / TOPS_SPAN;
+    row_tops_kernel<<<(unsigned)tops, 256, 0, s>>>(h->chunk_row, h->chunk_beg, h->csr_ptr, h->csr_val, h->nchunks, m, n, r,
+                                                   h->lrU, h->lrV, h->row_top, h->status);
     note_launch();
-    if (r > 0) {
-        SP_CHECK(fill_int(h->lr_top, r, kZeroRowExp, s));
-        SP_CHECK(row_exponents(h->lrV, n, r, n, h->lr_top, h->status, s));
-    }
     // ||A||_F
     const unsigned np = std::min<unsigned>(grid_of(std::max<int64_t>(nnz, 1), 256), (unsigned)norm_parts());
     sumsq_vals_kernel<<<np, 256, 0, s>>>(h->csr_val, nnz, h->norm_part);
@@ -1143,10 +1154,9 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
         v.B = h->lrV; v.b_rs = 1; v.b_cs = n;
         v.C = GV; v.c_rs = r; v.c_cs = 1;
         SP_CHECK(gemm64(v, h->part, h->part_elems, s));
-        lowrank_rows_kernel<<<1, 64, 0, s>>>(h->lr_top, r, GV, (double)n, h->lr_flat_dev);
-        note_launch();
     }
-    frobenius_total_kernel<<<1, 32, 0, s>>>(h->norm_part, (int)np, px, (int)nx, GU, GV, r, h->normA);
+    frobenius_total_kernel<<<1, 32, 0, s>>>(h->norm_part, (int)np, px, (int)nx, GU, GV, r, n, h->lr_top, h->lr_flat_dev,
+                                            h->normA);
     note_launch();
     SP_CHECK(cudaGetLastError());
     return RTPROJ_OK;
