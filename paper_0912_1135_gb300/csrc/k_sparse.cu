@@ -547,8 +547,8 @@ __global__ void pminus_kernel(const double* __restrict__ RinvT, const int32_t* _
 constexpr int LR_LO = 28;
 constexpr int LR_BITS = 57;            // 29 bits and the sign in the upper limb
 constexpr int LR_TERMS = 16;           // products whose upper sums (2^58 each) stay below 2^62
-constexpr int DC_STAGE = 32;           // columns of V staged at a time
-constexpr int DC_COLS = 4;             // columns c a thread works on at once
+constexpr int DC_STAGE_LG = 5;         // log2 of the columns of V staged at a time, at most
+constexpr int DC_COLS_LG = 2, DC_COLS = 1 << DC_COLS_LG;   // columns c a thread works on at once
 
 // An upper sum and the sum of the two middle products (2^-LR_LO of it).
 struct LimbSum { long long h, m; };
@@ -574,7 +574,9 @@ __device__ __forceinline__ int top_of(double x) {          // |x| < 2^top, tight
     return (e ? e : 1) - 1022;
 }
 
-// D(c, k): a thread per k (blockIdx.y picks blockDim of them), the CTA walks the columns c. The low-rank
+// D(c, k): a thread per k (blockIdx.y picks blockDim of them), the CTA walks the columns c, 2^lgst at a
+// time: 32, or fewer where that leaves less than eight CTAs an SM (a preconditioner of a 200 x 2000
+// matrix with 60 nonzeros a column took 1,713 us by 32, 1,438 by 4). The low-rank
 // part by limbs or in float64 (the words of ts and vs are then doubles).
 // dtop[k] (limbs; pre-filled with kZeroRowExp) gathers the frexp exponents of D(:, k)'s maxima.
 enum LowRank { LR_NONE, LR_LIMBS, LR_FLOAT64 };
@@ -583,12 +585,12 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
                                                        const double* __restrict__ cval, const double* __restrict__ Pm, int m,
                                                        int n, int r, const double* __restrict__ V,
                                                        const int32_t* __restrict__ vtop, const double* __restrict__ UtP,
-                                                       double* __restrict__ D, int32_t* __restrict__ dtop) {
+                                                       double* __restrict__ D, int32_t* __restrict__ dtop, int lgst) {
     extern __shared__ __align__(16) int2 d_smem[];
-    const int t = threadIdx.x, nt = blockDim.x, k = blockIdx.y * nt + t;
+    const int t = threadIdx.x, nt = blockDim.x, k = blockIdx.y * nt + t, stage = 1 << lgst;
     constexpr bool LOWRANK = LR != LR_NONE;
     int2* ts = d_smem;                                     // [r][nt]: (U^* P^-)(q, k) 2^{vtop[q]}
-    int2* vs = d_smem + (LOWRANK ? r * nt : 0);            // [DC_STAGE][r]
+    int2* vs = d_smem + (LOWRANK ? r * nt : 0);            // [stage][r]
     double* ts_d = reinterpret_cast<double*>(ts);
     double* vs_d = reinterpret_cast<double*>(vs);
     int ek = 0, tmax = kZeroRowExp;
@@ -606,11 +608,11 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
         for (int q = 0; q < r; ++q)
             ts[q * nt + t] = to_limbs<LR_LO>(k < m && !bad ? UtP[(int64_t)q * m + k] : 0.0, ek - vtop[q], LR_BITS);
     }
-    for (int64_t c0 = (int64_t)blockIdx.x * DC_STAGE; c0 < n; c0 += (int64_t)gridDim.x * DC_STAGE) {
+    for (int64_t c0 = (int64_t)blockIdx.x * stage; c0 < n; c0 += (int64_t)gridDim.x * stage) {
         if (LOWRANK) {
             __syncthreads();
-            for (int e = t; e < DC_STAGE * r; e += nt) {
-                const int q = e / DC_STAGE, cc = e % DC_STAGE;
+            for (int e = t; e < stage * r; e += nt) {
+                const int q = e >> lgst, cc = e & (stage - 1);
                 const double v = c0 + cc < n ? V[(int64_t)q * n + c0 + cc] : 0.0;
                 if (LR == LR_FLOAT64) vs_d[cc * r + q] = v;
                 else vs[cc * r + q] = to_limbs<LR_LO>(v, vtop[q], LR_BITS);
@@ -618,7 +620,7 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
             __syncthreads();
         }
         if (k >= m) continue;
-        const int cnt = (int)min((int64_t)DC_STAGE, n - c0);
+        const int cnt = (int)min((int64_t)stage, n - c0);
 #pragma unroll 1
         for (int cc = 0; cc < cnt; cc += DC_COLS) {
             double s[DC_COLS];
@@ -1210,17 +1212,20 @@ rtproj_status sparse_gram(rtproj_ctx* h) {
     note_launch();
     if (r > 0) SP_CHECK(ut_times(h, h->Pminus, m, m, h->lr_a, m));                    // U^* P^-
     const int nt = row_threads(m), kgroups = (m + nt - 1) / nt;
-    const dim3 dgrid((unsigned)std::max(1, std::min((n + DC_STAGE - 1) / DC_STAGE, sm_count() * 32 / kgroups)), (unsigned)kgroups);
+    int lgst = DC_STAGE_LG;
+    while (lgst > DC_COLS_LG && (int64_t)((n + (1 << lgst) - 1) >> lgst) * kgroups < 8 * sm_count()) --lgst;
+    const int stages = (n + (1 << lgst) - 1) >> lgst;
+    const dim3 dgrid((unsigned)std::max(1, std::min(stages, sm_count() * 32 / kgroups)), (unsigned)kgroups);
     auto run_d = [&](auto kern, size_t smem) {
-        const cudaError_t e = smem ? allow_dynamic_shared((const void*)kern, (size_t)kMaxLowRank * (256 + DC_STAGE) * sizeof(int2))
+        const cudaError_t e = smem ? allow_dynamic_shared((const void*)kern, (size_t)kMaxLowRank * (256 + (1 << DC_STAGE_LG)) * sizeof(int2))
                                    : cudaSuccess;
         if (e != cudaSuccess) return e;
         kern<<<dgrid, nt, smem, s>>>(h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, r, h->lrV, h->lr_top, h->lr_a, D,
-                                     h->d_top);
+                                     h->d_top, lgst);
         note_launch();
         return cudaGetLastError();
     };
-    const size_t smem = (size_t)r * (nt + DC_STAGE) * sizeof(int2);
+    const size_t smem = (size_t)r * (nt + (1 << lgst)) * sizeof(int2);
     if (r == 0) {
         SP_CHECK(run_d(sparse_d_kernel<LR_NONE>, 0));
     } else if (!h->lr_flat) {
