@@ -205,12 +205,17 @@ constexpr int SK_WARPS = SK_T / 32;
 constexpr int SK_LIMB = 30;                      // bits of the lower limb
 constexpr int SK_FLUSH = 1 << 16;                // products whose lower-limb sums fit 62 bits
 
+// A launch takes as many panels as stay in L2 together (their storage allowing), one on grid.y (grid.z
+// for V G): at 1000 x 5000, l = 1004, the 16 panels one after the other took 241 us, launches mostly.
+constexpr int64_t SK_L2_BYTES = (int64_t)32 << 20;
+
 // Panel entries (c, jj), jj < SK_COLS: N of G(c, j0 + jj), zero past column l. One warp per 4
 // (Gaussian) or 16 rows, two columns a lane.
 __global__ void __launch_bounds__(SK_T) omega_panel_kernel(int n, int l, int j0, int dist, uint32_t k0, uint32_t k1,
                                                            int16_t* __restrict__ P) {
     const int lane = threadIdx.x & 31;
-    const int j = j0 + 2 * lane;
+    const int j = j0 + blockIdx.y * SK_COLS + 2 * lane;
+    P += (int64_t)blockIdx.y * n * SK_COLS;
     const int per = dist == RTPROJ_OMEGA_GAUSSIAN ? 4 : 16;
     const int64_t groups = ((int64_t)n + per - 1) / per;
     for (int64_t q = (int64_t)blockIdx.x * SK_WARPS + (threadIdx.x >> 5); q < groups; q += (int64_t)gridDim.x * SK_WARPS) {
@@ -361,7 +366,7 @@ __host__ __device__ __forceinline__ int limb_bits(int64_t count) {
 // columns a lane. With a low-rank term, S(i, j) += sum_q U(i, q) (V G)(q, j).
 __global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __restrict__ rptr, const int32_t* __restrict__ col,
                                                              const double* __restrict__ val, const int32_t* __restrict__ top,
-                                                             const int16_t* __restrict__ P, int l, int j0, int gexp, int r,
+                                                             const int16_t* __restrict__ P, int n, int l, int j0, int gexp, int r,
                                                              const double* __restrict__ U, const double* __restrict__ VG,
                                                              int64_t ldvg, double* S, int64_t lds) {
     __shared__ int4 ent[SK_T];                     // upper limb, lower limb, column
@@ -376,7 +381,7 @@ __global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __re
         __syncthreads();
         if (p0 + t < e) {
             const int2 v = to_limbs(val[p0 + t], tp, bits);
-            ent[t] = make_int4(v.x, v.y, col[p0 + t], 0);
+            ent[t] = make_int4(v.x, v.y, col[p0 + t] + (int)blockIdx.y * n, 0);   // the panel's row
         } else {
             ent[t] = make_int4(0, 0, 0, 0);
         }
@@ -418,7 +423,7 @@ __global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __re
     atomicAdd(&sum[0][2 * lane + 1], (unsigned long long)h1);
     atomicAdd(&sum[1][2 * lane + 1], (unsigned long long)l1);
     __syncthreads();
-    const int j = j0 + t;
+    const int j = j0 + (int)blockIdx.y * SK_COLS + t;
     if (t < SK_COLS && j < l) {
         double s = limbs_to_double((long long)sum[0][t], (long long)sum[1][t], tp - bits + gexp);
         for (int q = 0; q < r; ++q) s = fma(U[(int64_t)i * r + q], VG[(int64_t)q * ldvg + j], s);
@@ -437,6 +442,8 @@ __global__ void __launch_bounds__(SK_T) lowrank_panel_kernel(const double* __res
     __shared__ int2 vs[VG_KC][VG_ROWS];
     __shared__ unsigned long long sum[2][VG_ROWS][SK_COLS];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, q0 = blockIdx.y * VG_ROWS;
+    P += (int64_t)blockIdx.z * n * SK_COLS;
+    part += (int64_t)blockIdx.z * gridDim.x * r * SK_COLS;
     const int64_t kb = (int64_t)blockIdx.x * chunk, ke = min((int64_t)n, kb + chunk);
     for (int e = t; e < 2 * VG_ROWS * SK_COLS; e += SK_T) (&sum[0][0][0])[e] = 0ull;
     long long h[VG_ROWS][2], lo[VG_ROWS][2];
@@ -499,6 +506,8 @@ __global__ void lowrank_panel_sum_kernel(const longlong2* __restrict__ part, con
                                          int l, int j0, int bits, int gexp, double* __restrict__ VG, int64_t ldvg) {
     const int idx = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     const int q = idx / SK_COLS, j = idx % SK_COLS;
+    j0 += blockIdx.y * SK_COLS;
+    part += (int64_t)blockIdx.y * chunks * r * SK_COLS;
     if (q >= r || j0 + j >= l) return;
     // the upper limbs' sums are below 2^62 a chunk: kept as a high and a low half
     long long hh = 0, hl = 0, lo = 0;
@@ -1168,21 +1177,26 @@ rtproj_status sparse_sketch(rtproj_ctx* h, uint64_t seed, int64_t l, double* S, 
     const uint32_t k0 = (uint32_t)(seed & 0xFFFFFFFFull), k1 = (uint32_t)(seed >> 32);
     const int m = (int)h->m, n = (int)h->n, r = h->lr, dist = h->opts.omega, gexp = omega_exp(dist);
     cudaStream_t s = h->stream;
+    const int64_t panel = (int64_t)n * SK_COLS * 2, room = panel_bytes(m, n) ? panel : (int64_t)m * n * 8;
+    const int total = (int)((l + SK_COLS - 1) / SK_COLS);
+    const int panels = (int)std::max<int64_t>(1, std::min<int64_t>(total, std::min(room, SK_L2_BYTES) / panel));   // a launch
     // the chunks of V G: up to four CTAs an SM, their partial sums within the scratch
-    const int64_t cap = std::max<int64_t>(1, (int64_t)(h->part_elems / ((size_t)std::max(r, 1) * SK_COLS * 2)));
-    int64_t chunks = std::min<int64_t>(cap, std::min<int64_t>(4 * sm_count(), ((int64_t)n + VG_KC - 1) / VG_KC));
+    const int64_t cap = std::max<int64_t>(1, (int64_t)(h->part_elems / ((size_t)std::max(r, 1) * SK_COLS * 2 * panels)));
+    int64_t chunks = std::min<int64_t>(cap, std::min<int64_t>(std::max(1, 4 * sm_count() / panels), ((int64_t)n + VG_KC - 1) / VG_KC));
     const int64_t chunk = (((int64_t)n + chunks - 1) / chunks + VG_KC - 1) / VG_KC * VG_KC;
     chunks = ((int64_t)n + chunk - 1) / chunk;
     const int vbits = limb_bits(chunk);
     const int per = dist == RTPROJ_OMEGA_GAUSSIAN ? 4 : 16;
     const unsigned pgrid = (unsigned)std::max<int64_t>(
         1, std::min<int64_t>(((int64_t)n + per * SK_WARPS - 1) / (per * SK_WARPS), (int64_t)sm_count() * 32));
-    for (int j0 = 0; j0 < (int)l; j0 += SK_COLS) {
-        omega_panel_kernel<<<pgrid, SK_T, 0, s>>>(n, (int)l, j0, dist, k0, k1, h->panel);
+    for (int p0 = 0; p0 < total; p0 += panels) {
+        const int j0 = p0 * SK_COLS;
+        const unsigned np = (unsigned)std::min(panels, total - p0);
+        omega_panel_kernel<<<dim3(pgrid, np), SK_T, 0, s>>>(n, (int)l, j0, dist, k0, k1, h->panel);
         if (r > 0) {   // V G (r x l), this panel's columns
             longlong2* part = reinterpret_cast<longlong2*>(h->part);
             const int groups = (r + 11) / 12, rows = (r + groups - 1) / groups;   // 1 .. 12 rows a CTA
-            const dim3 grid((unsigned)chunks, (unsigned)groups);
+            const dim3 grid((unsigned)chunks, (unsigned)groups, np);
             auto run = [&](auto kern) {
                 kern<<<grid, SK_T, 0, s>>>(h->lrV, h->lr_top, r, n, (int)chunk, vbits, h->panel, part);
             };
@@ -1190,12 +1204,12 @@ rtproj_status sparse_sketch(rtproj_ctx* h, uint64_t seed, int64_t l, double* S, 
             else if (rows <= 8) run(lowrank_panel_kernel<8>);
             else if (rows <= 10) run(lowrank_panel_kernel<10>);
             else run(lowrank_panel_kernel<12>);
-            lowrank_panel_sum_kernel<<<(unsigned)((r * SK_COLS + 7) / 8), 256, 0, s>>>(part, h->lr_top, (int)chunks, r, (int)l, j0,
-                                                                                       vbits, gexp, h->lr_a, l);
+            lowrank_panel_sum_kernel<<<dim3((unsigned)((r * SK_COLS + 7) / 8), np), 256, 0, s>>>(
+                part, h->lr_top, (int)chunks, r, (int)l, j0, vbits, gexp, h->lr_a, l);
             note_launch(2);
         }
-        sparse_sketch_kernel<<<(unsigned)m, SK_T, 0, s>>>(h->csr_ptr, h->csr_col, h->csr_val, h->row_top, h->panel, (int)l, j0,
-                                                          gexp, r, h->lrU, h->lr_a, l, S, lds);
+        sparse_sketch_kernel<<<dim3((unsigned)m, np), SK_T, 0, s>>>(h->csr_ptr, h->csr_col, h->csr_val, h->row_top, h->panel, n,
+                                                                    (int)l, j0, gexp, r, h->lrU, h->lr_a, l, S, lds);
         note_launch(2);
     }
     SP_CHECK(cudaGetLastError());
