@@ -172,8 +172,10 @@ __global__ void cross_term_kernel(const int64_t* __restrict__ rptr, const int32_
     double s = 0.0;
     for (int i = blockIdx.x; i < m; i += gridDim.x)
         for (int64_t p = rptr[i] + threadIdx.x; p < rptr[i + 1]; p += blockDim.x) {
+            const int c = col[p];
+            if (c < 0 || c >= n) continue;       // create fails on RTPROJ_EINVAL
             double uv = 0.0;
-            for (int q = 0; q < r; ++q) uv = fma(U[(int64_t)i * r + q], V[(int64_t)q * n + col[p]], uv);
+            for (int q = 0; q < r; ++q) uv = fma(U[(int64_t)i * r + q], V[(int64_t)q * n + c], uv);
             s = fma(val[p], uv, s);
         }
     const double t = block_sum(s, red);
