@@ -9,9 +9,10 @@
 // up, and the sum is shifted along. Bits lost in a shift lie below 2^-105 of that largest
 // product, and each addition loses less than one unit 2^E, so a sum of N products is within
 // N 2^-105 of the largest product's magnitude: the bound of a double-double sum, whose
-// every addition rounds at 2^-105 of the partial sum. Capacity: products enter at most
-// 2^115 units large, so 2^11 of them fit 127 bits (I128_MAX_TERMS); a longer sum is taken in parts
-// of at most that many, which are added in double-double (i128_flush).
+// every addition rounds at 2^-105 of the partial sum. A zero's product moves nothing; a subnormal
+// factor counts as 2^-1022 in "largest" (its own last place is 2^52 times coarser). Capacity: products
+// enter at most 2^115 units large, so 2^11 of them fit 127 bits (I128_MAX_TERMS); a longer sum is
+// taken in parts of at most that many, which are added in double-double (i128_flush).
 #pragma once
 
 #include <cstdint>
@@ -117,8 +118,8 @@ __device__ __forceinline__ void i128_add_signed(i128acc& a, uint32_t p0, uint32_
 __device__ __forceinline__ void i128_mac(i128acc& a, const i128op& x, const i128op& y, uint32_t flip = 0u) {
     const int e = x.e + y.e;
     int r = a.E - e;
-    if (r < 0) {                             // a larger product: the unit moves up
-        const int E = e + 9;
+    if (r < 0) {                             // a larger product: the unit moves up, but not for a zero's
+        const int E = (x.hi | x.lo) != 0u && (y.hi | y.lo) != 0u ? e + 9 : a.E;
         i128_sar(a, E - a.E);
         a.E = E;
         r = 9;

@@ -927,7 +927,7 @@ __global__ void __launch_bounds__(32 * SP_WARPS)
             acc[q] = i128_zero();
             bad[q] = false;
             const int j = j0 + q * KL;
-            uint32_t lo = 0u, hi = 0u;
+            uint32_t lo = 0u, hi = 0x3FF00000u;     // lanes past k: any value but zero
             if (j < k) {
                 const double y = Y[c * ldy + j];
                 lo = (uint32_t)__double2loint(y);
@@ -947,7 +947,8 @@ __global__ void __launch_bounds__(32 * SP_WARPS)
             uint32_t lo[JB], hi[JB];
 #pragma unroll
             for (int q = 0; q < JB; ++q) {
-                lo[q] = hi[q] = 0u;
+                lo[q] = 0u;
+                hi[q] = 0x3FF00000u;
                 if (j0 + q * KL < k) ldg_words(h + j0 + q * KL, lo[q], hi[q]);
             }
 #pragma unroll
