@@ -172,7 +172,8 @@ struct F64Arith {
     static __device__ __forceinline__ S mul(S a, S b) { return a * b; }
     static __device__ __forceinline__ S neg(S a) { return d(bits(a) ^ (1ull << 63)); }
     // Newton's iterations from the approximate functions (20 bits): x r^2 = 1 twice, then s^2 = x with
-    // the residual exact; 1 / a twice. Within an ulp or so, a third of the FP64 pipe's chain.
+    // the residual exact; 1 / a twice. Within a few units in the last place, far inside the QR's l 2^-53; a
+    // third of the FP64 pipe's chain.
     static __device__ __forceinline__ S sqrt(S a) {
         double r;
         asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
