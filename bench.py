@@ -350,9 +350,8 @@ def phase_work(mode, w, o):
 
 # DRAM bytes (read + write) per launch of a kernel, from one ncu capture of
 # `bench.py --steps 1 --warmup 3 --no-e2e --no-cpu-baseline --no-accuracy --no-fp64-form`
-# on the 512 x 65536 workload; to be replaced by None whenever that kernel changes.
-PROFILED_TRAFFIC = {("dense_512x65536", "qr_persistent_kernel"): 2160128 + 217600,
-                    ("dense_512x65536", "qr_persistent_ff_kernel"): 2189568 + 289024}
+# on the 512 x 65536 workload; None for a kernel that was not captured so or has changed since.
+PROFILED_TRAFFIC = {}
 
 
 def roofline_entry(mode, phase_ms, phase_cnt, steps, w, pk, opts):
@@ -364,6 +363,8 @@ def roofline_entry(mode, phase_ms, phase_cnt, steps, w, pk, opts):
         ms = phase_ms.get(ph, 0.0)
         if ms <= 0:
             continue
+        if ph == "qr" and not opts.async_ and opts.qr_form == 0 and (mode != "fp64" or w.l <= 2304):
+            kernel = "qr_regs_kernel"     # what a synchronous handle, on which the phases are timed, launches
         achieved = flops * steps / (ms * 1e-3) / 1e12
         peak = tensor_peak if bound == "tensor" else FP64_PEAK_TFLOPS
         phases[ph] = {"bound": bound, "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
