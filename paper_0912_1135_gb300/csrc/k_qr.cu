@@ -159,7 +159,8 @@ __global__ void qr_extract_r_kernel(const double* S, int m, int64_t lds, double*
 
 // ---------------------------------------------------------------------------------
 // Persistent form: one cooperative launch for all m steps; taken where the register form
-// (k_qr_regs.cu) is not: longer columns, factorizations side by side, a range it refuses. CTA b keeps columns
+// (k_qr_regs.cu) is not: longer columns, factorizations side by side, a range it refuses, fewer than 12
+// columns in float64. CTA b keeps columns
 // [b*cpc, b*cpc + cpc) of S^* (rows of S) in shared memory for the whole factorization,
 // one warp per column, and consecutive steps are separated by one grid-wide exchange.
 // The pivot rule is the textbook one (Businger-Golub with the norms recomputed every

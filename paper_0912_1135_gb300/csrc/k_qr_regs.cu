@@ -693,6 +693,10 @@ cudaError_t pivoted_qr_regs(const double* S, int m, int l, int64_t lds, double* 
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     const int sms = sm_count();
     if (!coop) return cudaSuccess;
+    // Float64 with few columns: the steps saved are less than the launch of the kernel behind (QR phase, us,
+    // persistent alone / this form: 1 x 5 14 / 21, 4 x 8 25 / 32, 8 x 12 39 / 44, 10 x 14 45 / 50, 12 x 16
+    // 59 / 56, 16 x 20 74 / 71).
+    if (f64 && m < 12) return cudaSuccess;
     // Warps per column, and row pairs a lane holds.
 #define QR_SHAPE(A, NP, WPC, MAXW) {(const void*)qr_regs_kernel<A, NP, WPC, MAXW, false>, NP, WPC, MAXW, false}
 #define QR_LONG(A, NP, WPC, MAXW) {(const void*)qr_regs_kernel<A, NP, WPC, MAXW, true>, NP, WPC, MAXW, true}
