@@ -19,6 +19,7 @@
 #include "i128.cuh"
 
 #include <algorithm>
+#include <climits>
 #include <cstring>
 #include <vector>
 
@@ -68,11 +69,20 @@ __device__ __forceinline__ int64_t block_inclusive_scan(int64_t v, int64_t* buf)
     return buf[threadIdx.x];
 }
 
-__global__ void block_totals_kernel(const int64_t* cnt, int n, int64_t* tot) {
+// *longest (zeroed before) = the largest count.
+__global__ void block_totals_kernel(const int64_t* cnt, int n, int64_t* tot, int* longest) {
     __shared__ int64_t buf[SCAN_T];
-    const int64_t i = (int64_t)blockIdx.x * SCAN_T + threadIdx.x;
-    const int64_t incl = block_inclusive_scan(i < n ? cnt[i] : 0, buf);
-    if (threadIdx.x == SCAN_T - 1) tot[blockIdx.x] = incl;
+    __shared__ int most;
+    const int64_t i = (int64_t)blockIdx.x * SCAN_T + threadIdx.x, v = i < n ? cnt[i] : 0;
+    if (threadIdx.x == 0) most = 0;
+    const int64_t incl = block_inclusive_scan(v, buf);        // and a barrier
+    const unsigned mine = __reduce_max_sync(0xffffffffu, (unsigned)min(v, (int64_t)INT_MAX));
+    if ((threadIdx.x & 31) == 0) atomicMax(&most, (int)mine);
+    __syncthreads();
+    if (threadIdx.x == SCAN_T - 1) {
+        tot[blockIdx.x] = incl;
+        atomicMax(longest, most);
+    }
 }
 
 // fill[0 .. nfill) = kZeroRowExp on the way (row_tops_kernel's maxima start from it).
@@ -559,7 +569,9 @@ constexpr int LR_LO = 28;
 constexpr int LR_BITS = 57;            // 29 bits and the sign in the upper limb
 constexpr int LR_TERMS = 16;           // products whose upper sums (2^58 each) stay below 2^62
 constexpr int DC_STAGE_LG = 5;         // log2 of the columns of V staged at a time, at most
-constexpr int DC_COLS_LG = 2, DC_COLS = 1 << DC_COLS_LG;   // columns c a thread works on at once
+constexpr int DC_COLS_LG = 2, DC_COLS = 1 << DC_COLS_LG;   // columns c a thread works on at once,
+constexpr int DC_TOGETHER = 16;                            // for their first entries
+constexpr int DC_LONG = 256;           // entries of a column that others should not wait for
 
 // An upper sum and the sum of the two middle products (2^-LR_LO of it).
 struct LimbSum { long long h, m; };
@@ -585,10 +597,11 @@ __device__ __forceinline__ int top_of(double x) {          // |x| < 2^top, tight
     return (e ? e : 1) - 1022;
 }
 
-// D(c, k): a thread per k (blockIdx.y picks blockDim of them), the CTA walks the columns c, 2^lgst at a
+// D(c, k): a thread per k (blockIdx.y picks blockDim of them), the CTA walks the columns c, 2^lgt at a
 // time: 32, or fewer where that leaves less than eight CTAs an SM (a preconditioner of a 200 x 2000
-// matrix with 60 nonzeros a column took 1,713 us by 32, 1,438 by 4). The low-rank
-// part by limbs or in float64 (the words of ts and vs are then doubles).
+// matrix with 60 nonzeros a column took 1,713 us by 32, 1,438 by 4), down to one where a column has
+// more than DC_LONG entries, which then has several of them in flight (three of 3,000 among 27: 2,814
+// and 683 us). The low-rank part by limbs or in float64 (the words of ts and vs are then doubles).
 // dtop[k] (limbs; pre-filled with kZeroRowExp) gathers the frexp exponents of D(:, k)'s maxima.
 enum LowRank { LR_NONE, LR_LIMBS, LR_FLOAT64 };
 template <LowRank LR>
@@ -596,9 +609,10 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
                                                        const double* __restrict__ cval, const double* __restrict__ Pm, int m,
                                                        int n, int r, const double* __restrict__ V,
                                                        const int32_t* __restrict__ vtop, const double* __restrict__ UtP,
-                                                       double* __restrict__ D, int32_t* __restrict__ dtop, int lgst) {
+                                                       double* __restrict__ D, int32_t* __restrict__ dtop, int lgt) {
     extern __shared__ __align__(16) int2 d_smem[];
-    const int t = threadIdx.x, nt = blockDim.x, k = blockIdx.y * nt + t, stage = 1 << lgst;
+    const int t = threadIdx.x, nt = blockDim.x, k = blockIdx.y * nt + t;
+    const int turn = 1 << lgt, lgst = max(lgt, DC_COLS_LG), stage = 1 << lgst;   // V's columns: DC_COLS of them at least
     constexpr bool LOWRANK = LR != LR_NONE;
     int2* ts = d_smem;                                     // [r][nt]: (U^* P^-)(q, k) 2^{vtop[q]}
     int2* vs = d_smem + (LOWRANK ? r * nt : 0);            // [stage][r]
@@ -619,7 +633,7 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
         for (int q = 0; q < r; ++q)
             ts[q * nt + t] = to_limbs<LR_LO>(k < m && !bad ? UtP[(int64_t)q * m + k] : 0.0, ek - vtop[q], LR_BITS);
     }
-    for (int64_t c0 = (int64_t)blockIdx.x * stage; c0 < n; c0 += (int64_t)gridDim.x * stage) {
+    for (int64_t c0 = (int64_t)blockIdx.x * turn; c0 < n; c0 += (int64_t)gridDim.x * turn) {
         if (LOWRANK) {
             __syncthreads();
             for (int e = t; e < stage * r; e += nt) {
@@ -631,7 +645,7 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
             __syncthreads();
         }
         if (k >= m) continue;
-        const int cnt = (int)min((int64_t)stage, n - c0);
+        const int cnt = (int)min((int64_t)turn, n - c0);
 #pragma unroll 1
         for (int cc = 0; cc < cnt; cc += DC_COLS) {
             double s[DC_COLS];
@@ -645,10 +659,16 @@ __global__ void __launch_bounds__(256) sparse_d_kernel(const int64_t* __restrict
                 most = max(most, len[u]);
                 s[u] = 0.0;
             }
-            for (int p = 0; p < most; ++p)
+            for (int p = 0; p < min(most, DC_TOGETHER); ++p)
 #pragma unroll
                 for (int u = 0; u < DC_COLS; ++u)
                     if (p < len[u]) s[u] = fma(cval[b[u] + p], __ldg(Pm + (int64_t)crow[b[u] + p] * m + k), s[u]);
+            if (most > DC_TOGETHER)              // long columns: each by itself, several of its entries in flight
+#pragma unroll
+                for (int u = 0; u < DC_COLS; ++u)
+#pragma unroll 4
+                    for (int p = DC_TOGETHER; p < len[u]; ++p)
+                        s[u] = fma(cval[b[u] + p], __ldg(Pm + (int64_t)crow[b[u] + p] * m + k), s[u]);
             if (LR == LR_FLOAT64) {
 #pragma unroll 2
                 for (int q = 0; q < r; ++q) {
@@ -1131,7 +1151,7 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
         count_cols_kernel<<<grid_of(nnz, 256), 256, 0, s>>>(h->csr_col, nnz, n, h->csc_cursor, h->status);
         note_launch();
     }
-    block_totals_kernel<<<nb, SCAN_T, 0, s>>>(h->csc_cursor, n, h->scan_tot);
+    block_totals_kernel<<<nb, SCAN_T, 0, s>>>(h->csc_cursor, n, h->scan_tot, h->longest_col_dev);
     scan_totals_kernel<<<1, SCAN_T, 0, s>>>(h->scan_tot, nb, h->row_top, m + r);
     block_scan_kernel<<<nb, SCAN_T, 0, s>>>(h->csc_cursor, n, h->scan_tot, h->csc_ptr);
     note_launch(3);
@@ -1229,20 +1249,21 @@ rtproj_status sparse_gram(rtproj_ctx* h) {
     note_launch();
     if (r > 0) SP_CHECK(ut_times(h, h->Pminus, m, m, h->lr_a, m));                    // U^* P^-
     const int nt = row_threads(m), kgroups = (m + nt - 1) / nt;
-    int lgst = DC_STAGE_LG;
-    while (lgst > DC_COLS_LG && (int64_t)((n + (1 << lgst) - 1) >> lgst) * kgroups < 8 * sm_count()) --lgst;
-    const int stages = (n + (1 << lgst) - 1) >> lgst;
-    const dim3 dgrid((unsigned)std::max(1, std::min(stages, sm_count() * 32 / kgroups)), (unsigned)kgroups);
+    int lgt = DC_STAGE_LG;
+    const int lgt_min = h->longest_col > DC_LONG ? 0 : DC_COLS_LG;
+    while (lgt > lgt_min && (int64_t)((n + (1 << lgt) - 1) >> lgt) * kgroups < 8 * sm_count()) --lgt;
+    const int turns = (n + (1 << lgt) - 1) >> lgt;
+    const dim3 dgrid((unsigned)std::max(1, std::min(turns, sm_count() * 32 / kgroups)), (unsigned)kgroups);
     auto run_d = [&](auto kern, size_t smem) {
         const cudaError_t e = smem ? allow_dynamic_shared((const void*)kern, (size_t)kMaxLowRank * (256 + (1 << DC_STAGE_LG)) * sizeof(int2))
                                    : cudaSuccess;
         if (e != cudaSuccess) return e;
         kern<<<dgrid, nt, smem, s>>>(h->csc_ptr, h->csc_row, h->csc_val, h->Pminus, m, n, r, h->lrV, h->lr_top, h->lr_a, D,
-                                     h->d_top, lgst);
+                                     h->d_top, lgt);
         note_launch();
         return cudaGetLastError();
     };
-    const size_t smem = (size_t)r * (nt + (1 << lgst)) * sizeof(int2);
+    const size_t smem = (size_t)r * (nt + (1 << std::max(lgt, DC_COLS_LG))) * sizeof(int2);
     if (r == 0) {
         SP_CHECK(run_d(sparse_d_kernel<LR_NONE>, 0));
     } else if (!h->lr_flat) {

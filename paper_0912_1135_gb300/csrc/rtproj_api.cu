@@ -311,6 +311,7 @@ rtproj_ctx* bind_handle(int64_t m, int64_t n, int64_t l_max, int64_t k_max, void
     h->status = (int*)(b + L.status);
     h->a_status_dev = h->status + 8;
     h->lr_flat_dev = h->status + 14;
+    h->longest_col_dev = h->status + 15;
     h->S = (double*)(b + L.S);
     h->qr_work = (double*)(b + L.qr_work);
     h->perm = (int32_t*)(b + L.perm);
@@ -348,7 +349,7 @@ rtproj_status finish_handle(rtproj_ctx* h) {
             if (cudaEventCreate(&h->timer.b[i]) != cudaSuccess || cudaEventCreate(&h->timer.e[i]) != cudaSuccess)
                 return RTPROJ_ECUDA;
     }
-    if (cudaMemsetAsync(h->status, 0, sizeof(int), h->stream) != cudaSuccess) return RTPROJ_ECUDA;
+    if (cudaMemsetAsync(h->status, 0, 16 * sizeof(int), h->stream) != cudaSuccess) return RTPROJ_ECUDA;   // L.status
     return RTPROJ_OK;
 }
 }  // namespace
@@ -475,6 +476,7 @@ rtproj_status rtproj_create_sparse(rtproj_t* out, int64_t m, int64_t n, int64_t 
         else
             st = (rtproj_status)words[0];
         h->lr_flat = r > 0 ? words[h->lr_flat_dev - h->status] : 0;
+        h->longest_col = words[h->longest_col_dev - h->status];
     }
     if (st != RTPROJ_OK) {
         rtproj_destroy(h);

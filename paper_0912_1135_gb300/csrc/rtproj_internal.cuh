@@ -475,6 +475,8 @@ struct rtproj_ctx {
     int32_t* lr_top = nullptr;        // r: the same of V's rows
     int* lr_flat_dev = nullptr;       // whether V's rows are flat enough for fixed point (k_sparse.cu)
     int lr_flat = 0;                  // the same on the host
+    int* longest_col_dev = nullptr;   // entries of the longest column of S
+    int longest_col = 0;              // the same on the host
     int32_t* d_top = nullptr;         // m: the same of the columns of D = A^* P^- (with a low-rank term)
     int16_t* panel = nullptr;         // n x 64 entries of G (as integers), the sketch's current panel
 

@@ -59,3 +59,45 @@ def test_products_by_groups_of_lanes(m, n, k, r):
     assert_rows_close(Z.cpu().numpy()[:few], Zx, tol, "Z")
     assert_rows_close(ROW.cpu().numpy()[:few], ROWx, 64 * tol, "ROW")
     assert_rows_close(back.cpu().numpy(), Z.cpu().numpy(), 2 * tol, "the vectors in the other order")
+
+
+@pytest.mark.parametrize("r,spike", [(0, False), (1, False), (5, False), (5, True), (20, True)])
+@pytest.mark.parametrize("m,n", [(20, 23), (33, 150), (300, 700), (25, 9000)])
+def test_gram_with_long_columns(m, n, r, spike):
+    """Columns of some hundreds to thousands of entries (duplicates that sum), which go one a turn where
+    columns are few; V by limbs or, with one large entry a row, in float64. L L^* against W W^*,
+    W = R^{-*} Pi A: the Gram test's bound with its terms counted as the longest column's."""
+    torch, rt = torch_cuda(), rt_module()
+    rng = np.random.default_rng(m + n + r)
+    per = rng.integers(1, 6, n)
+    longest = 1500
+    cols = rng.choice(n, 3, replace=False)
+    col = np.concatenate([np.repeat(np.arange(n), per), np.full(longest, cols[0]), np.full(300, cols[1]), np.full(257, cols[2])])
+    row = rng.integers(0, m, col.size)
+    row[np.cumsum(per) - per] = np.arange(n) % m
+    val = rng.standard_normal(col.size)
+    val[per.sum():] *= 0.05
+    order = np.argsort(row, kind="stable")
+    row, col, val = row[order], col[order].astype(np.int32), val[order]
+    rp = np.concatenate([[0], np.cumsum(np.bincount(row, minlength=m))]).astype(np.int64)
+    A = np.zeros((m, n))
+    np.add.at(A, (row, col), val)
+    U = V = None
+    if r:
+        r = min(r, m)
+        U, V = rng.standard_normal((m, r)) / np.sqrt(r) / 8, rng.standard_normal((r, n))
+        if spike:
+            V[np.arange(r), rng.integers(0, n, r)] *= 64.0
+        A = A + U @ V
+    kappa = np.linalg.cond(A)
+    assert kappa < 1e4
+    l = min(n, 2 * m + 8)
+    with rt.SparseProjector(to_dev(torch, rp), to_dev(torch, col), to_dev(torch, val), n,
+                            U=None if U is None else to_dev(torch, U), V=None if V is None else to_dev(torch, V),
+                            l_max=l) as P:
+        P.precondition(seed=3, l=l)
+        R, perm, L = P.export_state()
+    W = np.linalg.solve(R.T, A[perm])
+    X = W @ W.T
+    L = np.tril(L)
+    assert np.max(np.abs(L @ L.T - X)) <= 2 * longest * kappa ** 2 * 2.0 ** -50 * np.max(np.abs(X))
