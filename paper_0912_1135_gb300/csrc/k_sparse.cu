@@ -265,7 +265,8 @@ int omega_exp(int dist) { return dist == RTPROJ_OMEGA_GAUSSIAN ? -12 : dist == R
 // finite: a CTA per chunk of S, then per TOPS_SPAN entries of a row of V, then of U. top[i]
 // (pre-filled with kZeroRowExp, and left so for an empty or zero row) is the frexp exponent of row i's
 // largest magnitude: S's m rows, then V's r. (A CTA a row took 165 us of 966 at create for 2 x 500,000.)
-constexpr int TOPS_SPAN = 4096;
+constexpr int TOPS_SPAN = 2048;
+static_assert(TOPS_SPAN <= 8 * 256 && SP_CHUNK <= 8 * 256, "a CTA's values are loaded at once");
 __global__ void __launch_bounds__(256) row_tops_kernel(const int32_t* __restrict__ crow_of, const int64_t* __restrict__ cbeg,
                                                        const int64_t* __restrict__ rptr, const double* __restrict__ val,
                                                        int nchunks, int m, int n, int r, const double* __restrict__ U,
@@ -291,12 +292,17 @@ __global__ void __launch_bounds__(256) row_tops_kernel(const int32_t* __restrict
         b = u * TOPS_SPAN;
         e = min(b + (int64_t)TOPS_SPAN, (int64_t)m * r);
     }
-    uint32_t mxh = 0u, orl = 0u;
-    for (int64_t p = b + threadIdx.x; p < e; p += blockDim.x) {
-        uint32_t lo, hi;
-        ldg_words(x + p, lo, hi);
-        mxh = max(mxh, hi & 0x7FFFFFFFu);
-        orl |= lo;
+    uint32_t mxh = 0u, orl = 0u, lo[8], hi[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int64_t p = b + u * 256 + threadIdx.x;
+        lo[u] = hi[u] = 0u;
+        if (p < e) ldg_words(x + p, lo[u], hi[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        mxh = max(mxh, hi[u] & 0x7FFFFFFFu);
+        orl |= lo[u];
     }
     mxh = __reduce_max_sync(0xffffffffu, mxh);
     orl = __reduce_or_sync(0xffffffffu, orl);
@@ -1153,6 +1159,10 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
     }
     block_totals_kernel<<<nb, SCAN_T, 0, s>>>(h->csc_cursor, n, h->scan_tot, h->longest_col_dev);
     scan_totals_kernel<<<1, SCAN_T, 0, s>>>(h->scan_tot, nb, h->row_top, m + r);
+    const int64_t tops = h->nchunks + (int64_t)((n + TOPS_SPAN - 1) / TOPS_SPAN) * r + ((int64_t)m * r + TOPS_SPAN - 1) / TOPS_SPAN;
+    row_tops_kernel<<<(unsigned)tops, 256, 0, s>>>(h->chunk_row, h->chunk_beg, h->csr_ptr, h->csr_val, h->nchunks, m, n, r,
+                                                   h->lrU, h->lrV, h->row_top, h->status);
+    note_launch();
     block_scan_kernel<<<nb, SCAN_T, 0, s>>>(h->csc_cursor, n, h->scan_tot, h->csc_ptr);
     note_launch(3);
     SP_CHECK(cudaMemsetAsync(h->csc_cursor, 0, (size_t)n * 8, s));
@@ -1160,10 +1170,6 @@ rtproj_status sparse_prepare(rtproj_ctx* h) {
         h->csr_ptr, h->csr_col, h->csr_val, m, n, h->csc_ptr, h->csc_cursor, h->csc_row, h->csc_val);
     sort_columns_kernel<<<grid_of(n, 256), 256, 0, s>>>(h->csc_ptr, n, h->csc_row, h->csc_val);
     note_launch(2);
-    const int64_t tops = h->nchunks + (int64_t)((n + TOPS_SPAN - 1) / TOPS_SPAN) * r + ((int64_t)m * r + TOPS_SPAN - 1) / TOPS_SPAN;
-    row_tops_kernel<<<(unsigned)tops, 256, 0, s>>>(h->chunk_row, h->chunk_beg, h->csr_ptr, h->csr_val, h->nchunks, m, n, r,
-                                                   h->lrU, h->lrV, h->row_top, h->status);
-    note_launch();
     // ||A||_F
     const unsigned np = std::min<unsigned>(grid_of(std::max<int64_t>(nnz, 1), 256), (unsigned)norm_parts());
     sumsq_vals_kernel<<<np, 256, 0, s>>>(h->csr_val, nnz, h->norm_part);
