@@ -220,6 +220,10 @@ constexpr int SK_FLUSH = 1 << 16;                // products whose lower-limb su
 // A launch takes as many panels as stay in L2 together (their storage allowing), one on grid.y (grid.z
 // for V G): at 1000 x 5000, l = 1004, the 16 panels one after the other took 241 us, launches mostly.
 constexpr int64_t SK_L2_BYTES = (int64_t)32 << 20;
+// G is generated in place for rows of at most SK_GEN_ROW nonzeros and at most SK_GEN nonzeros times
+// panels: 64 x 512, two panels, 16 a row 41 us, by panels 46; 500 x 2000, eight panels, 2 a row 55 and 56,
+// 16 a row 68 and 62; 2000 x 20,000, 32 panels, 16 a row 487 and 375.
+constexpr int SK_GEN_ROW = 16, SK_GEN = 1 << 13;
 
 // Panel entries (c, jj), jj < SK_COLS: N of G(c, j0 + jj), zero past column l. One warp per 4
 // (Gaussian) or 16 rows, two columns a lane.
@@ -380,18 +384,61 @@ __host__ __device__ __forceinline__ int limb_bits(int64_t count) {
     return b;
 }
 
-// S(i, j0 .. j0 + SK_COLS - 1) for row i: the CTA's warps take the row's nonzeros in turn, two
-// columns a lane. With a low-rank term, S(i, j) += sum_q U(i, q) (V G)(q, j).
+// Rows of several chunks: which CTA sums what, and where the sums go.
+struct SharedRows {
+    const int32_t* chunk_row; const int64_t* chunk_beg; const int32_t* row_chunk;
+    int group;               // chunks a CTA
+    int slots;
+    longlong2* part;         // [panel][slot][SK_COLS]
+};
+// The place of a row's share s among the partial sums (`first`: the row's first chunk): rows do not overlap.
+__device__ __forceinline__ int sketch_slot(const SharedRows& a, int i, int first, int s) { return first / a.group + i + s; }
+
+// Entries (c, j) and (c, j + 1) of G as integers, one in each half.
+__device__ __forceinline__ int omega_pair(int c, int j, int l, int dist, uint32_t k0, uint32_t k1) {
+    int a, b;
+    if (dist == RTPROJ_OMEGA_GAUSSIAN) {           // as gauss_quad, the pair that holds row c only
+        const uint4 u = philox4x32_10(make_uint4((uint32_t)c >> 2, (uint32_t)j, 1u, 0u), k0, k1);
+        const uint4 v = philox4x32_10(make_uint4((uint32_t)c >> 2, (uint32_t)(j + 1), 1u, 0u), k0, k1);
+        int a1, b1;
+        gauss_pair(c & 2 ? u.z : u.x, c & 2 ? u.w : u.y, a, a1);
+        gauss_pair(c & 2 ? v.z : v.x, c & 2 ? v.w : v.y, b, b1);
+        if (c & 1) {
+            a = a1;
+            b = b1;
+        }
+    } else {
+        const float sc = dist == RTPROJ_OMEGA_RADEMACHER ? 1.0f : 256.0f;
+        const uint4 u = philox4x32_10(make_uint4((uint32_t)c >> 4, (uint32_t)j, 0u, 0u), k0, k1);
+        const uint4 v = philox4x32_10(make_uint4((uint32_t)c >> 4, (uint32_t)(j + 1), 0u, 0u), k0, k1);
+        a = (int)(omega_from_byte(block_byte(u, c & 15), dist) * sc);
+        b = (int)(omega_from_byte(block_byte(v, c & 15), dist) * sc);
+    }
+    return (j < l ? a & 0xFFFF : 0) | (j + 1 < l ? b << 16 : 0);
+}
+
+// S(i, j0 .. j0 + SK_COLS - 1): a CTA takes `group` chunks of a row, its warps the nonzeros in turn, two
+// columns a lane. A row of more chunks is summed by several CTAs and added by sketch_rows_kernel (one
+// CTA a row, panel after panel, took 11.4 ms for 888 x 250,000 with a tenth of the nonzeros in one row;
+// now 1.4). GEN: G's entries are generated where they are used, which for rows of a few nonzeros takes
+// less than the panels' launch.
+template <bool GEN, bool SHARED>
 __global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __restrict__ rptr, const int32_t* __restrict__ col,
                                                              const double* __restrict__ val, const int32_t* __restrict__ top,
                                                              const int16_t* __restrict__ P, int n, int l, int j0, int gexp, int r,
                                                              const double* __restrict__ U, const double* __restrict__ VG,
-                                                             int64_t ldvg, double* S, int64_t lds) {
+                                                             int64_t ldvg, double* S, int64_t lds, int dist, uint32_t k0,
+                                                             uint32_t k1, SharedRows a) {
     __shared__ int4 ent[SK_T];                     // upper limb, lower limb, column
     __shared__ unsigned long long sum[2][SK_COLS];
-    const int i = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int64_t b = rptr[i], e = rptr[i + 1];
+    const int i = SHARED ? a.chunk_row[blockIdx.x] : (int)blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int64_t b = rptr[i], e = rptr[i + 1];
     const int tp = max(top[i], -1073), bits = limb_bits(e - b);   // -1073: the smallest value's, or an empty row
+    if (SHARED) {
+        if (((int)blockIdx.x - a.row_chunk[i]) % a.group) return;
+        b = a.chunk_beg[blockIdx.x];
+        e = min(b + (int64_t)a.group * SP_CHUNK, e);
+    }
     if (t < SK_COLS) sum[0][t] = sum[1][t] = 0ull;
     long long h0 = 0, h1 = 0, l0 = 0, l1 = 0;
     int held = 0;
@@ -399,7 +446,7 @@ __global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __re
         __syncthreads();
         if (p0 + t < e) {
             const int2 v = to_limbs(val[p0 + t], tp, bits);
-            ent[t] = make_int4(v.x, v.y, col[p0 + t] + (int)blockIdx.y * n, 0);   // the panel's row
+            ent[t] = make_int4(v.x, v.y, col[p0 + t] + (GEN ? 0 : (int)blockIdx.y * n), 0);   // the panel's row
         } else {
             ent[t] = make_int4(0, 0, 0, 0);
         }
@@ -411,7 +458,9 @@ __global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __re
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 v[u] = ent[(q + u * SK_WARPS) & (SK_T - 1)];
-                N[u] = __ldg(reinterpret_cast<const int*>(P + (int64_t)v[u].z * SK_COLS) + lane);
+                if constexpr (GEN) N[u] = q + u * SK_WARPS < cnt ? omega_pair(v[u].z, j0 + (int)blockIdx.y * SK_COLS + 2 * lane,
+                                                                              l, dist, k0, k1) : 0;
+                else N[u] = __ldg(reinterpret_cast<const int*>(P + (int64_t)v[u].z * SK_COLS) + lane);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -442,11 +491,38 @@ __global__ void __launch_bounds__(SK_T) sparse_sketch_kernel(const int64_t* __re
     atomicAdd(&sum[1][2 * lane + 1], (unsigned long long)l1);
     __syncthreads();
     const int j = j0 + (int)blockIdx.y * SK_COLS + t;
-    if (t < SK_COLS && j < l) {
-        double s = limbs_to_double((long long)sum[0][t], (long long)sum[1][t], tp - bits + gexp);
-        for (int q = 0; q < r; ++q) s = fma(U[(int64_t)i * r + q], VG[(int64_t)q * ldvg + j], s);
-        S[(int64_t)i * lds + j] = s;
+    if (t >= SK_COLS || j >= l) return;
+    if (SHARED) {
+        const int first = a.row_chunk[i];
+        if (a.row_chunk[i + 1] - first > a.group) {
+            const int slot = sketch_slot(a, i, first, ((int)blockIdx.x - first) / a.group);
+            a.part[((int64_t)blockIdx.y * a.slots + slot) * SK_COLS + t] =
+                make_longlong2((long long)sum[0][t], (long long)sum[1][t]);
+            return;
+        }
     }
+    double s = limbs_to_double((long long)sum[0][t], (long long)sum[1][t], tp - bits + gexp);
+    for (int q = 0; q < r; ++q) s = fma(U[(int64_t)i * r + q], VG[(int64_t)q * ldvg + j], s);
+    S[(int64_t)i * lds + j] = s;
+}
+
+// The rows that several CTAs have summed.
+__global__ void __launch_bounds__(SK_COLS) sketch_rows_kernel(const int64_t* __restrict__ rptr, const int32_t* __restrict__ top,
+                                                              int l, int j0, int gexp, int r, const double* __restrict__ U,
+                                                              const double* __restrict__ VG, int64_t ldvg, double* S, int64_t lds,
+                                                              SharedRows a) {
+    const int i = blockIdx.x, j = j0 + (int)blockIdx.y * SK_COLS + (int)threadIdx.x;
+    const int first = a.row_chunk[i], chunks = a.row_chunk[i + 1] - first;
+    if (chunks <= a.group || j >= l) return;
+    const longlong2* p = a.part + ((int64_t)blockIdx.y * a.slots + sketch_slot(a, i, first, 0)) * SK_COLS + threadIdx.x;
+    long long h = 0, lo = 0;                       // h: within 2^62 over the whole row (limb_bits)
+    for (int s = 0; s < (chunks + a.group - 1) / a.group; ++s) {
+        h += p[(int64_t)s * SK_COLS].x;
+        lo += p[(int64_t)s * SK_COLS].y;
+    }
+    double s = limbs_to_double(h, lo, max(top[i], -1073) - limb_bits(rptr[i + 1] - rptr[i]) + gexp);
+    for (int q = 0; q < r; ++q) s = fma(U[(int64_t)i * r + q], VG[(int64_t)q * ldvg + j], s);
+    S[(int64_t)i * lds + j] = s;
 }
 
 // Partial sums of (V G)(q, j0 ..) over chunk blockIdx.x of the rows of G: rows q0 .. q0 + VG_ROWS - 1
@@ -1126,9 +1202,11 @@ rtproj_status sparse_chunks(rtproj_ctx* h, const int64_t* rp_host) {
     const int64_t m = h->m;
     std::vector<int32_t> crow, rch((size_t)m + 1);
     std::vector<int64_t> cbeg;
+    h->longest_row = 0;
     for (int64_t i = 0; i < m; ++i) {
         rch[(size_t)i] = (int32_t)crow.size();
         const int64_t b = rp_host[i], e = rp_host[i + 1];
+        h->longest_row = std::max(h->longest_row, e - b);
         int64_t p = b;
         do {
             crow.push_back((int32_t)i);
@@ -1208,7 +1286,16 @@ rtproj_status sparse_sketch(rtproj_ctx* h, uint64_t seed, int64_t l, double* S, 
     cudaStream_t s = h->stream;
     const int64_t panel = (int64_t)n * SK_COLS * 2, room = panel_bytes(m, n) ? panel : (int64_t)m * n * 8;
     const int total = (int)((l + SK_COLS - 1) / SK_COLS);
-    const int panels = (int)std::max<int64_t>(1, std::min<int64_t>(total, std::min(room, SK_L2_BYTES) / panel));   // a launch
+    const bool gen = r == 0 && h->longest_row <= SK_GEN_ROW && h->nnz * total <= SK_GEN;
+    int panels = gen ? total : (int)std::max<int64_t>(1, std::min<int64_t>(total, std::min(room, SK_L2_BYTES) / panel));   // a launch
+    panels = std::min(panels, 65535);
+    // chunks a CTA: as many as keep the CTAs at some eight an SM, and their partial sums within the scratch
+    SharedRows a = {h->chunk_row, h->chunk_beg, h->row_chunk, 1, 0, reinterpret_cast<longlong2*>(h->part)};
+    const bool shared_rows = h->nchunks > m;
+    const int64_t places = (int64_t)(h->part_elems / (2 * SK_COLS));
+    while (shared_rows && (h->nnz / ((int64_t)a.group * SP_CHUNK) > 8 * sm_count() || h->nchunks / a.group + m + 1 > places)) a.group *= 2;
+    a.slots = h->nchunks / a.group + m + 1;
+    if (shared_rows) panels = (int)std::max<int64_t>(1, std::min<int64_t>(panels, places / a.slots));
     // the chunks of V G: up to four CTAs an SM, their partial sums within the scratch
     const int64_t cap = std::max<int64_t>(1, (int64_t)(h->part_elems / ((size_t)std::max(r, 1) * SK_COLS * 2 * panels)));
     int64_t chunks = std::min<int64_t>(cap, std::min<int64_t>(std::max(1, 4 * sm_count() / panels), ((int64_t)n + VG_KC - 1) / VG_KC));
@@ -1221,7 +1308,10 @@ rtproj_status sparse_sketch(rtproj_ctx* h, uint64_t seed, int64_t l, double* S, 
     for (int p0 = 0; p0 < total; p0 += panels) {
         const int j0 = p0 * SK_COLS;
         const unsigned np = (unsigned)std::min(panels, total - p0);
-        omega_panel_kernel<<<dim3(pgrid, np), SK_T, 0, s>>>(n, (int)l, j0, dist, k0, k1, h->panel);
+        if (!gen) {
+            omega_panel_kernel<<<dim3(pgrid, np), SK_T, 0, s>>>(n, (int)l, j0, dist, k0, k1, h->panel);
+            note_launch();
+        }
         if (r > 0) {   // V G (r x l), this panel's columns
             longlong2* part = reinterpret_cast<longlong2*>(h->part);
             const int groups = (r + 11) / 12, rows = (r + groups - 1) / groups;   // 1 .. 12 rows a CTA
@@ -1237,9 +1327,20 @@ rtproj_status sparse_sketch(rtproj_ctx* h, uint64_t seed, int64_t l, double* S, 
                 part, h->lr_top, (int)chunks, r, (int)l, j0, vbits, gexp, h->lr_a, l);
             note_launch(2);
         }
-        sparse_sketch_kernel<<<dim3((unsigned)m, np), SK_T, 0, s>>>(h->csr_ptr, h->csr_col, h->csr_val, h->row_top, h->panel, n,
-                                                                    (int)l, j0, gexp, r, h->lrU, h->lr_a, l, S, lds);
-        note_launch(2);
+        const dim3 grid((unsigned)h->nchunks, np);
+        auto run = [&](auto kern) {
+            kern<<<grid, SK_T, 0, s>>>(h->csr_ptr, h->csr_col, h->csr_val, h->row_top, h->panel, n, (int)l, j0, gexp, r, h->lrU,
+                                       h->lr_a, l, S, lds, dist, k0, k1, a);
+        };
+        if (gen) run(sparse_sketch_kernel<true, false>);
+        else if (shared_rows) run(sparse_sketch_kernel<false, true>);
+        else run(sparse_sketch_kernel<false, false>);
+        note_launch();
+        if (shared_rows) {
+            sketch_rows_kernel<<<dim3((unsigned)m, np), SK_COLS, 0, s>>>(h->csr_ptr, h->row_top, (int)l, j0, gexp, r, h->lrU,
+                                                                         h->lr_a, l, S, lds, a);
+            note_launch();
+        }
     }
     SP_CHECK(cudaGetLastError());
     return RTPROJ_OK;

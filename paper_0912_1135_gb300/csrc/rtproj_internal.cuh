@@ -467,6 +467,7 @@ struct rtproj_ctx {
     double* lr_b = nullptr;           // r x k_max: V b or U^* h
     double* lr_small = nullptr;       // U^* U, V V^* and partial sums (||A||_F)
     int nchunks = 0;                  // rows cut into chunks of nonzeros for A x
+    int64_t longest_row = 0;          // nonzeros of the longest row
     int32_t* chunk_row = nullptr;     // row of each chunk
     int64_t* chunk_beg = nullptr;     // first nonzero of each chunk
     int32_t* row_chunk = nullptr;     // m + 1: first chunk of each row
